@@ -889,514 +889,6 @@ static distdl_status_t conv_impl(const distdl_partition *p, const void *const *i
 }
 
 // ---------------------------------------------------------------------------------------------
-// Generalized convolution layer: channels partitioned as well (Section 4, "Sparse layers": forward /
-// adjoint convolution algorithms with x on 1 x P_ci x P_0 x P_1, y on 1 x P_co x P_0 x P_1, weights on
-// P_co x P_ci and the work partition 1 x P_co x P_ci x P_0 x P_1).
-//   forward:  x <- H x;  x^ <- B x (to the P_co copies);  y^_{ijs} <- Conv(w_{ij}, b_i on j = 0; x^_{js});
-//             y_{is} <- R over j, in order.
-//   adjoint:  dy^ <- B dy (to the P_ci copies);  dx^_{ijs} <- [dConv]*(dy^_{ijs});  dx_{js} <- R over i, in
-//             order;  dx <- H* dx  (gather form: a correlation of dy with the rotated kernels).
-// With every shard in one memory the broadcasts are implicit and the sum-reduce is the running sum of
-// the block that owns an output tile: it walks through the blocks of the reduced channel partition in
-// worker order and through the channels of a block in channel order, so the order of the sum is fixed.
-// H / H* are fused as in the depthwise kernels (tiles staged with their ghost rows and columns from
-// the neighbouring shards' bulk).  A block owns 32 x 128 pixels of kCob output channels; a thread
-// 4 x 8 pixels of them, as packed pairs of neighbouring pixels.
-// ---------------------------------------------------------------------------------------------
-constexpr int kCob = 2;                 // output channels per block
-constexpr int kMaxChanBlocks = 8;       // P_co, P_ci
-constexpr int kMaxGroups = 128;         // groups of kCob output channels
-
-struct ConvGParams {
-    ConvParams base;                        // in = shards of the input tensor, out = shards of the output tensor
-    const float *w[kMaxChanBlocks * kMaxChanBlocks];   // weight blocks, worker order i * P_ci + j
-    const float *bias[kMaxChanBlocks];      // forward only; per block of output channels, may be null
-    int32_t cnt_out[kMaxChanBlocks], cnt_in[kMaxChanBlocks];   // channels per block of the output / input partition
-    int32_t p_out, p_in, pci;               // blocks of the output / input channel partition; P_ci
-    int32_t groups;                         // groups of up to kCob output channels, all blocks together
-    uint8_t grp_block[kMaxGroups], grp_first[kMaxGroups], grp_count[kMaxGroups];
-    int32_t tiles_y, total_tiles;
-    int32_t ooff;                           // ghost width of the output layout
-};
-
-// One input channel's contribution to the block's kCob x 32 x 128 outputs: per thread 4 x 8 pixels of kCob
-// channels as packed pairs.  wp: K * K * kCob (w, w) pairs of this input channel, [tap][channel].
-template <int K, bool ADJ>
-__device__ __forceinline__ void convg_accumulate(const float *tile, const uint64_t *wp, uint64_t (&acc)[kCob][kRowsPerThread][4]) {
-    using C = ConvCfg<K, ADJ>;
-    constexpr int XO = C::PADL - C::PH;                         // tile column of the first input of output column 0
-    constexpr int NF2 = ((XO + kColsPerThread + K - 1 + 3) / 4) * 4;   // floats of a thread's (aligned) window
-    constexpr int NP = NF2 / 2;
-    static_assert(kTileW - kColsPerThread + NF2 <= C::PITCH, "window beyond the tile row");
-    static_assert(kCob % 2 == 0, "weight pairs are read two channels at a time");
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const float *tbase = tile + (ty * kRowsPerThread) * C::PITCH + kColsPerThread * tx;
-#pragma unroll
-    for (int rho = 0; rho < kRowsPerThread + K - 1; ++rho) {
-        uint64_t Pr[NP], Qr[NP - 1];
-        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(tbase + rho * C::PITCH);
-#pragma unroll
-        for (int v = 0; v < NP / 2; ++v) {
-            const ulonglong2 q = src[v];
-            Pr[2 * v] = q.x;
-            Pr[2 * v + 1] = q.y;
-        }
-#pragma unroll
-        for (int i = 0; i < NP - 1; ++i) {
-            float a0, a1, b0, b1;
-            unpack2(Pr[i], a0, a1);
-            unpack2(Pr[i + 1], b0, b1);
-            Qr[i] = pack2(a1, b0);
-        }
-#pragma unroll
-        for (int r = 0; r < kRowsPerThread; ++r) {
-            const int a = rho - r;
-            if (a < 0 || a >= K) continue;
-#pragma unroll
-            for (int b = 0; b < K; ++b) {
-                // the pairs of all kCob channels of one tap sit side by side: one 16-byte read for two channels
-                uint64_t w2[kCob];
-#pragma unroll
-                for (int o = 0; o < kCob; o += 2) {
-                    const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(wp + (a * K + b) * kCob + o);
-                    w2[o] = q.x;
-                    w2[o + 1] = q.y;
-                }
-                // outputs (2 p2, 2 p2 + 1) read window floats XO + 2 p2 + b, + 1
-                const int j0 = XO + b;
-#pragma unroll
-                for (int p2 = 0; p2 < 4; ++p2) {
-                    const uint64_t X = (j0 & 1) ? Qr[p2 + (j0 - 1) / 2] : Pr[p2 + j0 / 2];
-#pragma unroll
-                    for (int o = 0; o < kCob; ++o) acc[o][r][p2] = fma2(w2[o], X, acc[o][r][p2]);
-                }
-            }
-        }
-    }
-}
-
-// (w, w) pairs of input channel (ib, cl) for the output channels of group (ob, o0, oc); layout [tap][channel]
-template <int K, bool ADJ>
-__device__ __forceinline__ void convg_stage_weights(const ConvGParams &G, int ob, int o0, int oc, int ib, int cl, uint64_t *dst) {
-    if ((int)threadIdx.x < kCob * K * K) {
-        const int tap = threadIdx.x / kCob, o = threadIdx.x - tap * kCob;
-        float w = 0.f;
-        if (o < oc) {
-            const float *blk = ADJ ? G.w[ib * G.pci + ob] : G.w[ob * G.pci + ib];
-            const int s_out = ADJ ? K * K : G.cnt_in[ib] * K * K, s_in = ADJ ? G.cnt_out[ob] * K * K : K * K;
-            w = __ldg(blk + (size_t)(o0 + o) * s_out + (size_t)cl * s_in + (ADJ ? K * K - 1 - tap : tap));   // adjoint: rotated
-        }
-        reinterpret_cast<float2 *>(dst)[threadIdx.x] = make_float2(w, w);
-    }
-}
-
-template <int K, bool ADJ>
-__device__ __forceinline__ void convg_store(const ConvGParams &G, const ConvTile &t, int n, int ob, int o0, int oc,
-                                            const uint64_t (&acc)[kCob][kRowsPerThread][4]) {
-    const ConvParams &P = G.base;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int spatial = P.ph_workers * P.pw_workers;
-    const int oo = G.ooff;
-    const uint32_t pitch_o = (uint32_t)(t.bw + 2 * oo), rows_o = (uint32_t)(t.bh + 2 * oo);
-    const int jo = t.j0 + kColsPerThread * tx;
-#pragma unroll
-    for (int o = 0; o < kCob; ++o) {
-        if (o >= oc) continue;
-        float *oplane = P.out[ob * spatial + t.shard] + ((size_t)n * G.cnt_out[ob] + (size_t)(o0 + o)) * rows_o * pitch_o;
-#pragma unroll
-        for (int r = 0; r < kRowsPerThread; ++r) {
-            const int io = t.i0 + ty * kRowsPerThread + r;
-            if (io >= t.bh || jo >= t.bw) continue;
-            float v[8];
-#pragma unroll
-            for (int p2 = 0; p2 < 4; ++p2) unpack2(acc[o][r][p2], v[2 * p2], v[2 * p2 + 1]);
-            float *dst = oplane + ((size_t)(io + oo) * pitch_o + (size_t)(jo + oo));
-            if (jo + 7 < t.bw && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-                *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-                *reinterpret_cast<float4 *>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (jo + q < t.bw) dst[q] = v[q];
-            }
-        }
-    }
-}
-
-template <int K, bool ADJ>
-__device__ __forceinline__ void convg_init(const ConvGParams &G, int ob, int o0, int oc, uint64_t (&acc)[kCob][kRowsPerThread][4]) {
-#pragma unroll
-    for (int o = 0; o < kCob; ++o) {
-        float b = 0.f;
-        if (!ADJ && G.bias[ob] && o < oc) b = __ldg(G.bias[ob] + o0 + o);
-#pragma unroll
-        for (int r = 0; r < kRowsPerThread; ++r)
-#pragma unroll
-            for (int p2 = 0; p2 < 4; ++p2) acc[o][r][p2] = pack2(b, b);
-    }
-}
-
-// General variant: tiles staged by per-thread asynchronous copies (any row pitch, any number of shards).
-template <int K, bool ADJ>
-__global__ void __launch_bounds__(kConvThreads, 3)
-convg_kernel(const __grid_constant__ ConvGParams G) {
-    using C = ConvCfg<K, ADJ>;
-    extern __shared__ __align__(16) float smem[];               // two x tiles, then two weight tables
-    float *tiles = smem;
-    uint64_t *wtab = reinterpret_cast<uint64_t *>(smem + 2 * C::TILE_FLOATS);   // [2][K * K][kCob] (w, w) pairs
-    const ConvParams &P = G.base;
-    const int spatial = P.ph_workers * P.pw_workers;
-
-    for (int tile = blockIdx.x; tile < G.total_tiles; tile += gridDim.x) {
-        ConvTile t = decode_tile(P, tile, G.tiles_y, 0);
-        if (!t.valid) continue;                                  // the same for every thread of the block
-        const int n = t.plane / G.groups, g = t.plane - n * G.groups;
-        const int ob = G.grp_block[g], o0 = G.grp_first[g], oc = G.grp_count[g];
-        uint64_t acc[kCob][kRowsPerThread][4];
-        convg_init<K, ADJ>(G, ob, o0, oc, acc);
-        // the channels of the reduced partition: block after block, channel after channel
-        auto stage = [&](int ib, int cl, int buf) {
-            ConvTile ti = t;
-            ti.plane = n * G.cnt_in[ib] + cl;
-            stage_tile<K, ADJ>(P, ti, tiles + buf * C::TILE_FLOATS, ib * spatial);
-            convg_stage_weights<K, ADJ>(G, ob, o0, oc, ib, cl, wtab + buf * (kCob * K * K));
-        };
-        int ib = 0, cl = 0, buf = 0;
-        stage(0, 0, 0);
-        cp_async_commit();
-        while (true) {
-            int nib = ib, ncl = cl + 1;
-            if (ncl == G.cnt_in[ib]) {
-                ncl = 0;
-                ++nib;
-            }
-            const bool has_next = nib < G.p_in;
-            if (has_next) stage(nib, ncl, buf ^ 1);
-            cp_async_commit();
-            cp_async_wait_group<1>();
-            __syncthreads();
-            convg_accumulate<K, ADJ>(tiles + buf * C::TILE_FLOATS, wtab + buf * (kCob * K * K), acc);
-            __syncthreads();
-            if (!has_next) break;
-            ib = nib;
-            cl = ncl;
-            buf ^= 1;
-        }
-        cp_async_wait_group<0>();
-        convg_store<K, ADJ>(G, t, n, ob, o0, oc, acc);
-        __syncthreads();
-    }
-}
-
-// TMA variant (at most kConvGTmaShards input shards, rows of whole 16-byte units): the tile body of every
-// input channel arrives by one bulk tensor copy, the halo strips cell by cell into a side buffer.
-constexpr int kConvGTmaShards = 32;
-struct ConvGTmaParams {
-    ConvGParams g;
-    CUtensorMap in_map[kConvGTmaShards];
-};
-
-// Four blocks per SM where the register tile allows it without spills (5 x 5), three otherwise.
-template <int K, bool ADJ>
-__global__ void __launch_bounds__(kConvThreads, K == 5 ? 4 : 3)
-convg_tma_kernel(const __grid_constant__ ConvGTmaParams Q) {
-    using C = ConvCfg<K, ADJ>;
-    using T = ConvTmaCfg<K, ADJ>;
-    extern __shared__ uint8_t smem_raw[];
-    const uint32_t raw = smem_u32(smem_raw);
-    float *tiles = reinterpret_cast<float *>(smem_raw + (((raw + 127u) & ~127u) - raw));
-    float *sides = tiles + 2 * T::TILE_STRIDE;
-    uint64_t *wtab = reinterpret_cast<uint64_t *>(sides + 2 * T::SIDE_STRIDE);          // [2][K * K][kCob]
-    const uint32_t bars = smem_u32(wtab + 2 * kCob * K * K);
-    const ConvGParams &G = Q.g;
-    const ConvParams &P = G.base;
-    const int spatial = P.ph_workers * P.pw_workers;
-    if (threadIdx.x == 0) {
-        mbar_init(bars, 1);
-        mbar_init(bars + 8, 1);
-        fence_barrier_init();
-    }
-    __syncthreads();
-    uint32_t phase0 = 0, phase1 = 0;
-    bool failed = false;
-
-    for (int tile = blockIdx.x; tile < G.total_tiles && !failed; tile += gridDim.x) {
-        ConvTile t = decode_tile(P, tile, G.tiles_y, 0);
-        if (!t.valid) continue;
-        const int n = t.plane / G.groups, g = t.plane - n * G.groups;
-        const int ob = G.grp_block[g], o0 = G.grp_first[g], oc = G.grp_count[g];
-        uint64_t acc[kCob][kRowsPerThread][4];
-        convg_init<K, ADJ>(G, ob, o0, oc, acc);
-        auto stage = [&](int ib, int cl, int buf) {
-            ConvTile ti = t;
-            ti.plane = n * G.cnt_in[ib] + cl;
-            if (threadIdx.x == 0) {
-                fence_proxy_async();
-                mbar_expect_tx(bars + 8 * buf, T::BOX_BYTES);
-                // forward: padded coordinates (bulk column j sits at j + PH); adjoint: bulk coordinates
-                const int x = ADJ ? t.j0 - C::PADL : t.j0;
-                const int y = ADJ ? t.i0 - C::PH : t.i0;
-                tma_load_3d(smem_u32(tiles + buf * T::TILE_STRIDE), &Q.in_map[ib * spatial + t.shard], x, y, ti.plane, bars + 8 * buf);
-            }
-            stage_halo_strips<K, ADJ>(P, ti, sides + buf * T::SIDE_STRIDE, ib * spatial);
-            convg_stage_weights<K, ADJ>(G, ob, o0, oc, ib, cl, wtab + buf * (kCob * K * K));
-        };
-        int ib = 0, cl = 0, buf = 0;
-        stage(0, 0, 0);
-        cp_async_commit();
-        while (true) {
-            int nib = ib, ncl = cl + 1;
-            if (ncl == G.cnt_in[ib]) {
-                ncl = 0;
-                ++nib;
-            }
-            const bool has_next = nib < G.p_in;
-            if (has_next) stage(nib, ncl, buf ^ 1);
-            cp_async_commit();
-            cp_async_wait_group<1>();
-            bool ok = true;
-            {
-                const uint32_t bar = bars + 8 * buf, parity = buf ? phase1 : phase0;
-                if (!mbar_try_wait(bar, parity)) {
-                    const uint64_t t0 = global_timer();
-                    while (!mbar_try_wait(bar, parity)) {
-                        if (global_timer() - t0 > kConvWaitLimitNs) {
-                            ok = false;
-                            break;
-                        }
-                    }
-                }
-                if (buf) phase1 ^= 1; else phase0 ^= 1;
-            }
-            if (__syncthreads_or(!ok)) {
-                if (threadIdx.x == 0) {
-                    atomicExch(&g_conv_status, (int)DISTDL_ERR_TIMEOUT);
-                    const uint64_t t0 = global_timer();
-                    while (global_timer() - t0 < 1000000ull) {}
-                }
-                failed = true;
-                break;
-            }
-            float *tl = tiles + buf * T::TILE_STRIDE;
-            {
-                const float *sd = sides + buf * T::SIDE_STRIDE;
-                for_each_patch_cell<K, ADJ>(t, [&](int q, int ry, int s2) { tl[ry * C::PITCH + s2] = sd[q]; });
-            }
-            __syncthreads();
-            convg_accumulate<K, ADJ>(tl, wtab + buf * (kCob * K * K), acc);
-            __syncthreads();
-            if (!has_next) break;
-            ib = nib;
-            cl = ncl;
-            buf ^= 1;
-        }
-        cp_async_wait_group<0>();
-        if (failed) break;
-        convg_store<K, ADJ>(G, t, n, ob, o0, oc, acc);
-        __syncthreads();
-    }
-}
-
-// Clears the ghost frame of every plane of the padded output shards (what H* leaves behind).
-struct GhostFrameParams {
-    float *shard[kConvMaxWorkers];
-    int32_t planes[kConvMaxWorkers], bh[kConvMaxWorkers], bw[kConvMaxWorkers];
-    int32_t h;
-};
-__global__ void clear_ghost_frame_kernel(const __grid_constant__ GhostFrameParams Q) {
-    const int s = blockIdx.y;
-    const int bh = Q.bh[s], bw = Q.bw[s], h = Q.h;
-    const int pw = bw + 2 * h, ph = bh + 2 * h;
-    const int frame = ph * pw - bh * bw;                  // ghost cells per plane
-    const long long total = (long long)Q.planes[s] * frame;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long long)gridDim.x * blockDim.x) {
-        const int plane = (int)(idx / frame);
-        int e = (int)(idx - (long long)plane * frame), row, col;
-        if (e < h * pw) {                                 // rows above the bulk
-            row = e / pw;
-            col = e - row * pw;
-        } else if (e < 2 * h * pw) {                      // rows below
-            e -= h * pw;
-            row = h + bh + e / pw;
-            col = e % pw;
-        } else {                                          // columns beside the bulk rows
-            e -= 2 * h * pw;
-            row = h + e / (2 * h);
-            const int c = e % (2 * h);
-            col = c < h ? c : bw + c;
-        }
-        Q.shard[s][((size_t)plane * ph + row) * pw + col] = 0.f;
-    }
-}
-
-template <int K, bool ADJ>
-static distdl_status_t launch_convg(const ConvGParams &G, int in_shards, const int64_t *in_planes, cudaStream_t s) {
-    using C = ConvCfg<K, ADJ>;
-    using T = ConvTmaCfg<K, ADJ>;
-    constexpr int smem_plain = 2 * C::TILE_FLOATS * 4 + 2 * kCob * K * K * 8;
-    constexpr int smem_tma = 2 * T::TILE_STRIDE * 4 + 2 * T::SIDE_STRIDE * 4 + 2 * kCob * K * K * 8 + 64 + 128;
-    // one-time set-up per device (kernel attributes, occupancy): a process may drive several GPUs
-    static bool configured_on[kMaxDevicesPerProcess] = {false};
-    int cur_dev = 0;
-    DISTDL_CUDA_CHECK(cudaGetDevice(&cur_dev));
-    if (cur_dev < 0 || cur_dev >= kMaxDevicesPerProcess)
-        return fail(DISTDL_ERR_UNSUPPORTED, "device index %d: at most %d devices per process", cur_dev, kMaxDevicesPerProcess);
-    std::lock_guard<std::mutex> setup_lock(setup_mutex());      // first calls from several threads set up once
-    bool &configured = configured_on[cur_dev];
-    static int blocks_plain_on[kMaxDevicesPerProcess] = {0}, blocks_tma_on[kMaxDevicesPerProcess] = {0};
-    int &blocks_plain = blocks_plain_on[cur_dev], &blocks_tma = blocks_tma_on[cur_dev];
-    if (!configured) {
-        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_kernel<K, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_plain));
-        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_tma_kernel<K, ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_tma));
-        int dev = 0, sms = 0, a = 0, b = 0;
-        DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
-        DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        DISTDL_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, convg_kernel<K, ADJ>, kConvThreads, smem_plain));
-        DISTDL_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, convg_tma_kernel<K, ADJ>, kConvThreads, smem_tma));
-        blocks_plain = sms * std::max(a, 1);
-        blocks_tma = sms * std::max(b, 1);
-        configured = true;
-    }
-    const ConvParams &P = G.base;
-    EncodeTiledFn enc = tensor_map_encoder();
-    bool tma = enc != nullptr && in_shards <= kConvGTmaShards;
-    for (int32_t c = 0; c < P.pw_workers; ++c) tma = tma && ((P.bw[c] + 2 * C::IOFF) % 4) == 0;
-    if (tma) {
-        ConvGTmaParams Q;
-        memset(&Q, 0, sizeof(Q));
-        Q.g = G;
-        const int spatial = P.ph_workers * P.pw_workers;
-        const cuuint32_t estr[3] = {1, 1, 1};
-        for (int k = 0; k < in_shards; ++k) {
-            const int r = (k % spatial) / P.pw_workers, c = k % P.pw_workers;
-            const cuuint64_t pitch = (cuuint64_t)(P.bw[c] + 2 * C::IOFF), rows = (cuuint64_t)(P.bh[r] + 2 * C::IOFF);
-            const cuuint64_t dims[3] = {pitch, rows, (cuuint64_t)in_planes[k / spatial]};
-            const cuuint64_t strides[2] = {pitch * 4, pitch * rows * 4};
-            const cuuint32_t box[3] = {(cuuint32_t)C::PITCH, (cuuint32_t)C::ROWS, 1};
-            if (enc(&Q.in_map[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(P.in[k]), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                return fail(DISTDL_ERR_CUDA, "convg: tensor map of input shard %d failed", k);
-        }
-        const int grid = G.total_tiles < blocks_tma ? G.total_tiles : blocks_tma;
-        convg_tma_kernel<K, ADJ><<<grid, kConvThreads, smem_tma, s>>>(Q);
-    } else {
-        const int grid = G.total_tiles < blocks_plain ? G.total_tiles : blocks_plain;
-        convg_kernel<K, ADJ><<<grid, kConvThreads, smem_plain, s>>>(G);
-    }
-    DISTDL_CUDA_CHECK(cudaGetLastError());
-    return DISTDL_OK;
-}
-
-// px: partition of the tensor with n_ci channels (x, dx); the other tensor (y, dy) has n_co channels on pco
-// blocks and the same spatial partition.  Forward: in = x (padded), out = y (bulk-shaped); adjoint: in = dy
-// (bulk-shaped), out = dx (padded, ghosts cleared).
-static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32_t pco, const void *const *in,
-                                  const void *const *w, const void *const *bias, int32_t kh, int32_t kw,
-                                  void *const *out, void *stream, bool adj, const char *what) {
-    clear_error();
-    if (!px || !in || !w || !out) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
-    if (px->rank != 4 || px->dtype != DISTDL_F32) return fail(DISTDL_ERR_SHAPE, "%s: needs a rank-4 F32 partition", what);
-    if (px->any_periodic()) return fail(DISTDL_ERR_UNSUPPORTED, "%s: periodic partitions are not supported by the fused layers", what);
-    if (px->pshape[0] != 1) return fail(DISTDL_ERR_UNSUPPORTED, "%s: the batch dimension may not be partitioned", what);
-    if (kh != kw || (kh != 3 && kh != 5 && kh != 7))
-        return fail(DISTDL_ERR_UNSUPPORTED, "%s: kernel %d x %d (supported: 3x3, 5x5, 7x7)", what, kh, kw);
-    const int32_t pci = px->pshape[1], ph = px->pshape[2], pw = px->pshape[3];
-    if (pco < 1 || nco < pco) return fail(DISTDL_ERR_SHAPE, "%s: %lld output channels on %d blocks", what, (long long)nco, pco);
-    if (pci > kMaxChanBlocks || pco > kMaxChanBlocks)
-        return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than %d blocks of a channel partition", what, kMaxChanBlocks);
-    if ((int64_t)std::max(pci, pco) * ph * pw > kConvMaxWorkers)
-        return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than %d shards of one tensor", what, kConvMaxWorkers);
-    const int h = kh / 2;
-    for (int k = 0; k < 4; ++k)
-        for (int32_t c = 0; c < px->pshape[k]; ++c) {
-            const int want = k < 2 ? 0 : h;
-            if (px->hlo[k][c] != want || px->hhi[k][c] != want)
-                return fail(DISTDL_ERR_SHAPE, "%s: halo widths must be 0,0,%d,%d on every side", what, h, h);
-        }
-    ConvGParams G;
-    memset(&G, 0, sizeof(G));
-    ConvParams &P = G.base;
-    int64_t max_bh = 0, max_bw = 0;
-    for (int32_t r = 0; r < ph; ++r) max_bh = std::max<int64_t>(max_bh, P.bh[r] = (int32_t)px->size[2][r]);
-    for (int32_t c = 0; c < pw; ++c) max_bw = std::max<int64_t>(max_bw, P.bw[c] = (int32_t)px->size[3][c]);
-    P.ph_workers = ph;
-    P.pw_workers = pw;
-    P.tiles_x = (int32_t)((max_bw + kTileW - 1) / kTileW);
-    G.tiles_y = (int32_t)((max_bh + kTileH - 1) / kTileH);
-    conv_set_divisor(P, 0, (uint32_t)P.tiles_x);
-    conv_set_divisor(P, 1, (uint32_t)pw);
-    conv_set_divisor(P, 2, (uint32_t)G.tiles_y);
-    conv_set_divisor(P, 3, (uint32_t)ph);
-    // channel blocks: the evenly split n_ci (from the partition) and n_co
-    std::vector<int64_t> co_start, co_size;
-    split_evenly(nco, pco, co_start, co_size);
-    const int32_t p_out = adj ? pci : pco, p_in = adj ? pco : pci;
-    for (int32_t b = 0; b < pci; ++b) (adj ? G.cnt_out : G.cnt_in)[b] = (int32_t)px->size[1][b];
-    for (int32_t b = 0; b < pco; ++b) (adj ? G.cnt_in : G.cnt_out)[b] = (int32_t)co_size[b];
-    G.p_out = p_out;
-    G.p_in = p_in;
-    G.pci = pci;
-    int groups = 0;
-    for (int32_t b = 0; b < p_out; ++b)
-        for (int32_t f = 0; f < G.cnt_out[b]; f += kCob) {
-            if (groups == kMaxGroups || f > 255) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many output channels", what);
-            G.grp_block[groups] = (uint8_t)b;
-            G.grp_first[groups] = (uint8_t)f;
-            G.grp_count[groups] = (uint8_t)std::min<int32_t>(kCob, G.cnt_out[b] - f);
-            ++groups;
-        }
-    G.groups = groups;
-    G.ooff = adj ? h : 0;
-    const int64_t total = (int64_t)P.tiles_x * G.tiles_y * ph * pw * px->global_shape[0] * groups;
-    if (total >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
-    G.total_tiles = (int32_t)total;
-    const int spatial = ph * pw;
-    for (int32_t k = 0; k < p_in * spatial; ++k) {
-        if (!in[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: input shard %d is NULL", what, k);
-        if (!aligned16(in[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: input shard %d is not 16-byte aligned", what, k);
-        P.in[k] = (const float *)in[k];
-    }
-    for (int32_t k = 0; k < p_out * spatial; ++k) {
-        if (!out[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: output shard %d is NULL", what, k);
-        if (!aligned16(out[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: output shard %d is not 16-byte aligned", what, k);
-        P.out[k] = (float *)out[k];
-    }
-    for (int32_t k = 0; k < pco * pci; ++k) {
-        if (!w[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: weight block %d is NULL", what, k);
-        G.w[k] = (const float *)w[k];
-    }
-    if (!adj && bias)
-        for (int32_t b = 0; b < pco; ++b) G.bias[b] = (const float *)bias[b];
-    cudaStream_t s = (cudaStream_t)stream;
-    distdl_status_t st;
-    int64_t in_planes[kMaxChanBlocks];
-    for (int32_t b = 0; b < p_in; ++b) in_planes[b] = px->global_shape[0] * G.cnt_in[b];
-    const int ins = p_in * spatial;
-    if (!adj) st = kh == 3 ? launch_convg<3, false>(G, ins, in_planes, s) : kh == 5 ? launch_convg<5, false>(G, ins, in_planes, s)
-                                                                        : launch_convg<7, false>(G, ins, in_planes, s);
-    else st = kh == 3 ? launch_convg<3, true>(G, ins, in_planes, s) : kh == 5 ? launch_convg<5, true>(G, ins, in_planes, s)
-                                                                     : launch_convg<7, true>(G, ins, in_planes, s);
-    if (st != DISTDL_OK || !adj) return st;
-    // adjoint: the ghosts of dx are zero, as H* leaves them
-    GhostFrameParams Q;
-    memset(&Q, 0, sizeof(Q));
-    Q.h = h;
-    for (int32_t b = 0; b < pci; ++b)
-        for (int32_t r = 0; r < ph; ++r)
-            for (int32_t c = 0; c < pw; ++c) {
-                const int k = (b * ph + r) * pw + c;
-                Q.shard[k] = (float *)out[k];
-                Q.planes[k] = (int32_t)(px->global_shape[0] * px->size[1][b]);
-                Q.bh[k] = P.bh[r];
-                Q.bw[k] = P.bw[c];
-            }
-    clear_ghost_frame_kernel<<<dim3(64, (unsigned)(pci * spatial)), 256, 0, s>>>(Q);
-    DISTDL_CUDA_CHECK(cudaGetLastError());
-    return DISTDL_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
 // Parameter gradients of the layer (adjoint convolution algorithm, Section 4 "Sparse layers"):
 //   dw^_k[c,a,b] = sum_{n,i,j} dy_k[n,c,i,j] * (H x)_k[n,c,i+a,j+b],   db^_k[c] = sum dy_k[n,c,i,j],
 //   dw = R_k dw^_k,  db = R_k db^_k      (every worker holds a copy of the kernel).
@@ -2033,16 +1525,6 @@ static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, 
 }
 
 }  // namespace distdl
-
-extern "C" distdl_status_t distdl_convg_fwd(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *x,
-                                            const void *const *w, const void *const *bias, int32_t kh, int32_t kw,
-                                            void *const *y, void *stream) {
-    return distdl::convg_impl(px, nco, pco, x, w, bias, kh, kw, y, stream, false, "convg_fwd");
-}
-extern "C" distdl_status_t distdl_convg_adj(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *dy,
-                                            const void *const *w, int32_t kh, int32_t kw, void *const *dx, void *stream) {
-    return distdl::convg_impl(px, nco, pco, dy, w, nullptr, kh, kw, dx, stream, true, "convg_adj");
-}
 
 extern "C" distdl_status_t distdl_convg_adj_params_workspace(const distdl_partition_t *px, int64_t nco, int32_t pco,
                                                              int32_t kh, int32_t kw, int64_t *bytes) {

@@ -1,0 +1,62 @@
+// Device helpers shared by the convolution kernels: packed fp32 arithmetic, asynchronous copies into shared memory,
+// division by a launch constant.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace distdl {
+
+constexpr int kConvMaxWorkers = 64;
+
+// n / d == umulhi(n, magic) >> shift for any n < 2^31 (magic 0 stands for d = 1): magic = ceil(2^(31+s) / d) with
+// s = ceil(log2 d) is below 2^32 and divides exactly.
+struct FastDiv {
+    uint32_t d, magic, shift;
+};
+inline FastDiv make_fast_div(uint32_t d) {
+    FastDiv f = {d, 0, 0};
+    if (d < 2) return f;
+    uint32_t sh = 0;
+    while ((1u << sh) < d) ++sh;
+    const uint64_t num = (uint64_t)1 << (31 + sh);
+    f.magic = (uint32_t)((num + d - 1) / d);
+    f.shift = sh - 1;
+    return f;
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ uint32_t fast_quot(const FastDiv &f, uint32_t n) {
+    return f.magic ? __umulhi(n, f.magic) >> f.shift : n;
+}
+// n = q * d + r: returns r and leaves q in n
+__device__ __forceinline__ uint32_t fast_rem(const FastDiv &f, uint32_t &n) {
+    const uint32_t q = fast_quot(f, n), r = n - q * f.d;
+    n = q;
+    return r;
+}
+
+// Packed fp32 pair arithmetic (two FMAs per instruction on sm_100).
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ void cp_async4_to(uint32_t smem, const float *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+#endif
+
+}  // namespace distdl

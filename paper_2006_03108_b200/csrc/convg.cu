@@ -1,0 +1,520 @@
+// Generalized convolution layer: channels partitioned as well (Section 4, "Sparse layers": forward /
+// adjoint convolution algorithms with x on 1 x P_ci x P_0 x P_1, y on 1 x P_co x P_0 x P_1, weights on
+// P_co x P_ci and the work partition 1 x P_co x P_ci x P_0 x P_1).
+//   forward:  x <- H x;  x^ <- B x (to the P_co copies);  y^_{ijs} <- Conv(w_{ij}, b_i on j = 0; x^_{js});
+//             y_{is} <- R over j, in order.
+//   adjoint:  dy^ <- B dy (to the P_ci copies);  dx^_{ijs} <- [dConv]*(dy^_{ijs});  dx_{js} <- R over i, in
+//             order;  dx <- H* dx  (gather form: a correlation of dy with the rotated kernels).
+// With every shard in one memory the broadcasts are implicit and the sum-reduce is the running sum of
+// the block that owns an output tile: it walks through the blocks of the reduced channel partition in
+// worker order and through the channels of a block in channel order, so the order of the sum is fixed.
+// H / H* are fused: a tile is staged with its ghost rows and columns straight from the bulk of the
+// neighbouring shards (zeros outside the tensor), and the adjoint writes the zeros that H* leaves in the
+// ghosts of dx together with the tile beside them.
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+#include "common.h"
+#include "conv_common.h"
+
+namespace distdl {
+
+constexpr int kCgThreads = 128;
+constexpr int kCgPx = 8;                // consecutive pixels of a row per thread
+constexpr int kCgMaxPairs = 4;          // output-channel pairs per thread
+constexpr int kMaxChanBlocks = 8;       // P_co, P_ci
+constexpr int kMaxGroups = 128;         // groups of up to 2 * kCgMaxPairs output channels
+
+// Shape of the tiles of one launch.  A tile is tn images x th rows x 8 * seg columns of one shard and one group of
+// output channels; thread -> (image, row, segment of eight columns).
+struct CgShape {
+    int32_t tn, th, seg;
+    int32_t rows, cols, pitch;          // staged rows and columns of one image, floats from row to row
+    int32_t tile_floats;                // one staged channel
+    int32_t entries;                    // staged cells: tn * rows * cols
+    int32_t smem_bytes;
+};
+
+struct ConvGParams {
+    const float *in[kConvMaxWorkers];       // shards of the input tensor, channel block after channel block
+    float *out[kConvMaxWorkers];
+    int32_t bh[kConvMaxWorkers], bw[kConvMaxWorkers];   // bulk rows / columns per worker row / column
+    const float *w[kMaxChanBlocks * kMaxChanBlocks];    // weight blocks, worker order i * P_ci + j
+    const float *bias[kMaxChanBlocks];      // forward only; per block of output channels, may be null
+    int32_t cnt_out[kMaxChanBlocks], cnt_in[kMaxChanBlocks];   // channels per block of the output / input partition
+    int32_t ph, pw, p_in, pci, batch;
+    uint8_t grp_block[kMaxGroups], grp_count[kMaxGroups];
+    uint16_t grp_first[kMaxGroups];
+    CgShape t;
+    FastDiv groups, tiles_x, pw_div, tiles_y, ph_div, cols, rows, tn, seg, half_th;
+};
+
+// What bounds it: the fp32 pipe.  A thread owns eight pixels of a row and up to eight output channels; the accumulators
+// are pairs of channels, so a weight pair is two neighbouring floats of the staged table (one 16-byte broadcast read
+// feeds two pairs) and an input value is duplicated once and used by every tap and channel: 5 x 5, eight channels, 800
+// packed FMAs per input channel and thread beside about 125 other instructions.  With pairs of pixels instead (two
+// channels per thread, as many packed FMAs as now for a quarter of the outputs) every input channel was staged four
+// times as often.
+//
+// Measured (forward / adjoint, B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.14 ms each = 47 TFLOP/s
+// (1.48 / 1.59 ms with two channels a block; packed FMAs alone, as an outer product in registers, reach 59 TFLOP/s);
+// 6 -> 16 channels, 256 images of 28 x 28 on 2 x 2 workers about 0.047 ms each (0.82 / 0.79 ms).
+//
+// Small images are packed: a tile may span several images, so 14 x 14 shards fill the threads (32 x 128 tiles left 95 %
+// of them idle).  Cells are staged one by one (4-byte asynchronous copies), which takes any row pitch and any mixture of
+// neighbours; where each cell comes from is worked out once per tile and kept in a table, a channel then costs one table
+// read, one pointer read and one copy per cell.  Two buffers, one barrier per input channel.
+template <int K, bool ADJ, int CP>
+__global__ void __launch_bounds__(kCgThreads, K == 7 ? 3 : 4)
+convg_kernel(const __grid_constant__ ConvGParams G) {
+    constexpr int PH = K / 2, CT = 2 * CP;
+    constexpr int NF = ((kCgPx + K - 1 + 3) / 4) * 4;      // floats of a thread's window per row
+    constexpr int WF = ((K * K * CT + 3) / 4) * 4;
+    constexpr int io = ADJ ? 0 : PH, oo = ADJ ? PH : 0;    // ghost width of the input / output layout
+    extern __shared__ __align__(16) float smem[];
+    const CgShape &T = G.t;
+    float *tiles = smem;
+    float *wbuf = tiles + 2 * T.tile_floats;
+    uint2 *table = reinterpret_cast<uint2 *>(wbuf + 2 * WF);
+    const float **ptrs = reinterpret_cast<const float **>(table + T.entries);     // [2][9 * tn]
+    const int tid = threadIdx.x;
+
+    uint32_t id = blockIdx.x;
+    const int g = (int)fast_rem(G.groups, id);             // groups fastest: they read the same input tile
+    const int tx = (int)fast_rem(G.tiles_x, id);
+    const int c = (int)fast_rem(G.pw_div, id);
+    const int ty = (int)fast_rem(G.tiles_y, id);
+    const int r = (int)fast_rem(G.ph_div, id);
+    const int n0 = (int)id * T.tn;
+    const int bh = G.bh[r], bw = G.bw[c];
+    const int i0 = ty * T.th, j0 = tx * kCgPx * T.seg;
+    if (i0 >= bh || j0 >= bw) return;                      // shards smaller than the largest
+    const int ob = G.grp_block[g], o0 = G.grp_first[g], oc = G.grp_count[g];
+    const int spatial = G.ph * G.pw;
+
+    // where every staged cell comes from (each thread reads back its own entries only)
+    for (int e = tid; e < T.entries; e += kCgThreads) {
+        uint32_t q = (uint32_t)e;
+        const int s = (int)fast_rem(G.cols, q);
+        const int ry = (int)fast_rem(G.rows, q);
+        const int tn = (int)q;
+        const int dst = (tn * T.rows + ry) * T.pitch + s;
+        int i = i0 - PH + ry, j = j0 - PH + s, dr = 1, dc = 1;
+        bool ok = n0 + tn < G.batch;
+        if (i < 0) {
+            dr = 0;
+            ok = ok && r > 0;
+            if (ok) i += G.bh[r - 1];
+            ok = ok && i >= 0;
+        } else if (i >= bh) {
+            dr = 2;
+            i -= bh;
+            ok = ok && r + 1 < G.ph;
+            if (ok) ok = i < G.bh[r + 1];
+        }
+        int w = bw;
+        if (j < 0) {
+            dc = 0;
+            ok = ok && c > 0;
+            if (ok) w = G.bw[c - 1];
+            j += w;
+            ok = ok && j >= 0;
+        } else if (j >= bw) {
+            dc = 2;
+            j -= bw;
+            ok = ok && c + 1 < G.pw;
+            if (ok) w = G.bw[c + 1];
+            ok = ok && j < w;
+        }
+        if (ok) {
+            table[e] = make_uint2((uint32_t)(i * (w + 2 * io) + j), (uint32_t)dst | ((uint32_t)((3 * dr + dc) * T.tn + tn) << 16));
+        } else {
+            table[e] = make_uint2(0xffffffffu, 0u);
+            tiles[dst] = 0.f;
+            tiles[T.tile_floats + dst] = 0.f;
+        }
+    }
+    if (oc < CT)
+        for (int idx = tid; idx < 2 * WF; idx += kCgThreads) wbuf[idx] = 0.f;
+
+    // first cell (bulk row 0, column 0) of the channel's plane in every neighbour, per image
+    auto set_pointers = [&](int ib, int cl, int b) {
+        for (int t = tid; t < 9 * T.tn; t += kCgThreads) {
+            uint32_t q = (uint32_t)t;
+            const int tn = (int)fast_rem(G.tn, q);
+            const int rr = r + (int)q / 3 - 1, cc = c + (int)q % 3 - 1;
+            const float *p = nullptr;
+            if (rr >= 0 && rr < G.ph && cc >= 0 && cc < G.pw) {
+                const uint32_t pitch = (uint32_t)(G.bw[cc] + 2 * io);
+                p = G.in[ib * spatial + rr * G.pw + cc] +
+                    (size_t)((n0 + tn) * G.cnt_in[ib] + cl) * ((uint32_t)(G.bh[rr] + 2 * io) * pitch) + (io * pitch + io);
+            }
+            ptrs[b * 9 * T.tn + t] = p;
+        }
+    };
+    const uint32_t tiles_s = (uint32_t)__cvta_generic_to_shared(tiles), wbuf_s = (uint32_t)__cvta_generic_to_shared(wbuf);
+    auto stage = [&](int ib, int cl, int b) {
+        const uint32_t dst0 = tiles_s + (uint32_t)(b * T.tile_floats) * 4u;
+        const float *const *pt = ptrs + b * 9 * T.tn;
+        for (int e = tid; e < T.entries; e += kCgThreads) {
+            const uint2 t = table[e];
+            if (t.x != 0xffffffffu) cp_async4_to(dst0 + (t.y & 0xffffu) * 4u, pt[t.y >> 16] + t.x);
+        }
+        const float *blk = ADJ ? G.w[ib * G.pci + ob] : G.w[ob * G.pci + ib];
+        const int s_out = ADJ ? K * K : G.cnt_in[ib] * K * K, s_in = ADJ ? G.cnt_out[ob] * K * K : K * K;
+        const float *wsrc = blk + (size_t)o0 * s_out + (size_t)cl * s_in;
+#pragma unroll
+        for (int k = 0; k < (K * K * CT + kCgThreads - 1) / kCgThreads; ++k) {
+            const int idx = tid + k * kCgThreads;
+            const int tap = idx / CT, o = idx - tap * CT;
+            if (idx < K * K * CT && o < oc)
+                cp_async4_to(wbuf_s + (uint32_t)(b * WF + idx) * 4u, wsrc + (size_t)o * s_out + (ADJ ? K * K - 1 - tap : tap));   // adjoint: rotated
+        }
+    };
+    auto advance = [&](int &ib, int &cl) {
+        if (++cl == G.cnt_in[ib]) {
+            cl = 0;
+            ++ib;
+        }
+    };
+
+    // this thread's item: neighbouring threads take the two rows of a pair, so that (with a row pitch of an odd number of
+    // float4s) the 16-byte reads of eight consecutive lanes fall into eight different bank groups
+    uint32_t rest = (uint32_t)tid >> 1;
+    const int seg = (int)fast_rem(G.seg, rest);
+    const int row = 2 * (int)fast_rem(G.half_th, rest) + (tid & 1);
+    const int img = (int)rest;
+    const bool active = img < T.tn && n0 + img < G.batch && i0 + row < bh && j0 + kCgPx * seg < bw;
+    const int xoff = (img * T.rows + row) * T.pitch + kCgPx * seg;
+
+    uint64_t acc[kCgPx][CP];
+#pragma unroll
+    for (int q = 0; q < CP; ++q) {
+        float b0 = 0.f, b1 = 0.f;
+        if (!ADJ && G.bias[ob]) {
+            if (2 * q < oc) b0 = __ldg(G.bias[ob] + o0 + 2 * q);
+            if (2 * q + 1 < oc) b1 = __ldg(G.bias[ob] + o0 + 2 * q + 1);
+        }
+#pragma unroll
+        for (int p = 0; p < kCgPx; ++p) acc[p][q] = pack2(b0, b1);
+    }
+
+    int sib = 0, scl = 0;                   // channel to stage next
+    int pib = 0, pcl = 0;                   // channel whose pointers are set next
+    set_pointers(pib, pcl, 0);
+    advance(pib, pcl);
+    __syncthreads();
+    stage(sib, scl, 0);
+    advance(sib, scl);
+    cp_async_commit();
+    if (pib < G.p_in) {
+        set_pointers(pib, pcl, 1);
+        advance(pib, pcl);
+    }
+    int buf = 0;
+    bool more = true;
+    while (more) {
+        cp_async_wait_group<0>();
+        __syncthreads();        // this channel has arrived; the other buffer has been read; the next pointers are set
+        more = sib < G.p_in;
+        if (more) {
+            stage(sib, scl, buf ^ 1);
+            advance(sib, scl);
+            cp_async_commit();
+            if (pib < G.p_in) {
+                set_pointers(pib, pcl, buf);
+                advance(pib, pcl);
+            }
+        }
+        if (active) {
+            const float *xb = tiles + buf * T.tile_floats + xoff;
+            const float *wb = wbuf + buf * WF;
+#pragma unroll 1
+            for (int a = 0; a < K; ++a) {
+                float x[NF];
+#pragma unroll
+                for (int v = 0; v < NF / 4; ++v) {
+                    const float4 f = *reinterpret_cast<const float4 *>(xb + 4 * v);
+                    x[4 * v] = f.x;
+                    x[4 * v + 1] = f.y;
+                    x[4 * v + 2] = f.z;
+                    x[4 * v + 3] = f.w;
+                }
+                uint64_t xx[kCgPx + K - 1];
+#pragma unroll
+                for (int v = 0; v < kCgPx + K - 1; ++v) xx[v] = pack2(x[v], x[v]);
+#pragma unroll
+                for (int b = 0; b < K; ++b) {
+                    uint64_t w[CP];
+                    if (CP % 2 == 0) {
+#pragma unroll
+                        for (int q = 0; q < CP; q += 2) {
+                            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(wb + b * CT + 2 * q);
+                            w[q] = v.x;
+                            w[q + 1] = v.y;
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < CP; ++q) w[q] = *reinterpret_cast<const uint64_t *>(wb + b * CT + 2 * q);
+                    }
+#pragma unroll
+                    for (int p = 0; p < kCgPx; ++p)
+#pragma unroll
+                        for (int q = 0; q < CP; ++q) acc[p][q] = fma2(xx[p + b], w[q], acc[p][q]);
+                }
+                xb += T.pitch;
+                wb += K * CT;
+            }
+        }
+        buf ^= 1;
+    }
+
+    // Store: two channels at a time through shared memory, so that a warp writes consecutive cells whatever the row pitch.
+    // The rectangle written is the tile, in the adjoint extended through the ghost layers wherever it touches a face.
+    const int th = min(T.th, bh - i0), tw = min(kCgPx * T.seg, bw - j0), imgs = min(T.tn, G.batch - n0);
+    const int top = ADJ && i0 == 0 ? oo : 0, bottom = ADJ && i0 + th == bh ? oo : 0;
+    const int left = ADJ && j0 == 0 ? oo : 0, right = ADJ && j0 + tw == bw ? oo : 0;
+    const int er = th + top + bottom, ew = tw + left + right;
+    const uint32_t pitch_o = (uint32_t)(bw + 2 * oo), plane_o = (uint32_t)(bh + 2 * oo) * pitch_o;
+    const int chan = G.cnt_out[ob];
+    float *obase = G.out[ob * spatial + r * G.pw + c] + ((size_t)n0 * chan + o0) * plane_o;
+    const int spitch = kCgPx * T.seg;
+    __syncthreads();                        // the tiles and the cell table are free
+    for (int idx = tid; idx < imgs * er; idx += kCgThreads) {
+        const int im = idx / er, y = idx - im * er;
+        const bool ghost = y < top || y >= top + th;
+        table[idx] = make_uint2((uint32_t)im * (uint32_t)chan * plane_o + (uint32_t)(i0 + oo - top + y) * pitch_o + (uint32_t)(j0 + oo - left),
+                                ghost ? 0xffffffffu : (uint32_t)((im * T.th + (y - top)) * spitch));
+    }
+    const int per_ch = T.tn * T.th * spitch;                                    // floats of one channel
+    const int vw = ADJ ? 0 : ((bw & 3) == 0 ? tw / 4 : 0);                      // whole rows of aligned float4s
+    const int cw = vw ? vw : ew;
+    const int step_row = kCgThreads / cw, step_col = kCgThreads - step_row * cw;
+#pragma unroll
+    for (int q = 0; q < CP; ++q) {
+        if (2 * q >= oc) break;
+        if (q > 0) __syncthreads();
+        if (active) {
+            float lo[kCgPx], hi[kCgPx];
+#pragma unroll
+            for (int p = 0; p < kCgPx; ++p) unpack2(acc[p][q], lo[p], hi[p]);
+            float *d = tiles + (img * T.th + row) * spitch + kCgPx * seg;
+            *reinterpret_cast<float4 *>(d) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+            *reinterpret_cast<float4 *>(d + 4) = make_float4(lo[4], lo[5], lo[6], lo[7]);
+            *reinterpret_cast<float4 *>(d + per_ch) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<float4 *>(d + per_ch + 4) = make_float4(hi[4], hi[5], hi[6], hi[7]);
+        }
+        __syncthreads();
+        float *o_lo = obase + (size_t)(2 * q) * plane_o;
+        const bool two = 2 * q + 1 < oc;
+        int y = tid / cw, x = tid - y * cw;
+        while (y < imgs * er) {
+            const uint2 t = table[y];
+            if (vw) {
+                const float *s = tiles + t.y + 4 * x;
+                *reinterpret_cast<float4 *>(o_lo + t.x + 4 * x) = *reinterpret_cast<const float4 *>(s);
+                if (two) *reinterpret_cast<float4 *>(o_lo + plane_o + t.x + 4 * x) = *reinterpret_cast<const float4 *>(s + per_ch);
+            } else {
+                const bool in = t.y != 0xffffffffu && (unsigned)(x - left) < (unsigned)tw;
+                const float *s = tiles + (in ? t.y + (uint32_t)(x - left) : 0u);
+                o_lo[t.x + x] = in ? s[0] : 0.f;
+                if (two) o_lo[plane_o + t.x + x] = in ? s[per_ch] : 0.f;
+            }
+            y += step_row;
+            x += step_col;
+            if (x >= cw) {
+                x -= cw;
+                ++y;
+            }
+        }
+    }
+}
+
+static CgShape cg_shape(int K, int tn, int th, int seg, int cp) {
+    CgShape t;
+    memset(&t, 0, sizeof(t));
+    const int nf = ((kCgPx + K - 1 + 3) / 4) * 4;
+    t.tn = tn;
+    t.th = th;
+    t.seg = seg;
+    t.rows = th + K - 1;
+    t.cols = kCgPx * seg + K - 1;
+    t.pitch = (std::max(t.cols, kCgPx * (seg - 1) + nf) + 3) / 4 * 4;
+    if ((t.pitch / 4) % 2 == 0) t.pitch += 4;
+    t.tile_floats = tn * t.rows * t.pitch;
+    t.entries = tn * t.rows * t.cols;
+    t.smem_bytes = 2 * t.tile_floats * 4 + 2 * ((K * K * 2 * cp + 3) / 4 * 4) * 4 + t.entries * 8 + 2 * 9 * tn * 8;
+    return t;
+}
+
+// Tile shape: the one with the smallest estimated time, tiles per SM times the cost of a tile in thread-cycles: the
+// packed FMAs of 128 threads (2.5 cycles each, as measured for a register outer product) plus the staging of its cells
+// (about eight instructions each).  Shards are cut into equal tiles; up to 56 KB of shared memory keep four blocks on an SM.
+static CgShape cg_choose(int K, int cp, int64_t max_bh, int64_t max_bw, int64_t batch, int64_t workers, int64_t groups, int sms) {
+    CgShape best;
+    memset(&best, 0, sizeof(best));
+    double best_cost = 0;
+    for (int seg = 1; seg <= 16; ++seg) {
+        const int64_t nx = (max_bw + kCgPx * seg - 1) / (kCgPx * seg);
+        if (seg > 1 && (max_bw + kCgPx * (seg - 1) - 1) / (kCgPx * (seg - 1)) == nx) continue;      // narrower tiles do as well
+        for (int th = 2; th * seg <= kCgThreads; th += 2) {
+            const int64_t ny = (max_bh + th - 1) / th;
+            if (th > 2 && (max_bh + th - 3) / (th - 2) == ny) continue;
+            const int room = kCgThreads / (th * seg);
+            for (int tn = 1; tn <= room && tn <= batch; tn = tn < room && tn < batch && 2 * tn > room ? room : 2 * tn) {
+                const int use = (int)std::min<int64_t>(tn, batch);
+                const CgShape t = cg_shape(K, use, th, seg, cp);
+                if (t.smem_bytes > 56 * 1024 || t.tile_floats > 32767) continue;
+                const int64_t tiles = nx * ny * workers * ((batch + use - 1) / use) * groups;
+                const double per_sm = std::max<double>(2.0, (double)((tiles + sms - 1) / sms));
+                const double cost = per_sm * (kCgThreads * (double)(K * K) * kCgPx * cp * 2.5 + 8.0 * t.entries);
+                if (best.tn == 0 || cost < best_cost) {
+                    best = t;
+                    best_cost = cost;
+                }
+            }
+        }
+    }
+    return best;
+}
+
+template <int K, bool ADJ, int CP>
+static distdl_status_t launch_convg(const ConvGParams &G, int64_t blocks, cudaStream_t s) {
+    static bool configured_on[kMaxDevicesPerProcess] = {false};
+    int dev = 0;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevicesPerProcess)
+        return fail(DISTDL_ERR_UNSUPPORTED, "device index %d: at most %d devices per process", dev, kMaxDevicesPerProcess);
+    {
+        std::lock_guard<std::mutex> setup_lock(setup_mutex());
+        if (!configured_on[dev]) {
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_kernel<K, ADJ, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 * 1024));
+            configured_on[dev] = true;
+        }
+    }
+    convg_kernel<K, ADJ, CP><<<(unsigned)blocks, kCgThreads, G.t.smem_bytes, s>>>(G);
+    DISTDL_CUDA_CHECK(cudaGetLastError());
+    return DISTDL_OK;
+}
+
+template <int K, bool ADJ>
+static distdl_status_t launch_convg_pairs(const ConvGParams &G, int cp, int64_t blocks, cudaStream_t s) {
+    switch (cp) {
+        case 1: return launch_convg<K, ADJ, 1>(G, blocks, s);
+        case 2: return launch_convg<K, ADJ, 2>(G, blocks, s);
+        case 3: return launch_convg<K, ADJ, 3>(G, blocks, s);
+        default: return launch_convg<K, ADJ, 4>(G, blocks, s);
+    }
+}
+
+// px: partition of the tensor with n_ci channels (x, dx); the other tensor (y, dy) has n_co channels on pco
+// blocks and the same spatial partition.  Forward: in = x (padded), out = y (bulk-shaped); adjoint: in = dy
+// (bulk-shaped), out = dx (padded, ghosts cleared).
+static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32_t pco, const void *const *in,
+                                  const void *const *w, const void *const *bias, int32_t kh, int32_t kw,
+                                  void *const *out, void *stream, bool adj, const char *what) {
+    clear_error();
+    if (!px || !in || !w || !out) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
+    if (px->rank != 4 || px->dtype != DISTDL_F32) return fail(DISTDL_ERR_SHAPE, "%s: needs a rank-4 F32 partition", what);
+    if (px->any_periodic()) return fail(DISTDL_ERR_UNSUPPORTED, "%s: periodic partitions are not supported by the fused layers", what);
+    if (px->pshape[0] != 1) return fail(DISTDL_ERR_UNSUPPORTED, "%s: the batch dimension may not be partitioned", what);
+    if (kh != kw || (kh != 3 && kh != 5 && kh != 7))
+        return fail(DISTDL_ERR_UNSUPPORTED, "%s: kernel %d x %d (supported: 3x3, 5x5, 7x7)", what, kh, kw);
+    const int32_t pci = px->pshape[1], ph = px->pshape[2], pw = px->pshape[3];
+    if (pco < 1 || nco < pco) return fail(DISTDL_ERR_SHAPE, "%s: %lld output channels on %d blocks", what, (long long)nco, pco);
+    if (pci > kMaxChanBlocks || pco > kMaxChanBlocks)
+        return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than %d blocks of a channel partition", what, kMaxChanBlocks);
+    if ((int64_t)std::max(pci, pco) * ph * pw > kConvMaxWorkers)
+        return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than %d shards of one tensor", what, kConvMaxWorkers);
+    const int h = kh / 2;
+    for (int k = 0; k < 4; ++k)
+        for (int32_t c = 0; c < px->pshape[k]; ++c) {
+            const int want = k < 2 ? 0 : h;
+            if (px->hlo[k][c] != want || px->hhi[k][c] != want)
+                return fail(DISTDL_ERR_SHAPE, "%s: halo widths must be 0,0,%d,%d on every side", what, h, h);
+        }
+    ConvGParams G;
+    memset(&G, 0, sizeof(G));
+    int64_t max_bh = 0, max_bw = 0;
+    for (int32_t r = 0; r < ph; ++r) max_bh = std::max<int64_t>(max_bh, G.bh[r] = (int32_t)px->size[2][r]);
+    for (int32_t c = 0; c < pw; ++c) max_bw = std::max<int64_t>(max_bw, G.bw[c] = (int32_t)px->size[3][c]);
+    G.ph = ph;
+    G.pw = pw;
+    G.batch = (int32_t)px->global_shape[0];
+    // channel blocks: the evenly split n_ci (from the partition) and n_co
+    std::vector<int64_t> co_start, co_size;
+    split_evenly(nco, pco, co_start, co_size);
+    const int32_t p_out = adj ? pci : pco, p_in = adj ? pco : pci;
+    for (int32_t b = 0; b < pci; ++b) (adj ? G.cnt_out : G.cnt_in)[b] = (int32_t)px->size[1][b];
+    for (int32_t b = 0; b < pco; ++b) (adj ? G.cnt_in : G.cnt_out)[b] = (int32_t)co_size[b];
+    G.p_in = p_in;
+    G.pci = pci;
+    // groups: as few as hold every channel of a block at up to eight per thread, of equal size
+    int groups = 0, cp = 1;
+    for (int32_t b = 0; b < p_out; ++b) {
+        const int64_t cnt = G.cnt_out[b], parts = (cnt + 2 * kCgMaxPairs - 1) / (2 * kCgMaxPairs);
+        if (groups + parts > kMaxGroups) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many output channels", what);
+        for (int64_t q = 0, first = 0; q < parts; ++q) {
+            const int64_t size = cnt / parts + (q < cnt % parts ? 1 : 0);
+            G.grp_block[groups] = (uint8_t)b;
+            G.grp_first[groups] = (uint16_t)first;
+            G.grp_count[groups] = (uint8_t)size;
+            cp = std::max(cp, (int)(size + 1) / 2);
+            first += size;
+            ++groups;
+        }
+    }
+    int dev = 0, sms = 148;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    G.t = cg_choose(kh, cp, max_bh, max_bw, G.batch, (int64_t)ph * pw, groups, sms);
+    const int64_t tiles_x = (max_bw + kCgPx * G.t.seg - 1) / (kCgPx * G.t.seg), tiles_y = (max_bh + G.t.th - 1) / G.t.th;
+    const int64_t total = tiles_x * tiles_y * ph * pw * ((G.batch + G.t.tn - 1) / G.t.tn) * groups;
+    if (total >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
+    G.groups = make_fast_div((uint32_t)groups);
+    G.tiles_x = make_fast_div((uint32_t)tiles_x);
+    G.pw_div = make_fast_div((uint32_t)pw);
+    G.tiles_y = make_fast_div((uint32_t)tiles_y);
+    G.ph_div = make_fast_div((uint32_t)ph);
+    G.cols = make_fast_div((uint32_t)G.t.cols);
+    G.rows = make_fast_div((uint32_t)G.t.rows);
+    G.tn = make_fast_div((uint32_t)G.t.tn);
+    G.seg = make_fast_div((uint32_t)G.t.seg);
+    G.half_th = make_fast_div((uint32_t)(G.t.th / 2));
+    const int spatial = ph * pw;
+    for (int32_t k = 0; k < p_in * spatial; ++k) {
+        if (!in[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: input shard %d is NULL", what, k);
+        if (!aligned16(in[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: input shard %d is not 16-byte aligned", what, k);
+        G.in[k] = (const float *)in[k];
+    }
+    for (int32_t k = 0; k < p_out * spatial; ++k) {
+        if (!out[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: output shard %d is NULL", what, k);
+        if (!aligned16(out[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: output shard %d is not 16-byte aligned", what, k);
+        G.out[k] = (float *)out[k];
+    }
+    for (int32_t k = 0; k < pco * pci; ++k) {
+        if (!w[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: weight block %d is NULL", what, k);
+        G.w[k] = (const float *)w[k];
+    }
+    if (!adj && bias)
+        for (int32_t b = 0; b < pco; ++b) G.bias[b] = (const float *)bias[b];
+    cudaStream_t s = (cudaStream_t)stream;
+    if (!adj)
+        return kh == 3 ? launch_convg_pairs<3, false>(G, cp, total, s) : kh == 5 ? launch_convg_pairs<5, false>(G, cp, total, s)
+                                                                                 : launch_convg_pairs<7, false>(G, cp, total, s);
+    return kh == 3 ? launch_convg_pairs<3, true>(G, cp, total, s) : kh == 5 ? launch_convg_pairs<5, true>(G, cp, total, s)
+                                                                            : launch_convg_pairs<7, true>(G, cp, total, s);
+}
+
+}  // namespace distdl
+
+extern "C" distdl_status_t distdl_convg_fwd(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *x,
+                                            const void *const *w, const void *const *bias, int32_t kh, int32_t kw,
+                                            void *const *y, void *stream) {
+    return distdl::convg_impl(px, nco, pco, x, w, bias, kh, kw, y, stream, false, "convg_fwd");
+}
+extern "C" distdl_status_t distdl_convg_adj(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *dy,
+                                            const void *const *w, int32_t kh, int32_t kw, void *const *dx, void *stream) {
+    return distdl::convg_impl(px, nco, pco, dy, w, nullptr, kh, kw, dx, stream, true, "convg_adj");
+}
