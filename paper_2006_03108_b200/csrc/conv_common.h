@@ -51,8 +51,15 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return d;
 }
 
+// x itself, as the result of an instruction: `zero` is a kernel parameter that holds 0.  A pair that is only put together by
+// register moves is put together again at every use when registers are short; the result of an exclusive-or is kept.
+__device__ __forceinline__ float fresh(float x, uint32_t zero) { return __uint_as_float(__float_as_uint(x) ^ zero); }
+
 __device__ __forceinline__ void cp_async4_to(uint32_t smem, const float *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16_to(uint32_t smem, const float *gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>

@@ -57,9 +57,9 @@ struct ConvGParams {
 // channels per thread, as many packed FMAs as now for a quarter of the outputs) every input channel was staged four
 // times as often.
 //
-// Measured (forward / adjoint, B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.14 ms each = 47 TFLOP/s
+// Measured (forward / adjoint, B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.14 / 1.16 ms = 47 TFLOP/s
 // (1.48 / 1.59 ms with two channels a block; packed FMAs alone, as an outer product in registers, reach 59 TFLOP/s);
-// 6 -> 16 channels, 256 images of 28 x 28 on 2 x 2 workers about 0.047 ms each (0.82 / 0.79 ms).
+// 6 -> 16 channels, 256 images of 28 x 28 on 2 x 2 workers 0.044 / 0.050 ms (0.82 / 0.79 ms).
 //
 // Small images are packed: a tile may span several images, so 14 x 14 shards fill the threads (32 x 128 tiles left 95 %
 // of them idle).  Cells are staged one by one (4-byte asynchronous copies), which takes any row pitch and any mixture of
@@ -507,6 +507,500 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
                                                                             : launch_convg_pairs<7, true>(G, cp, total, s);
 }
 
+// ---------------------------------------------------------------------------------------------
+// Parameter gradients (adjoint convolution algorithm):
+//   dw^_{ijs}[o,c,a,b] = sum_{n,i,j} dy_{is}[n,o,i,j] * (H x)_{js}[n,c,i+a,j+b],   db^_{is}[o] = sum dy_{is}[n,o,i,j],
+//   dw_{ij} = R_s dw^_{ijs},  db_i = R_s db^_{is}      (s: feature-space workers).
+// A work item is (group of output channels, group of input channels, slice): the tiles slice, slice + S, ... of all images
+// and workers, so the running sums stay in registers from tile to tile.  At the end of an item the block adds up its
+// splits in order and writes one row of K * K + 1 values per channel pair to the scratch table; a second small kernel adds
+// the rows of a pair in order.  The assignment of tiles to sums is static, so the result does not change from run to run.
+//
+// What bounds it: the fp32 pipe.  A thread owns one input channel c, one kernel row a and all OC output channels of the
+// group, and walks along the rows of the tile four pixels at a time: K * OC sums as pairs (even pixels, odd pixels), one new
+// 16-byte unit of x and OC broadcast units of dy per step, 2 K OC packed FMAs (80 for 5 x 5, eight channels, beside about
+// 20 other instructions).  The (c, a) combinations of a block share the staged dy, the rows of the tile are split over what
+// is left of the threads, and one more combination reads ones instead of x: its sums are db.  Lanes that own pixels
+// instead (all K * K sums of one or two channel pairs per lane) spend as many instructions on putting x pairs together and
+// on folding lanes as on FMAs.
+// Measured (B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.40 ms = 38 TFLOP/s (1.94 ms with one channel
+// pair per block, both its tiles staged again for every pair); 6 -> 16 channels, 256 images of 28 x 28 0.072 ms (1.61 ms).
+// Two steps per turn instead of moving the window: 1.63 ms (spills); 192 threads with 168 registers: 1.67 ms.
+// ---------------------------------------------------------------------------------------------
+constexpr int kGradRow = 64;            // floats per row of the scratch table (K * K + 1 <= 50 used)
+constexpr int kGgThreads = 256;
+constexpr int kGgSmem = 112 * 1024;     // two blocks per SM
+// output channels of a group: more would need more than the 128 registers of two blocks per SM
+constexpr int gg_max_oc(int k) { return k == 7 ? 4 : 8; }
+
+struct GgShape {
+    int32_t tn, th, seg;                // tile: tn images x th rows x 4 * seg columns
+    int32_t rows, units, pitch;         // staged x rows of one image, 16-byte units and floats per row
+    int32_t x_floats;                   // one staged input channel
+    int32_t px;                         // pixels of a tile = floats of one staged dy channel
+    int32_t buf_floats;                 // x of all input channels, then dy: per four pixels the units of all output channels
+    int32_t smem_bytes;
+};
+
+struct ConvGGradParams {
+    const float *x[kConvMaxWorkers], *dy[kConvMaxWorkers];
+    int32_t bh[kConvMaxWorkers], bw[kConvMaxWorkers];
+    int32_t x_start[8], x_cnt[8], y_start[8], y_cnt[8];     // channels of every block
+    int32_t cgrp[9], ogrp[9];           // first group of every block; [blocks]: all groups
+    int32_t x_blocks, y_blocks, ph, pw, batch, n_x;
+    int32_t slices;                     // slices per pair of groups
+    int32_t xc, splits;                 // input channels per block; splits of a tile's rows
+    int32_t tiles;                      // tiles of one channel: workers, images, rows, columns
+    uint32_t zero;                      // 0, see fresh()
+    float *partial;                     // [pairs][slices][kGradRow]
+    GgShape t;
+    FastDiv slice_div, cgrp_div, tiles_x, pw_div, tiles_y, ph_div, units, rows, seg, th;
+};
+
+// Coordinate i of a tile cell along one dimension -> owning worker coordinate (w - 1, w or w + 1) and index in its bulk;
+// false outside the tensor.
+__device__ __forceinline__ bool cg_owner(const int32_t *b, int workers, int w, int i, int &owner, int &index) {
+    owner = w;
+    index = i;
+    if (i < 0) {
+        owner = w - 1;
+        if (owner < 0) return false;
+        index = i + b[owner];
+        return index >= 0;
+    }
+    if (i >= b[w]) {
+        owner = w + 1;
+        if (owner >= workers) return false;
+        index = i - b[w];
+        return index < b[owner];
+    }
+    return true;
+}
+
+template <int K, int OC>
+__global__ void __launch_bounds__(kGgThreads, 2)
+convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
+    constexpr int PH = K / 2;
+    constexpr int NU = (4 + K - 1 + 3) / 4;                 // 16-byte units of x that four pixels of a kernel row need
+    extern __shared__ __align__(16) float smem[];           // two buffers, then a row of ones
+    const GgShape &T = G.t;
+    const int tid = threadIdx.x;
+    const int spatial = G.ph * G.pw;
+
+    uint32_t rest = blockIdx.x;
+    const int sl = (int)fast_rem(G.slice_div, rest);
+    const int cg = (int)fast_rem(G.cgrp_div, rest);
+    const int og = (int)rest;
+    int jb = 0, ib = 0;
+    while (cg >= G.cgrp[jb + 1]) ++jb;
+    while (og >= G.ogrp[ib + 1]) ++ib;
+    // groups of a block: equal sizes, the first ones one channel larger
+    const int cparts = G.cgrp[jb + 1] - G.cgrp[jb], cq = cg - G.cgrp[jb];
+    const int oparts = G.ogrp[ib + 1] - G.ogrp[ib], oq = og - G.ogrp[ib];
+    const int xcnt = G.x_cnt[jb], ycnt = G.y_cnt[ib];
+    const int cbase = xcnt / cparts, crem = xcnt - cbase * cparts, obase = ycnt / oparts, orem = ycnt - obase * oparts;
+    const int xc = cbase + (cq < crem ? 1 : 0), c0 = cq * cbase + min(cq, crem);
+    const int oc = obase + (oq < orem ? 1 : 0), o0 = oq * obase + min(oq, orem);
+
+    const int combos = G.xc * K + 1;
+    const int split = tid / combos, combo = tid - split * combos;
+    const bool is_ones = combo == combos - 1;
+    const int my_c = combo / K, my_a = combo - my_c * K;
+    const bool active = split < G.splits && (is_ones || my_c < xc);
+    const int x_pitch = is_ones ? 0 : T.pitch;
+    const uint32_t zero = G.zero;
+
+    uint64_t acc[OC][K];
+#pragma unroll
+    for (int k = 0; k < OC; ++k)
+#pragma unroll
+        for (int b = 0; b < K; ++b) acc[k][b] = 0ull;
+    for (int i = tid; i < T.pitch; i += kGgThreads) smem[2 * T.buf_floats + i] = 1.f;
+    for (int b = 0; b < 2; ++b)         // output channels that no copy ever writes
+        for (int i = tid; i < OC * T.px; i += kGgThreads)
+            if ((i >> 2) % OC >= oc) smem[b * T.buf_floats + G.xc * T.x_floats + i] = 0.f;
+
+    const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(smem);
+    // Cells are staged in units of four: one 16-byte copy where the unit lies inside one shard and its rows start on
+    // 16-byte boundaries, element by element otherwise.  Where a unit comes from is worked out once for all channels.
+    auto stage = [&](uint32_t L, int buf) {
+        const int tx = (int)fast_rem(G.tiles_x, L);
+        const int c = (int)fast_rem(G.pw_div, L);
+        const int ty = (int)fast_rem(G.tiles_y, L);
+        const int r = (int)fast_rem(G.ph_div, L);
+        const int n0 = (int)L * T.tn;
+        const int bh = G.bh[r], bw = G.bw[c];
+        const int i0 = ty * T.th, j0 = tx * 4 * T.seg;
+        if (i0 >= bh || j0 >= bw) return false;
+        const int th = min(T.th, bh - i0), tw = min(4 * T.seg, bw - j0);
+        const int need_rows = th + K - 1, need_cols = tw + K - 1;
+        const bool x_wide = ((bw + 2 * PH) & 3) == 0, y_wide = (bw & 3) == 0;
+        float *xs = smem + buf * T.buf_floats, *ds = xs + G.xc * T.x_floats;
+        const uint32_t xs_s = smem_s + (uint32_t)(buf * T.buf_floats) * 4u, ds_s = xs_s + (uint32_t)(G.xc * T.x_floats) * 4u;
+        for (int e = tid; e < T.tn * T.rows * T.units; e += kGgThreads) {
+            uint32_t q = (uint32_t)e;
+            const int s = 4 * (int)fast_rem(G.units, q);
+            const int line = (int)q;                        // row of all images
+            const int ry = (int)fast_rem(G.rows, q);
+            const int tn = (int)q;
+            const uint32_t dst = (uint32_t)(line * T.pitch + s);
+            int rr, i;
+            const bool row_ok = cg_owner(G.bh, G.ph, r, i0 - PH + ry, rr, i) && n0 + tn < G.batch && ry < need_rows;
+            const int j = j0 - PH + s;
+            if (row_ok && x_wide && j >= 0 && j + 4 <= bw && s + 4 <= need_cols) {
+                const uint32_t pitch = (uint32_t)(bw + 2 * PH), plane = (uint32_t)(G.bh[rr] + 2 * PH) * pitch;
+                const float *p = G.x[jb * spatial + rr * G.pw + c] + (size_t)((n0 + tn) * xcnt + c0) * plane +
+                                 ((uint32_t)(i + PH) * pitch + (uint32_t)(PH + j));
+                uint32_t d = xs_s + dst * 4u;
+#pragma unroll 1
+                for (int k = 0; k < xc; ++k, p += plane, d += (uint32_t)T.x_floats * 4u) cp_async16_to(d, p);
+            } else {
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    int cc, jj;
+                    // cells that no pixel of the tile reads are zero: they meet the zeros of the dy tile
+                    const bool ok = row_ok && s + f < need_cols && cg_owner(G.bw, G.pw, c, j + f, cc, jj);
+                    if (ok) {
+                        const uint32_t pitch = (uint32_t)(G.bw[cc] + 2 * PH), plane = (uint32_t)(G.bh[rr] + 2 * PH) * pitch;
+                        const float *p = G.x[jb * spatial + rr * G.pw + cc] + (size_t)((n0 + tn) * xcnt + c0) * plane +
+                                         ((uint32_t)(i + PH) * pitch + (uint32_t)(PH + jj));
+                        uint32_t d = xs_s + (dst + (uint32_t)f) * 4u;
+#pragma unroll 1
+                        for (int k = 0; k < xc; ++k, p += plane, d += (uint32_t)T.x_floats * 4u) cp_async4_to(d, p);
+                    } else {
+#pragma unroll 1
+                        for (int k = 0; k < xc; ++k) xs[k * T.x_floats + dst + f] = 0.f;
+                    }
+                }
+            }
+        }
+        const uint32_t plane_y = (uint32_t)bh * (uint32_t)bw;
+        const float *dysh = G.dy[ib * spatial + r * G.pw + c];
+        for (int e = tid; e < T.tn * T.th * T.seg; e += kGgThreads) {
+            uint32_t q = (uint32_t)e;
+            const int col = 4 * (int)fast_rem(G.seg, q);
+            const int row = (int)fast_rem(G.th, q);
+            const int tn = (int)q;
+            const bool row_ok = n0 + tn < G.batch && row < th;
+            const float *p = dysh + (size_t)((n0 + tn) * ycnt + o0) * plane_y + ((uint32_t)(i0 + row) * (uint32_t)bw + (uint32_t)(j0 + col));
+            if (row_ok && y_wide && col + 4 <= tw) {
+                uint32_t d = ds_s + (uint32_t)(e * OC) * 16u;
+#pragma unroll 1
+                for (int k = 0; k < oc; ++k, p += plane_y, d += 16u) cp_async16_to(d, p);
+            } else {
+#pragma unroll
+                for (int f = 0; f < 4; ++f) {
+                    if (row_ok && col + f < tw) {
+                        const float *pf = p + f;
+                        uint32_t d = ds_s + (uint32_t)(4 * e * OC + f) * 4u;
+#pragma unroll 1
+                        for (int k = 0; k < oc; ++k, pf += plane_y, d += 16u) cp_async4_to(d, pf);
+                    } else {
+#pragma unroll 1
+                        for (int k = 0; k < oc; ++k) ds[4 * (e * OC + k) + f] = 0.f;
+                    }
+                }
+            }
+        }
+        return true;
+    };
+
+    int L = sl, buf = 0;
+    bool cur = L < G.tiles && stage((uint32_t)L, 0);
+    cp_async_commit();
+    while (L < G.tiles) {
+        cp_async_wait_group<0>();
+        __syncthreads();                // this tile has arrived, the other buffer has been read
+        const int next = L + G.slices;
+        const bool nxt = next < G.tiles && stage((uint32_t)next, buf ^ 1);
+        cp_async_commit();
+        if (cur && active) {
+            const float *xt = is_ones ? smem + 2 * T.buf_floats : smem + buf * T.buf_floats + my_c * T.x_floats + my_a * T.pitch;
+            const float *dt = smem + buf * T.buf_floats + G.xc * T.x_floats;
+#pragma unroll 1
+            for (int line = split; line < T.tn * T.th; line += G.splits) {
+                const int img = (int)fast_quot(G.th, (uint32_t)line);
+                const float *xp = xt + (line + img * (K - 1)) * x_pitch;        // an image has th + K - 1 staged rows
+                const float *dp = dt + line * (4 * OC * T.seg);
+                uint64_t U[NU][2];
+#pragma unroll
+                for (int v = 0; v + 1 < NU; ++v) {
+                    const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(xp + 4 * v);
+                    U[v][0] = f.x;
+                    U[v][1] = f.y;
+                }
+                xp += 4 * (NU - 1);
+#pragma unroll 1
+                for (int q = 0; q < T.seg; ++q) {
+                    const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(xp);
+                    U[NU - 1][0] = f.x;
+                    U[NU - 1][1] = f.y;
+                    uint64_t Q[2 * NU - 1];                 // U holds (x[2i], x[2i+1]), Q (x[2i+1], x[2i+2])
+#pragma unroll
+                    for (int v = 0; v < 2 * NU - 1; ++v) {
+                        float a0, a1, b0, b1;
+                        unpack2(U[v / 2][v % 2], a0, a1);
+                        unpack2(U[(v + 1) / 2][(v + 1) % 2], b0, b1);
+                        Q[v] = pack2(fresh(a1, zero), fresh(b0, zero));
+                    }
+#pragma unroll
+                    for (int k = 0; k < OC; ++k) {
+                        const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(dp + 4 * k);
+#pragma unroll
+                        for (int b = 0; b < K; ++b) acc[k][b] = fma2((b & 1) ? Q[b / 2] : U[b / 4][b / 2 % 2], d.x, acc[k][b]);
+#pragma unroll
+                        for (int b = 0; b < K; ++b)
+                            acc[k][b] = fma2((b & 1) ? Q[b / 2 + 1] : U[(b / 2 + 1) / 2][(b / 2 + 1) % 2], d.y, acc[k][b]);
+                    }
+                    // the window moves on by one unit (moves: two steps per turn instead need registers that are not there)
+#pragma unroll
+                    for (int v = 0; v + 1 < NU; ++v) {
+                        U[v][0] = U[v + 1][0];
+                        U[v][1] = U[v + 1][1];
+                    }
+                    xp += 4;
+                    dp += 4 * OC;
+                }
+            }
+        }
+        cur = nxt;
+        L = next;
+        buf ^= 1;
+    }
+    // add up: the two halves of a pair, then the splits in order; one row per channel pair
+    __syncthreads();
+    if (active)
+#pragma unroll
+        for (int k = 0; k < OC; ++k)
+#pragma unroll
+            for (int b = 0; b < K; ++b) {
+                float lo, hi;
+                unpack2(acc[k][b], lo, hi);
+                smem[(k * K + b) * (G.splits * combos) + tid] = lo + hi;
+            }
+    __syncthreads();
+    for (int idx = tid; idx < oc * K * combos; idx += kGgThreads) {
+        const int kb = idx / combos, cb = idx - kb * combos;
+        const int k = kb / K, b = kb - k * K;
+        const bool ones = cb == combos - 1;
+        const int ch = ones ? 0 : cb / K;
+        if (ones ? b > 0 : ch >= xc) continue;              // the sums against ones are the same for every b
+        const float *src = smem + kb * (G.splits * combos) + cb;
+        float v = src[0];
+        for (int s = 1; s < G.splits; ++s) v += src[s * combos];
+        const size_t pair = (size_t)(G.y_start[ib] + o0 + k) * G.n_x + (G.x_start[jb] + c0 + ch);
+        G.partial[(pair * G.slices + sl) * kGradRow + (ones ? K * K : (cb - ch * K) * K + b)] = v;
+    }
+}
+
+// One block per channel pair: the rows of its slices added in a fixed order -- thread group h takes rows h, h + H, ..., the
+// groups' sums are added in order -- into tap t of dw block (i, j) at [o_local][c_local]; the last entry of the c = 0
+// pairs goes to db_i[o_local].
+constexpr int kGradFoldGroups = 8;
+struct ConvGGradOut {
+    float *dw[64];
+    float *db[8];
+};
+__global__ void __launch_bounds__(64 * kGradFoldGroups)
+convg_grad_finish_kernel(const __grid_constant__ ConvGGradParams G, const __grid_constant__ ConvGGradOut O, int taps) {
+    __shared__ float part[kGradFoldGroups][64];
+    const int q = blockIdx.x, t = threadIdx.x & 63, h = threadIdx.x >> 6;
+    const int o = q / G.n_x, c = q - o * G.n_x;
+    float v = 0.f;
+    if (t < taps || (t == taps && c == 0)) {
+        const float *row = G.partial + (size_t)q * G.slices * kGradRow + t;
+#pragma unroll 8
+        for (int s = h; s < G.slices; s += kGradFoldGroups) v += row[(size_t)s * kGradRow];
+    }
+    part[h][t] = v;
+    __syncthreads();
+    if (h > 0 || t > taps) return;
+    v = part[0][t];
+#pragma unroll
+    for (int k = 1; k < kGradFoldGroups; ++k) v += part[k][t];
+    int ib = 0, jb = 0;
+    while (ib + 1 < G.y_blocks && o >= G.y_start[ib + 1]) ++ib;
+    while (jb + 1 < G.x_blocks && c >= G.x_start[jb + 1]) ++jb;
+    if (t < taps) O.dw[ib * G.x_blocks + jb][((size_t)(o - G.y_start[ib]) * G.x_cnt[jb] + (c - G.x_start[jb])) * taps + t] = v;
+    else if (O.db[ib] && c == 0) O.db[ib][o - G.y_start[ib]] = v;
+}
+
+static GgShape gg_shape(int K, int tn, int th, int seg, int xc, int oc) {
+    GgShape t;
+    memset(&t, 0, sizeof(t));
+    const int nu = (4 + K - 1 + 3) / 4;
+    t.tn = tn;
+    t.th = th;
+    t.seg = seg;
+    t.rows = th + K - 1;
+    t.units = (4 * seg + K - 1 + 3) / 4;
+    // eight lanes are eight consecutive (channel, kernel row) combinations: an odd number of units per row and, from channel
+    // to channel, K rows' worth of units modulo eight put their 16-byte reads into eight different bank groups
+    int pu = std::max(t.units, seg - 1 + nu);
+    pu += 1 - pu % 2;
+    int xu = tn * t.rows * pu;
+    while ((xu - K * pu) % 8 != 0) ++xu;
+    t.pitch = 4 * pu;
+    t.x_floats = 4 * xu;
+    t.px = tn * th * 4 * seg;
+    t.buf_floats = xc * t.x_floats + oc * t.px;
+    const int fold = oc * K * kGgThreads * 4;               // the sums of all threads, at the end
+    t.smem_bytes = std::max((2 * t.buf_floats + t.pitch) * 4, fold);
+    return t;
+}
+
+// Tile shape with the smallest estimated time of a launch: tiles per block times warp instructions per tile (a packed FMA
+// counts 2.5: the rate of a register outer product), staging 40 per unit and 2 or 12 more per channel.
+static GgShape gg_choose(int K, int xc, int splits, int oc, int64_t max_bh, int64_t max_bw, int64_t batch, int64_t workers, int64_t slots) {
+    GgShape best;
+    memset(&best, 0, sizeof(best));
+    double best_cost = 0;
+    const bool x_wide = (max_bw + K - 1) % 4 == 0, y_wide = max_bw % 4 == 0;
+    for (int seg = 1; seg <= 32; ++seg) {
+        const int64_t nx = (max_bw + 4 * seg - 1) / (4 * seg);
+        if (seg > 1 && (max_bw + 4 * (seg - 1) - 1) / (4 * (seg - 1)) == nx) continue;
+        for (int th = 1; th <= 128; ++th) {
+            const int64_t ny = (max_bh + th - 1) / th;
+            if (th > 1 && (max_bh + th - 2) / (th - 1) == ny) continue;
+            for (int tn = 1; tn <= 64 && tn <= batch; ++tn) {
+                const GgShape t = gg_shape(K, tn, th, seg, xc, oc);
+                if (t.smem_bytes > kGgSmem) break;
+                const int64_t tiles = nx * ny * workers * ((batch + tn - 1) / tn);
+                const int64_t turns = (tiles + slots - 1) / slots;
+                const double compute = 8.0 * ((tn * th + splits - 1) / splits) * (seg * (2.0 * K * oc * 2.5 + oc + 10) + 20);
+                const double staging = (tn * t.rows * t.units * (40.0 + xc * (x_wide ? 2 : 12)) + tn * th * seg * (20.0 + oc * (y_wide ? 2 : 12))) / 32;
+                const double cost = turns * (compute + staging + 1200);
+                if (best.tn == 0 || cost < best_cost) {
+                    best = t;
+                    best_cost = cost;
+                }
+            }
+        }
+    }
+    return best;
+}
+
+// Geometry, groups and slices: shared by the workspace query and the launch.
+static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, int32_t pco, int32_t kh, int32_t kw,
+                                       const char *what, ConvGGradParams *G, int *oc_out, int *grid) {
+    if (!px) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL partition", what);
+    if (px->rank != 4 || px->dtype != DISTDL_F32) return fail(DISTDL_ERR_SHAPE, "%s: needs a rank-4 F32 partition", what);
+    if (px->any_periodic()) return fail(DISTDL_ERR_UNSUPPORTED, "%s: periodic partitions are not supported by the fused layers", what);
+    if (px->pshape[0] != 1) return fail(DISTDL_ERR_UNSUPPORTED, "%s: the batch dimension may not be partitioned", what);
+    if (kh != kw || (kh != 3 && kh != 5 && kh != 7))
+        return fail(DISTDL_ERR_UNSUPPORTED, "%s: kernel %d x %d (supported: 3x3, 5x5, 7x7)", what, kh, kw);
+    const int32_t pci = px->pshape[1], ph = px->pshape[2], pw = px->pshape[3];
+    if (pco < 1 || nco < pco) return fail(DISTDL_ERR_SHAPE, "%s: %lld output channels on %d blocks", what, (long long)nco, pco);
+    if (pci > 8 || pco > 8) return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than 8 blocks of a channel partition", what);
+    if ((int64_t)std::max(pci, pco) * ph * pw > kConvMaxWorkers)
+        return fail(DISTDL_ERR_UNSUPPORTED, "%s: more than %d shards of one tensor", what, kConvMaxWorkers);
+    const int h = kh / 2;
+    for (int k = 0; k < 4; ++k)
+        for (int32_t c = 0; c < px->pshape[k]; ++c) {
+            const int want = k < 2 ? 0 : h;
+            if (px->hlo[k][c] != want || px->hhi[k][c] != want)
+                return fail(DISTDL_ERR_SHAPE, "%s: halo widths must be 0,0,%d,%d on every side", what, h, h);
+        }
+    int64_t max_bh = 0, max_bw = 0;
+    for (int32_t r = 0; r < ph; ++r) max_bh = std::max<int64_t>(max_bh, G->bh[r] = (int32_t)px->size[2][r]);
+    for (int32_t c = 0; c < pw; ++c) max_bw = std::max<int64_t>(max_bw, G->bw[c] = (int32_t)px->size[3][c]);
+    const int64_t pairs = nco * px->global_shape[1];
+    if (pairs > 65536) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles or channel pairs", what);
+    G->ph = ph;
+    G->pw = pw;
+    G->batch = (int32_t)px->global_shape[0];
+    G->n_x = (int32_t)px->global_shape[1];
+    G->x_blocks = pci;
+    G->y_blocks = pco;
+    std::vector<int64_t> co_start, co_size;
+    split_evenly(nco, pco, co_start, co_size);
+    // output channels: as few groups as hold a block, of equal size
+    int max_x = 0, oc = 2;
+    G->cgrp[0] = G->ogrp[0] = 0;
+    for (int32_t b = 0; b < pco; ++b) {
+        G->y_start[b] = (int32_t)co_start[b];
+        const int cnt = G->y_cnt[b] = (int32_t)co_size[b];
+        const int parts = (cnt + gg_max_oc(kh) - 1) / gg_max_oc(kh);
+        oc = std::max(oc, ((cnt + parts - 1) / parts + 1) / 2 * 2);
+        G->ogrp[b + 1] = G->ogrp[b] + parts;
+    }
+    // input channels per block: threads that own no combination against staging dy for every group of them
+    for (int32_t b = 0; b < pci; ++b) max_x = std::max(max_x, (int)px->size[1][b]);
+    int xc = 1;
+    double best = -1;
+    for (int a = 1; a <= 8 && a <= max_x; ++a) {
+        const int g = (max_x + a - 1) / a, splits = kGgThreads / (a * kh + 1);
+        const double cost = g * (8.0 * kh * oc * 1.4 / splits + (1.4 * a + oc) * 0.06);
+        if (best < 0 || cost < best) {
+            best = cost;
+            xc = a;
+        }
+    }
+    for (int32_t b = 0; b < pci; ++b) {
+        G->x_start[b] = (int32_t)px->start[1][b];
+        G->x_cnt[b] = (int32_t)px->size[1][b];
+        G->cgrp[b + 1] = G->cgrp[b] + (G->x_cnt[b] + xc - 1) / xc;
+    }
+    G->xc = xc;
+    G->splits = kGgThreads / (xc * kh + 1);
+    int dev = 0, sms = 148;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // as many slices as fill the resident blocks once; never more than tiles
+    const int64_t group_pairs = (int64_t)G->cgrp[pci] * G->ogrp[pco];
+    const int64_t slots = std::max<int64_t>(1, 2 * (int64_t)sms / group_pairs);
+    G->t = gg_choose(kh, xc, G->splits, oc, max_bh, max_bw, G->batch, (int64_t)ph * pw, slots);
+    const int64_t tiles_x = (max_bw + 4 * G->t.seg - 1) / (4 * G->t.seg), tiles_y = (max_bh + G->t.th - 1) / G->t.th;
+    const int64_t tiles = tiles_x * tiles_y * ph * pw * ((G->batch + G->t.tn - 1) / G->t.tn);
+    if (tiles >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles or channel pairs", what);
+    G->tiles = (int32_t)tiles;
+    const int64_t slices = std::min<int64_t>(slots, tiles);
+    G->slices = (int32_t)slices;
+    G->slice_div = make_fast_div((uint32_t)slices);
+    G->cgrp_div = make_fast_div((uint32_t)G->cgrp[pci]);
+    G->tiles_x = make_fast_div((uint32_t)tiles_x);
+    G->pw_div = make_fast_div((uint32_t)pw);
+    G->tiles_y = make_fast_div((uint32_t)tiles_y);
+    G->ph_div = make_fast_div((uint32_t)ph);
+    G->units = make_fast_div((uint32_t)G->t.units);
+    G->rows = make_fast_div((uint32_t)G->t.rows);
+    G->seg = make_fast_div((uint32_t)G->t.seg);
+    G->th = make_fast_div((uint32_t)G->t.th);
+    *oc_out = oc;
+    *grid = (int)(slices * group_pairs);
+    return DISTDL_OK;
+}
+
+template <int K, int OC>
+static distdl_status_t launch_convg_grad(const ConvGGradParams &G, const ConvGGradOut &O, int grid, int pairs, cudaStream_t s) {
+    static bool configured_on[kMaxDevicesPerProcess] = {false};
+    int dev = 0;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevicesPerProcess)
+        return fail(DISTDL_ERR_UNSUPPORTED, "device index %d: at most %d devices per process", dev, kMaxDevicesPerProcess);
+    {
+        std::lock_guard<std::mutex> setup_lock(setup_mutex());
+        if (!configured_on[dev]) {
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_grad_kernel<K, OC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmem));
+            configured_on[dev] = true;
+        }
+    }
+    convg_grad_kernel<K, OC><<<grid, kGgThreads, G.t.smem_bytes, s>>>(G);
+    DISTDL_CUDA_CHECK(cudaGetLastError());
+    convg_grad_finish_kernel<<<pairs, 64 * kGradFoldGroups, 0, s>>>(G, O, K * K);
+    DISTDL_CUDA_CHECK(cudaGetLastError());
+    return DISTDL_OK;
+}
+
+template <int K>
+static distdl_status_t launch_convg_grad_channels(const ConvGGradParams &G, const ConvGGradOut &O, int oc, int grid, int pairs, cudaStream_t s) {
+    constexpr int most = gg_max_oc(K);
+    if (oc == 2) return launch_convg_grad<K, 2>(G, O, grid, pairs, s);
+    if (oc == 4) return launch_convg_grad<K, 4>(G, O, grid, pairs, s);
+    if (oc == 6) return launch_convg_grad<K, most < 6 ? most : 6>(G, O, grid, pairs, s);
+    return launch_convg_grad<K, most>(G, O, grid, pairs, s);
+}
+
 }  // namespace distdl
 
 extern "C" distdl_status_t distdl_convg_fwd(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *x,
@@ -517,4 +1011,61 @@ extern "C" distdl_status_t distdl_convg_fwd(const distdl_partition_t *px, int64_
 extern "C" distdl_status_t distdl_convg_adj(const distdl_partition_t *px, int64_t nco, int32_t pco, const void *const *dy,
                                             const void *const *w, int32_t kh, int32_t kw, void *const *dx, void *stream) {
     return distdl::convg_impl(px, nco, pco, dy, w, nullptr, kh, kw, dx, stream, true, "convg_adj");
+}
+
+extern "C" distdl_status_t distdl_convg_adj_params_workspace(const distdl_partition_t *px, int64_t nco, int32_t pco,
+                                                             int32_t kh, int32_t kw, int64_t *bytes) {
+    using namespace distdl;
+    clear_error();
+    if (!bytes) return fail(DISTDL_ERR_INVALID_ARG, "convg_adj_params_workspace: NULL argument");
+    ConvGGradParams G;
+    memset(&G, 0, sizeof(G));
+    int oc = 2, grid = 0;
+    const distdl_status_t st = convg_grad_plan(px, nco, pco, kh, kw, "convg_adj_params_workspace", &G, &oc, &grid);
+    if (st != DISTDL_OK) return st;
+    *bytes = nco * G.n_x * G.slices * kGradRow * (int64_t)sizeof(float);
+    return DISTDL_OK;
+}
+
+extern "C" distdl_status_t distdl_convg_adj_params(const distdl_partition_t *px, int64_t nco, int32_t pco,
+                                                   const void *const *x, const void *const *dy, int32_t kh, int32_t kw,
+                                                   void *const *dw, void *const *db, void *workspace,
+                                                   int64_t workspace_bytes, void *stream) {
+    using namespace distdl;
+    clear_error();
+    const char *what = "convg_adj_params";
+    if (!px || !x || !dy || !dw || !workspace) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
+    ConvGGradParams G;
+    memset(&G, 0, sizeof(G));
+    int oc = 2, grid = 0;
+    const distdl_status_t st = convg_grad_plan(px, nco, pco, kh, kw, what, &G, &oc, &grid);
+    if (st != DISTDL_OK) return st;
+    const int64_t need = nco * G.n_x * G.slices * kGradRow * (int64_t)sizeof(float);
+    if (workspace_bytes < need) return fail(DISTDL_ERR_INVALID_ARG, "%s: workspace of %lld bytes, %lld needed", what,
+                                            (long long)workspace_bytes, (long long)need);
+    if (!aligned16(workspace)) return fail(DISTDL_ERR_ALIGNMENT, "%s: workspace not 16-byte aligned", what);
+    for (int32_t k = 0; k < G.x_blocks * G.ph * G.pw; ++k) {
+        if (!x[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: x shard %d is NULL", what, k);
+        if (!aligned16(x[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: x shard %d is not 16-byte aligned", what, k);
+        G.x[k] = (const float *)x[k];
+    }
+    for (int32_t k = 0; k < G.y_blocks * G.ph * G.pw; ++k) {
+        if (!dy[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: dy shard %d is NULL", what, k);
+        if (!aligned16(dy[k])) return fail(DISTDL_ERR_ALIGNMENT, "%s: dy shard %d is not 16-byte aligned", what, k);
+        G.dy[k] = (const float *)dy[k];
+    }
+    ConvGGradOut O;
+    memset(&O, 0, sizeof(O));
+    for (int32_t k = 0; k < G.x_blocks * G.y_blocks; ++k) {
+        if (!dw[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: dw block %d is NULL", what, k);
+        O.dw[k] = (float *)dw[k];
+    }
+    if (db)
+        for (int32_t b = 0; b < G.y_blocks; ++b) O.db[b] = (float *)db[b];
+    G.partial = (float *)workspace;
+    cudaStream_t s = (cudaStream_t)stream;
+    const int pairs = (int)nco * G.n_x;
+    if (kh == 3) return launch_convg_grad_channels<3>(G, O, oc, grid, pairs, s);
+    if (kh == 5) return launch_convg_grad_channels<5>(G, O, oc, grid, pairs, s);
+    return launch_convg_grad_channels<7>(G, O, oc, grid, pairs, s);
 }
