@@ -55,6 +55,26 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 // register moves is put together again at every use when registers are short; the result of an exclusive-or is kept.
 __device__ __forceinline__ float fresh(float x, uint32_t zero) { return __uint_as_float(__float_as_uint(x) ^ zero); }
 
+// Coordinate i of a tile cell along one dimension -> owning worker coordinate (w - 1, w or w + 1) and index in its bulk;
+// false outside the tensor.
+__device__ __forceinline__ bool conv_owner(const int32_t *b, int workers, int w, int i, int &owner, int &index) {
+    owner = w;
+    index = i;
+    if (i < 0) {
+        owner = w - 1;
+        if (owner < 0) return false;
+        index = i + b[owner];
+        return index >= 0;
+    }
+    if (i >= b[w]) {
+        owner = w + 1;
+        if (owner >= workers) return false;
+        index = i - b[w];
+        return index < b[owner];
+    }
+    return true;
+}
+
 __device__ __forceinline__ void cp_async4_to(uint32_t smem, const float *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem), "l"(gmem) : "memory");
 }

@@ -557,26 +557,6 @@ struct ConvGGradParams {
     FastDiv slice_div, cgrp_div, tiles_x, pw_div, tiles_y, ph_div, units, rows, seg, th;
 };
 
-// Coordinate i of a tile cell along one dimension -> owning worker coordinate (w - 1, w or w + 1) and index in its bulk;
-// false outside the tensor.
-__device__ __forceinline__ bool cg_owner(const int32_t *b, int workers, int w, int i, int &owner, int &index) {
-    owner = w;
-    index = i;
-    if (i < 0) {
-        owner = w - 1;
-        if (owner < 0) return false;
-        index = i + b[owner];
-        return index >= 0;
-    }
-    if (i >= b[w]) {
-        owner = w + 1;
-        if (owner >= workers) return false;
-        index = i - b[w];
-        return index < b[owner];
-    }
-    return true;
-}
-
 template <int K, int OC>
 __global__ void __launch_bounds__(kGgThreads, 2)
 convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
@@ -645,7 +625,7 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
             const int tn = (int)q;
             const uint32_t dst = (uint32_t)(line * T.pitch + s);
             int rr, i;
-            const bool row_ok = cg_owner(G.bh, G.ph, r, i0 - PH + ry, rr, i) && n0 + tn < G.batch && ry < need_rows;
+            const bool row_ok = conv_owner(G.bh, G.ph, r, i0 - PH + ry, rr, i) && n0 + tn < G.batch && ry < need_rows;
             const int j = j0 - PH + s;
             if (row_ok && x_wide && j >= 0 && j + 4 <= bw && s + 4 <= need_cols) {
                 const uint32_t pitch = (uint32_t)(bw + 2 * PH), plane = (uint32_t)(G.bh[rr] + 2 * PH) * pitch;
@@ -659,7 +639,7 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
                 for (int f = 0; f < 4; ++f) {
                     int cc, jj;
                     // cells that no pixel of the tile reads are zero: they meet the zeros of the dy tile
-                    const bool ok = row_ok && s + f < need_cols && cg_owner(G.bw, G.pw, c, j + f, cc, jj);
+                    const bool ok = row_ok && s + f < need_cols && conv_owner(G.bw, G.pw, c, j + f, cc, jj);
                     if (ok) {
                         const uint32_t pitch = (uint32_t)(G.bw[cc] + 2 * PH), plane = (uint32_t)(G.bh[rr] + 2 * PH) * pitch;
                         const float *p = G.x[jb * spatial + rr * G.pw + cc] + (size_t)((n0 + tn) * xcnt + c0) * plane +

@@ -24,3 +24,25 @@ CONVG_EDGES = [
 def test_generalized_conv_tiles(case, integer):
     parity.test_generalized_conv_fwd_and_adj(case, integer)
     parity.test_generalized_conv_param_gradients(case, integer)
+
+
+# global NCHW, partition, kernel
+CONV_EDGES = [
+    ((1, 1, 5, 1), (1, 1, 1, 1), 3),         # one column
+    ((1, 2, 3, 3), (1, 1, 1, 1), 7),         # a kernel wider than the image
+    ((1, 2, 9, 66), (1, 1, 1, 1), 7),        # 64-column strips, the last of two columns, narrower than the halo
+    ((1, 1, 40, 129), (1, 1, 1, 1), 7),      # 128-column strips, the last of one column
+    ((2, 1, 23, 131), (1, 1, 1, 1), 5),      # the last row of a shard ends its array off a 16-byte boundary
+    ((1, 2, 50, 516), (1, 1, 1, 3), 5),      # 16-byte rows, strips of 128 and 44 columns
+    ((1, 2, 50, 510), (1, 1, 1, 3), 3),      # padded rows (172) on 16-byte boundaries, bulk rows (170) not
+    ((1, 1, 30, 408), (1, 1, 1, 3), 7),      # the other way round (142 / 136)
+    ((1, 1, 700, 70), (1, 1, 2, 1), 3),      # several row segments per shard
+    ((5, 3, 19, 45), (1, 1, 3, 2), 5),       # shards of 7, 6, 6 rows and 23, 22 columns
+]
+
+
+@pytest.mark.parametrize("case", CONV_EDGES, ids=[str(c) for c in CONV_EDGES])
+def test_depthwise_conv_strips(case):
+    parity.test_conv_fwd_and_adj(case)
+    parity.test_conv_param_gradients(case, True)
+    parity.test_conv_param_gradients(case, False)
