@@ -465,23 +465,6 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
             ++groups;
         }
     }
-    int dev = 0, sms = 148;
-    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
-    DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    G.t = cg_choose(kh, cp, max_bh, max_bw, G.batch, (int64_t)ph * pw, groups, sms);
-    const int64_t tiles_x = (max_bw + kCgPx * G.t.seg - 1) / (kCgPx * G.t.seg), tiles_y = (max_bh + G.t.th - 1) / G.t.th;
-    const int64_t total = tiles_x * tiles_y * ph * pw * ((G.batch + G.t.tn - 1) / G.t.tn) * groups;
-    if (total >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
-    G.groups = make_fast_div((uint32_t)groups);
-    G.tiles_x = make_fast_div((uint32_t)tiles_x);
-    G.pw_div = make_fast_div((uint32_t)pw);
-    G.tiles_y = make_fast_div((uint32_t)tiles_y);
-    G.ph_div = make_fast_div((uint32_t)ph);
-    G.cols = make_fast_div((uint32_t)G.t.cols);
-    G.rows = make_fast_div((uint32_t)G.t.rows);
-    G.tn = make_fast_div((uint32_t)G.t.tn);
-    G.seg = make_fast_div((uint32_t)G.t.seg);
-    G.half_th = make_fast_div((uint32_t)(G.t.th / 2));
     const int spatial = ph * pw;
     for (int32_t k = 0; k < p_in * spatial; ++k) {
         if (!in[k]) return fail(DISTDL_ERR_INVALID_ARG, "%s: input shard %d is NULL", what, k);
@@ -499,6 +482,23 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
     }
     if (!adj && bias)
         for (int32_t b = 0; b < pco; ++b) G.bias[b] = (const float *)bias[b];
+    int dev = 0, sms = 148;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    G.t = cg_choose(kh, cp, max_bh, max_bw, G.batch, (int64_t)ph * pw, groups, sms);
+    const int64_t tiles_x = (max_bw + kCgPx * G.t.seg - 1) / (kCgPx * G.t.seg), tiles_y = (max_bh + G.t.th - 1) / G.t.th;
+    const int64_t total = tiles_x * tiles_y * ph * pw * ((G.batch + G.t.tn - 1) / G.t.tn) * groups;
+    if (total >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
+    G.groups = make_fast_div((uint32_t)groups);
+    G.tiles_x = make_fast_div((uint32_t)tiles_x);
+    G.pw_div = make_fast_div((uint32_t)pw);
+    G.tiles_y = make_fast_div((uint32_t)tiles_y);
+    G.ph_div = make_fast_div((uint32_t)ph);
+    G.cols = make_fast_div((uint32_t)G.t.cols);
+    G.rows = make_fast_div((uint32_t)G.t.rows);
+    G.tn = make_fast_div((uint32_t)G.t.tn);
+    G.seg = make_fast_div((uint32_t)G.t.seg);
+    G.half_th = make_fast_div((uint32_t)(G.t.th / 2));
     cudaStream_t s = (cudaStream_t)stream;
     if (!adj)
         return kh == 3 ? launch_convg_pairs<3, false>(G, cp, total, s) : kh == 5 ? launch_convg_pairs<5, false>(G, cp, total, s)
