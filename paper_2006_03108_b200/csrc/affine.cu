@@ -1131,7 +1131,7 @@ extern "C" distdl_status_t distdl_affine_adj_params(int64_t nb, int64_t nfi, int
 }
 
 namespace distdl {
-int conv_take_status();   // conv.cu
+int conv_take_status();   // convd.cu
 
 // Self-test of the bounded wait: one thread waits, through the same mbar_wait as the kernels above, on a
 // barrier that nobody arrives at.  The wait gives up after `limit_cycles`, records DISTDL_ERR_TIMEOUT in the

@@ -81,6 +81,12 @@ struct HaloTile {
 };
 static_assert(sizeof(HaloTile) == 32, "HaloTile layout");
 
+// Copies and clears of boxes whose rows are long but not made of aligned 16-byte units go row by row: a warp takes a chunk of
+// a row, kRowUnroll elements per lane.
+constexpr int kRowUnroll = 16;
+constexpr int kRowMinUnits = 96;      // shorter rows: unit by unit (a chunk would leave lanes without an element)
+constexpr int kHaloWarps = 8;         // warps of a block
+
 struct HaloPlanHost {
     std::vector<HaloBox> boxes;
     std::vector<HaloSource> sources;

@@ -19,7 +19,7 @@ struct ShardPointers {
     void *p[DISTDL_MAX_WORKERS];
 };
 
-constexpr int kHaloThreads = 256;
+constexpr int kHaloThreads = 32 * kHaloWarps;
 
 // Element and 16-byte vector types of the sums, one addition per element, each the exact sum rounded
 // once to the type (fp32 / fp64 IEEE addition, add.rn.bf16).
@@ -92,6 +92,52 @@ __device__ __forceinline__ uint32_t dot_stride(const uint32_t *coord, const uint
 // Each thread keeps kCopyBatch independent loads in flight.
 // ---------------------------------------------------------------------------------------------
 constexpr int kCopyBatch = 8;
+
+// Long rows of elements: where a row starts is worked out once per chunk (by the whole warp alike) instead of once per
+// element, and a lane has kRowUnroll loads in flight.  What bounds it: device memory.  fp32 6001 x 7003 from eight row blocks to
+// eight column blocks (rows of 7003 cut into pieces of 875 / 876), 336 MB: 112 -> 59 us, back 113 -> 62 us.
+template <typename T>
+__device__ __forceinline__ void run_copy_rows(const HaloBox &box, const HaloSource *src, int nsrc,
+                                              const ShardPointers &sh, uint32_t first, uint32_t count) {
+    const int nd = box.ndim, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t inner = box.shape[nd - 1];
+    const uint32_t row0 = __umulhi(first, box.magic[nd - 1]) >> box.shift[nd - 1], col0 = first - row0 * inner;
+    const uint32_t last = first + count - 1;
+    const uint32_t row1 = __umulhi(last, box.magic[nd - 1]) >> box.shift[nd - 1], col1 = last - row1 * inner + 1;
+    const uint32_t chunks = (inner + 32 * kRowUnroll - 1) / (32 * kRowUnroll);
+    const uint32_t width = ((inner + chunks - 1) / chunks + 31) / 32 * 32;
+    T *dst = reinterpret_cast<T *>(sh.p[box.dst_shard]) + box.dst_offset;
+    const T *s0 = nsrc ? reinterpret_cast<const T *>(sh.p[src[0].shard]) + src[0].offset : nullptr;
+    const uint32_t total = (row1 - row0 + 1) * chunks;
+    for (uint32_t q = warp; q < total; q += kHaloWarps) {
+        const uint32_t r = q / chunks, c = (q - r * chunks) * width, row = row0 + r;
+        uint32_t n = row, doff = 0, soff = 0;
+#pragma unroll
+        for (int k = kMaxBoxDims - 2; k >= 0; --k) {
+            if (k < nd - 1) {
+                uint32_t coord = n;
+                if (k > 0) {
+                    n = __umulhi(coord, box.magic[k]) >> box.shift[k];
+                    coord -= n * box.shape[k];
+                }
+                doff += coord * box.dst_stride[k];
+                if (nsrc) soff += coord * src[0].stride[k];
+            }
+        }
+        const uint32_t lo = row == row0 ? col0 : 0u, hi = min(row == row1 ? col1 : inner, c + width);
+        T v[kRowUnroll];
+#pragma unroll
+        for (int u = 0; u < kRowUnroll; ++u) {
+            const uint32_t i = c + lane + 32u * u;
+            v[u] = nsrc && i >= lo && i < hi ? s0[soff + i] : zero_of<T>();
+        }
+#pragma unroll
+        for (int u = 0; u < kRowUnroll; ++u) {
+            const uint32_t i = c + lane + 32u * u;
+            if (i >= lo && i < hi) dst[doff + i] = v[u];
+        }
+    }
+}
 
 template <typename T>
 __device__ __forceinline__ void run_copy_tile(const HaloBox &box, const HaloSource *src, int nsrc,
@@ -268,8 +314,14 @@ halo_box_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict_
     }
     __syncthreads();
     if (!SUMS || nsrc <= 1) {
-        if (s_box.vec) run_copy_tile<uint4>(s_box, s_src, nsrc, sh, first, count);
-        else if (elem_bytes == 4) run_copy_tile<float>(s_box, s_src, nsrc, sh, first, count);
+        const int in = s_box.ndim - 1;
+        if (s_box.vec) {
+            run_copy_tile<uint4>(s_box, s_src, nsrc, sh, first, count);
+        } else if (s_box.shape[in] >= (uint32_t)kRowMinUnits && s_box.dst_stride[in] == 1 && (nsrc == 0 || s_src[0].stride[in] == 1)) {
+            if (elem_bytes == 4) run_copy_rows<float>(s_box, s_src, nsrc, sh, first, count);
+            else if (elem_bytes == 8) run_copy_rows<unsigned long long>(s_box, s_src, nsrc, sh, first, count);
+            else run_copy_rows<unsigned short>(s_box, s_src, nsrc, sh, first, count);
+        } else if (elem_bytes == 4) run_copy_tile<float>(s_box, s_src, nsrc, sh, first, count);
         else if (elem_bytes == 8) run_copy_tile<unsigned long long>(s_box, s_src, nsrc, sh, first, count);
         else run_copy_tile<unsigned short>(s_box, s_src, nsrc, sh, first, count);
     } else if (elem_bytes == 4) {

@@ -257,14 +257,23 @@ struct Builder {
         }
         const int32_t box_id = (int32_t)plan->boxes.size();
         plan->boxes.push_back(b);
-        for (int64_t at = 0; at < units; at += kTileUnits) {
+        // rows copied chunk by chunk: tiles of whole rows, as many as give every warp of a block the same number of chunks
+        int64_t tile_units = kTileUnits;
+        const int64_t inner = shape[nd_units - 1];
+        if (srcs.size() <= 1 && !vec && inner >= kRowMinUnits && inner <= kTileUnits && units > 4 * (int64_t)kTileUnits) {
+            const int64_t chunks = (inner + 32 * kRowUnroll - 1) / (32 * kRowUnroll);
+            int64_t step = kHaloWarps;
+            for (int64_t c = chunks; step > 1 && c % 2 == 0; c /= 2) step /= 2;
+            tile_units = inner * ((10240 / inner + step - 1) / step * step);
+        }
+        for (int64_t at = 0; at < units; at += tile_units) {
             HaloTile t;
             memset(&t, 0, sizeof(t));
             t.box = box_id;
             t.src_begin = src_begin;
             t.nsrc = (int32_t)srcs.size();
             t.first = (uint32_t)at;
-            t.count = (uint32_t)std::min<int64_t>(kTileUnits, units - at);
+            t.count = (uint32_t)std::min<int64_t>(tile_units, units - at);
             plan->tiles.push_back(t);
         }
         // algorithmic traffic: destination written once; every source read once; cleared sources

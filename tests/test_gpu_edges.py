@@ -46,3 +46,29 @@ def test_depthwise_conv_strips(case):
     parity.test_conv_fwd_and_adj(case)
     parity.test_conv_param_gradients(case, True)
     parity.test_conv_param_gradients(case, False)
+
+
+# Rows copied chunk by chunk: at least 96 elements, chunks of up to 512, tiles of whole rows
+REPART_EDGES = [
+    ((61, 1203), (4, 1), (1, 3)),            # pieces of 401
+    ((7, 95 * 3 + 1), (7, 1), (1, 3)),       # pieces of 96 and 95: one each side of the rule
+    ((300, 1537), (2, 1), (1, 3)),           # pieces of 513 and 512: two chunks and one; several tiles per box
+    ((3, 30001), (3, 1), (1, 2)),            # pieces longer than a tile
+]
+HALO_EDGES = [
+    ((40, 403), (2, 2), 1, 1),               # ghost rows of 201 / 202 cells
+    ((9, 10, 311), (2, 2, 1), (1, 2, 1), (2, 1, 1)),
+    ((5, 40001), (2, 1), (1, 0), (1, 0)),
+]
+
+
+@pytest.mark.parametrize("case", REPART_EDGES, ids=[str(c) for c in REPART_EDGES])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_repartition_rows(case, dtype):
+    parity.test_repartition_fwd_and_adj_bit_exact(case, dtype)
+
+
+@pytest.mark.parametrize("case", HALO_EDGES, ids=[str(c) for c in HALO_EDGES])
+def test_halo_long_rows(case):
+    parity.test_halo_fwd_and_adj_bit_exact(case)
+    parity.test_halo_fwd_and_adj_bf16_fp64_bit_exact(case)
