@@ -5,7 +5,7 @@
 //
 // All workers live in one device memory, so the broadcast is implicit (every thread block that
 // needs a block of x reads it through L2 -- no copy is materialised) and the sum-reduce is the
-// tensor-core accumulator itself: one thread block owns a 128 x 128 tile of the output and walks
+// tensor-core accumulator itself: a cluster of thread blocks owns a tile of the output and walks
 // through the workers of its grid row (forward) or grid column (adjoint) in worker order, so the
 // partial products y^_{ij} never exist in memory and the order of the sum is fixed.
 //
@@ -141,32 +141,29 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t adesc, 
 }
 
 // ------------------------------------------------------------------------------------------
-// Kernel.  PAIR = false: one thread block owns a 128 x 128 output tile (used when the batch fits
-// one 128-row tile).  PAIR = true: a cluster of two blocks owns a 256 x 128 tile; each block stages
-// its own 128 activation rows and its own half of the weight tile, one tcgen05.mma.cta_group::2
-// issued by the leader drives the tensor cores of both SMs and reads the weight halves from both
-// shared memories -- a quarter less shared-memory fill per flop, which buys a deeper ring.  The
-// leader's "full" barrier counts the bytes of both blocks' bulk copies; "empty" and "accumulator
-// ready" are signalled in both blocks at once by a multicast commit.
+// Pair variant: a cluster of two blocks owns a 256 x 128 output tile; each block stages its own 128
+// activation rows and its own half of the weight tile, one tcgen05.mma.cta_group::2 issued by the
+// leader drives the tensor cores of both SMs and reads the weight halves from both shared memories --
+// a quarter less shared-memory fill per flop, which buys a deeper ring.  The leader's "full" barrier
+// counts the bytes of both blocks' bulk copies; "empty" and "accumulator ready" are signalled in both
+// blocks at once by a multicast commit.
 //
 // The producer and the MMA issuer are single threads, so their loops are kept to a few dozen
 // instructions per k-block: counters advance incrementally (no divisions) and the shared-memory
 // descriptors are a precomputed base plus an offset.
 // Tiles are numbered row tile fastest, so blocks that share a weight tile run together.
 // ------------------------------------------------------------------------------------------
-template <bool PAIR>
-struct AffineCfg {
-    static constexpr int STAGES = PAIR ? 9 : 6;
+struct AffinePairCfg {
+    static constexpr int STAGES = 9;
     static constexpr int A_BYTES = kTileM * kBlockK * 2;                       // 16 KB
-    static constexpr int B_BYTES = (PAIR ? kTileN / 2 : kTileN) * kBlockK * 2; // 8 or 16 KB
+    static constexpr int B_BYTES = kTileN / 2 * kBlockK * 2;                   // 8 KB
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment*/ + 256 /*barriers*/;
 };
 
-template <bool PAIR>
 __global__ void __launch_bounds__(kAffineThreads, 1)
-affine_kernel(const __grid_constant__ AffineParams P) {
-    using C = AffineCfg<PAIR>;
+affine_kernel_pair(const __grid_constant__ AffineParams P) {
+    using C = AffinePairCfg;
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte alignment: the 128-byte swizzle pattern is a function of address bits [7,10)
     const uint32_t raw = smem_u32(smem_raw);
@@ -180,9 +177,9 @@ affine_kernel(const __grid_constant__ AffineParams P) {
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = PAIR ? cluster_ctarank() : 0;         // 0 = leader of the pair
-    const int rows_per_tile = PAIR ? 2 * kTileM : kTileM;
-    const int tile = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const uint32_t rank = cluster_ctarank();                    // 0 = leader of the pair
+    const int rows_per_tile = 2 * kTileM;
+    const int tile = (int)(blockIdx.x >> 1);
     const int row_tiles = (P.nb + rows_per_tile - 1) / rows_per_tile;
     const int m0 = (tile % row_tiles) * rows_per_tile + (int)rank * kTileM;   // this block's first row
     const int ntile = tile / row_tiles;
@@ -204,19 +201,12 @@ affine_kernel(const __grid_constant__ AffineParams P) {
     }
     if (warp == 1) {
         // 128 columns of tensor memory: one fp32 accumulator of 128 lanes x 128 columns per block
-        if (PAIR) {
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
-                         ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)kTileN) : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                         ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)kTileN) : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"((uint32_t)kTileN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tcgen05_fence_before();
-    if (PAIR) cluster_sync_all();    // both blocks' barriers exist before anyone signals them
-    else __syncthreads();
+    cluster_sync_all();              // both blocks' barriers exist before anyone signals them
     tcgen05_fence_after();
     const uint32_t tmem_acc = *tmem_slot;
 
@@ -227,28 +217,17 @@ affine_kernel(const __grid_constant__ AffineParams P) {
             // forward: W_{oblk, r}, next worker = next map; adjoint: W_{r, oblk}, next worker = next grid row
             const CUtensorMap *wmap = P.adjoint ? &P.w_map[oblk] : &P.w_map[oblk * P.pfi];
             const int wstep = P.adjoint ? P.pfi : 1;
-            const int nb0 = n0 + (PAIR ? (int)rank * (kTileN / 2) : 0);   // this block's part of the weight tile
+            const int nb0 = n0 + (int)rank * (kTileN / 2);   // this block's part of the weight tile
             uint32_t s = 0, phase = 0, sa = base;
             int k0 = 0, kin = 0;
             for (int kb = 0; kb < num_kblocks; ++kb) {
                 if (!mbar_wait(bar_empty + 8 * s, phase ^ 1, abort_flag)) break;
                 const uint32_t full = bar_full + 8 * s;
-                if (PAIR) {
-                    const uint32_t full_leader = map_to_cta(full, 0);
-                    if (rank == 0) mbar_expect_tx(full, 2 * C::STAGE_BYTES);      // both blocks' bytes
-                    tma_load_2d_pair(sa, amap, k0, m0, full_leader);
-                    if (!P.adjoint) tma_load_2d_pair(sa + C::A_BYTES, wmap, k0, nb0, full_leader);   // box {64 k, 64 rows}
-                    else tma_load_2d_pair(sa + C::A_BYTES, wmap, nb0, k0, full_leader);              // box {64 n, 64 k}
-                } else {
-                    mbar_expect_tx(full, C::STAGE_BYTES);
-                    tma_load_2d(sa, amap, k0, m0, full);                        // box {64 k, 128 rows}
-                    if (!P.adjoint) {
-                        tma_load_2d(sa + C::A_BYTES, wmap, k0, nb0, full);      // K-major: box {64 k, 128 rows}
-                    } else {                                                    // MN-major: two boxes {64 n, 64 k}
-                        tma_load_2d(sa + C::A_BYTES, wmap, nb0, k0, full);
-                        tma_load_2d(sa + C::A_BYTES + C::B_BYTES / 2, wmap, nb0 + 64, k0, full);
-                    }
-                }
+                const uint32_t full_leader = map_to_cta(full, 0);
+                if (rank == 0) mbar_expect_tx(full, 2 * C::STAGE_BYTES);          // both blocks' bytes
+                tma_load_2d_pair(sa, amap, k0, m0, full_leader);
+                if (!P.adjoint) tma_load_2d_pair(sa + C::A_BYTES, wmap, k0, nb0, full_leader);       // box {64 k, 64 rows}
+                else tma_load_2d_pair(sa + C::A_BYTES, wmap, nb0, k0, full_leader);                  // box {64 n, 64 k}
                 k0 += kBlockK;
                 if (++kin == kblocks_per_worker) {      // next worker of the grid row / column, in order
                     kin = 0;
@@ -272,13 +251,13 @@ affine_kernel(const __grid_constant__ AffineParams P) {
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0 && rank == 0) {
-            const uint32_t idesc = instr_desc(PAIR ? 2 * kTileM : kTileM, kTileN, P.adjoint ? 1 : 0);
+            const uint32_t idesc = instr_desc(2 * kTileM, kTileN, P.adjoint ? 1 : 0);
             // A, K-major: 8-row groups 1024 bytes apart; a K step of 16 elements is 32 bytes.
-            // B forward, K-major: the same.  B adjoint, MN-major: 64-column atoms B_BYTES/2 apart
-            // (leading offset; one atom per block in the pair variant), 8-k groups 1024 bytes apart; a
+            // B forward, K-major: the same.  B adjoint, MN-major: one 64-column atom per
+            // block, 8-k groups 1024 bytes apart; a
             // K step of 16 rows is 2048 bytes.  Descriptor addresses are in 16-byte units.
             const uint64_t a0 = smem_desc(base, 16, 1024);
-            const uint64_t b0 = P.adjoint ? smem_desc(base + C::A_BYTES, PAIR ? C::B_BYTES : C::B_BYTES / 2, 1024)
+            const uint64_t b0 = P.adjoint ? smem_desc(base + C::A_BYTES, C::B_BYTES, 1024)
                                           : smem_desc(base + C::A_BYTES, 16, 1024);
             const uint64_t bstep = P.adjoint ? (2048 >> 4) : (32 >> 4);
             uint32_t s = 0, phase = 0;
@@ -289,19 +268,11 @@ affine_kernel(const __grid_constant__ AffineParams P) {
                 if (!ok) break;
                 tcgen05_fence_after();
                 const uint64_t a = a0 + off, b = b0 + off;
-                if (PAIR) {
-                    umma_bf16_pair(tmem_acc, a, b, idesc, kb ? 1u : 0u);
-                    umma_bf16_pair(tmem_acc, a + 2, b + bstep, idesc, 1u);
-                    umma_bf16_pair(tmem_acc, a + 4, b + 2 * bstep, idesc, 1u);
-                    umma_bf16_pair(tmem_acc, a + 6, b + 3 * bstep, idesc, 1u);
-                    tcgen05_commit_pair(bar_empty + 8 * s);     // frees the stage in both blocks
-                } else {
-                    umma_bf16(tmem_acc, a, b, idesc, kb ? 1u : 0u);
-                    umma_bf16(tmem_acc, a + 2, b + bstep, idesc, 1u);
-                    umma_bf16(tmem_acc, a + 4, b + 2 * bstep, idesc, 1u);
-                    umma_bf16(tmem_acc, a + 6, b + 3 * bstep, idesc, 1u);
-                    tcgen05_commit(bar_empty + 8 * s);          // frees the stage once these MMAs retire
-                }
+                umma_bf16_pair(tmem_acc, a, b, idesc, kb ? 1u : 0u);
+                umma_bf16_pair(tmem_acc, a + 2, b + bstep, idesc, 1u);
+                umma_bf16_pair(tmem_acc, a + 4, b + 2 * bstep, idesc, 1u);
+                umma_bf16_pair(tmem_acc, a + 6, b + 3 * bstep, idesc, 1u);
+                tcgen05_commit_pair(bar_empty + 8 * s);         // frees the stage in both blocks
                 off += C::STAGE_BYTES >> 4;
                 if (++s == C::STAGES) {
                     s = 0;
@@ -309,10 +280,7 @@ affine_kernel(const __grid_constant__ AffineParams P) {
                     phase ^= 1;
                 }
             }
-            if (ok) {                                           // accumulator complete
-                if (PAIR) tcgen05_commit_pair(bar_acc);
-                else tcgen05_commit(bar_acc);
-            }
+            if (ok) tcgen05_commit_pair(bar_acc);               // accumulator complete
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps
@@ -360,14 +328,205 @@ affine_kernel(const __grid_constant__ AffineParams P) {
     // a block may not retire, or free its tensor memory, while its peer can still read its shared
     // memory or signal its barriers
     tcgen05_fence_before();
-    if (PAIR) cluster_sync_all();
-    else __syncthreads();
+    cluster_sync_all();
     if (warp == 1) {
         tcgen05_fence_after();
-        if (PAIR)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"((uint32_t)kTileN) : "memory");
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"((uint32_t)kTileN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"((uint32_t)kTileN) : "memory");
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// Few samples (a batch of at most 128): the weights are the M operand.  A cluster of S blocks owns 128
+// output features of the whole batch, every block contracts over its share of the k-blocks (shares in
+// worker order), and the partial sums are added in rank order through distributed shared memory, each
+// block finishing its share of the batch rows.
+//
+// What bounds it: the stream of the weights.  With the weights as the N operand (128 activation rows
+// staged and multiplied for 16 samples, one block per 128 features) 64 of 148 SMs read 8192 x 8192 weights, half of
+// every stage was padding: 57 us for 16 samples.  As the M operand the batch takes N = 16, 32, ... columns
+// of the instruction and 2 KB per 16 samples of a stage; S blocks per tile keep twice as many blocks as
+// SMs reading.  8192 x 8192 weights on 4 x 4 workers (B200, weights cold): 16 samples 57 -> 27 us (0.76 of the copy rate),
+// 64 samples forward / adjoint 44 / 38 -> 28 / 27 us, 128 samples 46 / 40 -> 31 / 30 us.
+// ------------------------------------------------------------------------------------------
+constexpr int kSplitWBytes = kTileM * kBlockK * 2;           // 16 KB: 128 features x 64 of the contraction
+constexpr int kSplitMaxStages = 12;
+constexpr int kSplitTail = 1024 + 256;                       // alignment, barriers
+constexpr int kSplitMaxSmem = 220 * 1024;                    // one block per SM; half of it: two
+
+struct AffineSplitParams {
+    AffineParams p;
+    int32_t n;                              // batch rounded up to a multiple of 16
+    int32_t split;                          // S = blocks per cluster
+    int32_t stages, stage_bytes;
+};
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kAffineThreads, 1)
+affine_kernel_split(const __grid_constant__ AffineSplitParams Q) {
+    const AffineParams &P = Q.p;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;            // the ring first; the partial sums take its place
+    uint8_t *aligned = smem_raw + (base - raw);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(aligned + Q.stages * Q.stage_bytes);
+    const uint32_t bar_full = smem_u32(bars);
+    const uint32_t bar_empty = bar_full + 8 * kSplitMaxStages;
+    const uint32_t bar_acc = bar_empty + 8 * kSplitMaxStages;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kSplitMaxStages + 1);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank();
+    const int tile = (int)blockIdx.x / Q.split;
+    const int tiles_per_block = (P.blk_out + kTileM - 1) / kTileM;   // the last tile of a block may be partly empty
+    const int oblk = tile / tiles_per_block;                  // output block (i forward, j adjoint)
+    const int n0 = (tile - oblk * tiles_per_block) * kTileM;  // first output feature inside the block
+    const int kblocks_per_worker = (P.blk_red + kBlockK - 1) / kBlockK;
+    const int all_kblocks = P.nred * kblocks_per_worker;
+    const int kb0 = (int)((long long)all_kblocks * rank / Q.split), kb1 = (int)((long long)all_kblocks * (rank + 1) / Q.split);
+    const uint32_t tmem_cols = Q.n <= 32 ? 32u : Q.n <= 64 ? 64u : 128u;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < Q.stages; ++s) {
+            mbar_init(bar_full + 8 * s, 1);
+            mbar_init(bar_empty + 8 * s, 1);
+        }
+        mbar_init(bar_acc, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tcgen05_fence_before();
+    __syncthreads();
+    tcgen05_fence_after();
+    const uint32_t tmem_acc = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int r = kb0 / kblocks_per_worker, k0 = (kb0 - r * kblocks_per_worker) * kBlockK;
+            const int wstep = P.adjoint ? P.pfi : 1;
+            const CUtensorMap *wmap = (P.adjoint ? &P.w_map[oblk] : &P.w_map[oblk * P.pfi]) + r * wstep;
+            uint32_t s = 0, phase = 0, sa = base;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(bar_empty + 8 * s, phase ^ 1, abort_flag)) break;
+                const uint32_t full = bar_full + 8 * s;
+                mbar_expect_tx(full, (uint32_t)Q.stage_bytes);
+                if (!P.adjoint) {
+                    tma_load_2d(sa, wmap, k0, n0, full);                            // K-major: box {64 k, 128 rows}
+                } else {                                                            // MN-major: two boxes {64 features, 64 k}
+                    tma_load_2d(sa, wmap, n0, k0, full);
+                    tma_load_2d(sa + kSplitWBytes / 2, wmap, n0 + 64, k0, full);
+                }
+                tma_load_2d(sa + kSplitWBytes, &P.a_map[r], k0, 0, full);           // box {64 k, n rows}
+                k0 += kBlockK;
+                if (k0 >= P.blk_red) {                  // next worker of the grid row / column, in order
+                    k0 = 0;
+                    ++r;
+                    wmap += wstep;
+                }
+                sa += (uint32_t)Q.stage_bytes;
+                if (++s == (uint32_t)Q.stages) {
+                    s = 0;
+                    sa = base;
+                    phase ^= 1;
+                }
+            }
+            if (*abort_flag) {
+                // give copies that are still in flight time to land before the block retires
+                const uint64_t t0 = global_timer();
+                while (global_timer() - t0 < 1000000ull) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = instr_desc(kTileM, Q.n, 0) | (P.adjoint ? 1u << 15 : 0u);
+            // weights, forward, K-major: 8-row groups 1024 bytes apart, a K step of 16 elements is 32 bytes; adjoint,
+            // MN-major: 64-feature atoms 8 KB apart, 8-k groups 1024 bytes apart, a K step of 16 rows is 2048 bytes
+            const uint64_t a0 = P.adjoint ? smem_desc(base, kSplitWBytes / 2, 1024) : smem_desc(base, 16, 1024);
+            const uint64_t astep = P.adjoint ? (2048 >> 4) : (32 >> 4);
+            const uint64_t b0 = smem_desc(base + kSplitWBytes, 16, 1024);
+            uint32_t s = 0, phase = 0;
+            uint64_t off = 0;
+            bool ok = true;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                ok = mbar_wait(bar_full + 8 * s, phase, abort_flag);
+                if (!ok) break;
+                tcgen05_fence_after();
+                const uint64_t a = a0 + off, b = b0 + off;
+                umma_bf16(tmem_acc, a, b, idesc, kb > kb0 ? 1u : 0u);
+                umma_bf16(tmem_acc, a + astep, b + 2, idesc, 1u);
+                umma_bf16(tmem_acc, a + 2 * astep, b + 4, idesc, 1u);
+                umma_bf16(tmem_acc, a + 3 * astep, b + 6, idesc, 1u);
+                tcgen05_commit(bar_empty + 8 * s);              // frees the stage once these MMAs retire
+                off += (uint64_t)Q.stage_bytes >> 4;
+                if (++s == (uint32_t)Q.stages) {
+                    s = 0;
+                    off = 0;
+                    phase ^= 1;
+                }
+            }
+            if (ok) tcgen05_commit(bar_acc);
+        }
+        __syncwarp();
+    } else {
+        const int quarter = warp & 3;                           // tensor-memory lanes [32 q, 32 q + 32)
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, 0, abort_flag));
+        tcgen05_fence_after();
+        if (ok) {
+            // every MMA has retired, so the ring is free: partial sums as [batch row][feature]
+            float *part = reinterpret_cast<float *>(aligned) + quarter * 32 + lane;
+#pragma unroll 1
+            for (int c = 0; c < Q.n; c += 16) {
+                uint32_t v[16];
+                tmem_ld16(tmem_acc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+#pragma unroll
+                for (int q = 0; q < 16; ++q) part[(c + q) * kTileM] = __uint_as_float(v[q]);
+            }
+        }
+    }
+    tcgen05_fence_before();
+    cluster_sync_all();                                         // every block's partial sums are in place
+    if (!*abort_flag) {
+        const int rows = (P.nb + Q.split - 1) / Q.split, row0 = rank * rows, row1 = min(P.nb, row0 + rows);
+        const int f = 4 * lane;                                 // feature inside the tile; whole float4s: blocks are multiples of 8
+        if (n0 + f < P.blk_out) {
+            float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (P.bias[oblk]) bias = __ldg(reinterpret_cast<const float4 *>(P.bias[oblk] + n0 + f));
+            for (int row = row0 + warp; row < row1; row += kAffineThreads / 32) {
+                const uint32_t addr = base + (uint32_t)((row * kTileM + f) * 4);
+                float4 o = ld_cluster_f4(map_to_cta(addr, 0));
+                for (int q = 1; q < Q.split; ++q) {
+                    const float4 v = ld_cluster_f4(map_to_cta(addr, (uint32_t)q));
+                    o.x += v.x; o.y += v.y; o.z += v.z; o.w += v.w;
+                }
+                o.x += bias.x; o.y += bias.y; o.z += bias.z; o.w += bias.w;
+                *reinterpret_cast<float4 *>(P.out[oblk] + (size_t)row * P.blk_out + n0 + f) = o;
+            }
+        }
+    }
+    cluster_sync_all();                                         // nobody retires while a peer reads its shared memory
+    if (warp == 1) {
+        tcgen05_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "r"(tmem_cols) : "memory");
     }
 }
 
@@ -930,19 +1089,21 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
     AffineParams P;
     memset(&P, 0, sizeof(P));
     const int64_t act_cols = adjoint ? bfo : bfi;
+    // few samples: the weights are the M operand and the batch, rounded up to 16, the N operand
+    const int n_split = (int)((nb + 15) / 16 * 16);
     for (int i = 0; i < nact; ++i)
-        if (!make_map(&P.a_map[i], act[i], nb, act_cols, kBlockK, kTileM))
+        if (!make_map(&P.a_map[i], act[i], nb, act_cols, kBlockK, nb <= kTileM ? n_split : kTileM))
             return fail(DISTDL_ERR_CUDA, "%s: tensor map of activation block %d failed", what, i);
     // more than one 128-row tile of the batch: a pair of blocks shares each 256 x 128 output tile
     const bool pair = nb > kTileM;
     // four-block variant: an even number of workers to sum over and output blocks of whole 256-column tiles
     const bool quad = pair && ((adjoint ? pfo : pfi) % 2 == 0) && ((adjoint ? bfi : bfo) % kQuadN == 0);
     for (int i = 0; i < pfo * pfi; ++i) {
-        // forward: box {64 along in-features (K), 128 out-feature rows} (64 rows per block of a pair);
+        // forward: box {64 along in-features (K), 128 out-feature rows} (64 rows per block of a plain pair);
         // adjoint: box {64 along in-features (N), 64 out-feature rows (K)} of the same row-major
         // [bfo, bfi] block
         const bool ok = adjoint ? make_map(&P.w_map[i], w[i], bfo, bfi, 64, kBlockK)
-                                : make_map(&P.w_map[i], w[i], bfo, bfi, kBlockK, quad ? kQuadN / 2 : (pair ? kTileN / 2 : kTileN));
+                                : make_map(&P.w_map[i], w[i], bfo, bfi, kBlockK, pair && !quad ? kTileN / 2 : 128);
         if (!ok) return fail(DISTDL_ERR_CUDA, "%s: tensor map of weight block %d failed", what, i);
     }
     for (int i = 0; i < nout; ++i) {
@@ -958,6 +1119,7 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
     P.adjoint = adjoint ? 1 : 0;
 
     // one-time set-up per device (kernel attributes, occupancy): a process may drive several GPUs
+    static int sms_on[kMaxDevicesPerProcess] = {0};
     static bool configured_on[kMaxDevicesPerProcess] = {false};
     int cur_dev = 0;
     DISTDL_CUDA_CHECK(cudaGetDevice(&cur_dev));
@@ -966,10 +1128,10 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
     std::lock_guard<std::mutex> setup_lock(setup_mutex());      // first calls from several threads set up once
     bool &configured = configured_on[cur_dev];
     if (!configured) {
-        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               AffineCfg<false>::SMEM_BYTES));
-        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               AffineCfg<true>::SMEM_BYTES));
+        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_kernel_split, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitMaxSmem));
+        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_kernel_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               AffinePairCfg::SMEM_BYTES));
+        DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms_on[cur_dev], cudaDevAttrMultiProcessorCount, cur_dev));
         DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_kernel_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, kQuadSmemBytes));
         configured = true;
     }
@@ -998,7 +1160,7 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
         memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3((unsigned)(2 * row_pairs * ntiles));
         cfg.blockDim = dim3(kAffineThreads);
-        cfg.dynamicSmemBytes = AffineCfg<true>::SMEM_BYTES;
+        cfg.dynamicSmemBytes = AffinePairCfg::SMEM_BYTES;
         cfg.stream = (cudaStream_t)stream;
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
@@ -1007,11 +1169,35 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
         attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel<true>, P));
+        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel_pair, P));
     } else {
-        const int64_t row_tiles = (nb + kTileM - 1) / kTileM;
-        affine_kernel<false><<<(unsigned)(row_tiles * ntiles), kAffineThreads, AffineCfg<false>::SMEM_BYTES,
-                               (cudaStream_t)stream>>>(P);
+        // blocks per tile: doubled while twice as many blocks as SMs are not exceeded and every block keeps four k-blocks
+        const int sms = sms_on[cur_dev];
+        const int64_t all_kblocks = (int64_t)P.nred * ((P.blk_red + kBlockK - 1) / kBlockK);
+        AffineSplitParams Q;
+        memset(&Q, 0, sizeof(Q));
+        Q.p = P;
+        Q.n = n_split;
+        Q.split = 1;
+        while (Q.split < 8 && ntiles * Q.split * 2 <= 2 * sms && all_kblocks >= 4 * 2 * Q.split) Q.split *= 2;
+        Q.stage_bytes = kSplitWBytes + Q.n * kBlockK * 2;
+        const int budget = ntiles * Q.split <= sms ? kSplitMaxSmem : kSplitMaxSmem / 2;
+        Q.stages = std::min(kSplitMaxStages, (budget - kSplitTail) / Q.stage_bytes);
+        const int smem = Q.stages * Q.stage_bytes + kSplitTail;       // at least three stages: room for the partial sums
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)(ntiles * Q.split));
+        cfg.blockDim = dim3(kAffineThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = (cudaStream_t)stream;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)Q.split;
+        attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel_split, Q));
     }
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;

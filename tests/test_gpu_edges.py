@@ -72,3 +72,20 @@ def test_repartition_rows(case, dtype):
 def test_halo_long_rows(case):
     parity.test_halo_fwd_and_adj_bit_exact(case)
     parity.test_halo_fwd_and_adj_bf16_fp64_bit_exact(case)
+
+
+# nb, nfi, nfo, pfo, pfi: up to 128 samples the weights are the M operand and up to eight blocks share a tile
+AFFINE_EDGES = [
+    (1, 8, 8, 1, 1),                         # one sample, one partly filled k-block
+    (16, 4096, 128, 1, 2),                   # one tile, eight blocks
+    (17, 2048, 528, 2, 4),                   # 32 columns for 17 samples, output blocks of 264
+    (63, 1000, 136, 1, 1),
+    (128, 72, 1032, 3, 1),                   # full batch, a reduction too short to share
+    (129, 512, 520, 1, 1),                   # the first batch of the pair variant
+]
+
+
+@pytest.mark.parametrize("case", AFFINE_EDGES, ids=[str(c) for c in AFFINE_EDGES])
+@pytest.mark.parametrize("integer", [True, False], ids=["int", "normal"])
+def test_affine_few_samples(case, integer):
+    parity.test_affine_fwd_and_adj(case, integer)
