@@ -109,87 +109,183 @@ pool_adj_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Variants with the kernel and stride fixed at compile time (2 x 2 / 2 and 3 x 3 / 2, the pooling
-// layers of the usual networks): index arithmetic in shifts, and four outputs (forward) or cells
-// (adjoint) per thread, 32 columns apart, so that the lanes of a warp always touch neighbouring
-// addresses.  Same sums in the same order as the general kernels above.
+// Variants with the kernel and stride fixed at compile time (2 x 2 / 2, 3 x 3 / 2 and 3 x 3 / 1, the pooling layers of the
+// usual networks).  A warp owns 64 columns (of outputs, adjoint: of groups of SH x SW cells) and marches down `rows` rows:
+// what overlapping windows share stays in registers, the loads of the next step are issued before this step's arithmetic,
+// and neighbouring lanes touch neighbouring addresses.  Same results as the general kernels above.
+//
+// What bounds them: device memory, instruction issue close behind.  Measured (B200, with the H / H* around them, forward /
+// adjoint, us; before: four outputs or groups of one row per thread, nothing shared between rows; 3 x 3 / 1: the general kernels):
+//   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    370 / 437   (368 / 538)
+//   2 x 2 / 2 max, the same                                   249 / 262   (257 / 312)
+//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      530 / 651   (1653 / 2687)
+// A maximum is taken per input row first (value, first
+// position); a NaN counts as the scan in window order counts it: it wins only as the window's first cell.
 // ---------------------------------------------------------------------------------------------
-constexpr int kPoolPerThread = 4;
+constexpr int kPoolCols = 2;           // columns per lane, 32 apart
+
+template <int KW>
+struct PoolRow {
+    float x[KW];                       // AVG: the cells;  MAX: x[0] = first cell of the row inside the tensor
+    float m;                           // MAX: largest cell that is a number, the first of equals
+    int b;                             // and its column in the window
+    __device__ __forceinline__ void set(const float (&v)[KW]) {
+#pragma unroll
+        for (int c = 0; c < KW; ++c) x[c] = v[c];
+    }
+    __device__ __forceinline__ void reduce() {
+        float top = x[0];
+#pragma unroll
+        for (int c = 1; c < KW; ++c) top = fmaxf(top, x[c]);
+        m = x[KW - 1];
+        b = KW - 1;
+#pragma unroll
+        for (int c = KW - 2; c >= 0; --c)
+            if (x[c] == top) {
+                m = x[c];
+                b = c;
+            }
+    }
+    // the cells [lo, hi) of the row lie inside the tensor (at least one)
+    __device__ __forceinline__ void reduce_clipped(int lo, int hi) {
+        float first = 0.f;
+        bool have = false;
+        m = 0.f;
+        b = 0;
+#pragma unroll
+        for (int c = 0; c < KW; ++c)
+            if (c >= lo && c < hi) {
+                if (!have) first = x[c];
+                if (!have || x[c] > m || (m != m && x[c] == x[c])) {
+                    m = x[c];
+                    b = c;
+                }
+                have = true;
+            }
+        x[0] = first;
+    }
+};
 
 template <int KH, int KW, int SH, int SW, int MODE>
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
-pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
+pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
     rest /= tiles_x;
     const int ty = rest % tiles_y;
     const int plane = rest / tiles_y;
-    const int jb = tx * kPoolThreadsX * kPoolPerThread + threadIdx.x, i = ty * kPoolThreadsY + threadIdx.y;
-    if (i >= S.oh) return;
-    const int r0 = S.i0 + i * SH;
-    const float *row = S.in + ((size_t)plane * S.ph + r0) * S.pw + S.j0;
-    float *orow = S.out + ((size_t)plane * S.oh + i) * S.ow;
-    int32_t *arow = (MODE == DISTDL_POOL_MAX && S.arg) ? S.arg + ((size_t)plane * S.oh + i) * S.ow : nullptr;
-    bool row_in[KH];
+    const int lane = threadIdx.x, jb = tx * (32 * kPoolCols) + lane, i_begin = (ty * kPoolThreadsY + (int)threadIdx.y) * rows;
+    const int i_end = min(i_begin + rows, S.oh);
+    if (i_begin >= i_end || tx * (32 * kPoolCols) >= S.ow) return;
+    bool on[kPoolCols], inside = true;
+    int lo[kPoolCols], hi[kPoolCols];                       // window columns inside the tensor
+    const float *src[kPoolCols];
+    const float *base = S.in + ((size_t)plane * S.ph + (S.i0 + i_begin * SH)) * S.pw + S.j0;
 #pragma unroll
-    for (int a = 0; a < KH; ++a) row_in[a] = S.g0h + r0 + a >= 0 && S.g0h + r0 + a < P.hg;
-    bool rows_inside = true;
+    for (int u = 0; u < kPoolCols; ++u) {
+        const int j = min(jb + 32 * u, S.ow - 1);
+        on[u] = jb + 32 * u < S.ow;
+        src[u] = base + j * SW;
+        const int gj = S.g0w + S.j0 + j * SW;
+        lo[u] = max(0, -gj);
+        hi[u] = min(KW, P.wg - gj);
+        inside = inside && lo[u] == 0 && hi[u] == KW;
+    }
+    inside = __all_sync(0xffffffffu, inside);
+    float next[SH][kPoolCols][KW];
+    PoolRow<KW> row[KH][kPoolCols];
+    auto load = [&](float (&v)[kPoolCols][KW]) {            // one input row, and on to the next
 #pragma unroll
-    for (int a = 0; a < KH; ++a) rows_inside = rows_inside && row_in[a];
+        for (int u = 0; u < kPoolCols; ++u) {
 #pragma unroll
-    for (int u = 0; u < kPoolPerThread; ++u) {
-        const int j = jb + u * kPoolThreadsX;
-        if (j >= S.ow) break;
-        const float *src = row + j * SW;
-        const int gj0 = S.g0w + S.j0 + j * SW;
-        float acc = 0.f;
-        int where = -1;
-        if (MODE == DISTDL_POOL_AVG) {
-#pragma unroll
-            for (int a = 0; a < KH; ++a)
-#pragma unroll
-                for (int b = 0; b < KW; ++b) acc = __fadd_rn(acc, src[a * S.pw + b]);
-            acc = __fmul_rn(acc, 1.0f / (float)(KH * KW));
-        } else if (rows_inside && gj0 >= 0 && gj0 + KW <= P.wg) {
-            // the whole window lies inside the tensor: no cell to exclude
-            acc = src[0];
-            where = 0;
-#pragma unroll
-            for (int a = 0; a < KH; ++a)
-#pragma unroll
-                for (int b = 0; b < KW; ++b) {
-                    if (a == 0 && b == 0) continue;
-                    const float v = src[a * S.pw + b];
-                    if (v > acc) {
-                        acc = v;
-                        where = a * KW + b;
-                    }
-                }
-        } else {
-#pragma unroll
-            for (int a = 0; a < KH; ++a)
-#pragma unroll
-                for (int b = 0; b < KW; ++b) {
-                    const float v = src[a * S.pw + b];
-                    if (row_in[a] && gj0 + b >= 0 && gj0 + b < P.wg && (where < 0 || v > acc)) {
-                        acc = v;
-                        where = a * KW + b;
-                    }
-                }
+            for (int c = 0; c < KW; ++c) v[u][c] = __ldg(src[u] + c);
+            src[u] += S.pw;
         }
-        orow[j] = acc;
-        if (arow) arow[j] = where < 0 ? 0 : where;
+    };
+    auto take = [&](int a, const float (&v)[kPoolCols][KW]) {
+#pragma unroll
+        for (int u = 0; u < kPoolCols; ++u) {
+            row[a][u].set(v[u]);
+            if (MODE == DISTDL_POOL_MAX) {
+                if (inside) row[a][u].reduce();
+                else row[a][u].reduce_clipped(lo[u], hi[u]);
+            }
+        }
+    };
+    // the rows that the first window shares with the one before it, then one step ahead
+#pragma unroll
+    for (int a = 0; a < KH - SH; ++a) {
+        float v[kPoolCols][KW];
+        load(v);
+        take(a, v);
+    }
+#pragma unroll
+    for (int a = 0; a < SH; ++a) load(next[a]);
+    float *out = S.out + ((size_t)plane * S.oh + i_begin) * S.ow + jb;
+    int32_t *arg = MODE == DISTDL_POOL_MAX && S.arg ? S.arg + ((size_t)plane * S.oh + i_begin) * S.ow + jb : nullptr;
+    for (int i = i_begin; i < i_end; ++i) {
+        float v[SH][kPoolCols][KW];
+#pragma unroll
+        for (int a = 0; a < SH; ++a)
+#pragma unroll
+            for (int u = 0; u < kPoolCols; ++u)
+#pragma unroll
+                for (int c = 0; c < KW; ++c) v[a][u][c] = next[a][u][c];
+        if (i + 1 < i_end)
+#pragma unroll
+            for (int a = 0; a < SH; ++a) load(next[a]);
+#pragma unroll
+        for (int a = 0; a < SH; ++a) take(KH - SH + a, v[a]);
+        const int gi = S.g0h + S.i0 + i * SH;               // tensor row of window row 0
+#pragma unroll
+        for (int u = 0; u < kPoolCols; ++u) {
+            float best = 0.f;
+            int where = 0;
+            if (MODE == DISTDL_POOL_AVG) {
+#pragma unroll
+                for (int a = 0; a < KH; ++a)
+#pragma unroll
+                    for (int c = 0; c < KW; ++c) best = __fadd_rn(best, row[a][u].x[c]);
+                best = __fmul_rn(best, 1.0f / (float)(KH * KW));
+            } else {
+                bool have = false;
+#pragma unroll
+                for (int a = 0; a < KH; ++a) {
+                    if (gi + a < 0 || gi + a >= P.hg || lo[u] >= hi[u]) continue;
+                    const PoolRow<KW> &r = row[a][u];
+                    if (!have) {
+                        const bool nan = r.x[0] != r.x[0];
+                        best = nan ? r.x[0] : r.m;
+                        where = a * KW + (nan ? lo[u] : r.b);
+                        have = true;
+                    } else if (r.m > best) {
+                        best = r.m;
+                        where = a * KW + r.b;
+                    }
+                }
+            }
+            if (on[u]) {
+                out[32 * u] = best;
+                if (arg) arg[32 * u] = where;
+            }
+        }
+        out += S.ow;
+        if (arg) arg += S.ow;
+#pragma unroll
+        for (int a = 0; a < KH - SH; ++a)
+#pragma unroll
+            for (int u = 0; u < kPoolCols; ++u) row[a][u] = row[a + SH][u];
     }
 }
 
-// Adjoint: a thread owns the SH x SW cells {i0 + SH*gi + r, j0 + SW*gj + c}.  The outputs whose window holds
-// cell (r, c) of the group are (gi - t, gj - v) with window positions a = r + t*SH < KH, b = c + v*SW < KW, all
-// known at compile time; the thread loads the NI x NJ candidate outputs once and every cell picks its terms
-// (ascending output order = descending t, v).  tiles count groups: row group = first group + tile row, and so on.
+// Adjoint: a lane owns the SH x SW cells {i0 + SH * gi + r, j0 + SW * gj + c} of a group and marches down gi.  The outputs whose
+// window holds cell (r, c) of the group are (gi - t, gj - v) with window positions a = r + t * SH < KH, b = c + v * SW < KW, all
+// known at compile time; the outputs (gi - t, .) of the rows above stay in registers, and every cell picks its terms
+// (ascending output order = descending t, v).
 template <int KH, int KW, int SH, int SW, int MODE>
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
-pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
+pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
@@ -198,93 +294,95 @@ pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
     const int plane = rest / tiles_y;
     constexpr int NI = (KH + SH - 1) / SH, NJ = (KW + SW - 1) / SW;
     // the first group holds padded row / column 0
-    const int gi = div_floor(-S.i0, SH) + ty * kPoolThreadsY + (int)threadIdx.y;
-    const int gjb = div_floor(-S.j0, SW) + tx * kPoolThreadsX * kPoolPerThread + (int)threadIdx.x;
-    const int p0 = S.i0 + gi * SH;
-    if (p0 >= S.ph) return;
+    const int gi0 = div_floor(-S.i0, SH) + (ty * kPoolThreadsY + (int)threadIdx.y) * rows;
+    const int gj0 = div_floor(-S.j0, SW) + tx * (32 * kPoolCols) + (int)threadIdx.x;
+    if (S.i0 + gi0 * SH >= S.ph) return;
     const float *dy = S.in + (size_t)plane * S.oh * S.ow;
     const int32_t *arg = MODE == DISTDL_POOL_MAX ? S.arg + (size_t)plane * S.oh * S.ow : nullptr;
-    float *oplane = S.out + (size_t)plane * S.ph * S.pw;
+    float *out = S.out + ((size_t)plane * S.ph + (S.i0 + gi0 * SH)) * S.pw + (S.j0 + gj0 * SW);
+    bool jok[kPoolCols][NJ], cok[kPoolCols][SW];
 #pragma unroll
-    for (int u = 0; u < kPoolPerThread; ++u) {
-        const int gj = gjb + u * kPoolThreadsX;
-        const int q0 = S.j0 + gj * SW;
-        if (q0 >= S.pw) break;
-        float g[NI][NJ];
-        int code[NI][NJ];          // MAX: recorded position, -1 for an absent output; AVG: 0 present, -1 absent
-        const bool interior = gi - (NI - 1) >= 0 && gi < S.oh && gj - (NJ - 1) >= 0 && gj < S.ow && p0 >= 0 &&
-                              p0 + SH <= S.ph && q0 >= 0 && q0 + SW <= S.pw;
-        if (interior) {
-            // every candidate output exists and every cell of the group lies in the shard: no tests, 32-bit offsets
-            const uint32_t o = (uint32_t)(gi * S.ow + gj);
+    for (int u = 0; u < kPoolCols; ++u) {
+        const int gj = gj0 + 32 * u;
 #pragma unroll
-            for (int t = 0; t < NI; ++t)
+        for (int v = 0; v < NJ; ++v) jok[u][v] = (unsigned)(gj - v) < (unsigned)S.ow;
 #pragma unroll
-                for (int v = 0; v < NJ; ++v) {
-                    g[t][v] = dy[o - (uint32_t)(t * S.ow + v)];
-                    code[t][v] = MODE == DISTDL_POOL_MAX ? arg[o - (uint32_t)(t * S.ow + v)] : 0;
-                }
-            float *dst = oplane + (uint32_t)(p0 * S.pw + q0);
+        for (int c = 0; c < SW; ++c) cok[u][c] = (unsigned)(S.j0 + gj * SW + c) < (unsigned)S.pw;
+    }
+    // MAX: recorded position, -1 for an absent output;  AVG: 0 present, -1 absent
+    float g[NI][kPoolCols][NJ], gn[kPoolCols][NJ];
+    int code[NI][kPoolCols][NJ], cn[kPoolCols][NJ];
+    auto load = [&](int i, float (&gv)[kPoolCols][NJ], int (&cv)[kPoolCols][NJ]) {
+        const bool ok = (unsigned)i < (unsigned)S.oh;
+        const int o = i * S.ow + gj0;
 #pragma unroll
-            for (int r = 0; r < SH; ++r)
-#pragma unroll
-                for (int c = 0; c < SW; ++c) {
-                    float acc = 0.f;
-#pragma unroll
-                    for (int t = NI - 1; t >= 0; --t)
-#pragma unroll
-                        for (int v = NJ - 1; v >= 0; --v) {
-                            if (r + t * SH >= KH || c + v * SW >= KW) continue;      // compile-time
-                            if (MODE == DISTDL_POOL_AVG) acc = __fadd_rn(acc, g[t][v]);
-                            else if (code[t][v] == (r + t * SH) * KW + (c + v * SW)) acc = __fadd_rn(acc, g[t][v]);
-                        }
-                    if (MODE == DISTDL_POOL_AVG) acc = __fmul_rn(acc, 1.0f / (float)(KH * KW));
-                    dst[r * S.pw + c] = acc;
-                }
-            continue;
-        }
-#pragma unroll
-        for (int t = 0; t < NI; ++t)
+        for (int u = 0; u < kPoolCols; ++u)
 #pragma unroll
             for (int v = 0; v < NJ; ++v) {
-                const int i = gi - t, j = gj - v;
-                const bool in = i >= 0 && i < S.oh && j >= 0 && j < S.ow;
-                g[t][v] = in ? dy[i * S.ow + j] : 0.f;
-                code[t][v] = !in ? -1 : (MODE == DISTDL_POOL_MAX ? arg[i * S.ow + j] : 0);
+                gv[u][v] = 0.f;
+                cv[u][v] = -1;
+                if (ok && jok[u][v]) {
+                    gv[u][v] = __ldg(dy + o + (32 * u - v));
+                    cv[u][v] = MODE == DISTDL_POOL_MAX ? __ldg(arg + o + (32 * u - v)) : 0;
+                }
             }
+    };
+#pragma unroll
+    for (int t = 1; t < NI; ++t) load(gi0 - t, g[t], code[t]);
+    load(gi0, gn, cn);
+    for (int gi = gi0; gi < gi0 + rows; ++gi) {
+        const int p0 = S.i0 + gi * SH;
+        if (p0 >= S.ph) break;
+#pragma unroll
+        for (int u = 0; u < kPoolCols; ++u)
+#pragma unroll
+            for (int v = 0; v < NJ; ++v) {
+                g[0][u][v] = gn[u][v];
+                code[0][u][v] = cn[u][v];
+            }
+        if (gi + 1 < gi0 + rows) load(gi + 1, gn, cn);
 #pragma unroll
         for (int r = 0; r < SH; ++r) {
-            const int p = p0 + r;
-            if (p < 0 || p >= S.ph) continue;
+            if ((unsigned)(p0 + r) < (unsigned)S.ph) {
 #pragma unroll
-            for (int c = 0; c < SW; ++c) {
-                const int q = q0 + c;
-                if (q < 0 || q >= S.pw) continue;
-                float acc = 0.f;
+                for (int u = 0; u < kPoolCols; ++u)
 #pragma unroll
-                for (int t = NI - 1; t >= 0; --t)
+                    for (int c = 0; c < SW; ++c) {
+                        float acc = 0.f;
 #pragma unroll
-                    for (int v = NJ - 1; v >= 0; --v) {
-                        if (r + t * SH >= KH || c + v * SW >= KW) continue;      // compile-time
-                        const bool take = MODE == DISTDL_POOL_AVG ? code[t][v] == 0
-                                                                  : code[t][v] == (r + t * SH) * KW + (c + v * SW);
-                        if (take) acc = __fadd_rn(acc, g[t][v]);
+                        for (int t = NI - 1; t >= 0; --t)
+#pragma unroll
+                            for (int v = NJ - 1; v >= 0; --v) {
+                                if (r + t * SH >= KH || c + v * SW >= KW) continue;      // compile-time
+                                const bool take = code[t][u][v] == (MODE == DISTDL_POOL_AVG ? 0 : (r + t * SH) * KW + (c + v * SW));
+                                if (take) acc = __fadd_rn(acc, g[t][u][v]);
+                            }
+                        if (MODE == DISTDL_POOL_AVG) acc = __fmul_rn(acc, 1.0f / (float)(KH * KW));
+                        if (cok[u][c]) out[32 * SW * u + c] = acc;
                     }
-                if (MODE == DISTDL_POOL_AVG) acc = __fmul_rn(acc, 1.0f / (float)(KH * KW));
-                oplane[(size_t)p * S.pw + q] = acc;
             }
+            out += S.pw;
         }
+#pragma unroll
+        for (int t = NI - 1; t > 0; --t)
+#pragma unroll
+            for (int u = 0; u < kPoolCols; ++u)
+#pragma unroll
+                for (int v = 0; v < NJ; ++v) {
+                    g[t][u][v] = g[t - 1][u][v];
+                    code[t][u][v] = code[t - 1][u][v];
+                }
     }
 }
 
 template <int KH, int KW, int SH, int SW>
-static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int tiles_x, int tiles_y, bool adjoint, cudaStream_t s) {
+static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int tiles_x, int tiles_y, int rows, bool adjoint, cudaStream_t s) {
     if (!adjoint) {
-        if (P.mode == DISTDL_POOL_AVG) pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
-        else pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
+        if (P.mode == DISTDL_POOL_AVG) pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
+        else pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
     } else {
-        if (P.mode == DISTDL_POOL_AVG) pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
-        else pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
+        if (P.mode == DISTDL_POOL_AVG) pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
+        else pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
     }
 }
 
@@ -379,16 +477,18 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         max_cols = std::max<int64_t>(max_cols, adjoint ? S.pw : S.ow);
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // the compile-time variants handle four outputs / cells per thread along a row
-    const int fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2 : 0;
-    const int per_thread = fixed ? kPoolPerThread : 1;
+    // the compile-time variants: 64 columns and up to 16 rows per warp (fewer where eight warps would leave some without a row)
+    const int fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
+                    : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
     if (fixed && adjoint) {
         // the compile-time adjoint walks groups of sh x sw cells; the group lattice starts up to one group before cell 0
         max_rows = max_rows / sh + 2;
         max_cols = max_cols / sw + 2;
     }
-    const int tiles_x = (int)((max_cols + kPoolThreadsX * per_thread - 1) / (kPoolThreadsX * per_thread));
-    const int tiles_y = (int)((max_rows + kPoolThreadsY - 1) / kPoolThreadsY);
+    const int rows = fixed ? (int)std::min<int64_t>(16, std::max<int64_t>(2, (max_rows + kPoolThreadsY - 1) / kPoolThreadsY)) : 1;
+    const int cols = fixed ? 32 * kPoolCols : kPoolThreadsX;
+    const int tiles_x = (int)((max_cols + cols - 1) / cols);
+    const int tiles_y = (int)((max_rows + kPoolThreadsY * rows - 1) / (kPoolThreadsY * rows));
     const int64_t blocks = (int64_t)tiles_x * tiles_y * P.planes;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     const dim3 grid((unsigned)blocks, (unsigned)p->num_workers), block(kPoolThreadsX, kPoolThreadsY);
@@ -398,8 +498,9 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         if (st != DISTDL_OK) return st;
     }
     if (blocks > 0) {
-        if (fixed == 1) launch_pool_fixed<2, 2, 2, 2>(P, grid, block, tiles_x, tiles_y, adjoint, s);
-        else if (fixed == 2) launch_pool_fixed<3, 3, 2, 2>(P, grid, block, tiles_x, tiles_y, adjoint, s);
+        if (fixed == 1) launch_pool_fixed<2, 2, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
+        else if (fixed == 2) launch_pool_fixed<3, 3, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
+        else if (fixed == 3) launch_pool_fixed<3, 3, 1, 1>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
         else if (!adjoint) pool_fwd_kernel<<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
         else pool_adj_kernel<<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
     }

@@ -1,6 +1,7 @@
 """GPU parity at the edges of the kernels' tiles and dispatch rules: the checks (and their bounds) are those of
 test_gpu_parity.py, the cases are the sizes where a tile is ragged, a tile holds several images, or a variant begins or ends."""
 
+import numpy as np
 import pytest
 
 import test_gpu_parity as parity
@@ -89,3 +90,44 @@ AFFINE_EDGES = [
 @pytest.mark.parametrize("integer", [True, False], ids=["int", "normal"])
 def test_affine_few_samples(case, integer):
     parity.test_affine_fwd_and_adj(case, integer)
+
+
+# global shape, partition, kernel, stride, padding
+POOL_EDGES = [
+    ((1, 1, 7, 5), (1, 1, 1, 1), (3, 3), (1, 1), ((1, 1), (1, 1))),         # every window of a border column is clipped
+    ((2, 1, 70, 131), (1, 1, 2, 2), (3, 3), (1, 1), ((1, 1), (1, 1))),
+    ((1, 2, 37, 67), (1, 1, 1, 1), (3, 3), (2, 2), ((0, 0), (0, 0))),
+    ((1, 1, 300, 22), (1, 1, 2, 1), (2, 2), (2, 2), ((0, 0), (0, 0))),      # several 128-row tiles of warps
+    ((1, 3, 9, 260), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),       # 65 outputs: one column past a warp's 64
+]
+
+
+@pytest.mark.parametrize("case", POOL_EDGES, ids=[str(c[:4]) for c in POOL_EDGES])
+@pytest.mark.parametrize("mode", ["avg", "max"])
+def test_pool_marching(case, mode):
+    parity.test_pool_fwd_and_adj(case, mode)
+
+
+@pytest.mark.parametrize("stride", [1, 2])
+def test_pool_max_of_special_values(stride):
+    """NaN, infinities and signed zeros: the first largest cell in window order, a NaN only as the window's first cell."""
+    torch, distdl = parity.torch, parity.distdl
+    n = 41
+    x = np.random.default_rng(5).choice(np.array([np.nan, -np.inf, np.inf, -0.0, 0.0, 1.0, -1.0], dtype=np.float32), size=(n, n))
+    w = distdl.halo_widths_1d(n, 1, 3, stride, 1, 1, 1)
+    part = distdl.Partition((1, 1, n, n), (1, 1, 1, 1), [0, 0, w[0], w[0]], [0, 0, w[1], w[1]])
+    m = (n + 2 - 3) // stride + 1
+    pad = np.zeros(part.padded_shape(0), dtype=np.float32)
+    pad[0, 0, w[0][0]:w[0][0] + n, w[0][0]:w[0][0] + n] = x
+    y, a = torch.empty((1, 1, m, m), device=parity.DEV), torch.empty((1, 1, m, m), dtype=torch.int32, device=parity.DEV)
+    distdl.pool_fwd(part, [parity.dev(pad)], (3, 3), (stride, stride), ((1, 1), (1, 1)), distdl.POOL_MAX, [y], [a])
+    yr, ar = np.empty((m, m), dtype=np.float32), np.empty((m, m), dtype=np.int32)
+    for i in range(m):
+        for j in range(m):
+            best, where = None, 0
+            for k in range(9):
+                p, q = i * stride - 1 + k // 3, j * stride - 1 + k % 3
+                if 0 <= p < n and 0 <= q < n and (best is None or x[p, q] > best):
+                    best, where = x[p, q], k
+            yr[i, j], ar[i, j] = best, where
+    assert parity.same_bits(parity.host(y)[0, 0], yr) and parity.same_bits(parity.host(a)[0, 0], ar)
