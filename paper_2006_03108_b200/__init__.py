@@ -111,17 +111,31 @@ def _ptr(t):
     return t.data_ptr()
 
 
+_array_types = {}
+
+
 def _ptr_array(ts):
-    arr = (ctypes.c_void_p * len(ts))()
-    for i, t in enumerate(ts):
-        arr[i] = _ptr(t)
-    return arr
+    n = len(ts)
+    kind = _array_types.get(n)
+    if kind is None:
+        kind = _array_types[n] = ctypes.c_void_p * n
+    return kind(*[t if t is None or isinstance(t, int) else t.data_ptr() for t in ts])
+
+
+_raw_stream = None
 
 
 def _stream(stream):
+    """Handle of a stream (an int, or an object with `cuda_stream`); None: PyTorch's current stream of the current device."""
+    global _raw_stream
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None:
+            # The handle alone: building a Stream object around it costs 3 us, a third of a small call (10.4 -> 7 us for H of
+            # 256 x 256 on 2 x 2 workers)
+            import torch
+            get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+            _raw_stream = (lambda: get(device())) if get else (lambda: torch.cuda.current_stream().cuda_stream)
+        return _raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
