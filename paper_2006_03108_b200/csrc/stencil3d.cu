@@ -11,18 +11,24 @@
 // written into the bulk of the padded dx shards whose ghosts are cleared as H* leaves them.
 //
 // Blocking: a block (four warps) owns 8 rows x 128 columns of one shard and marches through a chunk
-// of planes.  A thread owns 4 consecutive columns of two consecutive rows; the 2R+1 planes around the
-// current one live in its registers (z neighbours), the current plane with R extra rows above /
-// below and R extra columns left / right lives in shared memory (y and x neighbours; a star needs
-// no corners).  The two rows of a thread share their y neighbours: 2R + 2 plane rows, two of them its
-// own, serve both, which halves the shared-memory reads per output.  The values of the next plane --
-// the thread's own cells R planes ahead, its vectors of the extra rows, one cell of an extra column
-// -- are fetched one step early, so their latency is covered by the arithmetic of the current plane.
-// Two plane buffers, one barrier per plane.
+// of planes.  A thread owns 4 consecutive columns of two consecutive rows and keeps the running sums of the
+// 2R+1 outputs around the current plane in registers: a cell of plane p is tap 2R - i of output p - R + i, and the
+// sum moves from slot i + 1 to slot i as the destination of that very FMA (a queue of the 2R+1 input planes instead costs
+// 2R+1 register moves per cell).  The current plane with R extra rows above / below and R extra columns left / right
+// lies in shared memory (y and x neighbours, added to the output in the middle; a star needs no corners); the two rows of a
+// thread share their y neighbours, 2R + 2 plane rows, two of them its own.  Planes arrive by asynchronous copies
+// straight into a ring of five, four planes ahead: a plane's cells are needed at once when it becomes the current one, so
+// one plane of registers does not cover the latency of device memory.  One barrier per plane.  Rows that do not start on
+// 16-byte boundaries (R < 4 on the padded side) are copied four bytes a lane, a warp's cells next to one another.
+// Issue bounds it, not memory: 116 of ~300 instructions a plane are the warp's FMA (25 taps on eight cells, pairs
+// packed but for the odd column shifts), and a fourth block per multiprocessor spills (301 against 233 us).  At 512^3, R = 4,
+// forward 308 -> 233 us, adjoint 365 -> 264 us, where reading and writing the bulk once takes 164 us and 170 us.  The rest
+// of the radii and sizes gain by the rule for the chunks as well (200^3, R = 2: 61 -> 32 and 78 -> 31 us; 64^3, R = 4: 40 -> 6.4 us).
 #include <algorithm>
 #include <cstring>
 
 #include "common.h"
+#include "conv_common.h"
 
 namespace distdl {
 
@@ -33,9 +39,11 @@ constexpr int kStRpt = 2;             // consecutive rows per thread
 constexpr int kStThreads = 128;
 constexpr int kStRows = kStRpt * (kStThreads / 32);   // rows of a tile: 8
 constexpr int kStCols = 128;          // columns of a tile = 32 lanes x 4
-constexpr int kStChunk = 64;          // planes a block marches through
 constexpr int kStLead = 4;            // shared-memory column of the tile's first column (keeps rows 16-byte aligned)
 constexpr int kStPitch = kStLead + kStCols + 4;   // 136 floats
+constexpr int kStDepth = 5;           // planes in the ring (4 and 6 measure the same within 2 %)
+template <int R>
+constexpr int kStBlocks = R <= 2 ? 4 : 3;   // blocks per multiprocessor (registers: 128 / 168)
 
 struct StencilParams {
     const float *in[kStMaxWorkers];
@@ -44,8 +52,12 @@ struct StencilParams {
     int32_t pz, py, px;
     int32_t in_off, out_off;          // ghost width of the input / output layout (R or 0)
     int32_t tiles_y, tiles_x, chunks_z;
+    int32_t chunk;                    // planes a block marches through
     int32_t clear_ghosts;             // adjoint: the ghosts of the output shards are set to zero
-    float w[3][2 * kStMaxR + 1];      // taps; [d][k + R], already reversed for the adjoint
+    int32_t vec_out;                  // rows of the output start on 16-byte boundaries and hold whole vectors
+    // taps [d][k + R], already reversed for the adjoint; the three centre taps meet the same cell and are added up in [0][R]
+    float w[3][2 * kStMaxR + 1];
+    uint64_t w2[3][2 * kStMaxR + 1];  // the same as (w, w) pairs
 };
 
 // Owner of coordinate c along one dimension, seen from worker coordinate s: the worker itself, or the
@@ -68,10 +80,42 @@ __device__ __forceinline__ bool st_owner(const int32_t *b, int p, int s, int c, 
     return true;
 }
 
+// Copy of 16 / 4 bytes, or that many zeros (bytes = 0: nothing is read); nothing at all where `on` is false.
+__device__ __forceinline__ void st_copy16(uint32_t dst, const float *src, uint32_t bytes, bool on) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n@p cp.async.cg.shared.global [%0], [%1], 16, %2;\n}"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void st_copy4(uint32_t dst, const float *src, uint32_t bytes, bool on) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n@p cp.async.ca.shared.global [%0], [%1], 4, %2;\n}"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"((uint32_t)on) : "memory");
+}
+
+template <int R>
+constexpr int st_smem_bytes() { return kStDepth * (kStRows + 2 * R) * kStPitch * 4; }
+
+// Ghost shell of an output shard but for the row ends, which the threads that write the rows clear: the ghost planes below and
+// above, and the ghost rows of each bulk plane, which lie next to those of the plane before it in memory.  All of them are
+// contiguous runs and every block of the shard takes an equal share (block j of n).
+template <bool VEC>
+__device__ __forceinline__ void st_clear(float *out, int bz, int opy, int opx, int oo, int j, int n) {
+    auto zero = [&](size_t at, size_t end) {
+        if (VEC)
+            for (at += 4 * threadIdx.x; at < end; at += 4 * kStThreads) *reinterpret_cast<float4 *>(out + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+        else
+            for (at += threadIdx.x; at < end; at += kStThreads) out[at] = 0.f;
+    };
+    const size_t plane = (size_t)opy * opx, rows = (size_t)oo * opx, ghosts = oo * plane;
+    for (int i = j; i <= bz; i += n) zero((i + oo) * plane - (i > 0 ? rows : 0), (i + oo) * plane + (i < bz ? rows : 0));
+    const size_t piece = (ghosts + 4 * (size_t)n - 1) / (4 * (size_t)n) * 4, lo = min(j * piece, ghosts), hi = min(lo + piece, ghosts);
+    zero(lo, hi);
+    zero((bz + oo) * plane + lo, (bz + oo) * plane + hi);
+}
+
 template <int R, bool VEC>
-__global__ void __launch_bounds__(kStThreads, 4)
+__global__ void __launch_bounds__(kStThreads, kStBlocks<R>)
 stencil3d_kernel(const __grid_constant__ StencilParams P) {
-    __shared__ __align__(16) float plane[2][kStRows + 2 * R][kStPitch];
+    extern __shared__ __align__(16) float ring[];          // planes of kStRows + 2 R rows
+    constexpr int kPlane = (kStRows + 2 * R) * kStPitch;
     constexpr int N = 2 * R + 1;
     constexpr int kWarps = kStThreads / 32;
     constexpr int HR = (2 * R + kWarps - 1) / kWarps;     // extra rows a warp fetches per plane
@@ -86,9 +130,11 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
     const int shard = rest / P.chunks_z;
     const int sx = shard % P.px, sy = (shard / P.px) % P.py, sz = shard / (P.px * P.py);
     const int bz = P.bz[sz], by = P.by[sy], bx = P.bx[sx];
-    const int x0 = tx * kStCols, y0 = ty * kStRows, z0 = cz * kStChunk;
+    const int oo = P.out_off;
+    const int opy = by + 2 * oo, opx = bx + 2 * oo;
+    const int x0 = tx * kStCols, y0 = ty * kStRows, z0 = cz * P.chunk;
     if (x0 >= bx || y0 >= by || z0 >= bz) return;
-    const int z1 = min(z0 + kStChunk, bz);
+    const int z1 = min(z0 + P.chunk, bz);
     const int th = min(kStRows, by - y0), tw = min(kStCols, bx - x0);
     const int io = P.in_off;
     const int ipx = bx + 2 * io;                       // input row pitch of every shard in this worker column
@@ -100,217 +146,138 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
 #pragma unroll
     for (int r = 0; r < kStRpt; ++r) row_ok[r] = y0 + rw + r < by;
 
-    // Everything that does not change from plane to plane is resolved once: for each kind of load a
-    // base pointer (plane 0 of the owning shard, the thread's row and column; nullptr = zeros) and the
-    // plane stride of that shard, in elements (a shard holds fewer than 2^31 of them).
-    auto load4 = [&](const float *src) -> float4 {
-        if (VEC) return __ldg(reinterpret_cast<const float4 *>(src));
-        float4 v = make_float4(__ldg(src), 0.f, 0.f, 0.f);
-        if (x + 1 < bx) v.y = __ldg(src + 1);
-        if (x + 2 < bx) v.z = __ldg(src + 2);
-        if (x + 3 < bx) v.w = __ldg(src + 3);
-        return v;
-    };
-    const uint32_t ipy = (uint32_t)(by + 2 * io);
-    const uint32_t own_stride = ipy * (uint32_t)ipx;                   // the same in the shards below and above
-    const uint32_t own_off = (uint32_t)(y0 + rw + io) * (uint32_t)ipx + (uint32_t)(x + io);   // row 0 of the thread
-    const float *own_mid = col_ok ? P.in[shard] + own_off : nullptr;
-    const float *own_lo = col_ok && sz > 0 ? P.in[shard - P.py * P.px] + own_off : nullptr;
-    const float *own_hi = col_ok && sz + 1 < P.pz ? P.in[shard + P.py * P.px] + own_off : nullptr;
-    const int bz_lo = sz > 0 ? P.bz[sz - 1] : 0, bz_hi = sz + 1 < P.pz ? P.bz[sz + 1] : 0;
-    // this thread's cells of plane zp (any plane within R of the chunk), zeros outside the tensor
-    auto load_own = [&](int zp, float4 (&v)[kStRpt]) {
-        const float *base = own_mid;
-        if (zp < 0) {
-            base = own_lo;
-            zp += bz_lo;
-            if (zp < 0) base = nullptr;
-        } else if (zp >= bz) {
-            base = own_hi;
-            zp -= bz;
-            if (zp >= bz_hi) base = nullptr;
-        }
+    // Everything that does not change from plane to plane is resolved once: for each kind of copy a pointer that walks from plane to
+    // plane, the step (the plane stride of the owning shard, in elements: a shard holds fewer than 2^31 of them) and the bytes
+    // to read (0: zeros, and the pointer stands still)
+    // the columns that this thread copies of a row: its own four, or where rows are not aligned every 32nd
+    const int xc = VEC ? x : x0 + lane;
+    bool col_in[4];
 #pragma unroll
-        for (int r = 0; r < kStRpt; ++r) {
-            v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (base && row_ok[r]) v[r] = load4(base + (uint32_t)(zp + io) * own_stride + (uint32_t)(r * ipx));
+    for (int e = 0; e < 4; ++e) col_in[e] = VEC ? col_ok : xc + 32 * e < bx;
+    auto copy4 = [&](uint32_t dst, const float *src, uint32_t bytes, bool on) {
+        if (VEC) {
+            st_copy16(dst, src, bytes, on && col_ok);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) st_copy4(dst + 128 * e, src + 32 * e, bytes, on && col_in[e]);
         }
+    };
+    constexpr uint32_t kBytes = VEC ? 16 : 4;
+    const uint32_t copy_dst = (uint32_t)((kStLead + (VEC ? 4 : 1) * lane) * 4);
+    const uint32_t ipy = (uint32_t)(by + 2 * io);
+    const uint32_t own_off = (uint32_t)(y0 + rw + io) * (uint32_t)ipx + (uint32_t)(xc + io);   // row 0 of the thread
+    const uint32_t own_stride = ipy * (uint32_t)ipx;                   // the same in the shards below and above
+    const float *own_p = P.in[shard];
+    uint32_t own_bytes = 0;
+    // this thread's cell of plane zp (any plane within R of the chunk)
+    auto own_at = [&](int zp) {
+        int s3 = shard, n = bz;
+        if (zp < 0) {
+            s3 = sz > 0 ? shard - P.py * P.px : -1;
+            n = sz > 0 ? P.bz[sz - 1] : 0;
+            zp += n;
+        } else if (zp >= bz) {
+            s3 = sz + 1 < P.pz ? shard + P.py * P.px : -1;
+            n = sz + 1 < P.pz ? P.bz[sz + 1] : 0;
+            zp -= bz;
+        }
+        own_bytes = s3 >= 0 && col_in[0] && (unsigned)zp < (unsigned)n ? kBytes : 0u;
+        own_p = own_bytes ? P.in[s3] + ((uint32_t)(zp + io) * own_stride + own_off) : P.in[shard];
     };
     // extra rows of the current plane: row h of the 2R (R above the tile, R below) goes to warp h % kWarps
-    const float *hrow_base[HR];
-    uint32_t hrow_stride[HR];
-    int hrow_s[HR];
+    const float *hrow_p[HR];
+    uint32_t hrow_step[HR], hrow_bytes[HR], hrow_dst[HR];
 #pragma unroll
     for (int i = 0; i < HR; ++i) {
         const int h = warp + kWarps * i;
-        hrow_base[i] = nullptr;
-        hrow_stride[i] = 0;
-        hrow_s[i] = h < R ? h : R + th + (h - R);                      // its row in the shared-memory plane
+        hrow_p[i] = P.in[shard];
+        hrow_step[i] = hrow_bytes[i] = 0;
+        // its row in the shared-memory plane: the rows below follow the tile's last one
+        hrow_dst[i] = (uint32_t)(((h < R ? h : th + h) * kStPitch) * 4) + copy_dst;
         const int hy = h < R ? y0 - R + h : y0 + th + (h - R);
         int so, yo;
-        if (h < 2 * R && col_ok && st_owner(P.by, P.py, sy, hy, so, yo)) {
-            hrow_stride[i] = (uint32_t)(P.by[so] + 2 * io) * (uint32_t)ipx;
-            hrow_base[i] = P.in[(sz * P.py + so) * P.px + sx] + (uint32_t)(yo + io) * (uint32_t)ipx + (uint32_t)(x + io);
+        if (h < 2 * R && col_in[0] && st_owner(P.by, P.py, sy, hy, so, yo)) {
+            hrow_bytes[i] = kBytes;
+            hrow_step[i] = (uint32_t)(P.by[so] + 2 * io) * (uint32_t)ipx;
+            hrow_p[i] = P.in[(sz * P.py + so) * P.px + sx] + (uint32_t)(z0 + io) * hrow_step[i] +
+                        ((uint32_t)(yo + io) * (uint32_t)ipx + (uint32_t)(xc + io));
         }
     }
-    auto load_hrow = [&](int zp, float4 (&v)[HR]) {
-#pragma unroll
-        for (int i = 0; i < HR; ++i)
-            v[i] = hrow_base[i] ? load4(hrow_base[i] + (uint32_t)(zp + io) * hrow_stride[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    };
-    // threads 0 .. 8 * 2R - 1: one cell of an extra column of plane zp
+    // threads 0 .. 8 * 2R - 1: one cell of an extra column
     const int hc_row = threadIdx.x / (2 * R), hc_c = threadIdx.x % (2 * R);
     const bool hc_active = (int)threadIdx.x < kStRows * 2 * R && y0 + hc_row < by;
     const int hc_x = hc_c < R ? x0 - R + hc_c : x0 + tw + (hc_c - R);
-    const int hc_s = kStLead + (hc_x - x0);                               // its column in the shared-memory plane
-    const float *hcol_base = nullptr;
-    uint32_t hcol_stride = 0;
+    const uint32_t hcol_dst = (uint32_t)(((R + hc_row) * kStPitch + kStLead + (hc_x - x0)) * 4);
+    const float *hcol_p = P.in[shard];
+    uint32_t hcol_step = 0, hcol_bytes = 0;
     {
         int so, xo;
         if (hc_active && st_owner(P.bx, P.px, sx, hc_x, so, xo)) {
             const uint32_t pitch = (uint32_t)(P.bx[so] + 2 * io);
-            hcol_stride = ipy * pitch;
-            hcol_base = P.in[(sz * P.py + sy) * P.px + so] + (uint32_t)(y0 + hc_row + io) * pitch + (uint32_t)(xo + io);
+            hcol_bytes = 4u;
+            hcol_step = ipy * pitch;
+            hcol_p = P.in[(sz * P.py + sy) * P.px + so] + (uint32_t)(z0 + io) * hcol_step + ((uint32_t)(y0 + hc_row + io) * pitch + (uint32_t)(xo + io));
         }
     }
-    auto load_hcol = [&](int zp) -> float {
-        return hcol_base ? __ldg(hcol_base + (uint32_t)(zp + io) * hcol_stride) : 0.f;
-    };
-
-    // prime: planes z0 - R .. z0 + R, extra rows / column of plane z0
-    float4 q[N][kStRpt];
+    const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+    const uint32_t own_dst = ring_s + (uint32_t)((R + rw) * kStPitch * 4) + copy_dst;
+    own_at(z0 - R);
+    // plane zp into the slot `at` bytes into the ring: own cells, and if it is to be the current one a vector of each extra row and
+    // one extra-column cell; cells beyond the bulk are written by the extra-row / extra-column threads only
+    auto issue = [&](int zp, uint32_t at) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) load_own(z0 - R + i, q[i]);
-    float4 hrow[HR];
-    load_hrow(z0, hrow);
-    float hcol = load_hcol(z0);
-
-    const int oo = P.out_off;
-    const int opy = by + 2 * oo, opx = bx + 2 * oo;
-    float *optr = P.out[shard] + ((size_t)(z0 + oo) * opy + (size_t)(y0 + rw + oo)) * opx + (x + oo);
-    const size_t oplane = (size_t)opy * opx;
-    const bool clear_x = P.clear_ghosts && oo > 0;
-
-    auto put4 = [&](float *d, const float4 &v) {      // own / extra-row cells into the shared-memory plane
-        if (VEC) {
-            *reinterpret_cast<float4 *>(d) = v;
-        } else {
-            d[0] = v.x;
-            if (x + 1 < bx) d[1] = v.y;
-            if (x + 2 < bx) d[2] = v.z;
-            if (x + 3 < bx) d[3] = v.w;
+        for (int r = 0; r < kStRpt; ++r) copy4(own_dst + at + (uint32_t)(r * kStPitch * 4), own_p + r * ipx, own_bytes, row_ok[r]);
+        if (zp + 1 == 0 || zp + 1 == bz) own_at(zp + 1);
+        else own_p += own_bytes ? own_stride : 0u;
+        if (zp >= z0 && zp < z1) {
+#pragma unroll
+            for (int i = 0; i < HR; ++i) {
+                copy4(ring_s + at + hrow_dst[i], hrow_p[i], hrow_bytes[i], (2 * R) % kWarps == 0 || warp + kWarps * i < 2 * R);
+                hrow_p[i] += hrow_step[i];
+            }
+            st_copy4(ring_s + at + hcol_dst, hcol_p, hcol_bytes, hc_active);
+            hcol_p += hcol_step;
         }
     };
 
-    // One plane per turn; q[j] is the plane j - R away from the current one.  The queue is shifted by
-    // register moves at the end of a turn: rotating it at compile time instead needs 2R+1 copies of the
-    // loop body, which no longer fit the instruction cache (measured: 13 % slower).
-    for (int z = z0; z < z1; ++z) {
-        float(*pl)[kStPitch] = plane[(z - z0) & 1];
-        // current plane into shared memory: own cells, the extra-row vectors, one extra-column cell.
-        // Cells beyond the bulk are written by the extra-row / extra-column threads only.
-        if (col_ok) {
+    // sums of the outputs p - R .. p + R around plane p
+    uint64_t acc[N][kStRpt][2];
 #pragma unroll
-            for (int r = 0; r < kStRpt; ++r)
-                if (row_ok[r]) put4(&pl[R + rw + r][kStLead + 4 * lane], q[R][r]);
+    for (int i = 0; i < N; ++i)
 #pragma unroll
-            for (int i = 0; i < HR; ++i)
-                if (warp + kWarps * i < 2 * R) put4(&pl[hrow_s[i]][kStLead + 4 * lane], hrow[i]);
-        }
-        if (hc_active) pl[R + hc_row][hc_s] = hcol;
-        // next plane's values, one step early
-        float4 lead[kStRpt], hrow_n[HR];
-        float hcol_n = 0.f;
-        if (z + 1 < z1) {
-            load_own(z + 1 + R, lead);
-            load_hrow(z + 1, hrow_n);
-            hcol_n = load_hcol(z + 1);
-        } else {
+        for (int r = 0; r < kStRpt; ++r) acc[i][r][0] = acc[i][r][1] = 0ull;
+    // a plane's cells as z neighbours (the middle tap: the three centre taps together); the sums move on by one slot
+    auto z_taps = [&](const float4 (&v)[kStRpt]) {
 #pragma unroll
-            for (int r = 0; r < kStRpt; ++r) lead[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int i = 0; i < HR; ++i) hrow_n[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-
-        if (col_ok && row_ok[0]) {
-            float o[kStRpt][4];
-#pragma unroll
-            for (int r = 0; r < kStRpt; ++r)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) o[r][e] = 0.f;
-            // z neighbours: registers
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const float wz = P.w[0][k];
-#pragma unroll
-                for (int r = 0; r < kStRpt; ++r) {
-                    const float4 v = q[k][r];
-                    o[r][0] = fmaf(wz, v.x, o[r][0]);
-                    o[r][1] = fmaf(wz, v.y, o[r][1]);
-                    o[r][2] = fmaf(wz, v.z, o[r][2]);
-                    o[r][3] = fmaf(wz, v.w, o[r][3]);
-                }
-            }
-            // y neighbours: the rows rw .. rw + 2R + RPT - 1 of the plane, each read once and used by every
-            // row of the thread it is a neighbour of (tap k of row r is plane row rw + r + k)
-#pragma unroll
-            for (int j = 0; j < N + kStRpt - 1; ++j) {
-                float4 v;
-                // the thread's own rows come from its registers -- unless such a row lies beyond the bulk (a ragged
-                // last tile): then that plane row holds an extra row fetched from the shard below
-                const bool own = j >= R && j < R + kStRpt && row_ok[j >= R && j < R + kStRpt ? j - R : 0];
-                if (own) v = q[R][j >= R && j < R + kStRpt ? j - R : 0];
-                else if (VEC) v = *reinterpret_cast<const float4 *>(&pl[rw + j][kStLead + 4 * lane]);
-                else {
-                    const float *s = &pl[rw + j][kStLead + 4 * lane];
-                    v = make_float4(s[0], s[1], s[2], s[3]);
-                }
-#pragma unroll
-                for (int r = 0; r < kStRpt; ++r) {
-                    const int k = j - r;
-                    if (k < 0 || k >= N) continue;
-                    const float wy = P.w[1][k];
-                    o[r][0] = fmaf(wy, v.x, o[r][0]);
-                    o[r][1] = fmaf(wy, v.y, o[r][1]);
-                    o[r][2] = fmaf(wy, v.z, o[r][2]);
-                    o[r][3] = fmaf(wy, v.w, o[r][3]);
-                }
-            }
-            // x neighbours: the vectors left and right of the own one
+        for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int r = 0; r < kStRpt; ++r) {
-                float xs[12];
-                const float4 l = *reinterpret_cast<const float4 *>(&pl[R + rw + r][4 * lane]);
-                const float4 rt = *reinterpret_cast<const float4 *>(&pl[R + rw + r][4 * lane + 8]);
-                xs[0] = l.x; xs[1] = l.y; xs[2] = l.z; xs[3] = l.w;
-                if (VEC) {
-                    const float4 c = q[R][r];
-                    xs[4] = c.x; xs[5] = c.y; xs[6] = c.z; xs[7] = c.w;
-                } else {
-                    // a ragged last vector: its cells beyond the bulk are extra-column cells, not the thread's own
-                    const float4 c = *reinterpret_cast<const float4 *>(&pl[R + rw + r][kStLead + 4 * lane]);
-                    xs[4] = c.x; xs[5] = c.y; xs[6] = c.z; xs[7] = c.w;
-                }
-                xs[8] = rt.x; xs[9] = rt.y; xs[10] = rt.z; xs[11] = rt.w;
-#pragma unroll
-                for (int k = 0; k < N; ++k) {
-                    const float wx = P.w[2][k];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) o[r][e] = fmaf(wx, xs[4 + e + k - R], o[r][e]);
-                }
+                acc[i][r][0] = fma2(P.w2[0][2 * R - i], pack2(v[r].x, v[r].y), i + 1 < N ? acc[i + 1 < N ? i + 1 : i][r][0] : 0ull);
+                acc[i][r][1] = fma2(P.w2[0][2 * R - i], pack2(v[r].z, v[r].w), i + 1 < N ? acc[i + 1 < N ? i + 1 : i][r][1] : 0ull);
             }
+    };
+
+    float *optr = P.out[shard] + ((size_t)(z0 + oo) * opy + (size_t)(y0 + rw + oo)) * opx + (x + oo);
+    const size_t oplane = (size_t)opy * opx;
+    const bool clear_x = P.clear_ghosts && oo > 0 && (x == 0 || x + 4 >= bx);   // threads at the row ends
+
+    // output plane z - R is complete
+    auto store = [&]() {
+        if (col_ok && row_ok[0]) {
 #pragma unroll
             for (int r = 0; r < kStRpt; ++r) {
                 if (!row_ok[r]) continue;
+                float o[4];
+                unpack2(acc[0][r][0], o[0], o[1]);
+                unpack2(acc[0][r][1], o[2], o[3]);
                 float *op = optr + (size_t)r * opx;
-                if (VEC) {
-                    *reinterpret_cast<float4 *>(op) = make_float4(o[r][0], o[r][1], o[r][2], o[r][3]);
+                if (R == 4 ? VEC : P.vec_out) {
+                    *reinterpret_cast<float4 *>(op) = make_float4(o[0], o[1], o[2], o[3]);
                 } else {
-                    op[0] = o[r][0];
-                    if (x + 1 < bx) op[1] = o[r][1];
-                    if (x + 2 < bx) op[2] = o[r][2];
-                    if (x + 3 < bx) op[3] = o[r][3];
+                    op[0] = o[0];
+                    if (x + 1 < bx) op[1] = o[1];
+                    if (x + 2 < bx) op[2] = o[2];
+                    if (x + 3 < bx) op[3] = o[3];
                 }
                 // adjoint: the ghost columns beside this row are cleared by the threads that write the row's
                 // ends, so that they land in the same lines of memory as the row itself
@@ -329,53 +296,123 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
             }
         }
         optr += oplane;
-#pragma unroll
-        for (int i = 0; i + 1 < N; ++i)
-#pragma unroll
-            for (int r = 0; r < kStRpt; ++r) q[i][r] = q[i + 1][r];
-#pragma unroll
-        for (int r = 0; r < kStRpt; ++r) q[N - 1][r] = lead[r];
-#pragma unroll
-        for (int i = 0; i < HR; ++i) hrow[i] = hrow_n[i];
-        hcol = hcol_n;
+    };
+#pragma unroll 1
+    for (int i = 0; i < kStDepth - 1; ++i) {
+        if (z0 - R + i < z1 + R) issue(z0 - R + i, i * kPlane * 4);
+        cp_async_commit();
     }
-
+    // in the shadow of the first planes' arrival (ahead of their copies it costs 12 us of 233 at 512^3, clearing or not)
     if (P.clear_ghosts && oo > 0) {
-        // this block's part of the ghost shell of the output shard: its box of bulk cells, extended
-        // through the ghost layers wherever it touches a face of the shard
-        const int zl = z0 == 0 ? 0 : z0 + oo, zh = z1 == bz ? bz + 2 * oo : z1 + oo;
-        const int yl = y0 == 0 ? 0 : y0 + oo, yh = y0 + th == by ? by + 2 * oo : y0 + th + oo;
-        const int xl = x0 == 0 ? 0 : x0 + oo, xh = x0 + tw == bx ? bx + 2 * oo : x0 + tw + oo;
-        float *ob = P.out[shard];
-        const int ny = yh - yl, nx = xh - xl;
-        // whole planes of the ghost layers below / above
-        for (int pz = zl; pz < zh; ++pz) {
-            if (pz >= oo && pz < bz + oo) continue;
-            for (int idx = threadIdx.x; idx < ny * nx; idx += kStThreads)
-                ob[((size_t)pz * opy + (yl + idx / nx)) * opx + (xl + idx % nx)] = 0.f;
+        const int ny = (by + kStRows - 1) / kStRows, nx = (bx + kStCols - 1) / kStCols;   // this shard's blocks
+        st_clear<VEC && R == 4>(P.out[shard], bz, opy, opx, oo, (cz * ny + ty) * nx + tx, (bz + P.chunk - 1) / P.chunk * ny * nx);
+    }
+    uint32_t at = 0;                                       // slot of this plane, in bytes; the one before it is free
+#pragma unroll 1
+    for (int z = z0 - R; z < z1 + R; ++z) {
+        const bool centre = z >= z0 && z < z1;             // the planes around the chunk are only z neighbours
+        cp_async_wait_group<kStDepth - 2>();
+        __syncthreads();                                   // this plane has arrived; the one before it has been read
+        if (z + kStDepth - 1 < z1 + R) issue(z + kStDepth - 1, at == 0 ? (kStDepth - 1) * kPlane * 4 : at - kPlane * 4);
+        cp_async_commit();
+        const float *pl = reinterpret_cast<const float *>(reinterpret_cast<const char *>(ring) + at);
+        at = at == (kStDepth - 1) * kPlane * 4 ? 0u : at + kPlane * 4;
+        float4 cur[kStRpt];
+#pragma unroll
+        for (int r = 0; r < kStRpt; ++r) {
+            const float *c = pl + (R + rw + r) * kStPitch + kStLead + 4 * lane;
+            cur[r] = *reinterpret_cast<const float4 *>(c);
         }
-        // planes of the bulk: ghost rows over the whole width (the ghost columns beside bulk rows were
-        // cleared together with those rows)
-        const int gy_lo = y0 == 0 ? oo : 0, gy = gy_lo + (y0 + th == by ? oo : 0);
-        const int per_plane = gy * nx;
-        if (per_plane > 0) {
-            const int total = (z1 - z0) * per_plane;
-            for (int idx = threadIdx.x; idx < total; idx += kStThreads) {
-                const int pz = z0 + oo + idx / per_plane;
-                const int e = idx % per_plane, r = e / nx;
-                const int py = r < gy_lo ? r : by + oo + (r - gy_lo);
-                ob[((size_t)pz * opy + py) * opx + (xl + e % nx)] = 0.f;
+        z_taps(cur);
+        if (centre && col_ok && row_ok[0]) {
+            // x neighbours: the vectors left and right of the own one; shifts by an even number of columns as pairs
+#pragma unroll
+            for (int r = 0; r < kStRpt; ++r) {
+                float xs[12], o[4];
+                const float4 l = *reinterpret_cast<const float4 *>(pl + (R + rw + r) * kStPitch + 4 * lane);
+                const float4 rt = *reinterpret_cast<const float4 *>(pl + (R + rw + r) * kStPitch + 4 * lane + 8);
+                xs[0] = l.x; xs[1] = l.y; xs[2] = l.z; xs[3] = l.w;
+                const float4 c = cur[r];
+                xs[4] = c.x; xs[5] = c.y; xs[6] = c.z; xs[7] = c.w;
+                xs[8] = rt.x; xs[9] = rt.y; xs[10] = rt.z; xs[11] = rt.w;
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    if (k == R || ((k - R) & 1)) continue;
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+                        acc[R][r][p] = fma2(P.w2[2][k], pack2(xs[4 + 2 * p + k - R], xs[5 + 2 * p + k - R]), acc[R][r][p]);
+                }
+                unpack2(acc[R][r][0], o[0], o[1]);
+                unpack2(acc[R][r][1], o[2], o[3]);
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    if (!((k - R) & 1)) continue;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[e] = fmaf(P.w[2][k], xs[4 + e + k - R], o[e]);
+                }
+                acc[R][r][0] = pack2(o[0], o[1]);
+                acc[R][r][1] = pack2(o[2], o[3]);
             }
+            // y neighbours: the rows rw .. rw + 2R + RPT - 1 of the plane, each read once and used by every
+            // row of the thread it is a neighbour of (tap k of row r is plane row rw + r + k)
+            auto y_taps = [&](int j, const float4 &v) {
+#pragma unroll
+                for (int r = 0; r < kStRpt; ++r) {
+                    const int k = j - r;
+                    if (k < 0 || k >= N || k == R) continue;
+                    acc[R][r][0] = fma2(P.w2[1][k], pack2(v.x, v.y), acc[R][r][0]);
+                    acc[R][r][1] = fma2(P.w2[1][k], pack2(v.z, v.w), acc[R][r][1]);
+                }
+            };
+            // its own rows are in registers already (in a ragged last tile such a row may be an extra row of the plane)
+#pragma unroll
+            for (int r = 0; r < kStRpt; ++r) y_taps(R + r, cur[r]);
+#pragma unroll
+            for (int j = 0; j < N + kStRpt - 1; ++j)
+                if (j < R || j >= R + kStRpt) y_taps(j, *reinterpret_cast<const float4 *>(pl + (rw + j) * kStPitch + kStLead + 4 * lane));
         }
+        if (z >= z0 + R) store();
     }
 }
 
 template <int R>
 static distdl_status_t launch_stencil(const StencilParams &P, unsigned grid, bool vec, cudaStream_t s) {
-    if (vec) stencil3d_kernel<R, true><<<grid, kStThreads, 0, s>>>(P);
-    else stencil3d_kernel<R, false><<<grid, kStThreads, 0, s>>>(P);
+    constexpr int smem = st_smem_bytes<R>();
+    static bool configured_on[kMaxDevicesPerProcess] = {false};
+    int dev = 0;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevicesPerProcess)
+        return fail(DISTDL_ERR_UNSUPPORTED, "device index %d: at most %d devices per process", dev, kMaxDevicesPerProcess);
+    {
+        std::lock_guard<std::mutex> setup_lock(setup_mutex());
+        if (!configured_on[dev]) {
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            configured_on[dev] = true;
+        }
+    }
+    if (vec) stencil3d_kernel<R, true><<<grid, kStThreads, smem, s>>>(P);
+    else stencil3d_kernel<R, false><<<grid, kStThreads, smem, s>>>(P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
+}
+
+// Planes per block.  A block's time goes with its planes and the 2R around them, and with how many blocks share its
+// multiprocessor: 0.62 / 0.79 / 0.96 us a plane for one, two, three of them.  Small chunks fill the device and even out its last
+// wave, long ones read fewer planes twice: of the chunks in steps of a quarter the one with the least time by this count.
+static int32_t st_chunk(int64_t planes, int64_t tiles, int radius, int sms) {
+    const int64_t resident = radius <= 2 ? kStBlocks<2> : kStBlocks<4>;
+    int64_t best = planes, best_cost = INT64_MAX;
+    for (int64_t c = 4;; c += std::max<int64_t>(1, c / 4)) {
+        const int64_t chunks = (planes + c - 1) / c, chunk = (planes + chunks - 1) / chunks;
+        const int64_t n = (tiles * chunks + sms - 1) / sms, last = n % resident;
+        const int64_t cost = (n / resident * (45 + 17 * resident) + (last ? 45 + 17 * last : 0)) * (chunk + 2 * radius);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = chunk;
+        }
+        if (c >= planes) return (int32_t)best;
+    }
 }
 
 static distdl_status_t stencil_impl(const distdl_partition *p, const void *const *in, const float *w, int32_t radius,
@@ -407,12 +444,20 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
     P.clear_ghosts = adj ? 1 : 0;
     P.tiles_x = (int32_t)((mx + kStCols - 1) / kStCols);
     P.tiles_y = (int32_t)((my + kStRows - 1) / kStRows);
-    P.chunks_z = (int32_t)((mz + kStChunk - 1) / kStChunk);
     for (int d = 0; d < 3; ++d)
         for (int k = 0; k <= 2 * radius; ++k) P.w[d][k] = adj ? w[d * (2 * radius + 1) + (2 * radius - k)] : w[d * (2 * radius + 1) + k];
-    // 16-byte accesses: every row of every layout starts on a 16-byte boundary and holds whole vectors
-    bool vec = (P.in_off % 4) == 0 && (P.out_off % 4) == 0;
-    for (int32_t c = 0; c < p->pshape[2]; ++c) vec = vec && (P.bx[c] % 4) == 0;
+    P.w[0][radius] = (float)((double)P.w[0][radius] + (double)P.w[1][radius] + (double)P.w[2][radius]);
+    for (int d = 0; d < 3; ++d)
+        for (int k = 0; k <= 2 * radius; ++k) {
+            uint32_t bits;
+            memcpy(&bits, &P.w[d][k], 4);
+            P.w2[d][k] = (uint64_t)bits << 32 | bits;
+        }
+    // 16-byte accesses: every row of the layout starts on a 16-byte boundary and holds whole vectors
+    bool whole = true;
+    for (int32_t c = 0; c < p->pshape[2]; ++c) whole = whole && (P.bx[c] % 4) == 0;
+    const bool vec = whole && P.in_off % 4 == 0;
+    P.vec_out = whole && P.out_off % 4 == 0;
     for (int32_t wk = 0; wk < p->num_workers; ++wk) {
         if (!in[wk] || !out[wk]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shard pointer %d is NULL", what, wk);
         if (!aligned16(in[wk]) || !aligned16(out[wk])) return fail(DISTDL_ERR_ALIGNMENT, "%s: shard %d is not 16-byte aligned", what, wk);
@@ -420,6 +465,11 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
         P.in[wk] = (const float *)in[wk];
         P.out[wk] = (float *)out[wk];
     }
+    int dev = 0, sms = 0;
+    DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+    DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    P.chunk = st_chunk(mz, (int64_t)p->num_workers * P.tiles_y * P.tiles_x, radius, sms);
+    P.chunks_z = (int32_t)((mz + P.chunk - 1) / P.chunk);
     const int64_t blocks = (int64_t)p->num_workers * P.chunks_z * P.tiles_y * P.tiles_x;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     cudaStream_t s = (cudaStream_t)stream;

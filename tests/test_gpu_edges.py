@@ -131,3 +131,20 @@ def test_pool_max_of_special_values(stride):
                     best, where = x[p, q], k
             yr[i, j], ar[i, j] = best, where
     assert parity.same_bits(parity.host(y)[0, 0], yr) and parity.same_bits(parity.host(a)[0, 0], ar)
+
+
+# global shape, partition, radius
+STENCIL_EDGES = [
+    ((3, 3, 3), (1, 1, 1), 4),               # a shard smaller than the radius
+    ((1, 1, 5), (1, 1, 1), 1),               # one plane, one row
+    ((9, 10, 64), (1, 1, 1), 2),             # whole vectors on one side only: scalar copies in, vectors out, and the other way round
+    ((6, 21, 132), (1, 1, 1), 3),            # a second column tile of one vector, a last row tile of five rows
+    ((301, 8, 12), (1, 1, 1), 3),            # many chunks of planes, the last one short
+    ((10, 17, 258), (2, 2, 2), 4),           # rows 9 and 8, columns 129: shards with different numbers of tiles share the clearing
+    ((13, 9, 260), (3, 1, 2), 4),            # planes 5, 4, 4: neighbours exactly as deep as the radius
+]
+
+
+@pytest.mark.parametrize("case", STENCIL_EDGES, ids=[str(c) for c in STENCIL_EDGES])
+def test_stencil_planes_and_rows(case):
+    parity.test_stencil3d_fwd_and_adj(case)
