@@ -21,7 +21,7 @@
 // one plane of registers does not cover the latency of device memory.  One barrier per plane.  Rows that do not start on
 // 16-byte boundaries (R < 4 on the padded side) are copied four bytes a lane, a warp's cells next to one another.
 // Issue bounds it, not memory: 116 of ~300 instructions a plane are the warp's FMA (25 taps on eight cells, pairs
-// packed but for the odd column shifts), and a fourth block per multiprocessor spills (301 against 233 us).  At 512^3, R = 4,
+// packed but for the odd column shifts), and a fourth block per multiprocessor makes it 301 us from 233.  At 512^3, R = 4,
 // forward 308 -> 233 us, adjoint 365 -> 264 us, where reading and writing the bulk once takes 164 us and 170 us.  The rest
 // of the radii and sizes gain by the rule for the chunks as well (200^3, R = 2: 61 -> 32 and 78 -> 31 us; 64^3, R = 4: 40 -> 6.4 us).
 #include <algorithm>
@@ -42,8 +42,11 @@ constexpr int kStCols = 128;          // columns of a tile = 32 lanes x 4
 constexpr int kStLead = 4;            // shared-memory column of the tile's first column (keeps rows 16-byte aligned)
 constexpr int kStPitch = kStLead + kStCols + 4;   // 136 floats
 constexpr int kStDepth = 5;           // planes in the ring (4 and 6 measure the same within 2 %)
-template <int R>
-constexpr int kStBlocks = R <= 2 ? 4 : 3;   // blocks per multiprocessor (registers: 128 / 168)
+// Blocks per multiprocessor.  With 16-byte copies a fourth block of the wide stars costs more in registers (128 instead of 168: moves and
+// spills) than it hides; scalar copies have latency left for it (22 x 126 x 103 shards, R = 4, 576 blocks: 56 -> 48 and 74 -> 58 us; a
+// single 240 x 155 x 201 shard: 35 -> 39 us).
+template <int R, bool VEC>
+constexpr int kStBlocks = VEC && R >= 3 ? 3 : 4;
 
 struct StencilParams {
     const float *in[kStMaxWorkers];
@@ -112,7 +115,7 @@ __device__ __forceinline__ void st_clear(float *out, int bz, int opy, int opx, i
 }
 
 template <int R, bool VEC>
-__global__ void __launch_bounds__(kStThreads, kStBlocks<R>)
+__global__ void __launch_bounds__(kStThreads, kStBlocks<R, VEC>)
 stencil3d_kernel(const __grid_constant__ StencilParams P) {
     extern __shared__ __align__(16) float ring[];          // planes of kStRows + 2 R rows
     constexpr int kPlane = (kStRows + 2 * R) * kStPitch;
@@ -400,8 +403,8 @@ static distdl_status_t launch_stencil(const StencilParams &P, unsigned grid, boo
 // Planes per block.  A block's time goes with its planes and the 2R around them, and with how many blocks share its
 // multiprocessor: 0.62 / 0.79 / 0.96 us a plane for one, two, three of them.  Small chunks fill the device and even out its last
 // wave, long ones read fewer planes twice: of the chunks in steps of a quarter the one with the least time by this count.
-static int32_t st_chunk(int64_t planes, int64_t tiles, int radius, int sms) {
-    const int64_t resident = radius <= 2 ? kStBlocks<2> : kStBlocks<4>;
+static int32_t st_chunk(int64_t planes, int64_t tiles, int radius, bool vec, int sms) {
+    const int64_t resident = !vec ? kStBlocks<4, false> : radius <= 2 ? kStBlocks<2, true> : kStBlocks<4, true>;
     int64_t best = planes, best_cost = INT64_MAX;
     for (int64_t c = 4;; c += std::max<int64_t>(1, c / 4)) {
         const int64_t chunks = (planes + c - 1) / c, chunk = (planes + chunks - 1) / chunks;
@@ -468,7 +471,7 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
     int dev = 0, sms = 0;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
     DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    P.chunk = st_chunk(mz, (int64_t)p->num_workers * P.tiles_y * P.tiles_x, radius, sms);
+    P.chunk = st_chunk(mz, (int64_t)p->num_workers * P.tiles_y * P.tiles_x, radius, vec, sms);
     P.chunks_z = (int32_t)((mz + P.chunk - 1) / P.chunk);
     const int64_t blocks = (int64_t)p->num_workers * P.chunks_z * P.tiles_y * P.tiles_x;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
