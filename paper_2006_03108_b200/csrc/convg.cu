@@ -21,14 +21,14 @@
 namespace distdl {
 
 constexpr int kCgThreads = 128;
-constexpr int kCgPx = 8;                // consecutive pixels of a row per thread
 constexpr int kCgMaxPairs = 4;          // output-channel pairs per thread
 constexpr int kMaxChanBlocks = 8;       // P_co, P_ci
 constexpr int kMaxGroups = 128;         // groups of up to 2 * kCgMaxPairs output channels
 
-// Shape of the tiles of one launch.  A tile is tn images x th rows x 8 * seg columns of one shard and one group of
-// output channels; thread -> (image, row, segment of eight columns).
+// Shape of the tiles of one launch.  A tile is tn images x th rows x px * seg columns of one shard and one group of
+// output channels; thread -> (image, row, segment of px columns).
 struct CgShape {
+    int32_t px;                         // consecutive pixels of a row per thread: 8 or 4
     int32_t tn, th, seg;
     int32_t rows, cols, pitch;          // staged rows and columns of one image, floats from row to row
     int32_t tile_floats;                // one staged channel
@@ -50,26 +50,31 @@ struct ConvGParams {
     FastDiv groups, tiles_x, pw_div, tiles_y, ph_div, cols, rows, tn, seg, half_th;
 };
 
-// What bounds it: the fp32 pipe.  A thread owns eight pixels of a row and up to eight output channels; the accumulators
+// Blocks per SM that the registers allow: 168 a thread for eight pixels (a whole row of taps read ahead), 128 for four.
+constexpr int cg_blocks(int px) { return px == 8 ? 3 : 4; }
+
+// What bounds it: the fp32 pipe.  A thread owns PX pixels of a row and up to eight output channels; the accumulators
 // are pairs of channels, so a weight pair is two neighbouring floats of the staged table (one 16-byte broadcast read
-// feeds two pairs) and an input value is duplicated once and used by every tap and channel: 5 x 5, eight channels, 800
-// packed FMAs per input channel and thread beside about 125 other instructions.  With pairs of pixels instead (two
-// channels per thread, as many packed FMAs as now for a quarter of the outputs) every input channel was staged four
-// times as often.
+// feeds two pairs) and an input value is duplicated once and used by every tap and channel: 5 x 5, eight channels, eight
+// pixels, 800 packed FMAs per input channel and thread beside about 125 other instructions.  With pairs of pixels instead
+// (two channels per thread, as many packed FMAs as now for a quarter of the outputs) every input channel was staged four
+// times as often.  The rows of taps are unrolled, so that the next row's reads overlap the FMAs of this one; that takes
+// 168 registers with eight pixels, and three blocks an SM are faster with it than four without (1.14 -> 1.10 ms below).
+// Blocks of one or two warps instead, one image each: 54 us instead of 40, the weights are staged for fewer outputs.
 //
-// Measured (forward / adjoint, B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.14 / 1.16 ms = 47 TFLOP/s
+// Measured (forward / adjoint, B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.10 / 1.12 ms = 49 TFLOP/s
 // (1.48 / 1.59 ms with two channels a block; packed FMAs alone, as an outer product in registers, reach 59 TFLOP/s);
-// 6 -> 16 channels, 256 images of 28 x 28 on 2 x 2 workers 0.044 / 0.050 ms (0.82 / 0.79 ms).
+// 6 -> 16 channels, 256 images of 28 x 28 on 2 x 2 workers 0.040 / 0.044 ms (0.82 / 0.79 ms).
 //
 // Small images are packed: a tile may span several images, so 14 x 14 shards fill the threads (32 x 128 tiles left 95 %
 // of them idle).  Cells are staged one by one (4-byte asynchronous copies), which takes any row pitch and any mixture of
 // neighbours; where each cell comes from is worked out once per tile and kept in a table, a channel then costs one table
 // read, one pointer read and one copy per cell.  Two buffers, one barrier per input channel.
-template <int K, bool ADJ, int CP>
-__global__ void __launch_bounds__(kCgThreads, K == 7 ? 3 : 4)
+template <int K, bool ADJ, int CP, int PX>
+__global__ void __launch_bounds__(kCgThreads, cg_blocks(PX))
 convg_kernel(const __grid_constant__ ConvGParams G) {
     constexpr int PH = K / 2, CT = 2 * CP;
-    constexpr int NF = ((kCgPx + K - 1 + 3) / 4) * 4;      // floats of a thread's window per row
+    constexpr int NF = ((PX + K - 1 + 3) / 4) * 4;         // floats of a thread's window per row
     constexpr int WF = ((K * K * CT + 3) / 4) * 4;
     constexpr int io = ADJ ? 0 : PH, oo = ADJ ? PH : 0;    // ghost width of the input / output layout
     extern __shared__ __align__(16) float smem[];
@@ -88,7 +93,7 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
     const int r = (int)fast_rem(G.ph_div, id);
     const int n0 = (int)id * T.tn;
     const int bh = G.bh[r], bw = G.bw[c];
-    const int i0 = ty * T.th, j0 = tx * kCgPx * T.seg;
+    const int i0 = ty * T.th, j0 = tx * PX * T.seg;
     if (i0 >= bh || j0 >= bw) return;                      // shards smaller than the largest
     const int ob = G.grp_block[g], o0 = G.grp_first[g], oc = G.grp_count[g];
     const int spatial = G.ph * G.pw;
@@ -185,10 +190,10 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
     const int seg = (int)fast_rem(G.seg, rest);
     const int row = 2 * (int)fast_rem(G.half_th, rest) + (tid & 1);
     const int img = (int)rest;
-    const bool active = img < T.tn && n0 + img < G.batch && i0 + row < bh && j0 + kCgPx * seg < bw;
-    const int xoff = (img * T.rows + row) * T.pitch + kCgPx * seg;
+    const bool active = img < T.tn && n0 + img < G.batch && i0 + row < bh && j0 + PX * seg < bw;
+    const int xoff = (img * T.rows + row) * T.pitch + PX * seg;
 
-    uint64_t acc[kCgPx][CP];
+    uint64_t acc[PX][CP];
 #pragma unroll
     for (int q = 0; q < CP; ++q) {
         float b0 = 0.f, b1 = 0.f;
@@ -197,7 +202,7 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
             if (2 * q + 1 < oc) b1 = __ldg(G.bias[ob] + o0 + 2 * q + 1);
         }
 #pragma unroll
-        for (int p = 0; p < kCgPx; ++p) acc[p][q] = pack2(b0, b1);
+        for (int p = 0; p < PX; ++p) acc[p][q] = pack2(b0, b1);
     }
 
     int sib = 0, scl = 0;                   // channel to stage next
@@ -230,7 +235,7 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
         if (active) {
             const float *xb = tiles + buf * T.tile_floats + xoff;
             const float *wb = wbuf + buf * WF;
-#pragma unroll 1
+#pragma unroll
             for (int a = 0; a < K; ++a) {
                 float x[NF];
 #pragma unroll
@@ -241,9 +246,9 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
                     x[4 * v + 2] = f.z;
                     x[4 * v + 3] = f.w;
                 }
-                uint64_t xx[kCgPx + K - 1];
+                uint64_t xx[PX + K - 1];
 #pragma unroll
-                for (int v = 0; v < kCgPx + K - 1; ++v) xx[v] = pack2(x[v], x[v]);
+                for (int v = 0; v < PX + K - 1; ++v) xx[v] = pack2(x[v], x[v]);
 #pragma unroll
                 for (int b = 0; b < K; ++b) {
                     uint64_t w[CP];
@@ -259,7 +264,7 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
                         for (int q = 0; q < CP; ++q) w[q] = *reinterpret_cast<const uint64_t *>(wb + b * CT + 2 * q);
                     }
 #pragma unroll
-                    for (int p = 0; p < kCgPx; ++p)
+                    for (int p = 0; p < PX; ++p)
 #pragma unroll
                         for (int q = 0; q < CP; ++q) acc[p][q] = fma2(xx[p + b], w[q], acc[p][q]);
                 }
@@ -272,14 +277,14 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
 
     // Store: two channels at a time through shared memory, so that a warp writes consecutive cells whatever the row pitch.
     // The rectangle written is the tile, in the adjoint extended through the ghost layers wherever it touches a face.
-    const int th = min(T.th, bh - i0), tw = min(kCgPx * T.seg, bw - j0), imgs = min(T.tn, G.batch - n0);
+    const int th = min(T.th, bh - i0), tw = min(PX * T.seg, bw - j0), imgs = min(T.tn, G.batch - n0);
     const int top = ADJ && i0 == 0 ? oo : 0, bottom = ADJ && i0 + th == bh ? oo : 0;
     const int left = ADJ && j0 == 0 ? oo : 0, right = ADJ && j0 + tw == bw ? oo : 0;
     const int er = th + top + bottom, ew = tw + left + right;
     const uint32_t pitch_o = (uint32_t)(bw + 2 * oo), plane_o = (uint32_t)(bh + 2 * oo) * pitch_o;
     const int chan = G.cnt_out[ob];
     float *obase = G.out[ob * spatial + r * G.pw + c] + ((size_t)n0 * chan + o0) * plane_o;
-    const int spitch = kCgPx * T.seg;
+    const int spitch = PX * T.seg;
     __syncthreads();                        // the tiles and the cell table are free
     for (int idx = tid; idx < imgs * er; idx += kCgThreads) {
         const int im = idx / er, y = idx - im * er;
@@ -296,14 +301,15 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
         if (2 * q >= oc) break;
         if (q > 0) __syncthreads();
         if (active) {
-            float lo[kCgPx], hi[kCgPx];
+            float lo[PX], hi[PX];
 #pragma unroll
-            for (int p = 0; p < kCgPx; ++p) unpack2(acc[p][q], lo[p], hi[p]);
-            float *d = tiles + (img * T.th + row) * spitch + kCgPx * seg;
-            *reinterpret_cast<float4 *>(d) = make_float4(lo[0], lo[1], lo[2], lo[3]);
-            *reinterpret_cast<float4 *>(d + 4) = make_float4(lo[4], lo[5], lo[6], lo[7]);
-            *reinterpret_cast<float4 *>(d + per_ch) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-            *reinterpret_cast<float4 *>(d + per_ch + 4) = make_float4(hi[4], hi[5], hi[6], hi[7]);
+            for (int p = 0; p < PX; ++p) unpack2(acc[p][q], lo[p], hi[p]);
+            float *d = tiles + (img * T.th + row) * spitch + PX * seg;
+#pragma unroll
+            for (int p = 0; p < PX; p += 4) {
+                *reinterpret_cast<float4 *>(d + p) = make_float4(lo[p], lo[p + 1], lo[p + 2], lo[p + 3]);
+                *reinterpret_cast<float4 *>(d + per_ch + p) = make_float4(hi[p], hi[p + 1], hi[p + 2], hi[p + 3]);
+            }
         }
         __syncthreads();
         float *o_lo = obase + (size_t)(2 * q) * plane_o;
@@ -331,16 +337,17 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
     }
 }
 
-static CgShape cg_shape(int K, int tn, int th, int seg, int cp) {
+static CgShape cg_shape(int K, int px, int tn, int th, int seg, int cp) {
     CgShape t;
     memset(&t, 0, sizeof(t));
-    const int nf = ((kCgPx + K - 1 + 3) / 4) * 4;
+    const int nf = ((px + K - 1 + 3) / 4) * 4;
+    t.px = px;
     t.tn = tn;
     t.th = th;
     t.seg = seg;
     t.rows = th + K - 1;
-    t.cols = kCgPx * seg + K - 1;
-    t.pitch = (std::max(t.cols, kCgPx * (seg - 1) + nf) + 3) / 4 * 4;
+    t.cols = px * seg + K - 1;
+    t.pitch = (std::max(t.cols, px * (seg - 1) + nf) + 3) / 4 * 4;
     if ((t.pitch / 4) % 2 == 0) t.pitch += 4;
     t.tile_floats = tn * t.rows * t.pitch;
     t.entries = tn * t.rows * t.cols;
@@ -350,28 +357,44 @@ static CgShape cg_shape(int K, int tn, int th, int seg, int cp) {
 
 // Tile shape: the one with the smallest estimated time, tiles per SM times the cost of a tile in thread-cycles: the
 // packed FMAs of 128 threads (2.5 cycles each, as measured for a register outer product) plus the staging of its cells
-// (about eight instructions each).  Shards are cut into equal tiles; up to 56 KB of shared memory keep four blocks on an SM.
-static CgShape cg_choose(int K, int cp, int64_t max_bh, int64_t max_bw, int64_t batch, int64_t workers, int64_t groups, int sms) {
+// (about eight instructions each); the last wave of an SM takes 0.45 of a full one, whatever is in it, and 0.55 in proportion.
+// Up to 56 KB of shared memory keep four blocks on an SM.  Sizes are tried from the largest down in steps of a fifth, shards cut
+// into that many equal tiles, and what cannot win by its FMAs alone is passed over: 1 to 2 us of host time.  Four pixels a thread spend a tenth more on the same outputs (weights are read for
+// half as many FMAs), but make twice the warps: 16 images of 28 x 28, 6 -> 16 channels, forward 12.6 us with eight pixels,
+// 9.8 with four; 256 images 46.8 and 39.6; 1024 images 148 and 146, their adjoint 138 and 153.
+static CgShape cg_choose(int K, int cp, int max_bh, int max_bw, int batch, int workers, int groups, int sms) {
     CgShape best;
     memset(&best, 0, sizeof(best));
     double best_cost = 0;
-    for (int seg = 1; seg <= 16; ++seg) {
-        const int64_t nx = (max_bw + kCgPx * seg - 1) / (kCgPx * seg);
-        if (seg > 1 && (max_bw + kCgPx * (seg - 1) - 1) / (kCgPx * (seg - 1)) == nx) continue;      // narrower tiles do as well
-        for (int th = 2; th * seg <= kCgThreads; th += 2) {
-            const int64_t ny = (max_bh + th - 1) / th;
-            if (th > 2 && (max_bh + th - 3) / (th - 2) == ny) continue;
-            const int room = kCgThreads / (th * seg);
-            for (int tn = 1; tn <= room && tn <= batch; tn = tn < room && tn < batch && 2 * tn > room ? room : 2 * tn) {
-                const int use = (int)std::min<int64_t>(tn, batch);
-                const CgShape t = cg_shape(K, use, th, seg, cp);
-                if (t.smem_bytes > 56 * 1024 || t.tile_floats > 32767) continue;
-                const int64_t tiles = nx * ny * workers * ((batch + use - 1) / use) * groups;
-                const double per_sm = std::max<double>(2.0, (double)((tiles + sms - 1) / sms));
-                const double cost = per_sm * (kCgThreads * (double)(K * K) * kCgPx * cp * 2.5 + 8.0 * t.entries);
-                if (best.tn == 0 || cost < best_cost) {
-                    best = t;
-                    best_cost = cost;
+    const double per_tile = 1.0 / sms;
+    for (int px = 8; px >= 4; px -= 4) {
+        const double fma = kCgThreads * (double)(K * K) * px * cp * (px == 4 ? 2.75 : 2.5);
+        const int res = cg_blocks(px);
+        int nx_before = 0;
+        for (int try_seg = kCgThreads / px; try_seg >= 1; try_seg -= std::max(1, try_seg / 5)) {
+            const int nx = (max_bw + px * try_seg - 1) / (px * try_seg);
+            if (nx == nx_before) continue;
+            nx_before = nx;
+            const int seg = (max_bw + px * nx - 1) / (px * nx);
+            int ny_before = 0;
+            for (int try_th = kCgThreads / seg / 2 * 2; try_th >= 2; try_th -= std::max(2, try_th / 10 * 2)) {
+                const int ny = (max_bh + try_th - 1) / try_th;
+                if (ny == ny_before) continue;
+                ny_before = ny;
+                const int th = ((max_bh + ny - 1) / ny + 1) & ~1;
+                const int room = kCgThreads / (th * seg);
+                for (int tn = std::min(room, batch); tn >= 1; tn /= 2) {
+                    const int64_t tiles = (int64_t)(nx * ny) * ((int64_t)(workers * groups) * (tn == 1 ? batch : (batch + tn - 1) / tn));
+                    const int per_sm = (int)(int64_t)((double)(tiles + sms - 1) * per_tile), last = per_sm % res;
+                    const double waves = per_sm - last + (last ? 0.45 * res + 0.55 * last : 0.0);
+                    if (best.tn != 0 && waves * fma >= best_cost) continue;
+                    const CgShape t = cg_shape(K, px, tn, th, seg, cp);
+                    if (t.smem_bytes > 56 * 1024 || t.tile_floats > 32767) continue;
+                    const double cost = waves * (fma + 8.0 * t.entries);
+                    if (best.tn == 0 || cost < best_cost) {
+                        best = t;
+                        best_cost = cost;
+                    }
                 }
             }
         }
@@ -379,7 +402,7 @@ static CgShape cg_choose(int K, int cp, int64_t max_bh, int64_t max_bw, int64_t 
     return best;
 }
 
-template <int K, bool ADJ, int CP>
+template <int K, bool ADJ, int CP, int PX>
 static distdl_status_t launch_convg(const ConvGParams &G, int64_t blocks, cudaStream_t s) {
     static bool configured_on[kMaxDevicesPerProcess] = {false};
     int dev = 0;
@@ -389,11 +412,11 @@ static distdl_status_t launch_convg(const ConvGParams &G, int64_t blocks, cudaSt
     {
         std::lock_guard<std::mutex> setup_lock(setup_mutex());
         if (!configured_on[dev]) {
-            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_kernel<K, ADJ, CP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 * 1024));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_kernel<K, ADJ, CP, PX>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 * 1024));
             configured_on[dev] = true;
         }
     }
-    convg_kernel<K, ADJ, CP><<<(unsigned)blocks, kCgThreads, G.t.smem_bytes, s>>>(G);
+    convg_kernel<K, ADJ, CP, PX><<<(unsigned)blocks, kCgThreads, G.t.smem_bytes, s>>>(G);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -401,10 +424,10 @@ static distdl_status_t launch_convg(const ConvGParams &G, int64_t blocks, cudaSt
 template <int K, bool ADJ>
 static distdl_status_t launch_convg_pairs(const ConvGParams &G, int cp, int64_t blocks, cudaStream_t s) {
     switch (cp) {
-        case 1: return launch_convg<K, ADJ, 1>(G, blocks, s);
-        case 2: return launch_convg<K, ADJ, 2>(G, blocks, s);
-        case 3: return launch_convg<K, ADJ, 3>(G, blocks, s);
-        default: return launch_convg<K, ADJ, 4>(G, blocks, s);
+        case 1: return G.t.px == 8 ? launch_convg<K, ADJ, 1, 8>(G, blocks, s) : launch_convg<K, ADJ, 1, 4>(G, blocks, s);
+        case 2: return G.t.px == 8 ? launch_convg<K, ADJ, 2, 8>(G, blocks, s) : launch_convg<K, ADJ, 2, 4>(G, blocks, s);
+        case 3: return G.t.px == 8 ? launch_convg<K, ADJ, 3, 8>(G, blocks, s) : launch_convg<K, ADJ, 3, 4>(G, blocks, s);
+        default: return G.t.px == 8 ? launch_convg<K, ADJ, 4, 8>(G, blocks, s) : launch_convg<K, ADJ, 4, 4>(G, blocks, s);
     }
 }
 
@@ -485,8 +508,8 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
     int dev = 0, sms = 148;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
     DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    G.t = cg_choose(kh, cp, max_bh, max_bw, G.batch, (int64_t)ph * pw, groups, sms);
-    const int64_t tiles_x = (max_bw + kCgPx * G.t.seg - 1) / (kCgPx * G.t.seg), tiles_y = (max_bh + G.t.th - 1) / G.t.th;
+    G.t = cg_choose(kh, cp, (int)max_bh, (int)max_bw, G.batch, ph * pw, groups, sms);
+    const int64_t tiles_x = (max_bw + G.t.px * G.t.seg - 1) / (G.t.px * G.t.seg), tiles_y = (max_bh + G.t.th - 1) / G.t.th;
     const int64_t total = tiles_x * tiles_y * ph * pw * ((G.batch + G.t.tn - 1) / G.t.tn) * groups;
     if (total >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     G.groups = make_fast_div((uint32_t)groups);
@@ -524,7 +547,7 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
 // instead (all K * K sums of one or two channel pairs per lane) spend as many instructions on putting x pairs together and
 // on folding lanes as on FMAs.
 // Measured (B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.40 ms = 38 TFLOP/s (1.94 ms with one channel
-// pair per block, both its tiles staged again for every pair); 6 -> 16 channels, 256 images of 28 x 28 0.072 ms (1.61 ms).
+// pair per block, both its tiles staged again for every pair); 6 -> 16 channels, 256 images of 28 x 28 0.063 ms (1.61 ms).
 // Two steps per turn instead of moving the window: 1.63 ms (spills); 192 threads with 168 registers: 1.67 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int kGradRow = 64;            // floats per row of the scratch table (K * K + 1 <= 50 used)
@@ -830,24 +853,35 @@ static GgShape gg_shape(int K, int tn, int th, int seg, int xc, int oc) {
 }
 
 // Tile shape with the smallest estimated time of a launch: tiles per block times warp instructions per tile (a packed FMA
-// counts 2.5: the rate of a register outer product), staging 40 per unit and 2 or 12 more per channel.
-static GgShape gg_choose(int K, int xc, int splits, int oc, int64_t max_bh, int64_t max_bw, int64_t batch, int64_t workers, int64_t slots) {
+// counts 2.5: the rate of a register outer product), staging 40 per unit and 2 or 12 more per channel.  Sizes are tried from
+// the largest down in steps of a fifth, shards cut into that many equal tiles, and what cannot win by its FMAs alone is passed
+// over: 3 to 7 us of host time (7 to 27 us with every size in turn).
+static GgShape gg_choose(int K, int xc, int splits, int oc, int max_bh, int max_bw, int batch, int workers, int slots) {
     GgShape best;
     memset(&best, 0, sizeof(best));
     double best_cost = 0;
     const bool x_wide = (max_bw + K - 1) % 4 == 0, y_wide = max_bw % 4 == 0;
-    for (int seg = 1; seg <= 32; ++seg) {
-        const int64_t nx = (max_bw + 4 * seg - 1) / (4 * seg);
-        if (seg > 1 && (max_bw + 4 * (seg - 1) - 1) / (4 * (seg - 1)) == nx) continue;
-        for (int th = 1; th <= 128; ++th) {
-            const int64_t ny = (max_bh + th - 1) / th;
-            if (th > 1 && (max_bh + th - 2) / (th - 1) == ny) continue;
-            for (int tn = 1; tn <= 64 && tn <= batch; ++tn) {
-                const GgShape t = gg_shape(K, tn, th, seg, xc, oc);
-                if (t.smem_bytes > kGgSmem) break;
-                const int64_t tiles = nx * ny * workers * ((batch + tn - 1) / tn);
-                const int64_t turns = (tiles + slots - 1) / slots;
+    int nx_before = 0;
+    for (int try_seg = 32; try_seg >= 1; try_seg -= std::max(1, try_seg / 5)) {
+        const int nx = (max_bw + 4 * try_seg - 1) / (4 * try_seg);
+        if (nx == nx_before) continue;
+        nx_before = nx;
+        const int seg = (max_bw + 4 * nx - 1) / (4 * nx);
+        int ny_before = 0;
+        for (int try_th = 128; try_th >= 1; try_th -= std::max(1, try_th / 5)) {
+            const int ny = (max_bh + try_th - 1) / try_th;
+            if (ny == ny_before) continue;
+            ny_before = ny;
+            const int th = (max_bh + ny - 1) / ny;
+            // the sums of all threads and one image's dy alone bound the images of a tile
+            const int room = std::min(64, kGgSmem / (2 * 4 * (oc * th * 4 * seg + xc * (th + K - 1) * 4 * seg)));
+            for (int tn = std::min(room, batch); tn >= 1; tn -= std::max(1, tn / 5)) {
+                const int64_t tiles = (int64_t)(nx * ny) * ((int64_t)workers * (tn == 1 ? batch : (batch + tn - 1) / tn));
+                const double turns = (double)((tiles + slots - 1) / slots);
                 const double compute = 8.0 * ((tn * th + splits - 1) / splits) * (seg * (2.0 * K * oc * 2.5 + oc + 10) + 20);
+                if (best.tn != 0 && turns * (compute + 1200) >= best_cost) continue;
+                const GgShape t = gg_shape(K, tn, th, seg, xc, oc);
+                if (t.smem_bytes > kGgSmem) continue;
                 const double staging = (tn * t.rows * t.units * (40.0 + xc * (x_wide ? 2 : 12)) + tn * th * seg * (20.0 + oc * (y_wide ? 2 : 12))) / 32;
                 const double cost = turns * (compute + staging + 1200);
                 if (best.tn == 0 || cost < best_cost) {
@@ -929,7 +963,7 @@ static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, 
     // as many slices as fill the resident blocks once; never more than tiles
     const int64_t group_pairs = (int64_t)G->cgrp[pci] * G->ogrp[pco];
     const int64_t slots = std::max<int64_t>(1, 2 * (int64_t)sms / group_pairs);
-    G->t = gg_choose(kh, xc, G->splits, oc, max_bh, max_bw, G->batch, (int64_t)ph * pw, slots);
+    G->t = gg_choose(kh, xc, G->splits, oc, (int)max_bh, (int)max_bw, G->batch, ph * pw, slots);
     const int64_t tiles_x = (max_bw + 4 * G->t.seg - 1) / (4 * G->t.seg), tiles_y = (max_bh + G->t.th - 1) / G->t.th;
     const int64_t tiles = tiles_x * tiles_y * ph * pw * ((G->batch + G->t.tn - 1) / G->t.tn);
     if (tiles >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles or channel pairs", what);

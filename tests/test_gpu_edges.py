@@ -17,6 +17,9 @@ CONVG_EDGES = [
     (2, 9, 3, 18, 40, 2, 1, 1, 1, 7),        # 16-float windows, uneven input blocks (5, 4)
     (1, 2, 17, 33, 129, 1, 2, 1, 1, 5),      # 9 and 8 channels: groups of 5, 4 and 8; one cell past tile edges
     (3, 6, 5, 20, 31, 1, 1, 3, 1, 3),        # uneven rows (7, 7, 6) beside odd columns
+    (4, 2, 8, 301, 310, 1, 1, 1, 1, 3),      # tiles enough for several waves: eight pixels a thread, all of four pairs / one pair
+    (300, 4, 7, 30, 39, 1, 1, 1, 1, 5),      # the same with tiles of several images; rows that end inside a thread's pixels
+    (200, 4, 10, 29, 31, 1, 2, 1, 1, 7),     # the same, 7 x 7 and two blocks of channels
 ]
 
 
