@@ -772,7 +772,7 @@ affine_kernel_quad(const __grid_constant__ AffineParams P) {
 //   dW_{ij} = dy^_{ij}^T x^_{ij}  with dy^_{ij} = dy_i (B along grid rows), x^_{ij} = x_j (B along grid
 //   columns, kept from the forward pass);  db_i = column sums of dy_i (the bias lives on grid column 0).
 // The weights are distributed over the worker grid itself, so nothing is reduced afterwards: each
-// thread block owns one 128 x 128 tile of one worker's dW block and contracts over the batch.
+// thread block owns one 128 x 128 or 128 x 256 tile of one worker's dW block at a time and contracts over the batch.
 // Both operands are MN-major for the tensor cores (dy_i is [nb, out] row-major: the M index is
 // contiguous; x_j is [nb, in]: the N index is contiguous), staged by TMA as 64 x 64 swizzled atoms.
 // The output (fp32, nfo x nfi) dominates the traffic: the epilogue stages the tile in (swizzled)
@@ -780,19 +780,23 @@ affine_kernel_quad(const __grid_constant__ AffineParams P) {
 // MMAs of the next tile run.
 // ------------------------------------------------------------------------------------------
 constexpr int kDwThreads = 192;                              // warp 0: TMA, warp 1: MMA + TMEM, warps 2..5: epilogue
-constexpr int kDwStages = 4;
-constexpr int kDwOperandBytes = 2 * 64 * kBlockK * 2;        // two 64 x 64 bf16 atoms = 16 KB
-constexpr int kDwStageBytes = 2 * kDwOperandBytes;           // A and B
-constexpr int kDwOutBytes = kTileM * kTileN * 4;             // 64 KB: the fp32 tile as four 128 x 32 boxes
-constexpr int kDwSmemBytes = kDwStages * kDwStageBytes + kDwOutBytes + 1024 + 128;
-constexpr int kDwTmemCols = 2 * kTileN;                      // two accumulators
+constexpr int kDwAtomBytes = 64 * kBlockK * 2;               // a 64 x 64 bf16 atom = 8 KB
+constexpr int kDwOutBytes = 4 * kTileM * 32 * 4;             // 64 KB: four 128 x 32 boxes of the fp32 tile
+template <int TN>
+struct DwShape {                                             // tile 128 x TN
+    static constexpr int kStages = TN == 256 ? 3 : 4;
+    static constexpr int kABytes = 2 * kDwAtomBytes;
+    static constexpr int kStageBytes = (2 + TN / 64) * kDwAtomBytes;
+    static constexpr int kSmemBytes = kStages * kStageBytes + kDwOutBytes + 1024 + 128;
+    static constexpr int kTmemCols = 2 * TN;                 // two accumulators
+};
 
 struct AffineDwParams {
     CUtensorMap dy_map[8];                  // dy_i  [nb, bfo] bf16, box {64 out, 64 batch}
     CUtensorMap x_map[8];                   // x_j   [nb, bfi] bf16, box {64 in, 64 batch}
     CUtensorMap dw_map[kMaxMaps - 8];       // dW_ij [bfo, bfi] fp32, box {32 in, 128 out}
     int32_t nb, pfi;
-    int32_t tiles_m, tiles_n;               // 128 x 128 tiles per worker block
+    int32_t tiles_m, tiles_n;               // 128 x TN tiles per worker block
     int32_t total_tiles;
     int32_t bfi;                            // columns of a dW block
 };
@@ -819,11 +823,12 @@ __device__ __forceinline__ bool epilogue_all(bool pred) {
 struct DwTile {
     int wi, wj, m0, n0;
 };
+template <int TN>
 __device__ __forceinline__ DwTile dw_tile(const AffineDwParams &P, int tile) {
     // tile id: column tile fastest, then row tile, then worker j, then worker i
     DwTile t;
     int rest = tile;
-    t.n0 = (rest % P.tiles_n) * kTileN;
+    t.n0 = (rest % P.tiles_n) * TN;
     rest /= P.tiles_n;
     t.m0 = (rest % P.tiles_m) * kTileM;
     rest /= P.tiles_m;
@@ -833,11 +838,19 @@ __device__ __forceinline__ DwTile dw_tile(const AffineDwParams &P, int tile) {
 }
 
 // Persistent: one block per SM walks over tiles blockIdx.x, + gridDim.x, ...  The producer runs ahead
-// through a four-stage ring (a whole tile at batch 256), the accumulator alternates between two
-// 128-column halves of tensor memory, and the epilogue of tile t (tensor memory -> swizzled shared
+// through a ring of four (three wide) stages, the accumulator alternates between two
+// halves of tensor memory, and the epilogue of tile t (tensor memory -> swizzled shared
 // memory -> TMA stores) runs while the tensor cores work on tile t + 1.
+//
+// What bounds it: the SM's port into L2, and the store of the fp32 result.  A 128 x 128 tile takes 128 KB of operands in
+// for 64 KB out at batch 256, a 128 x 256 tile 192 KB for 128 KB, a sixth less for the same output.  8192 x 8192 on 4 x 4 workers, db
+// with it (B200): batch 256 67.0 -> 59.6 us (63.6 by the bias gradient in its shadow alone), where writing dW takes 41 us at the
+// copy rate; 4096 x 4096, batch 1024: 71 -> 58 us.
+template <int TN>
 __global__ void __launch_bounds__(kDwThreads, 1)
 affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
+    constexpr int kDwStages = DwShape<TN>::kStages, kDwStageBytes = DwShape<TN>::kStageBytes, kDwABytes = DwShape<TN>::kABytes;
+    constexpr int kDwTmemCols = DwShape<TN>::kTmemCols;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -881,7 +894,7 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
             uint32_t s = 0, phase = 0;
             bool ok = true;
             for (int tile = blockIdx.x; tile < P.total_tiles && ok; tile += gridDim.x) {
-                const DwTile t = dw_tile(P, tile);
+                const DwTile t = dw_tile<TN>(P, tile);
                 const CUtensorMap *amap = &P.dy_map[t.wi], *bmap = &P.x_map[t.wj];
                 for (int kb = 0; kb < num_kblocks; ++kb) {
                     ok = mbar_wait(bar_empty + 8 * s, phase ^ 1, abort_flag);
@@ -890,9 +903,10 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
                     mbar_expect_tx(full, kDwStageBytes);
                     const int k0 = kb * kBlockK;
                     tma_load_2d(sa, amap, t.m0, k0, full);                                 // atom: out features m0 .. m0 + 63
-                    tma_load_2d(sa + kDwOperandBytes / 2, amap, t.m0 + 64, k0, full);
-                    tma_load_2d(sa + kDwOperandBytes, bmap, t.n0, k0, full);               // atom: in features n0 .. n0 + 63
-                    tma_load_2d(sa + kDwOperandBytes + kDwOperandBytes / 2, bmap, t.n0 + 64, k0, full);
+                    tma_load_2d(sa + kDwAtomBytes, amap, t.m0 + 64, k0, full);
+#pragma unroll
+                    for (int q = 0; q < TN / 64; ++q)                                      // atom: in features n0 + 64 q ..
+                        tma_load_2d(sa + kDwABytes + q * kDwAtomBytes, bmap, t.n0 + 64 * q, k0, full);
                     if (++s == kDwStages) {
                         s = 0;
                         phase ^= 1;
@@ -909,7 +923,7 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
         if (lane == 0) {
             // both operands MN-major (bits 15 and 16): 64-wide atoms 8 KB apart (leading offset), groups of
             // eight batch rows 1024 bytes apart (stride offset), a K step of 16 batch rows is 2048 bytes
-            const uint32_t idesc = instr_desc(kTileM, kTileN, 1) | (1u << 15);
+            const uint32_t idesc = instr_desc(kTileM, TN, 1) | (1u << 15);
             uint32_t s = 0, phase = 0;
             bool ok = true;
             int it = 0;
@@ -919,14 +933,14 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
                 ok = mbar_wait(bar_acc_empty + 8 * buf, (((uint32_t)it >> 1) & 1u) ^ 1u, abort_flag);
                 if (!ok) break;
                 tcgen05_fence_after();
-                const uint32_t tmem_acc = tmem_base + buf * (uint32_t)kTileN;
+                const uint32_t tmem_acc = tmem_base + buf * (uint32_t)TN;
                 for (int kb = 0; kb < num_kblocks; ++kb) {
                     ok = mbar_wait(bar_full + 8 * s, phase, abort_flag);
                     if (!ok) break;
                     tcgen05_fence_after();
                     const uint32_t sa = base + s * kDwStageBytes;
-                    const uint64_t a = smem_desc(sa, kDwOperandBytes / 2, 1024);
-                    const uint64_t b = smem_desc(sa + kDwOperandBytes, kDwOperandBytes / 2, 1024);
+                    const uint64_t a = smem_desc(sa, kDwAtomBytes, 1024);
+                    const uint64_t b = smem_desc(sa + kDwABytes, kDwAtomBytes, 1024);
                     constexpr uint64_t kstep = 2048 >> 4;
                     umma_bf16(tmem_acc, a, b, idesc, kb ? 1u : 0u);
                     umma_bf16(tmem_acc, a + kstep, b + kstep, idesc, 1u);
@@ -956,26 +970,26 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
             const bool mine = mbar_wait(bar_acc_full + 8 * buf, ((uint32_t)it >> 1) & 1u, abort_flag);
             if (!epilogue_all(mine)) break;
             tcgen05_fence_after();
-            const uint32_t tmem_acc = tmem_base + buf * (uint32_t)kTileN;
-            const DwTile t = dw_tile(P, tile);
+            const uint32_t tmem_acc = tmem_base + buf * (uint32_t)TN;
+            const DwTile t = dw_tile<TN>(P, tile);
             const CUtensorMap *omap = &P.dw_map[t.wi * P.pfi + t.wj];
             // box by box, so that the read-out of one box by its store (which runs at the rate of the SM's
             // port into the memory system) overlaps the copy of the next box out of tensor memory
 #pragma unroll 1
-            for (int q = 0; q < kTileN / 32; ++q) {
+            for (int q = 0; q < TN / 32; ++q) {
                 // at most three stores in flight: the one that read this box for the previous tile is done
                 if (issuer) asm volatile("cp.async.bulk.wait_group.read 3;" ::: "memory");
                 asm volatile("bar.sync 1, 128;" ::: "memory");
                 uint32_t v[32];
                 tmem_ld32(tmem_acc + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(32 * q), v);
-                const uint32_t boxaddr = out_base + (uint32_t)q * (kTileM * 128);
+                const uint32_t boxaddr = out_base + (uint32_t)(q & 3) * (kTileM * 128);
                 const uint32_t rowaddr = boxaddr + (uint32_t)row * 128;
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
                                  ::"r"(rowaddr + (uint32_t)((c ^ (row & 7)) << 4)), "r"(v[4 * c]), "r"(v[4 * c + 1]),
                                    "r"(v[4 * c + 2]), "r"(v[4 * c + 3]) : "memory");
-                if (q == kTileN / 32 - 1) {
+                if (q == TN / 32 - 1) {
                     // this half of tensor memory may be overwritten by the tile after the next
                     tcgen05_fence_before();
                     __syncwarp();
@@ -993,6 +1007,8 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
         }
         if (issuer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores done before the block retires
     }
+    // launched to overlap the bias gradient's kernel, which nothing here reads; what follows in the stream waits for both
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     tcgen05_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -1012,6 +1028,7 @@ struct AffineDbParams {
 constexpr int kDbThreads = 256;
 __global__ void __launch_bounds__(kDbThreads) affine_db_kernel(const AffineDbParams P) {
     __shared__ float part[kDbThreads / 32][64];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int col = blockIdx.x * 64 + 2 * lane;
     const int i = blockIdx.y;
@@ -1243,8 +1260,9 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
     }
     if (!encode_fn()) return fail(DISTDL_ERR_CUDA, "%s: cuTensorMapEncodeTiled is not available", what);
     // tiles past the end of a block are partly empty: loads are zero-filled and stores clipped by TMA
-    const int64_t tiles = ((bfo + kTileM - 1) / kTileM) * ((bfi + kTileN - 1) / kTileN) * pfo * pfi;
+    const int64_t tiles = ((bfo + kTileM - 1) / kTileM) * ((bfi + 127) / 128) * pfo * pfi;
     if (tiles >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
+    const int64_t wide_tiles = ((bfo + kTileM - 1) / kTileM) * ((bfi + 255) / 256) * pfo * pfi;
 
     AffineDwParams P;
     memset(&P, 0, sizeof(P));
@@ -1257,8 +1275,6 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
     P.nb = (int32_t)nb;
     P.pfi = pfi;
     P.tiles_m = (int32_t)((bfo + kTileM - 1) / kTileM);
-    P.tiles_n = (int32_t)((bfi + kTileN - 1) / kTileN);
-    P.total_tiles = (int32_t)tiles;
     P.bfi = (int32_t)bfi;
     // one-time set-up per device (kernel attributes, occupancy): a process may drive several GPUs
     static bool configured_on[kMaxDevicesPerProcess] = {false};
@@ -1271,15 +1287,18 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
     static int sms_on[kMaxDevicesPerProcess] = {0};
     int &sms = sms_on[cur_dev];
     if (!configured) {
-        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmemBytes));
+        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_dw_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DwShape<128>::kSmemBytes));
+        DISTDL_CUDA_CHECK(cudaFuncSetAttribute(affine_dw_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, DwShape<256>::kSmemBytes));
         int dev = 0;
         DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
         DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         configured = true;
     }
-    const unsigned grid = (unsigned)std::min<int64_t>(tiles, sms > 0 ? sms : 1);
-    affine_dw_kernel<<<grid, kDwThreads, kDwSmemBytes, (cudaStream_t)stream>>>(P);
-    DISTDL_CUDA_CHECK(cudaGetLastError());
+    const int64_t slots = sms > 0 ? sms : 1;
+    // what a tile moves between L2 and its SM bounds it: 128 KB of operands and 64 KB out, or 192 KB and 128 KB (batch 256)
+    const bool wide = (wide_tiles + slots - 1) / slots * (192 + 128) < (tiles + slots - 1) / slots * (128 + 64);
+    P.tiles_n = (int32_t)(wide ? (bfi + 255) / 256 : (bfi + 127) / 128);
+    P.total_tiles = (int32_t)(wide ? wide_tiles : tiles);
     if (db) {
         AffineDbParams B;
         memset(&B, 0, sizeof(B));
@@ -1293,6 +1312,18 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
         affine_db_kernel<<<grid, kDbThreads, 0, (cudaStream_t)stream>>>(B);
         DISTDL_CUDA_CHECK(cudaGetLastError());
     }
+    // dW does not read db: its blocks start beside those of the kernel before it (and wait for that kernel at their end)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(P.total_tiles, slots));
+    cfg.blockDim = dim3(kDwThreads);
+    cfg.dynamicSmemBytes = wide ? DwShape<256>::kSmemBytes : DwShape<128>::kSmemBytes;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = db ? 1 : 0;
+    DISTDL_CUDA_CHECK(wide ? cudaLaunchKernelEx(&cfg, affine_dw_kernel<256>, P) : cudaLaunchKernelEx(&cfg, affine_dw_kernel<128>, P));
     return DISTDL_OK;
 }
 

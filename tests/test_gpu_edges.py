@@ -95,6 +95,13 @@ def test_affine_few_samples(case, integer):
     parity.test_affine_fwd_and_adj(case, integer)
 
 
+@pytest.mark.parametrize("case", [(40, 3592, 2048, 1, 1), (70, 7184, 1032, 1, 2)], ids=str)
+@pytest.mark.parametrize("integer", [True, False], ids=["int", "normal"])
+def test_affine_wide_gradient_tiles(case, integer):
+    """Tiles enough for 256 columns each; the last one holds eight columns, the last row tile all or eight of its rows."""
+    parity.test_affine_param_gradients(case, integer)
+
+
 # global shape, partition, kernel, stride, padding
 POOL_EDGES = [
     ((1, 1, 7, 5), (1, 1, 1, 1), (3, 3), (1, 1), ((1, 1), (1, 1))),         # every window of a border column is clipped
