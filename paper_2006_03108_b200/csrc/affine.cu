@@ -208,6 +208,7 @@ affine_kernel_pair(const __grid_constant__ AffineParams P) {
     tcgen05_fence_before();
     cluster_sync_all();              // both blocks' barriers exist before anyone signals them
     tcgen05_fence_after();
+    stream_enter();
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
@@ -417,6 +418,7 @@ affine_kernel_split(const __grid_constant__ AffineSplitParams Q) {
     tcgen05_fence_before();
     __syncthreads();
     tcgen05_fence_after();
+    stream_enter();
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
@@ -628,6 +630,7 @@ affine_kernel_quad(const __grid_constant__ AffineParams P) {
     tcgen05_fence_before();
     cluster_sync_all();
     tcgen05_fence_after();
+    stream_enter();
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
@@ -799,6 +802,7 @@ struct AffineDwParams {
     int32_t tiles_m, tiles_n;               // 128 x TN tiles per worker block
     int32_t total_tiles;
     int32_t bfi;                            // columns of a dW block
+    int32_t after_db;                       // the kernel before it in the stream is the bias gradient's, which it does not depend on
 };
 
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int32_t c0, int32_t c1) {
@@ -887,6 +891,8 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
     tcgen05_fence_before();
     __syncthreads();
     tcgen05_fence_after();
+    if (P.after_db) stream_enter_beside();
+    else stream_enter();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
@@ -1007,8 +1013,7 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
         }
         if (issuer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores done before the block retires
     }
-    // launched to overlap the bias gradient's kernel, which nothing here reads; what follows in the stream waits for both
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (P.after_db) stream_leave_beside();
     tcgen05_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -1028,7 +1033,7 @@ struct AffineDbParams {
 constexpr int kDbThreads = 256;
 __global__ void __launch_bounds__(kDbThreads) affine_db_kernel(const AffineDbParams P) {
     __shared__ float part[kDbThreads / 32][64];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    stream_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int col = blockIdx.x * 64 + 2 * lane;
     const int i = blockIdx.y;
@@ -1157,36 +1162,10 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
     if (quad) {
         const int64_t row_pairs = (nb + 2 * kTileM - 1) / (2 * kTileM);
         const int64_t qtiles = (adjoint ? nfi : nfo) / kQuadN;
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3((unsigned)(4 * row_pairs * qtiles));
-        cfg.blockDim = dim3(kQuadThreads);
-        cfg.dynamicSmemBytes = kQuadSmemBytes;
-        cfg.stream = (cudaStream_t)stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 4;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel_quad, P));
+        launch_clusters_in_stream(affine_kernel_quad, 4, dim3((unsigned)(4 * row_pairs * qtiles)), kQuadThreads, kQuadSmemBytes, (cudaStream_t)stream, P);
     } else if (pair) {
         const int64_t row_pairs = (nb + 2 * kTileM - 1) / (2 * kTileM);
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3((unsigned)(2 * row_pairs * ntiles));
-        cfg.blockDim = dim3(kAffineThreads);
-        cfg.dynamicSmemBytes = AffinePairCfg::SMEM_BYTES;
-        cfg.stream = (cudaStream_t)stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 2;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel_pair, P));
+        launch_clusters_in_stream(affine_kernel_pair, 2, dim3((unsigned)(2 * row_pairs * ntiles)), kAffineThreads, AffinePairCfg::SMEM_BYTES, (cudaStream_t)stream, P);
     } else {
         // blocks per tile: doubled while twice as many blocks as SMs are not exceeded and every block keeps four k-blocks
         const int sms = sms_on[cur_dev];
@@ -1201,20 +1180,7 @@ static distdl_status_t affine_impl(int64_t nb, int64_t nfi, int64_t nfo, int32_t
         const int budget = ntiles * Q.split <= sms ? kSplitMaxSmem : kSplitMaxSmem / 2;
         Q.stages = std::min(kSplitMaxStages, (budget - kSplitTail) / Q.stage_bytes);
         const int smem = Q.stages * Q.stage_bytes + kSplitTail;       // at least three stages: room for the partial sums
-        cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3((unsigned)(ntiles * Q.split));
-        cfg.blockDim = dim3(kAffineThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = (cudaStream_t)stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)Q.split;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        DISTDL_CUDA_CHECK(cudaLaunchKernelEx(&cfg, affine_kernel_split, Q));
+        launch_clusters_in_stream(affine_kernel_split, (unsigned)Q.split, dim3((unsigned)(ntiles * Q.split)), kAffineThreads, smem, (cudaStream_t)stream, Q);
     }
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
@@ -1309,21 +1275,14 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
         B.nb = (int32_t)nb;
         B.bfo = (int32_t)bfo;
         dim3 grid((unsigned)((bfo + 63) / 64), (unsigned)pfo);
-        affine_db_kernel<<<grid, kDbThreads, 0, (cudaStream_t)stream>>>(B);
+        launch_in_stream(affine_db_kernel, grid, kDbThreads, 0, (cudaStream_t)stream, B);
         DISTDL_CUDA_CHECK(cudaGetLastError());
     }
-    // dW does not read db: its blocks start beside those of the kernel before it (and wait for that kernel at their end)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>(P.total_tiles, slots));
-    cfg.blockDim = dim3(kDwThreads);
-    cfg.dynamicSmemBytes = wide ? DwShape<256>::kSmemBytes : DwShape<128>::kSmemBytes;
-    cfg.stream = (cudaStream_t)stream;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = db ? 1 : 0;
-    DISTDL_CUDA_CHECK(wide ? cudaLaunchKernelEx(&cfg, affine_dw_kernel<256>, P) : cudaLaunchKernelEx(&cfg, affine_dw_kernel<128>, P));
+    P.after_db = db ? 1 : 0;
+    const dim3 dw_grid((unsigned)std::min<int64_t>(P.total_tiles, slots));
+    if (wide) launch_in_stream(affine_dw_kernel<256>, dw_grid, kDwThreads, DwShape<256>::kSmemBytes, (cudaStream_t)stream, P);
+    else launch_in_stream(affine_dw_kernel<128>, dw_grid, kDwThreads, DwShape<128>::kSmemBytes, (cudaStream_t)stream, P);
+    DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
 

@@ -39,6 +39,7 @@ __device__ __forceinline__ void st_stream(uint4 *p, uint4 v) {
 // dst[j][i] = src[i] for j < k; nvec 16-byte vectors, then `tail` trailing bytes.
 __global__ void __launch_bounds__(kStreamThreads)
 broadcast_kernel(const uint4 *__restrict__ src, const __grid_constant__ FanPointers dst, int k, size_t nvec, int tail) {
+    stream_enter();
     const size_t stride = (size_t)gridDim.x * kStreamThreads;
     size_t i = (size_t)blockIdx.x * kStreamThreads + threadIdx.x;
     for (; i + (kUnroll - 1) * stride < nvec; i += kUnroll * stride) {
@@ -102,6 +103,7 @@ __device__ __forceinline__ uint4 add_vec(uint4 a, uint4 b) {
 template <int K, int DT>
 __global__ void __launch_bounds__(kStreamThreads)
 sumreduce_kernel(const __grid_constant__ FanPointers src, void *__restrict__ dst, int k_runtime, size_t nvec, int tail) {
+    stream_enter();
     const int k = K > 0 ? K : k_runtime;
     const size_t stride = (size_t)gridDim.x * kStreamThreads;
     for (size_t i = (size_t)blockIdx.x * kStreamThreads + threadIdx.x; i < nvec; i += stride) {
@@ -163,6 +165,7 @@ inline bool aligned32(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 constexpr int kUnroll32 = 4;
 __global__ void __launch_bounds__(kStreamThreads)
 broadcast_kernel32(const Vec32 *__restrict__ src, const __grid_constant__ FanPointers dst, int k, size_t nvec32) {
+    stream_enter();
     const size_t stride = (size_t)gridDim.x * kStreamThreads;
     size_t i = (size_t)blockIdx.x * kStreamThreads + threadIdx.x;
     for (; i + (kUnroll32 - 1) * stride < nvec32; i += kUnroll32 * stride) {
@@ -218,19 +221,17 @@ static distdl_status_t broadcast_impl(const void *src, void *const *dst, int32_t
             if (wide) {
                 // 256-bit accesses for the body, the 16-byte kernel for what is left (under 32 bytes)
                 const size_t nvec32 = bytes / 32;
-                broadcast_kernel32<<<stream_grid(nvec32, kUnroll32), kStreamThreads, 0, (cudaStream_t)stream>>>(
-                    (const Vec32 *)src, fp, filled, nvec32);
+                launch_in_stream(broadcast_kernel32, stream_grid(nvec32, kUnroll32), kStreamThreads, 0, (cudaStream_t)stream, (const Vec32 *)src, fp, filled, nvec32);
                 DISTDL_CUDA_CHECK(cudaGetLastError());
                 const size_t done = nvec32 * 32;
                 if (done < bytes) {
                     FanPointers rest;
                     for (int r = 0; r < kMaxFan; ++r) rest.p[r] = fp.p[r] ? (char *)fp.p[r] + done : nullptr;
-                    broadcast_kernel<<<1, kStreamThreads, 0, (cudaStream_t)stream>>>(
-                        (const uint4 *)((const char *)src + done), rest, filled, (bytes - done) / 16, tail);
+                    launch_in_stream(broadcast_kernel, 1, kStreamThreads, 0, (cudaStream_t)stream, (const uint4 *)((const char *)src + done), rest, filled, (bytes - done) / 16, tail);
                     DISTDL_CUDA_CHECK(cudaGetLastError());
                 }
             } else {
-                broadcast_kernel<<<grid, kStreamThreads, 0, (cudaStream_t)stream>>>((const uint4 *)src, fp, filled, nvec, tail);
+                launch_in_stream(broadcast_kernel, grid, kStreamThreads, 0, (cudaStream_t)stream, (const uint4 *)src, fp, filled, nvec, tail);
                 DISTDL_CUDA_CHECK(cudaGetLastError());
             }
             filled = 0;
@@ -242,9 +243,9 @@ static distdl_status_t broadcast_impl(const void *src, void *const *dst, int32_t
 template <int K>
 static void launch_sum(const FanPointers &fp, void *dst, int k, size_t nvec, int tail, int grid, distdl_dtype_t t,
                        cudaStream_t s) {
-    if (t == DISTDL_F32) sumreduce_kernel<K, 0><<<grid, kStreamThreads, 0, s>>>(fp, dst, k, nvec, tail);
-    else if (t == DISTDL_BF16) sumreduce_kernel<K, 1><<<grid, kStreamThreads, 0, s>>>(fp, dst, k, nvec, tail);
-    else sumreduce_kernel<K, 2><<<grid, kStreamThreads, 0, s>>>(fp, dst, k, nvec, tail);
+    if (t == DISTDL_F32) launch_in_stream(sumreduce_kernel<K, 0>, grid, kStreamThreads, 0, s, fp, dst, k, nvec, tail);
+    else if (t == DISTDL_BF16) launch_in_stream(sumreduce_kernel<K, 1>, grid, kStreamThreads, 0, s, fp, dst, k, nvec, tail);
+    else launch_in_stream(sumreduce_kernel<K, 2>, grid, kStreamThreads, 0, s, fp, dst, k, nvec, tail);
 }
 
 static distdl_status_t sumreduce_impl(const void *const *src, void *dst, int32_t k, int64_t n, distdl_dtype_t t,

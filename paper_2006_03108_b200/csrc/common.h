@@ -27,6 +27,48 @@ void clear_error();
 constexpr int kMaxDevicesPerProcess = 64;   // per-device one-time set-up flags are kept for this many devices
 std::mutex &setup_mutex();                  // guards the one-time, per-device set-up of the operator entry points
 
+#ifdef __CUDACC__
+// Kernels follow one another in a stream without the gap between a kernel's last block and the next one's first: a kernel is
+// launched while its predecessor runs, and its blocks come to a multiprocessor as soon as there is room.  stream_enter() is every
+// such kernel's first access to memory: it returns when all that came before in the stream is complete and visible, and only
+// then lets the successor's blocks come.
+// Measured (B200): back to back from the host, thirty random layers and exchanges take 1.10 times less time in the geometric mean (a
+// halo exchange of 8 x 8 x 53 x 49 and its adjoint 16.6 -> 12.4 us); in a captured graph, where the gap is smaller, the last microsecond of it.
+__device__ __forceinline__ void stream_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// For a kernel that does not depend on the kernel right before it in the stream (but on what came before that): it runs beside
+// it and waits for it at the end, so that what follows in the stream comes after both.
+__device__ __forceinline__ void stream_enter_beside() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void stream_leave_beside() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_clusters_in_stream(void (*kernel)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                      const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attrs[2] = {};
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[0].val.programmaticStreamSerializationAllowed = 1;
+    attrs[1].id = cudaLaunchAttributeClusterDimension;
+    attrs[1].val.clusterDim.x = cluster;
+    attrs[1].val.clusterDim.y = 1;
+    attrs[1].val.clusterDim.z = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = cluster ? 2 : 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);      // an error is found by cudaGetLastError, as after any launch
+}
+template <typename... P, typename... A>
+inline void launch_in_stream(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A &...args) {
+    launch_clusters_in_stream(kernel, 0, grid, block, smem, stream, args...);
+}
+#endif
+
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 inline int elem_size(distdl_dtype_t t) { return t == DISTDL_F32 ? 4 : (t == DISTDL_F64 ? 8 : 2); }
 inline bool valid_dtype(distdl_dtype_t t) { return t == DISTDL_F32 || t == DISTDL_BF16 || t == DISTDL_F64; }

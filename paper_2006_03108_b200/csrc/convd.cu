@@ -344,6 +344,7 @@ struct DwWindow<K, -1> {
 template <int K, bool ADJ, int NC, bool VEC>
 __global__ void __launch_bounds__(kDwThreads, K == 7 ? 3 : 4)
 conv_rows_kernel(const __grid_constant__ DwParams P) {
+    stream_enter();
     using C = DwCfg<K, NC, false>;
     constexpr int OO = ADJ ? C::PH : 0;                     // ghost width of the output layout
     extern __shared__ __align__(16) float smem[];
@@ -476,6 +477,7 @@ constexpr int kGradRow = 64;   // floats per (channel, slice) row of the scratch
 template <int K, int NC, bool VEC>
 __global__ void __launch_bounds__(kDwThreads, K == 7 ? 3 : 4)
 conv_grad_rows_kernel(const __grid_constant__ DwParams P) {
+    stream_enter();
     using C = DwCfg<K, NC, true>;
     extern __shared__ __align__(16) float smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -584,6 +586,7 @@ conv_grad_rows_kernel(const __grid_constant__ DwParams P) {
 constexpr int kDwFoldGroups = 16;
 __global__ void __launch_bounds__(64 * kDwFoldGroups)
 conv_grad_finish_kernel(const float *partial, int slices, int taps, float *dw, float *db) {
+    stream_enter();
     __shared__ float part[kDwFoldGroups][64];
     const int ch = blockIdx.x, t = threadIdx.x & 63, h = threadIdx.x >> 6;
     float v = 0.f;
@@ -719,7 +722,7 @@ static distdl_status_t launch_conv_rows(DwParams &P, int64_t max_bh, int64_t max
     if (st != DISTDL_OK) return st;
     st = dw_items(&P, K, max_bh, max_bw, 32 * NC, DwCfg<K, NC, false>::G, P.planes, (int64_t)blocks * kDwWarps, what);
     if (st != DISTDL_OK) return st;
-    conv_rows_kernel<K, ADJ, NC, VEC><<<(unsigned)((P.items + kDwWarps - 1) / kDwWarps), kDwThreads, smem, s>>>(P);
+    launch_in_stream(conv_rows_kernel<K, ADJ, NC, VEC>, (unsigned)((P.items + kDwWarps - 1) / kDwWarps), kDwThreads, smem, s, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -795,11 +798,11 @@ static distdl_status_t grad_plan(const distdl_partition *p, int32_t kh, int32_t 
 template <int K>
 static distdl_status_t launch_grad(const DwParams &P, DwGradKind kind, float *dw, float *db, cudaStream_t s) {
     const unsigned grid = (unsigned)(P.slices * P.channels);
-    if (kind == kDwNarrow) conv_grad_rows_kernel<K, 2, false><<<grid, kDwThreads, dw_smem_bytes<K, 2>(true), s>>>(P);
-    else if (kind == kDwVector && K == 5) conv_grad_rows_kernel<5, 4, true><<<grid, kDwThreads, dw_smem_bytes<5, 4>(true), s>>>(P);
-    else conv_grad_rows_kernel<K, 4, false><<<grid, kDwThreads, dw_smem_bytes<K, 4>(true), s>>>(P);
+    if (kind == kDwNarrow) launch_in_stream(conv_grad_rows_kernel<K, 2, false>, grid, kDwThreads, dw_smem_bytes<K, 2>(true), s, P);
+    else if (kind == kDwVector && K == 5) launch_in_stream(conv_grad_rows_kernel<5, 4, true>, grid, kDwThreads, dw_smem_bytes<5, 4>(true), s, P);
+    else launch_in_stream(conv_grad_rows_kernel<K, 4, false>, grid, kDwThreads, dw_smem_bytes<K, 4>(true), s, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
-    conv_grad_finish_kernel<<<P.channels, 64 * kDwFoldGroups, 0, s>>>(P.partial, P.slices, K * K, dw, db);
+    launch_in_stream(conv_grad_finish_kernel, P.channels, 64 * kDwFoldGroups, 0, s, P.partial, P.slices, K * K, dw, db);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }

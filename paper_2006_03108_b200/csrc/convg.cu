@@ -73,6 +73,7 @@ constexpr int cg_blocks(int px) { return px == 8 ? 3 : 4; }
 template <int K, bool ADJ, int CP, int PX>
 __global__ void __launch_bounds__(kCgThreads, cg_blocks(PX))
 convg_kernel(const __grid_constant__ ConvGParams G) {
+    stream_enter();
     constexpr int PH = K / 2, CT = 2 * CP;
     constexpr int NF = ((PX + K - 1 + 3) / 4) * 4;         // floats of a thread's window per row
     constexpr int WF = ((K * K * CT + 3) / 4) * 4;
@@ -416,7 +417,7 @@ static distdl_status_t launch_convg(const ConvGParams &G, int64_t blocks, cudaSt
             configured_on[dev] = true;
         }
     }
-    convg_kernel<K, ADJ, CP, PX><<<(unsigned)blocks, kCgThreads, G.t.smem_bytes, s>>>(G);
+    launch_in_stream(convg_kernel<K, ADJ, CP, PX>, (unsigned)blocks, kCgThreads, G.t.smem_bytes, s, G);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -583,6 +584,7 @@ struct ConvGGradParams {
 template <int K, int OC>
 __global__ void __launch_bounds__(kGgThreads, 2)
 convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
+    stream_enter();
     constexpr int PH = K / 2;
     constexpr int NU = (4 + K - 1 + 3) / 4;                 // 16-byte units of x that four pixels of a kernel row need
     extern __shared__ __align__(16) float smem[];           // two buffers, then a row of ones
@@ -806,6 +808,7 @@ struct ConvGGradOut {
 };
 __global__ void __launch_bounds__(64 * kGradFoldGroups)
 convg_grad_finish_kernel(const __grid_constant__ ConvGGradParams G, const __grid_constant__ ConvGGradOut O, int taps) {
+    stream_enter();
     __shared__ float part[kGradFoldGroups][64];
     const int q = blockIdx.x, t = threadIdx.x & 63, h = threadIdx.x >> 6;
     const int o = q / G.n_x, c = q - o * G.n_x;
@@ -999,9 +1002,9 @@ static distdl_status_t launch_convg_grad(const ConvGGradParams &G, const ConvGGr
             configured_on[dev] = true;
         }
     }
-    convg_grad_kernel<K, OC><<<grid, kGgThreads, G.t.smem_bytes, s>>>(G);
+    launch_in_stream(convg_grad_kernel<K, OC>, grid, kGgThreads, G.t.smem_bytes, s, G);
     DISTDL_CUDA_CHECK(cudaGetLastError());
-    convg_grad_finish_kernel<<<pairs, 64 * kGradFoldGroups, 0, s>>>(G, O, K * K);
+    launch_in_stream(convg_grad_finish_kernel, pairs, 64 * kGradFoldGroups, 0, s, G, O, K * K);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }

@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(kHaloThreads, SUMS ? 2 : 4)
 halo_box_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict__ sources,
                 const HaloTile *__restrict__ tiles, int32_t elem_bytes,
                 const __grid_constant__ ShardPointers sh) {
+    stream_enter();
     __shared__ __align__(16) HaloBox s_box;
     __shared__ __align__(16) HaloSource s_src[kMaxSources];
     // every thread reads the (uniform) tile record; box and sources are staged in shared memory
@@ -555,6 +556,7 @@ __device__ __forceinline__ void fast_line_rows(const FastHeader &H, const FastDi
 __global__ void __launch_bounds__(kFastThreads)
 halo_fast_fwd_kernel(const __grid_constant__ FastHeader H, const FastDim *__restrict__ dims_g,
                      const __grid_constant__ ShardPointers sh) {
+    stream_enter();
     __shared__ FastDim dims[kMaxFastCoords];
     __shared__ __align__(16) unsigned char scratch[kFastMaxSlots * 16];
     fast_load_records(H, dims_g, dims);
@@ -652,9 +654,7 @@ halo_fast_fwd_kernel(const __grid_constant__ FastHeader H, const FastDim *__rest
 // in memory order, with the neighbour's ghost value taken from shared memory.
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(kFastThreads)
-halo_fast_adj_lines_kernel(const __grid_constant__ FastHeader H, const FastDim *__restrict__ dims_g,
-                           const __grid_constant__ ShardPointers sh) {
+__device__ __forceinline__ void halo_fast_adj_lines(const FastHeader &H, const FastDim *__restrict__ dims_g, const ShardPointers &sh) {
     __shared__ FastDim dims[kMaxFastCoords];
     __shared__ __align__(16) unsigned char scratch[kFastMaxSlots * 16];
     fast_load_records(H, dims_g, dims);
@@ -735,6 +735,18 @@ halo_fast_adj_lines_kernel(const __grid_constant__ FastHeader H, const FastDim *
     }
 }
 
+// The boxes' kernel, if there is one, is the one before it in the stream: its cells are others, so the two run side by side where
+// the first one's last blocks leave room (512^3 over 4 x 4 x 4 workers, widths 4: 120 -> 116 us).
+template <typename T>
+__global__ void __launch_bounds__(kFastThreads)
+halo_fast_adj_lines_kernel(const __grid_constant__ FastHeader H, const FastDim *__restrict__ dims_g,
+                           const __grid_constant__ ShardPointers sh, bool after_boxes) {
+    if (after_boxes) stream_enter_beside();
+    else stream_enter();
+    halo_fast_adj_lines<T>(H, dims_g, sh);
+    if (after_boxes) stream_leave_beside();
+}
+
 static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &plan, void *const *shards,
                               void *stream, bool adjoint, const char *what) {
     clear_error();
@@ -765,18 +777,15 @@ static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &p
     }();
     if (box_only) {
         if (adjoint)
-            halo_box_kernel<true><<<plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream>>>(
-                plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
+            launch_in_stream(halo_box_kernel<true>, plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream, plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
         else
-            halo_box_kernel<false><<<plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream>>>(
-                plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
+            launch_in_stream(halo_box_kernel<false>, plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream, plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
         DISTDL_CUDA_CHECK(cudaGetLastError());
         return DISTDL_OK;
     }
     if (!adjoint && p->fast.usable && p->fast_dims_dev) {
         const FastHeader &h = p->fast.hdr;
-        halo_fast_fwd_kernel<<<(unsigned)h.num_groups * (unsigned)(h.group[0] + h.group[1]), kFastThreads, 0,
-                               (cudaStream_t)stream>>>(h, p->fast_dims_dev, sh);
+        launch_in_stream(halo_fast_fwd_kernel, (unsigned)h.num_groups * (unsigned)(h.group[0] + h.group[1]), kFastThreads, 0, (cudaStream_t)stream, h, p->fast_dims_dev, sh);
         DISTDL_CUDA_CHECK(cudaGetLastError());
         return DISTDL_OK;
     }
@@ -784,23 +793,21 @@ static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &p
         cudaStream_t st = (cudaStream_t)stream;
         const HaloPlanDevice &rest = p->adj_rest_dev;      // everything but the row ends of the rows out of outer reach
         if (rest.num_tiles > 0) {
-            halo_box_kernel<true><<<rest.num_tiles, kHaloThreads, 0, st>>>(rest.boxes, rest.sources, rest.tiles, elem_size(p->dtype), sh);
+            launch_in_stream(halo_box_kernel<true>, rest.num_tiles, kHaloThreads, 0, st, rest.boxes, rest.sources, rest.tiles, elem_size(p->dtype), sh);
             DISTDL_CUDA_CHECK(cudaGetLastError());
         }
         const FastHeader &h = p->fast.adj_hdr;
         const unsigned grid = (unsigned)h.num_groups * (unsigned)(h.group[0] + h.group[1]);
-        if (p->dtype == DISTDL_F32) halo_fast_adj_lines_kernel<float4><<<grid, kFastThreads, 0, st>>>(h, p->fast_dims_dev, sh);
-        else if (p->dtype == DISTDL_F64) halo_fast_adj_lines_kernel<double2><<<grid, kFastThreads, 0, st>>>(h, p->fast_dims_dev, sh);
-        else halo_fast_adj_lines_kernel<bf16x8><<<grid, kFastThreads, 0, st>>>(h, p->fast_dims_dev, sh);
+        if (p->dtype == DISTDL_F32) launch_in_stream(halo_fast_adj_lines_kernel<float4>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
+        else if (p->dtype == DISTDL_F64) launch_in_stream(halo_fast_adj_lines_kernel<double2>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
+        else launch_in_stream(halo_fast_adj_lines_kernel<bf16x8>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
         DISTDL_CUDA_CHECK(cudaGetLastError());
         return DISTDL_OK;
     }
     if (adjoint)
-        halo_box_kernel<true><<<plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream>>>(
-            plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
+        launch_in_stream(halo_box_kernel<true>, plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream, plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
     else
-        halo_box_kernel<false><<<plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream>>>(
-            plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
+        launch_in_stream(halo_box_kernel<false>, plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream, plan.boxes, plan.sources, plan.tiles, elem_size(p->dtype), sh);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -886,9 +893,7 @@ static distdl_status_t halo_fwd_noalloc_impl(int32_t rank, const int64_t *global
     if (!h.sources.empty())
         DISTDL_CUDA_CHECK(cudaMemcpyAsync(base + bz, h.sources.data(), h.sources.size() * sizeof(HaloSource), cudaMemcpyHostToDevice, s));
     DISTDL_CUDA_CHECK(cudaMemcpyAsync(base + bz + sz, h.tiles.data(), h.tiles.size() * sizeof(HaloTile), cudaMemcpyHostToDevice, s));
-    halo_box_kernel<false><<<(unsigned)h.tiles.size(), kHaloThreads, 0, s>>>(
-        reinterpret_cast<const HaloBox *>(base), reinterpret_cast<const HaloSource *>(base + bz),
-        reinterpret_cast<const HaloTile *>(base + bz + sz), elem_size(p->dtype), sh);
+    launch_in_stream(halo_box_kernel<false>, (unsigned)h.tiles.size(), kHaloThreads, 0, s, reinterpret_cast<const HaloBox *>(base), reinterpret_cast<const HaloSource *>(base + bz), reinterpret_cast<const HaloTile *>(base + bz + sz), elem_size(p->dtype), sh);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -939,8 +944,7 @@ static distdl_status_t repartition_launch(const distdl_repartition *r, const voi
     }
     const HaloPlanDevice &plan = adjoint ? r->adj_dev : r->fwd_dev;
     if (plan.num_tiles == 0) return DISTDL_OK;
-    halo_box_kernel<false><<<plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream>>>(plan.boxes, plan.sources, plan.tiles,
-                                                                                       elem_size(r->dtype), sh);
+    launch_in_stream(halo_box_kernel<false>, plan.num_tiles, kHaloThreads, 0, (cudaStream_t)stream, plan.boxes, plan.sources, plan.tiles, elem_size(r->dtype), sh);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }

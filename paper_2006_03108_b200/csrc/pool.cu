@@ -37,6 +37,7 @@ struct PoolParams {
 // One thread per output.  blockIdx.y = worker, blockIdx.x = (plane, row tile, column tile).
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_fwd_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
+    stream_enter();
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
@@ -81,6 +82,7 @@ __device__ __forceinline__ int div_floor(int a, int b) { return a >= 0 ? a / b :
 // 0 <= p - i0 - i*sh < kh and likewise for the columns.
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_adj_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
+    stream_enter();
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
@@ -169,6 +171,7 @@ struct PoolRow {
 template <int KH, int KW, int SH, int SW, int MODE>
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {
+    stream_enter();
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
@@ -286,6 +289,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
 template <int KH, int KW, int SH, int SW, int MODE>
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {
+    stream_enter();
     const PoolShard &S = P.s[blockIdx.y];
     int rest = blockIdx.x;
     const int tx = rest % tiles_x;
@@ -378,11 +382,11 @@ pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
 template <int KH, int KW, int SH, int SW>
 static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int tiles_x, int tiles_y, int rows, bool adjoint, cudaStream_t s) {
     if (!adjoint) {
-        if (P.mode == DISTDL_POOL_AVG) pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
-        else pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
+        if (P.mode == DISTDL_POOL_AVG) launch_in_stream(pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
+        else launch_in_stream(pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
     } else {
-        if (P.mode == DISTDL_POOL_AVG) pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
-        else pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX><<<grid, block, 0, s>>>(P, tiles_x, tiles_y, rows);
+        if (P.mode == DISTDL_POOL_AVG) launch_in_stream(pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
+        else launch_in_stream(pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
     }
 }
 
@@ -501,8 +505,8 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         if (fixed == 1) launch_pool_fixed<2, 2, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
         else if (fixed == 2) launch_pool_fixed<3, 3, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
         else if (fixed == 3) launch_pool_fixed<3, 3, 1, 1>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
-        else if (!adjoint) pool_fwd_kernel<<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
-        else pool_adj_kernel<<<grid, block, 0, s>>>(P, tiles_x, tiles_y);
+        else if (!adjoint) launch_in_stream(pool_fwd_kernel, grid, block, 0, s, P, tiles_x, tiles_y);
+        else launch_in_stream(pool_adj_kernel, grid, block, 0, s, P, tiles_x, tiles_y);
     }
     DISTDL_CUDA_CHECK(cudaGetLastError());
     if (!adjoint) return DISTDL_OK;

@@ -117,6 +117,7 @@ __device__ __forceinline__ void st_clear(float *out, int bz, int opy, int opx, i
 template <int R, bool VEC>
 __global__ void __launch_bounds__(kStThreads, kStBlocks<R, VEC>)
 stencil3d_kernel(const __grid_constant__ StencilParams P) {
+    stream_enter();
     extern __shared__ __align__(16) float ring[];          // planes of kStRows + 2 R rows
     constexpr int kPlane = (kStRows + 2 * R) * kStPitch;
     constexpr int N = 2 * R + 1;
@@ -394,8 +395,8 @@ static distdl_status_t launch_stencil(const StencilParams &P, unsigned grid, boo
             configured_on[dev] = true;
         }
     }
-    if (vec) stencil3d_kernel<R, true><<<grid, kStThreads, smem, s>>>(P);
-    else stencil3d_kernel<R, false><<<grid, kStThreads, smem, s>>>(P);
+    if (vec) launch_in_stream(stencil3d_kernel<R, true>, grid, kStThreads, smem, s, P);
+    else launch_in_stream(stencil3d_kernel<R, false>, grid, kStThreads, smem, s, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }

@@ -158,3 +158,43 @@ STENCIL_EDGES = [
 @pytest.mark.parametrize("case", STENCIL_EDGES, ids=[str(c) for c in STENCIL_EDGES])
 def test_stencil_planes_and_rows(case):
     parity.test_stencil3d_fwd_and_adj(case)
+
+
+@pytest.mark.parametrize("n", [1 << 20, 1000])
+@pytest.mark.parametrize("captured", [False, True], ids=["eager", "graph"])
+def test_kernels_follow_copies_and_foreign_kernels_in_order(n, captured):
+    """Copies, memsets, other libraries' kernels and a second stream between the operators: each sees what came before it."""
+    torch, distdl, dev = parity.torch, parity.distdl, parity.DEV
+    x = torch.arange(n, device=dev, dtype=torch.float32)
+    y, z, w, out = (torch.empty_like(x) for _ in range(4))
+    pinned = torch.empty(n, pin_memory=True)
+    s, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def body():
+        y.copy_(x)
+        distdl.broadcast_fwd(y, [z, w])
+        w.zero_()
+        distdl.sumreduce_fwd([z, y, w], out)        # 2 x
+        out.mul_(2)
+        distdl.broadcast_fwd(out, [z])              # 4 x
+        pinned.copy_(z, non_blocking=True)
+        s2.wait_stream(s)
+        with torch.cuda.stream(s2):
+            distdl.broadcast_fwd(z, [w])
+        s.wait_stream(s2)
+        distdl.sumreduce_fwd([w, z], y)             # 8 x
+
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            body()
+        run = graph.replay
+    else:
+        def run():
+            with torch.cuda.stream(s):
+                body()
+    torch.cuda.synchronize()
+    for _ in range(20):
+        run()
+    torch.cuda.synchronize()
+    assert torch.equal(y, 8 * x) and torch.equal(z, 4 * x) and torch.equal(pinned, (4 * x).cpu())
