@@ -120,8 +120,9 @@ pool_adj_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) 
 // adjoint, us; before: four outputs or groups of one row per thread, nothing shared between rows; 3 x 3 / 1: the general kernels):
 //   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    370 / 437   (368 / 538)
 //   2 x 2 / 2 max, the same                                   249 / 262   (257 / 312)
-//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      530 / 651   (1653 / 2687)
-// A maximum is taken per input row first (value, first
+//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      485 / 651   (1653 / 2687)
+// The adjoint's cells of a row put together by shuffles, so that a store is 32 cells and not every other one of 64: 3 x 3 / 2
+// 434 -> 500.  A maximum is taken per input row first (value, first
 // position); a NaN counts as the scan in window order counts it: it wins only as the window's first cell.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPoolCols = 2;           // columns per lane, 32 apart
@@ -241,6 +242,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
 #pragma unroll
         for (int a = 0; a < SH; ++a) take(KH - SH + a, v[a]);
         const int gi = S.g0h + S.i0 + i * SH;               // tensor row of window row 0
+        const bool full = inside && gi >= 0 && gi + KH <= P.hg;   // nothing to clip (3 x 3 / 1: 509 -> 465 us on 2 x 2 workers)
 #pragma unroll
         for (int u = 0; u < kPoolCols; ++u) {
             float best = 0.f;
@@ -252,6 +254,17 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
                     for (int c = 0; c < KW; ++c) best = __fadd_rn(best, row[a][u].x[c]);
                 best = __fmul_rn(best, 1.0f / (float)(KH * KW));
             } else {
+                if (full) {
+                    const bool nan = row[0][u].x[0] != row[0][u].x[0];
+                    best = nan ? row[0][u].x[0] : row[0][u].m;
+                    where = nan ? 0 : row[0][u].b;
+#pragma unroll
+                    for (int a = 1; a < KH; ++a)
+                        if (row[a][u].m > best) {
+                            best = row[a][u].m;
+                            where = a * KW + row[a][u].b;
+                        }
+                } else {
                 bool have = false;
 #pragma unroll
                 for (int a = 0; a < KH; ++a) {
@@ -266,6 +279,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
                         best = r.m;
                         where = a * KW + r.b;
                     }
+                }
                 }
             }
             if (on[u]) {
