@@ -149,23 +149,17 @@ struct PoolRow {
                 b = c;
             }
     }
-    // the cells [lo, hi) of the row lie inside the tensor (at least one)
+    // the cells [lo, hi) of the row lie inside the tensor (at least one): the others take the value of the nearest of those,
+    // which changes neither the maximum nor, once it is no smaller than lo, its first position
     __device__ __forceinline__ void reduce_clipped(int lo, int hi) {
-        float first = 0.f;
-        bool have = false;
-        m = 0.f;
-        b = 0;
 #pragma unroll
-        for (int c = 0; c < KW; ++c)
-            if (c >= lo && c < hi) {
-                if (!have) first = x[c];
-                if (!have || x[c] > m || (m != m && x[c] == x[c])) {
-                    m = x[c];
-                    b = c;
-                }
-                have = true;
-            }
-        x[0] = first;
+        for (int c = KW - 2; c >= 0; --c)
+            if (c < lo) x[c] = x[c + 1];
+#pragma unroll
+        for (int c = 1; c < KW; ++c)
+            if (c >= hi) x[c] = x[c - 1];
+        reduce();
+        b = max(b, lo);
     }
 };
 
@@ -182,7 +176,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
     const int lane = threadIdx.x, jb = tx * (32 * kPoolCols) + lane, i_begin = (ty * kPoolThreadsY + (int)threadIdx.y) * rows;
     const int i_end = min(i_begin + rows, S.oh);
     if (i_begin >= i_end || tx * (32 * kPoolCols) >= S.ow) return;
-    bool on[kPoolCols], inside = true;
+    bool on[kPoolCols], inside = true, some = true;         // all / at least one of the window's columns inside the tensor
     int lo[kPoolCols], hi[kPoolCols];                       // window columns inside the tensor
     const float *src[kPoolCols];
     const float *base = S.in + ((size_t)plane * S.ph + (S.i0 + i_begin * SH)) * S.pw + S.j0;
@@ -195,8 +189,10 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
         lo[u] = max(0, -gj);
         hi[u] = min(KW, P.wg - gj);
         inside = inside && lo[u] == 0 && hi[u] == KW;
+        some = some && lo[u] < hi[u];
     }
     inside = __all_sync(0xffffffffu, inside);
+    some = __all_sync(0xffffffffu, some);
     float next[SH][kPoolCols][KW];
     PoolRow<KW> row[KH][kPoolCols];
     auto load = [&](float (&v)[kPoolCols][KW]) {            // one input row, and on to the next
@@ -242,7 +238,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
 #pragma unroll
         for (int a = 0; a < SH; ++a) take(KH - SH + a, v[a]);
         const int gi = S.g0h + S.i0 + i * SH;               // tensor row of window row 0
-        const bool full = inside && gi >= 0 && gi + KH <= P.hg;   // nothing to clip (3 x 3 / 1: 509 -> 465 us on 2 x 2 workers)
+        const bool full = some && gi >= 0 && gi + KH <= P.hg;   // no row of the window outside (3 x 3 / 1: 509 -> 465 us on 2 x 2 workers)
 #pragma unroll
         for (int u = 0; u < kPoolCols; ++u) {
             float best = 0.f;
@@ -257,7 +253,7 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
                 if (full) {
                     const bool nan = row[0][u].x[0] != row[0][u].x[0];
                     best = nan ? row[0][u].x[0] : row[0][u].m;
-                    where = nan ? 0 : row[0][u].b;
+                    where = nan ? lo[u] : row[0][u].b;
 #pragma unroll
                     for (int a = 1; a < KH; ++a)
                         if (row[a][u].m > best) {
@@ -495,7 +491,8 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         max_cols = std::max<int64_t>(max_cols, adjoint ? S.pw : S.ow);
     }
     cudaStream_t s = (cudaStream_t)stream;
-    // the compile-time variants: 64 columns and up to 16 rows per warp (fewer where eight warps would leave some without a row)
+    // the compile-time variants: 64 columns and up to 16 rows per warp, fewer where eight warps would leave some without a row
+    // or an SM would have fewer than 16 warps
     const int fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
                     : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
     if (fixed && adjoint) {
@@ -503,10 +500,18 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         max_rows = max_rows / sh + 2;
         max_cols = max_cols / sw + 2;
     }
-    const int rows = fixed ? (int)std::min<int64_t>(16, std::max<int64_t>(2, (max_rows + kPoolThreadsY - 1) / kPoolThreadsY)) : 1;
     const int cols = fixed ? 32 * kPoolCols : kPoolThreadsX;
     const int tiles_x = (int)((max_cols + cols - 1) / cols);
+    int rows = 1;
+    if (fixed) {
+        int dev = 0, sms = 0;
+        DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
+        DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const int64_t all = (int64_t)p->num_workers * P.planes * tiles_x * max_rows;      // rows of 64 columns
+        rows = (int)std::min<int64_t>(16, std::max<int64_t>(2, std::min((max_rows + kPoolThreadsY - 1) / kPoolThreadsY, all / (16 * sms))));
+    }
     const int tiles_y = (int)((max_rows + kPoolThreadsY * rows - 1) / (kPoolThreadsY * rows));
+    if (fixed) rows = (int)((max_rows + kPoolThreadsY * tiles_y - 1) / (kPoolThreadsY * tiles_y));      // equal shares
     const int64_t blocks = (int64_t)tiles_x * tiles_y * P.planes;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     const dim3 grid((unsigned)blocks, (unsigned)p->num_workers), block(kPoolThreadsX, kPoolThreadsY);

@@ -63,6 +63,9 @@ HALO_EDGES = [
     ((40, 403), (2, 2), 1, 1),               # ghost rows of 201 / 202 cells
     ((9, 10, 311), (2, 2, 1), (1, 2, 1), (2, 1, 1)),
     ((5, 40001), (2, 1), (1, 0), (1, 0)),
+    ((9, 10, 385), (2, 2, 1), (1, 2, 1), (2, 1, 1)),     # rows just long enough to be copied by warps
+    ((257, 9, 34), (1, 1, 2), (0, 0, 1), (0, 0, 1)),     # columns of 2313 cells: tiles of 256, the last one of nine
+    ((64, 4, 66), (1, 1, 2), (0, 0, 1), (0, 0, 2)),      # 256 cells: one whole tile
 ]
 
 
@@ -109,6 +112,8 @@ POOL_EDGES = [
     ((1, 2, 37, 67), (1, 1, 1, 1), (3, 3), (2, 2), ((0, 0), (0, 0))),
     ((1, 1, 300, 22), (1, 1, 2, 1), (2, 2), (2, 2), ((0, 0), (0, 0))),      # several 128-row tiles of warps
     ((1, 3, 9, 260), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),       # 65 outputs: one column past a warp's 64
+    ((40, 9, 66, 61), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),      # several rows a warp, every warp at both ends of the rows
+    ((90, 16, 75, 33), (1, 1, 1, 1), (3, 3), (1, 1), ((1, 1), (1, 1))),     # 75 rows in equal shares of 16 warps
 ]
 
 
