@@ -126,15 +126,33 @@ static_assert(sizeof(HaloTile) == 32, "HaloTile layout");
 // Copies and clears of boxes whose rows are long but not made of aligned 16-byte units go row by row: a warp takes a chunk of
 // a row, kRowUnroll elements per lane.
 constexpr int kRowUnroll = 16;
-constexpr int kRowMinUnits = 96;      // shorter rows: unit by unit (a chunk would leave lanes without an element)
+// Shorter rows go unit by unit, with eight loads of a thread in flight whatever the rows: a warp alone with a row of 100 to 200 units waits
+// for it (H of 200^3 on 2 x 2 x 2 workers, widths 2, and of the pooling layer below: 14.5 -> 7.3 and 29.6 -> 17.8 us with the forward pooling;
+// 1400 x 2000 from row to column blocks, rows of 175 and 250: 10.3 -> 10.7 us).
+constexpr int kRowMinUnits = 384;
 constexpr int kHaloWarps = 8;         // warps of a block
 
 struct HaloPlanHost {
     std::vector<HaloBox> boxes;
     std::vector<HaloSource> sources;
     std::vector<HaloTile> tiles;
+    struct Cut {                   // how a box is cut into tiles
+        int32_t src_begin, nsrc;
+        int64_t units;
+        int64_t row_tile;          // tiles of whole rows: their units;  0: any tile size
+    };
+    std::vector<Cut> cuts;         // per box
     int64_t algorithmic_bytes = 0; // bytes read + written by the in-place method
 };
+
+// Tiles of kTileUnits units, or (fine) of as many as make about eight blocks per multiprocessor with the blocks that small boxes make
+// anyway, a unit for every thread at least: the cells of thin ghost layers are requests of their own to the memory system, which a
+// multiprocessor serves one by one, and 4096 to a block leave most of them idle (H / H* of 292 x 58 x 92 fp64 on 4 x 3 x 2 workers,
+// widths 1: 6.7 / 9.8 -> 5.1 / 7.8 us; max pooling of 8 x 8 x 512 x 512 on 2 x 2 workers with its H / H*: 32.1 / 39.5 -> 30.1 / 33.4 us;
+// 3226 x 101 from columns to rows: 5.4 -> 4.0 us.  Boxes not counted: 88 x 49 x 58 on 4 x 3 x 4, widths 3, 6.4 / 9.9 instead of 6.0 / 8.4 us).
+constexpr int64_t kTileUnits = 4096;
+constexpr int64_t kPlanBlocks = 8 * 148;
+void cut_tiles(HaloPlanHost *plan, bool fine);
 
 struct HaloPlanDevice {
     HaloBox *boxes = nullptr;

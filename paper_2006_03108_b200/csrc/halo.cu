@@ -858,10 +858,14 @@ static distdl_status_t halo_fwd_noalloc_impl(int32_t rank, const int64_t *global
         distdl_partition *p;
         ~Guard() { delete p; }
     } guard{p};
-    const HaloPlanHost &h = p->fwd_host;
+    HaloPlanHost &h = p->fwd_host;
     auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
-    const size_t bz = up(h.boxes.size() * sizeof(HaloBox)), sz = up(h.sources.size() * sizeof(HaloSource)),
-                 tz = up(h.tiles.size() * sizeof(HaloTile));
+    const size_t bz = up(h.boxes.size() * sizeof(HaloBox)), sz = up(h.sources.size() * sizeof(HaloSource));
+    size_t tz = up(h.tiles.size() * sizeof(HaloTile));
+    if (bz + sz + tz > kStaticPlanBytes) {
+        cut_tiles(&h, false);                          // the coarse tiles take less of it
+        tz = up(h.tiles.size() * sizeof(HaloTile));
+    }
     if (bz + sz + tz > kStaticPlanBytes)
         return fail(DISTDL_ERR_UNSUPPORTED,
                     "%s: the plan of this partition needs %zu bytes of tables, the fixed device array holds %zu "

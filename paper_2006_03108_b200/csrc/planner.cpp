@@ -85,6 +85,30 @@ extern "C" distdl_status_t distdl_halo_widths_1d(int64_t n, int32_t p, int32_t k
 // ---------------------------------------------------------------------------------------------
 // Box construction
 // ---------------------------------------------------------------------------------------------
+void distdl::cut_tiles(HaloPlanHost *plan, bool fine) {
+    constexpr int64_t kTileThreads = 32 * kHaloWarps;
+    int64_t total = 0;
+    for (const HaloPlanHost::Cut &c : plan->cuts) total += c.units;
+    const int64_t share = total / std::max<int64_t>(kPlanBlocks / 8, kPlanBlocks - (int64_t)plan->cuts.size()) + 1;
+    const int64_t whole = std::max<int64_t>(1, (share + kTileThreads - 1) / kTileThreads) * kTileThreads;
+    const int64_t size = fine ? std::min(kTileUnits, whole) : kTileUnits;
+    plan->tiles.clear();
+    for (size_t box = 0; box < plan->cuts.size(); ++box) {
+        const HaloPlanHost::Cut &c = plan->cuts[box];
+        const int64_t step = c.row_tile ? c.row_tile : size;
+        for (int64_t at = 0; at < c.units; at += step) {
+            HaloTile t;
+            memset(&t, 0, sizeof(t));
+            t.box = (int32_t)box;
+            t.src_begin = c.src_begin;
+            t.nsrc = c.nsrc;
+            t.first = (uint32_t)at;
+            t.count = (uint32_t)std::min<int64_t>(step, c.units - at);
+            plan->tiles.push_back(t);
+        }
+    }
+}
+
 namespace {
 
 struct Region {             // a rectangular set of cells of one shard, in padded-local indices
@@ -98,8 +122,6 @@ struct PendingSource {
     int32_t close;
     int32_t clear_after;
 };
-
-constexpr uint32_t kTileUnits = 4096;
 
 struct Builder {
     HaloPlanHost *plan;
@@ -255,10 +277,9 @@ struct Builder {
             for (int i = 0; i < nd_units; ++i) s.stride[i] = (uint32_t)ss[j][i];
             plan->sources.push_back(s);
         }
-        const int32_t box_id = (int32_t)plan->boxes.size();
         plan->boxes.push_back(b);
         // rows copied chunk by chunk: tiles of whole rows, as many as give every warp of a block the same number of chunks
-        int64_t tile_units = kTileUnits;
+        int64_t tile_units = 0;
         const int64_t inner = shape[nd_units - 1];
         if (srcs.size() <= 1 && !vec && inner >= kRowMinUnits && inner <= kTileUnits && units > 4 * (int64_t)kTileUnits) {
             const int64_t chunks = (inner + 32 * kRowUnroll - 1) / (32 * kRowUnroll);
@@ -266,16 +287,7 @@ struct Builder {
             for (int64_t c = chunks; step > 1 && c % 2 == 0; c /= 2) step /= 2;
             tile_units = inner * ((10240 / inner + step - 1) / step * step);
         }
-        for (int64_t at = 0; at < units; at += tile_units) {
-            HaloTile t;
-            memset(&t, 0, sizeof(t));
-            t.box = box_id;
-            t.src_begin = src_begin;
-            t.nsrc = (int32_t)srcs.size();
-            t.first = (uint32_t)at;
-            t.count = (uint32_t)std::min<int64_t>(tile_units, units - at);
-            plan->tiles.push_back(t);
-        }
+        plan->cuts.push_back({src_begin, (int32_t)srcs.size(), units, tile_units});
         // algorithmic traffic: destination written once; every source read once; cleared sources
         // written once; the destination's own previous value is source 0 of a sum (counted there).
         int64_t bytes = cells * esize;
@@ -407,6 +419,7 @@ distdl_status_t build_halo_plans(distdl_partition *p, bool forward_only) {
             }
         } while (next_delta(delta, d));
     }
+    cut_tiles(&p->fwd_host, true);
     // The forward-only form serves the entry point that builds its plan at every call: the pairwise check of the
     // destination boxes (quadratic in their number) is left to partition_create, which builds the same boxes.
     if (forward_only) return DISTDL_OK;
@@ -508,6 +521,8 @@ distdl_status_t build_halo_plans(distdl_partition *p, bool forward_only) {
     }
     if (!ab.destinations_disjoint()) return fail(DISTDL_ERR_SHAPE, "halo plan: adjoint boxes overlap");
     if (split_adj && !rb.destinations_disjoint()) return fail(DISTDL_ERR_SHAPE, "halo plan: adjoint boxes overlap");
+    cut_tiles(&p->adj_host, true);
+    cut_tiles(&p->adj_rest_host, true);
     return DISTDL_OK;
 }
 
@@ -568,6 +583,8 @@ distdl_status_t build_repartition_plans(distdl_repartition *r) {
     }
     if (!fb.destinations_disjoint() || !ab.destinations_disjoint())
         return fail(DISTDL_ERR_SHAPE, "repartition plan: boxes overlap");
+    cut_tiles(&r->fwd_host, true);
+    cut_tiles(&r->adj_host, true);
     return DISTDL_OK;
 }
 
