@@ -8,6 +8,7 @@
 // same nested sum the d reversed phases would produce -- own value, low neighbour, high
 // neighbour within a dimension; dimension 0 outermost -- so the result is bit-identical to the
 // phase-by-phase order.  Each ghost cell is read by exactly one thread, which also clears it.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -747,6 +748,36 @@ halo_fast_adj_lines_kernel(const __grid_constant__ FastHeader H, const FastDim *
     if (after_boxes) stream_leave_beside();
 }
 
+// Whether any of the arrays may overlap: in address order, does one begin before all before it have ended.  (Pair by pair, 48
+// workers' exchange and its adjoint spent 22 of 48 us here, 36 workers' 13 of 34.)
+struct Span {
+    const char *begin, *end;
+};
+static bool may_overlap(Span *spans, int n) {
+    std::sort(spans, spans + n, [](const Span &a, const Span &b) { return a.begin < b.begin; });
+    const char *end = nullptr;
+    for (int i = 0; i < n; ++i) {
+        if (i > 0 && spans[i].begin < end) return true;
+        end = i > 0 ? std::max(end, spans[i].end) : spans[i].end;
+    }
+    return false;
+}
+
+// shards must not overlap (each is written in place); the pair named is the first one
+static distdl_status_t check_disjoint(const distdl_partition *p, const void *const *shards, const char *what) {
+    const int64_t es = elem_size(p->dtype);
+    Span spans[DISTDL_MAX_WORKERS];
+    for (int32_t w = 0; w < p->num_workers; ++w) spans[w] = {(const char *)shards[w], (const char *)shards[w] + p->shard_elems(w) * es};
+    if (!may_overlap(spans, p->num_workers)) return DISTDL_OK;
+    for (int32_t a = 0; a < p->num_workers; ++a)
+        for (int32_t b = a + 1; b < p->num_workers; ++b) {
+            const char *a0 = (const char *)shards[a], *a1 = a0 + p->shard_elems(a) * es;
+            const char *b0 = (const char *)shards[b], *b1 = b0 + p->shard_elems(b) * es;
+            if (a0 < b1 && b0 < a1) return fail(DISTDL_ERR_INVALID_ARG, "%s: shards %d and %d overlap", what, a, b);
+        }
+    return DISTDL_OK;
+}
+
 static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &plan, void *const *shards,
                               void *stream, bool adjoint, const char *what) {
     clear_error();
@@ -758,16 +789,7 @@ static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &p
         if (!aligned16(shards[w])) return fail(DISTDL_ERR_ALIGNMENT, "%s: shards[%d] is not 16-byte aligned", what, w);
         sh.p[w] = shards[w];
     }
-    // shards must not overlap (each is written in place)
-    {
-        const int64_t es = elem_size(p->dtype);
-        for (int32_t a = 0; a < p->num_workers; ++a)
-            for (int32_t b = a + 1; b < p->num_workers; ++b) {
-                const char *a0 = (const char *)shards[a], *a1 = a0 + p->shard_elems(a) * es;
-                const char *b0 = (const char *)shards[b], *b1 = b0 + p->shard_elems(b) * es;
-                if (a0 < b1 && b0 < a1) return fail(DISTDL_ERR_INVALID_ARG, "%s: shards %d and %d overlap", what, a, b);
-            }
-    }
+    if (const distdl_status_t st = check_disjoint(p, shards, what)) return st;
     for (int32_t w = p->num_workers; w < DISTDL_MAX_WORKERS; ++w) sh.p[w] = nullptr;
     if (plan.num_tiles == 0) return DISTDL_OK;
     // DISTDL_HALO_PLAN=box in the environment sends every call through the general box plan (for comparisons)
@@ -872,18 +894,12 @@ static distdl_status_t halo_fwd_noalloc_impl(int32_t rank, const int64_t *global
                     "(use distdl_partition_create + distdl_halo_fwd for larger partitions)",
                     what, bz + sz + tz, kStaticPlanBytes);
     ShardPointers sh;
-    const int64_t es = elem_size(p->dtype);
     for (int32_t w = 0; w < p->num_workers; ++w) {
         if (!shards[w]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shards[%d] is NULL", what, w);
         if (!aligned16(shards[w])) return fail(DISTDL_ERR_ALIGNMENT, "%s: shards[%d] is not 16-byte aligned", what, w);
         sh.p[w] = shards[w];
     }
-    for (int32_t a = 0; a < p->num_workers; ++a)
-        for (int32_t b = a + 1; b < p->num_workers; ++b) {
-            const char *a0 = (const char *)shards[a], *a1 = a0 + p->shard_elems(a) * es;
-            const char *b0 = (const char *)shards[b], *b1 = b0 + p->shard_elems(b) * es;
-            if (a0 < b1 && b0 < a1) return fail(DISTDL_ERR_INVALID_ARG, "%s: shards %d and %d overlap", what, a, b);
-        }
+    if (const distdl_status_t overlap = check_disjoint(p, shards, what)) return overlap;
     for (int32_t w = p->num_workers; w < DISTDL_MAX_WORKERS; ++w) sh.p[w] = nullptr;
     if (h.tiles.empty()) return DISTDL_OK;
     unsigned char *base = nullptr;

@@ -203,3 +203,18 @@ def test_kernels_follow_copies_and_foreign_kernels_in_order(n, captured):
         run()
     torch.cuda.synchronize()
     assert torch.equal(y, 8 * x) and torch.equal(z, 4 * x) and torch.equal(pinned, (4 * x).cpu())
+
+
+def test_halo_names_the_first_overlapping_pair():
+    torch, distdl = parity.torch, parity.distdl
+    part = distdl.Partition((12, 40), (3, 2), [1, 1], [1, 1])
+    size = [int(np.prod(part.padded_shape(w))) for w in range(6)]
+    pool = torch.zeros(6 * 4096, device=parity.DEV)
+    at = [5 * 4096, 3 * 4096, 4096, 4 * 4096, 4096 + 4, 0]          # shards 2 and 4 share cells, in no address order
+    shards = [pool[a:a + n] for a, n in zip(at, size)]
+    for op in (distdl.halo_fwd, distdl.halo_adj):
+        with pytest.raises(distdl.DistdlError, match="shards 2 and 4 overlap"):
+            op(part, shards)
+    shards[4] = pool[2 * 4096:2 * 4096 + size[4]]
+    distdl.halo_fwd(part, shards)
+    torch.cuda.synchronize()
