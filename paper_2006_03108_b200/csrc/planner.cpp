@@ -298,10 +298,13 @@ struct Builder {
 
     bool destinations_disjoint() const {
         const int d = rank;
-        for (size_t a = 0; a < dst_regions.size(); ++a)
-            for (size_t b = a + 1; b < dst_regions.size(); ++b) {
-                const Region &x = dst_regions[a], &y = dst_regions[b];
-                if (x.shard != y.shard) continue;
+        // in shard order: only boxes of one shard can meet (every pair of a plan's boxes took half of partition_create at 512^3 on 64 workers)
+        std::vector<const Region *> order;
+        for (const Region &r : dst_regions) order.push_back(&r);
+        std::stable_sort(order.begin(), order.end(), [](const Region *x, const Region *y) { return x->shard < y->shard; });
+        for (size_t a = 0; a < order.size(); ++a)
+            for (size_t b = a + 1; b < order.size() && order[b]->shard == order[a]->shard; ++b) {
+                const Region &x = *order[a], &y = *order[b];
                 bool overlap = true;
                 for (int k = 0; k < d && overlap; ++k)
                     overlap = x.start[k] < y.start[k] + y.extent[k] && y.start[k] < x.start[k] + x.extent[k];
