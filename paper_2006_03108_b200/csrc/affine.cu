@@ -346,7 +346,7 @@ affine_kernel_pair(const __grid_constant__ AffineParams P) {
 // staged and multiplied for 16 samples, one block per 128 features) 64 of 148 SMs read 8192 x 8192 weights, half of
 // every stage was padding: 57 us for 16 samples.  As the M operand the batch takes N = 16, 32, ... columns
 // of the instruction and 2 KB per 16 samples of a stage; S blocks per tile keep twice as many blocks as
-// SMs reading.  8192 x 8192 weights on 4 x 4 workers (B200, weights cold): 16 samples 57 -> 27 us (0.76 of the copy rate),
+// SMs reading.  8192 x 8192 weights on 4 x 4 workers (B200, weights cold): 16 samples 57 -> 26 us (0.8 of the copy rate),
 // 64 samples forward / adjoint 44 / 38 -> 28 / 27 us, 128 samples 46 / 40 -> 31 / 30 us.
 // ------------------------------------------------------------------------------------------
 constexpr int kSplitWBytes = kTileM * kBlockK * 2;           // 16 KB: 128 features x 64 of the contraction

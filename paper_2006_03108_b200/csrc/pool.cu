@@ -118,9 +118,9 @@ pool_adj_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) 
 //
 // What bounds them: device memory, instruction issue close behind.  Measured (B200, with the H / H* around them, forward /
 // adjoint, us; before: four outputs or groups of one row per thread, nothing shared between rows; 3 x 3 / 1: the general kernels):
-//   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    370 / 437   (368 / 538)
-//   2 x 2 / 2 max, the same                                   249 / 262   (257 / 312)
-//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      485 / 651   (1653 / 2687)
+//   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    358 / 421   (368 / 538)
+//   2 x 2 / 2 max, the same                                   260 / 252   (259 / 313)
+//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      457 / 651   (1653 / 2687)
 // The adjoint's cells of a row put together by shuffles, so that a store is 32 cells and not every other one of 64: 3 x 3 / 2
 // 434 -> 500.  A maximum is taken per input row first (value, first
 // position); a NaN counts as the scan in window order counts it: it wins only as the window's first cell.
