@@ -93,6 +93,7 @@ def lib():
     L.distdl_device_status.argtypes = [vp]
     L.distdl_selftest_wait_timeout.argtypes = [c_i64, vp]
     L.distdl_selftest_row_plan.argtypes = [vp, c_i32, pi32, c_i32, pi32, c_i32, pi32]
+    L.distdl_selftest_conv_row_reads.argtypes = [vp, c_i32, c_i32, pi64, pi64]
     _lib = L
     return L
 
@@ -491,3 +492,11 @@ def selftest_row_plan(part, adjoint=False):
     n = ctypes.c_int32(0)
     _check(lib().distdl_selftest_row_plan(part.handle, 1 if adjoint else 0, hdr, 64, rec, 16 * 64, ctypes.byref(n)))
     return list(hdr), [list(rec[16 * i:16 * i + 16]) for i in range(n.value)]
+
+
+def selftest_conv_row_reads(part, k, gradients=False):
+    """(floats read past the end of a shard's array at most, rows copied cell by cell) of the depthwise convolution's copies
+    from arrays without ghosts (include/distdl_selftest.h)."""
+    past, cells = ctypes.c_int64(0), ctypes.c_int64(0)
+    _check(lib().distdl_selftest_conv_row_reads(part.handle, int(k), 1 if gradients else 0, ctypes.byref(past), ctypes.byref(cells)))
+    return past.value, cells.value

@@ -33,6 +33,10 @@ def test_generalized_conv_tiles(case, integer):
 # global NCHW, partition, kernel
 CONV_EDGES = [
     ((1, 1, 5, 1), (1, 1, 1, 1), 3),         # one column
+    ((1, 1, 6, 1), (1, 1, 1, 1), 3),         # the array ends inside the 16-byte block of the row before the last
+    ((1, 1, 7, 1), (1, 1, 1, 1), 5),         # and of the row before that
+    ((1, 3, 1, 1), (1, 1, 1, 1), 3),         # of the planes before the last
+    ((1, 1, 6, 3), (1, 1, 1, 3), 3),         # the same in three shards
     ((1, 2, 3, 3), (1, 1, 1, 1), 7),         # a kernel wider than the image
     ((1, 2, 9, 66), (1, 1, 1, 1), 7),        # 64-column strips, the last of two columns, narrower than the halo
     ((1, 1, 40, 129), (1, 1, 1, 1), 7),      # 128-column strips, the last of one column

@@ -286,3 +286,21 @@ def test_partition_broadcast_rejects_shapes_that_do_not_broadcast():
     assert call((2, 1), (1, 2)) == 2
     assert call((1,), (512,)) == 4                                                        # DISTDL_ERR_UNSUPPORTED
     assert lib.distdl_partition_broadcast_fwd(1, None, None, elems, ptrs, ptrs, distdl.F32, None) == 1
+
+
+@pytest.mark.parametrize("gradients", [False, True])
+@pytest.mark.parametrize("k", [3, 5, 7])
+def test_depthwise_convolution_copies_end_inside_their_arrays(k, gradients):
+    """Rows of arrays without ghosts travel in 16-byte blocks: none may begin before the array's end and reach past it, and
+    the rows that would are the few of the last 12 bytes."""
+    h = (0, 0, k // 2, k // 2)
+    for planes in (1, 2, 3, 4):
+        for rows in range(1, 12):
+            for cols in (1, 2, 3, 4, 5, 9, 66, 130):
+                part = distdl.Partition((1, planes, rows, cols), (1, 1, 1, 1), h, h)
+                past, by_cell = distdl.selftest_conv_row_reads(part, k, gradients)
+                assert past <= 0 and by_cell <= 3, (planes, rows, cols, past, by_cell)
+    if k == 3:
+        part = distdl.Partition((1, 1, 6, 3), (1, 1, 1, 3), h, h)
+        past, by_cell = distdl.selftest_conv_row_reads(part, k, gradients)
+        assert past <= 0 and by_cell <= 3 * 3
