@@ -783,6 +783,7 @@ affine_kernel_quad(const __grid_constant__ AffineParams P) {
 // MMAs of the next tile run.
 // ------------------------------------------------------------------------------------------
 constexpr int kDwThreads = 192;                              // warp 0: TMA, warp 1: MMA + TMEM, warps 2..5: epilogue
+constexpr int kDbWarps = 8;                                  // with db: warps 6..13
 constexpr int kDwAtomBytes = 64 * kBlockK * 2;               // a 64 x 64 bf16 atom = 8 KB
 constexpr int kDwOutBytes = 4 * kTileM * 32 * 4;             // 64 KB: four 128 x 32 boxes of the fp32 tile
 template <int TN>
@@ -802,7 +803,9 @@ struct AffineDwParams {
     int32_t tiles_m, tiles_n;               // 128 x TN tiles per worker block
     int32_t total_tiles;
     int32_t bfi;                            // columns of a dW block
-    int32_t after_db;                       // the kernel before it in the stream is the bias gradient's, which it does not depend on
+    const uint16_t *dy[8];                  // the bias gradient: dy_i, db_i (null: none wanted), columns of a dy block
+    float *db[8];
+    int32_t pfo, bfo;
 };
 
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int32_t c0, int32_t c1) {
@@ -841,17 +844,50 @@ __device__ __forceinline__ DwTile dw_tile(const AffineDwParams &P, int tile) {
     return t;
 }
 
+// db_i[o] = sum over the batch of dy_i[b, o], fp32 sums of bf16 values in a fixed order: the batch is cut
+// into eight contiguous chunks (one per warp, rows ascending inside a chunk) and the chunk sums are
+// added in chunk order.  64 columns of one dy block at a time; thirty-two loads of a lane in flight.
+__device__ __forceinline__ void affine_db_columns(const AffineDwParams &P, int warp, int lane) {
+    __shared__ float part[kDbWarps][64];
+    const int groups = (P.bfo + 63) / 64, t = 32 * warp + lane;
+    const int chunk = (P.nb + kDbWarps - 1) / kDbWarps, b0 = warp * chunk, b1 = min(P.nb, b0 + chunk);
+    for (int g = blockIdx.x; g < P.pfo * groups; g += gridDim.x) {
+        const int i = g / groups, col0 = (g - i * groups) * 64;
+        float s0 = 0.f, s1 = 0.f;
+        if (col0 + 2 * lane < P.bfo) {
+            const uint16_t *src = P.dy[i] + col0 + 2 * lane;
+#pragma unroll 32
+            for (int b = b0; b < b1; ++b) {
+                const uint32_t two = __ldg(reinterpret_cast<const uint32_t *>(src + (size_t)b * P.bfo));
+                s0 += __uint_as_float(two << 16);
+                s1 += __uint_as_float(two & 0xffff0000u);
+            }
+        }
+        part[warp][2 * lane] = s0;
+        part[warp][2 * lane + 1] = s1;
+        asm volatile("bar.sync 2, %0;" ::"n"(32 * kDbWarps) : "memory");
+        if (t < 64) {
+            float v = part[0][t];
+#pragma unroll
+            for (int w = 1; w < kDbWarps; ++w) v += part[w][t];
+            if (col0 + t < P.bfo) P.db[i][col0 + t] = v;
+        }
+        asm volatile("bar.sync 2, %0;" ::"n"(32 * kDbWarps) : "memory");
+    }
+}
+
 // Persistent: one block per SM walks over tiles blockIdx.x, + gridDim.x, ...  The producer runs ahead
 // through a ring of four (three wide) stages, the accumulator alternates between two
 // halves of tensor memory, and the epilogue of tile t (tensor memory -> swizzled shared
 // memory -> TMA stores) runs while the tensor cores work on tile t + 1.
 //
 // What bounds it: the SM's port into L2, and the store of the fp32 result.  A 128 x 128 tile takes 128 KB of operands in
-// for 64 KB out at batch 256, a 128 x 256 tile 192 KB for 128 KB, a sixth less for the same output.  8192 x 8192 on 4 x 4 workers, db
-// with it (B200): batch 256 67.0 -> 59.6 us (63.6 by the bias gradient in its shadow alone), where writing dW takes 41 us at the
-// copy rate; 4096 x 4096, batch 1024: 71 -> 58 us.
+// for 64 KB out at batch 256, a 128 x 256 tile 192 KB for 128 KB, a sixth less for the same output.  db is the work of eight warps
+// of its own, beside the tiles of their block.  8192 x 8192 on 4 x 4 workers, batch 256 (B200): 56.4 us without db, 56.5 with it,
+// where writing dW takes 41 us at the copy rate (db as a launch of its own that dW's blocks came in behind: 57.7); 4096 x 4096, batch
+// 1024: 35.3 (36.9); 2048 x 2048 on 2 x 2, batch 64: 9.5 (11.6); 128 x 128, batch 16384: 102 (135).
 template <int TN>
-__global__ void __launch_bounds__(kDwThreads, 1)
+__global__ void __launch_bounds__(kDwThreads + 32 * kDbWarps, 1)
 affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
     constexpr int kDwStages = DwShape<TN>::kStages, kDwStageBytes = DwShape<TN>::kStageBytes, kDwABytes = DwShape<TN>::kABytes;
     constexpr int kDwTmemCols = DwShape<TN>::kTmemCols;
@@ -891,8 +927,7 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
     tcgen05_fence_before();
     __syncthreads();
     tcgen05_fence_after();
-    if (P.after_db) stream_enter_beside();
-    else stream_enter();
+    stream_enter();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
@@ -962,6 +997,8 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
             }
         }
         __syncwarp();
+    } else if (warp >= kDwThreads / 32) {
+        affine_db_columns(P, warp - kDwThreads / 32, lane);
     } else {
         // epilogue.  Box q of the staging buffer (columns 32 q .. 32 q + 31) is a 128 x 32 fp32 array of
         // 128-byte rows with the 16-byte chunks of row r stored at chunk ^ (r & 7): the layout of a
@@ -1013,50 +1050,11 @@ affine_dw_kernel(const __grid_constant__ AffineDwParams P) {
         }
         if (issuer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // all stores done before the block retires
     }
-    if (P.after_db) stream_leave_beside();
     tcgen05_fence_before();
     __syncthreads();
     if (warp == 1) {
         tcgen05_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)kDwTmemCols) : "memory");
-    }
-}
-
-// db_i[o] = sum over the batch of dy_i[b, o], fp32 sums of bf16 values in a fixed order: the batch is cut
-// into eight contiguous chunks (one per warp, rows ascending inside a chunk) and the chunk sums are
-// added in chunk order.  A block covers 64 columns of one dy block.
-struct AffineDbParams {
-    const uint16_t *dy[8];
-    float *db[8];
-    int32_t nb, bfo;
-};
-constexpr int kDbThreads = 256;
-__global__ void __launch_bounds__(kDbThreads) affine_db_kernel(const AffineDbParams P) {
-    __shared__ float part[kDbThreads / 32][64];
-    stream_enter();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int col = blockIdx.x * 64 + 2 * lane;
-    const int i = blockIdx.y;
-    const int chunk = (P.nb + kDbThreads / 32 - 1) / (kDbThreads / 32);
-    const int b0 = warp * chunk, b1 = min(P.nb, b0 + chunk);
-    const uint16_t *src = P.dy[i] + col;
-    float s0 = 0.f, s1 = 0.f;
-    if (col < P.bfo) {
-#pragma unroll 8
-        for (int b = b0; b < b1; ++b) {
-            const uint32_t two = *reinterpret_cast<const uint32_t *>(src + (size_t)b * P.bfo);
-            s0 += __uint_as_float(two << 16);
-            s1 += __uint_as_float(two & 0xffff0000u);
-        }
-    }
-    part[warp][2 * lane] = s0;
-    part[warp][2 * lane + 1] = s1;
-    __syncthreads();
-    if (threadIdx.x < 64) {
-        float v = part[0][threadIdx.x];
-#pragma unroll
-        for (int w = 1; w < kDbThreads / 32; ++w) v += part[w][threadIdx.x];
-        if (blockIdx.x * 64 + (int)threadIdx.x < P.bfo) P.db[i][blockIdx.x * 64 + threadIdx.x] = v;
     }
 }
 
@@ -1265,23 +1263,17 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
     const bool wide = (wide_tiles + slots - 1) / slots * (192 + 128) < (tiles + slots - 1) / slots * (128 + 64);
     P.tiles_n = (int32_t)(wide ? (bfi + 255) / 256 : (bfi + 127) / 128);
     P.total_tiles = (int32_t)(wide ? wide_tiles : tiles);
-    if (db) {
-        AffineDbParams B;
-        memset(&B, 0, sizeof(B));
+    P.pfo = pfo;
+    P.bfo = (int32_t)bfo;
+    if (db)
         for (int i = 0; i < pfo; ++i) {
-            B.dy[i] = (const uint16_t *)dy[i];
-            B.db[i] = (float *)db[i];
+            P.dy[i] = (const uint16_t *)dy[i];
+            P.db[i] = (float *)db[i];
         }
-        B.nb = (int32_t)nb;
-        B.bfo = (int32_t)bfo;
-        dim3 grid((unsigned)((bfo + 63) / 64), (unsigned)pfo);
-        launch_in_stream(affine_db_kernel, grid, kDbThreads, 0, (cudaStream_t)stream, B);
-        DISTDL_CUDA_CHECK(cudaGetLastError());
-    }
-    P.after_db = db ? 1 : 0;
+    const int threads = kDwThreads + (db ? 32 * kDbWarps : 0);
     const dim3 dw_grid((unsigned)std::min<int64_t>(P.total_tiles, slots));
-    if (wide) launch_in_stream(affine_dw_kernel<256>, dw_grid, kDwThreads, DwShape<256>::kSmemBytes, (cudaStream_t)stream, P);
-    else launch_in_stream(affine_dw_kernel<128>, dw_grid, kDwThreads, DwShape<128>::kSmemBytes, (cudaStream_t)stream, P);
+    if (wide) launch_in_stream(affine_dw_kernel<256>, dw_grid, threads, DwShape<256>::kSmemBytes, (cudaStream_t)stream, P);
+    else launch_in_stream(affine_dw_kernel<128>, dw_grid, threads, DwShape<128>::kSmemBytes, (cudaStream_t)stream, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }

@@ -39,11 +39,6 @@ __device__ __forceinline__ void stream_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// For a kernel that does not depend on the kernel right before it in the stream (but on what came before that): it runs beside
-// it and waits for it at the end, so that what follows in the stream comes after both.
-__device__ __forceinline__ void stream_enter_beside() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void stream_leave_beside() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 template <typename... P, typename... A>
 inline void launch_clusters_in_stream(void (*kernel)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                       const A &...args) {

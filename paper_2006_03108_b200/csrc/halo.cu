@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "common.h"
 
@@ -190,16 +191,20 @@ __device__ __forceinline__ void stores_after(const double &v) { asm volatile("" 
 __device__ __forceinline__ void stores_after(const bf16x8 &v) { asm volatile("" ::"r"(v.v.x), "r"(v.v.y), "r"(v.v.z), "r"(v.v.w) : "memory"); }
 __device__ __forceinline__ void stores_after(const bf16x1 &v) { asm volatile("" ::"h"(v.v) : "memory"); }
 
-template <typename T, int NSRC>
+// U: units per thread per batch; SHORT: an address is kept as 32-bit offset (fewer registers) instead of pointer.
+template <typename T, int NSRC, int U, bool SHORT>
 __device__ __forceinline__ void run_sum_tile_balanced(const HaloBox &box, const HaloSource *src,
                                                       const ShardPointers &sh, uint32_t first, uint32_t count) {
-    constexpr int U = NSRC >= 8 ? 1 : (NSRC == 4 ? 2 : 8);   // units per thread per batch
     const int nd = box.ndim;
     T *base[NSRC];
 #pragma unroll
     for (int j = 0; j < NSRC; ++j) base[j] = reinterpret_cast<T *>(sh.p[src[j].shard]) + src[j].offset;
     for (uint32_t b0 = threadIdx.x; b0 < count; b0 += kHaloThreads * U) {
-        T *ptr[U][NSRC];
+        typename std::conditional<SHORT, uint32_t, T *>::type at[U][NSRC];
+        auto cell = [&](int u, int j) -> T & {
+            if constexpr (SHORT) return base[j][at[u][j]];
+            else return *at[u][j];
+        };
         T v[U][NSRC];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -209,8 +214,9 @@ __device__ __forceinline__ void run_sum_tile_balanced(const HaloBox &box, const 
                 decompose(box, first + i, c);
 #pragma unroll
                 for (int j = 0; j < NSRC; ++j) {
-                    ptr[u][j] = base[j] + dot_stride(c, src[j].stride, nd);
-                    v[u][j] = *ptr[u][j];
+                    if constexpr (SHORT) at[u][j] = dot_stride(c, src[j].stride, nd);
+                    else at[u][j] = base[j] + dot_stride(c, src[j].stride, nd);
+                    v[u][j] = cell(u, j);
                 }
             }
         }
@@ -227,9 +233,9 @@ __device__ __forceinline__ void run_sum_tile_balanced(const HaloBox &box, const 
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (b0 + u * kHaloThreads < count) {
-                *ptr[u][0] = v[u][0];
+                cell(u, 0) = v[u][0];
 #pragma unroll
-                for (int j = 1; j < NSRC; ++j) *ptr[u][j] = zero_of<T>();
+                for (int j = 1; j < NSRC; ++j) cell(u, j) = zero_of<T>();
             }
         }
     }
@@ -280,27 +286,25 @@ __device__ __forceinline__ void run_sum_tile_general(const HaloBox &box, const H
     }
 }
 
-template <typename T>
+// BLOCKS: blocks per multiprocessor, which the loads in flight are shared among.
+template <typename T, int BLOCKS>
 __device__ __forceinline__ void run_sum_tile(const HaloBox &box, const HaloSource *src, int nsrc,
                                              const ShardPointers &sh, uint32_t first, uint32_t count) {
-    if (box.balanced && nsrc == 2) run_sum_tile_balanced<T, 2>(box, src, sh, first, count);
-    else if (box.balanced && nsrc == 4) run_sum_tile_balanced<T, 4>(box, src, sh, first, count);
-    else if (box.balanced && nsrc == 8) run_sum_tile_balanced<T, 8>(box, src, sh, first, count);
+    if (box.balanced && nsrc == 2) run_sum_tile_balanced<T, 2, 16 / BLOCKS, (BLOCKS > 2)>(box, src, sh, first, count);
+    else if (box.balanced && nsrc == 4) run_sum_tile_balanced<T, 4, 4 / BLOCKS, (BLOCKS > 2)>(box, src, sh, first, count);
+    else if (box.balanced && nsrc == 8) run_sum_tile_balanced<T, 8, 1, (BLOCKS > 2)>(box, src, sh, first, count);
     else run_sum_tile_general<T>(box, src, nsrc, sh, first, count);
 }
 
 // One thread block per tile.  SUMS = false: the forward plan (copies and clears only).
-template <bool SUMS>
-__global__ void __launch_bounds__(kHaloThreads, SUMS ? 2 : 4)
-halo_box_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict__ sources,
-                const HaloTile *__restrict__ tiles, int32_t elem_bytes,
-                const __grid_constant__ ShardPointers sh) {
-    stream_enter();
+template <bool SUMS, int BLOCKS>
+__device__ __forceinline__ void halo_box_block(const HaloBox *__restrict__ boxes, const HaloSource *__restrict__ sources,
+                                               const HaloTile *__restrict__ tiles, int32_t elem_bytes, const ShardPointers &sh, uint32_t block) {
     __shared__ __align__(16) HaloBox s_box;
     __shared__ __align__(16) HaloSource s_src[kMaxSources];
     // every thread reads the (uniform) tile record; box and sources are staged in shared memory
-    const uint4 t0 = __ldg(reinterpret_cast<const uint4 *>(tiles + blockIdx.x));
-    const uint32_t count = __ldg(&tiles[blockIdx.x].count);
+    const uint4 t0 = __ldg(reinterpret_cast<const uint4 *>(tiles + block));
+    const uint32_t count = __ldg(&tiles[block].count);
     const int box_id = (int)t0.x, src_begin = (int)t0.y, nsrc = (int)t0.z;
     const uint32_t first = t0.w;
     {
@@ -327,17 +331,25 @@ halo_box_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict_
         else if (elem_bytes == 8) run_copy_tile<unsigned long long>(s_box, s_src, nsrc, sh, first, count);
         else run_copy_tile<unsigned short>(s_box, s_src, nsrc, sh, first, count);
     } else if (elem_bytes == 4) {
-        if (s_box.vec) run_sum_tile<float4>(s_box, s_src, nsrc, sh, first, count);
-        else run_sum_tile<float>(s_box, s_src, nsrc, sh, first, count);
+        if (s_box.vec) run_sum_tile<float4, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
+        else run_sum_tile<float, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
     } else if (elem_bytes == 8) {
-        if (s_box.vec) run_sum_tile<double2>(s_box, s_src, nsrc, sh, first, count);
-        else run_sum_tile<double>(s_box, s_src, nsrc, sh, first, count);
+        if (s_box.vec) run_sum_tile<double2, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
+        else run_sum_tile<double, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
     } else {
-        if (s_box.vec) run_sum_tile<bf16x8>(s_box, s_src, nsrc, sh, first, count);
-        else run_sum_tile<bf16x1>(s_box, s_src, nsrc, sh, first, count);
+        if (s_box.vec) run_sum_tile<bf16x8, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
+        else run_sum_tile<bf16x1, BLOCKS>(s_box, s_src, nsrc, sh, first, count);
     }
 }
 
+template <bool SUMS>
+__global__ void __launch_bounds__(kHaloThreads, SUMS ? 2 : 4)
+halo_box_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict__ sources,
+                const HaloTile *__restrict__ tiles, int32_t elem_bytes,
+                const __grid_constant__ ShardPointers sh) {
+    stream_enter();
+    halo_box_block<SUMS, SUMS ? 2 : 4>(boxes, sources, tiles, elem_bytes, sh, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------------------------
 // Row plan kernels (see FastDim): H, and the row ends of H*, for partitions whose innermost
@@ -369,10 +381,10 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t x, uint32_t magic, uint32_
 }
 
 // Which kind of block this is, and its index among the blocks of that kind.
-__device__ __forceinline__ int fast_block_kind(const FastHeader &H, uint32_t *tile_id) {
+__device__ __forceinline__ int fast_block_kind(const FastHeader &H, uint32_t block, uint32_t *tile_id) {
     const uint32_t per_group = (uint32_t)(H.group[0] + H.group[1]);
-    const uint32_t group = blockIdx.x / per_group;
-    uint32_t in_group = blockIdx.x - group * per_group;
+    const uint32_t group = block / per_group;
+    uint32_t in_group = block - group * per_group;
     int kind = 0;
     if (in_group >= (uint32_t)H.group[0]) {
         in_group -= (uint32_t)H.group[0];
@@ -563,7 +575,7 @@ halo_fast_fwd_kernel(const __grid_constant__ FastHeader H, const FastDim *__rest
     fast_load_records(H, dims_g, dims);
     const int d = H.rank;
     uint32_t tile_id;
-    const int kind = fast_block_kind(H, &tile_id);
+    const int kind = fast_block_kind(H, blockIdx.x, &tile_id);
     if (kind == 0) {
         const uint32_t s = tile_id / (uint32_t)H.tiles_per_owner[0];
         if (s < (uint32_t)H.num_workers) fast_ghost_rows(H, dims, sh, scratch, s, tile_id - s * (uint32_t)H.tiles_per_owner[0]);
@@ -647,21 +659,27 @@ halo_fast_fwd_kernel(const __grid_constant__ FastHeader H, const FastDim *__rest
 // H* at the row ends.  T: 16-byte vector of the element type (float4, double2, bf16x8).
 //
 // The box plan is at its best where rows are long; where a partition is split along the innermost
-// dimension, most of its boxes are columns a few units wide.  For those H* runs in two launches that
-// touch disjoint cells: the box kernel on a plan without the row-end columns of the bulk rows that no
-// outer neighbour reaches, and this kernel on exactly those.  There a bulk unit near a row end receives
+// dimension, most of its boxes are columns a few units wide.  For those H* has two kinds of block, of disjoint
+// cells: tiles of a box plan without the row-end columns of the bulk rows that no
+// outer neighbour reaches, and line blocks on exactly those.  There a bulk unit near a row end receives
 // from one ghost unit of the neighbour along the row, and every unit involved -- low ghost, low
 // receiving, high receiving, high ghost of every worker of the line -- is read once and written once,
 // in memory order, with the neighbour's ghost value taken from shared memory.
+//
+// What bounds it: requests to memory, a 16-byte row end each.  Both kinds are one launch, the tiles first, so that the line blocks
+// fill the tiles' last wave; four blocks per multiprocessor with half as many units of a sum in flight per thread as the box
+// kernel has with two, and up to 1024 row ends a block, four in flight per thread.  H* of 512^3 over 4 x 4 x 4 workers, widths 4:
+// 110 us; as two launches, each waiting for the one before, 122 (256^3 over 2 x 2 x 2: 11.3 and 18.6); blocks of
+// 512 row ends 120 (11.8); two blocks per multiprocessor 131 (14.7).
 // ---------------------------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ void halo_fast_adj_lines(const FastHeader &H, const FastDim *__restrict__ dims_g, const ShardPointers &sh) {
+__device__ __forceinline__ void halo_line_block(const FastHeader &H, const FastDim *__restrict__ dims_g, const ShardPointers &sh, uint32_t block) {
     __shared__ FastDim dims[kMaxFastCoords];
     __shared__ __align__(16) unsigned char scratch[kFastMaxSlots * 16];
     fast_load_records(H, dims_g, dims);
     const int d = H.rank;
     uint32_t tile_id;
-    if (fast_block_kind(H, &tile_id) != 1) return;
+    if (fast_block_kind(H, block, &tile_id) != 1) return;
     // both ends of the bulk rows that are out of reach in every outer dimension, for all workers of the line
     const uint32_t line = tile_id / (uint32_t)H.tiles_per_owner[1];
     if (line >= (uint32_t)H.num_lines) return;
@@ -693,59 +711,80 @@ __device__ __forceinline__ void halo_fast_adj_lines(const FastHeader &H, const F
     __syncthreads();
     T *slots = reinterpret_cast<T *>(scratch);
     const uint32_t EC = cum_e[px];
-    // pass 1: every unit of the row ends into shared memory, in memory order per worker
-    for (uint32_t q = threadIdx.x; q < nrows * EC; q += kFastThreads) {
-        int a = 0;
-        while (q >= nrows * cum_e[a + 1]) ++a;
-        const uint32_t qa = q - nrows * cum_e[a];
-        const FastDim &f = xd[a];
+    // Unit q of the row ends, in memory order per worker: its worker, its slot's row and place in the row, its address.
+    struct Unit {
+        int a;
+        uint32_t rl, u, col;
+    };
+    auto unit = [&](uint32_t q) {
+        Unit r;
+        r.a = 0;
+        while (q >= nrows * cum_e[r.a + 1]) ++r.a;
+        const uint32_t qa = q - nrows * cum_e[r.a];
+        const FastDim &f = xd[r.a];
         const uint32_t ec = (uint32_t)(f.n - f.b + f.rlo + f.rhi), lo_end = (uint32_t)(f.hlo + f.rlo);
-        const uint32_t rl = qa / ec, u = qa - rl * ec;
-        const uint32_t col = u < lo_end ? u : u - lo_end + (uint32_t)(f.hlo + f.b - f.rhi);
-        const bool ghost = col < (uint32_t)f.hlo || col >= (uint32_t)(f.hlo + f.b);
-        const bool outside = ghost && (col < (uint32_t)f.hlo ? f.lo_c < 0 : f.hi_c < 0);      // never read: only cleared
-        if (!outside) slots[q] = reinterpret_cast<const T *>(sh.p[first_worker + a])[rowlin[rl] * (uint32_t)f.n + col];
+        r.rl = qa / ec;
+        r.u = qa - r.rl * ec;
+        r.col = r.u < lo_end ? r.u : r.u - lo_end + (uint32_t)(f.hlo + f.b - f.rhi);
+        return r;
+    };
+    constexpr int U = 4;
+    // pass 1: every unit of the row ends into shared memory
+    const uint32_t all = nrows * EC;
+    for (uint32_t q0 = threadIdx.x; q0 < all; q0 += U * kFastThreads) {
+        T v[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const uint32_t q = q0 + k * kFastThreads;
+            v[k] = zero_of<T>();
+            if (q < all) {
+                const Unit r = unit(q);
+                const FastDim &f = xd[r.a];
+                // ghosts outside the tensor are never read: only cleared
+                const bool outside = (r.col < (uint32_t)f.hlo && f.lo_c < 0) || (r.col >= (uint32_t)(f.hlo + f.b) && f.hi_c < 0);
+                if (!outside) v[k] = reinterpret_cast<const T *>(sh.p[first_worker + r.a])[rowlin[r.rl] * (uint32_t)f.n + r.col];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (q0 + k * kFastThreads < all) slots[q0 + k * kFastThreads] = v[k];
     }
     __syncthreads();
     // pass 2: ghosts <- 0, receiving units <- own value + the neighbour's ghost copy, same order
-    for (uint32_t q = threadIdx.x; q < nrows * EC; q += kFastThreads) {
-        int a = 0;
-        while (q >= nrows * cum_e[a + 1]) ++a;
-        const uint32_t qa = q - nrows * cum_e[a];
-        const FastDim &f = xd[a];
-        const uint32_t ec = (uint32_t)(f.n - f.b + f.rlo + f.rhi), lo_end = (uint32_t)(f.hlo + f.rlo);
-        const uint32_t rl = qa / ec, u = qa - rl * ec;
-        const uint32_t col = u < lo_end ? u : u - lo_end + (uint32_t)(f.hlo + f.b - f.rhi);
+    for (uint32_t q = threadIdx.x; q < all; q += kFastThreads) {
+        const Unit r = unit(q);
+        const FastDim &f = xd[r.a];
         T v = zero_of<T>();
-        if (col >= (uint32_t)f.hlo && col < (uint32_t)(f.hlo + f.b)) {
+        if (r.col >= (uint32_t)f.hlo && r.col < (uint32_t)(f.hlo + f.b)) {
             v = slots[q];
-            if (u < lo_end) {
+            if (r.u < (uint32_t)(f.hlo + f.rlo)) {
                 if (f.lo_c >= 0) {      // the low neighbour's high ghost unit of the same cell: the last units of its row ends
                     const FastDim &g = xd[f.lo_c];
                     const uint32_t gec = (uint32_t)(g.n - g.b + g.rlo + g.rhi);
-                    const uint32_t gu = (uint32_t)(g.hlo + g.rlo + g.rhi) + (u - (uint32_t)f.hlo);
-                    v = vadd(v, slots[nrows * cum_e[f.lo_c] + rl * gec + gu]);
+                    const uint32_t gu = (uint32_t)(g.hlo + g.rlo + g.rhi) + (r.u - (uint32_t)f.hlo);
+                    v = vadd(v, slots[nrows * cum_e[f.lo_c] + r.rl * gec + gu]);
                 }
             } else if (f.hi_c >= 0) {   // the high neighbour's low ghost unit: the first units of its row
                 const FastDim &g = xd[f.hi_c];
                 const uint32_t gec = (uint32_t)(g.n - g.b + g.rlo + g.rhi);
-                v = vadd(v, slots[nrows * cum_e[f.hi_c] + rl * gec + (u - lo_end)]);
+                v = vadd(v, slots[nrows * cum_e[f.hi_c] + r.rl * gec + (r.u - (uint32_t)(f.hlo + f.rlo))]);
             }
         }
-        reinterpret_cast<T *>(sh.p[first_worker + a])[rowlin[rl] * (uint32_t)f.n + col] = v;
+        reinterpret_cast<T *>(sh.p[first_worker + r.a])[rowlin[r.rl] * (uint32_t)f.n + r.col] = v;
     }
 }
 
-// The boxes' kernel, if there is one, is the one before it in the stream: its cells are others, so the two run side by side where
-// the first one's last blocks leave room (512^3 over 4 x 4 x 4 workers, widths 4: 120 -> 116 us).
+// H* of such a partition: the tiles of the boxes, then the blocks of the row ends.
 template <typename T>
-__global__ void __launch_bounds__(kFastThreads)
-halo_fast_adj_lines_kernel(const __grid_constant__ FastHeader H, const FastDim *__restrict__ dims_g,
-                           const __grid_constant__ ShardPointers sh, bool after_boxes) {
-    if (after_boxes) stream_enter_beside();
-    else stream_enter();
-    halo_fast_adj_lines<T>(H, dims_g, sh);
-    if (after_boxes) stream_leave_beside();
+__global__ void __launch_bounds__(kHaloThreads, 4)
+halo_adj_kernel(const HaloBox *__restrict__ boxes, const HaloSource *__restrict__ sources, const HaloTile *__restrict__ tiles,
+                uint32_t num_tiles, const __grid_constant__ FastHeader H, const FastDim *__restrict__ dims_g,
+                const __grid_constant__ ShardPointers sh) {
+    static_assert(kHaloThreads == kFastThreads, "both kinds of block");
+    constexpr int kBytes = std::is_same<T, float4>::value ? 4 : std::is_same<T, double2>::value ? 8 : 2;
+    stream_enter();
+    if (blockIdx.x < num_tiles) halo_box_block<true, 4>(boxes, sources, tiles, kBytes, sh, blockIdx.x);
+    else halo_line_block<T>(H, dims_g, sh, blockIdx.x - num_tiles);
 }
 
 // Whether any of the arrays may overlap: in address order, does one begin before all before it have ended.  (Pair by pair, 48
@@ -814,15 +853,14 @@ static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &p
     if (adjoint && p->fast.adj_usable && p->fast_dims_dev) {
         cudaStream_t st = (cudaStream_t)stream;
         const HaloPlanDevice &rest = p->adj_rest_dev;      // everything but the row ends of the rows out of outer reach
-        if (rest.num_tiles > 0) {
-            launch_in_stream(halo_box_kernel<true>, rest.num_tiles, kHaloThreads, 0, st, rest.boxes, rest.sources, rest.tiles, elem_size(p->dtype), sh);
-            DISTDL_CUDA_CHECK(cudaGetLastError());
-        }
         const FastHeader &h = p->fast.adj_hdr;
-        const unsigned grid = (unsigned)h.num_groups * (unsigned)(h.group[0] + h.group[1]);
-        if (p->dtype == DISTDL_F32) launch_in_stream(halo_fast_adj_lines_kernel<float4>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
-        else if (p->dtype == DISTDL_F64) launch_in_stream(halo_fast_adj_lines_kernel<double2>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
-        else launch_in_stream(halo_fast_adj_lines_kernel<bf16x8>, grid, kFastThreads, 0, st, h, p->fast_dims_dev, sh, rest.num_tiles > 0);
+        const unsigned grid = (unsigned)rest.num_tiles + (unsigned)h.num_groups * (unsigned)(h.group[0] + h.group[1]);
+        const auto run = [&](auto kernel) {
+            launch_in_stream(kernel, grid, kHaloThreads, 0, st, rest.boxes, rest.sources, rest.tiles, (uint32_t)rest.num_tiles, h, p->fast_dims_dev, sh);
+        };
+        if (p->dtype == DISTDL_F32) run(halo_adj_kernel<float4>);
+        else if (p->dtype == DISTDL_F64) run(halo_adj_kernel<double2>);
+        else run(halo_adj_kernel<bf16x8>);
         DISTDL_CUDA_CHECK(cudaGetLastError());
         return DISTDL_OK;
     }

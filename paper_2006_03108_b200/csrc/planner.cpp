@@ -731,7 +731,7 @@ void build_fast_plan(distdl_partition *p) {
     a = h;
     memset(a.rows_per_tile, 0, sizeof(a.rows_per_tile));
     memset(a.tiles_per_owner, 0, sizeof(a.tiles_per_owner));
-    a.rows_per_tile[1] = (int32_t)std::min<int64_t>(128, std::max<int64_t>(1, 512 / ec));
+    a.rows_per_tile[1] = (int32_t)std::min<int64_t>(128, std::max<int64_t>(1, 1024 / ec));     // as many units as a block can stage
     a.tiles_per_owner[1] = tiles(inner_rows_max, a.rows_per_tile[1]);
     {
         const int64_t total[2] = {0, (int64_t)a.tiles_per_owner[1] * a.num_lines};

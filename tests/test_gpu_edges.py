@@ -209,6 +209,65 @@ def test_kernels_follow_copies_and_foreign_kernels_in_order(n, captured):
     assert torch.equal(y, 8 * x) and torch.equal(z, 4 * x) and torch.equal(pinned, (4 * x).cpu())
 
 
+@pytest.mark.parametrize("captured", [False, True], ids=["eager", "graph"])
+@pytest.mark.parametrize("op", ["halo_adj", "affine_adj_params"])
+def test_operators_of_two_kinds_of_work_see_what_came_before(op, captured):
+    """H* with a plan for its row ends, and dW with db: a writer of their inputs, the operator, a reader of its results, with no
+    wait of the host between passes and other inputs in each; against the same passes with a wait after every step."""
+    torch, distdl, dev = parity.torch, parity.distdl, parity.DEV
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(3)
+    if op == "halo_adj":
+        part = distdl.Partition((72, 96, 128), (2, 2, 2), (4,) * 3, (4,) * 3)
+        assert part.uses_row_plan(adjoint=True)
+        base = [torch.rand(part.padded_shape(w), device=dev, generator=gen) for w in range(8)]
+        ins = outs = [torch.empty_like(b) for b in base]
+        call = lambda: distdl.halo_adj(part, ins)
+    else:
+        base = [torch.randn(192, 520, device=dev, generator=gen).bfloat16(), torch.randn(192, 1032, device=dev, generator=gen).bfloat16()]
+        ins = [torch.empty_like(b) for b in base]
+        outs = [torch.empty(520, 1032, device=dev), torch.empty(520, device=dev)]
+        call = lambda: distdl.affine_adj_params(192, 1032, 520, 1, 1, [ins[0]], [ins[1]], [outs[0]], [outs[1]])
+    scale = torch.ones((), device=dev)
+
+    def body(wait=lambda: None):
+        for i, b in zip(ins, base):
+            torch.mul(b, scale, out=i)          # the operator's input, by a kernel of another library
+            wait()
+        call()
+        wait()
+        got = [o.clone() for o in outs]
+        wait()
+        return got
+
+    stream = torch.cuda.Stream()
+    want = []
+    for n in range(20):
+        scale.fill_(n - 7.5)
+        want.append(body(torch.cuda.synchronize))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        body()                                  # kernels loaded before the capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph() if captured else None
+    if captured:
+        with torch.cuda.graph(graph, stream=stream):
+            held = body()
+    torch.cuda.synchronize()
+    got = []
+    with torch.cuda.stream(stream):
+        for n in range(20):
+            scale.fill_(n - 7.5)
+            if captured:
+                graph.replay()
+                got.append([h.clone() for h in held])
+            else:
+                got.append(body())
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert all(torch.equal(p.view(torch.int32), q.view(torch.int32)) for p, q in zip(a, b))
+
+
 def test_halo_names_the_first_overlapping_pair():
     torch, distdl = parity.torch, parity.distdl
     part = distdl.Partition((12, 40), (3, 2), [1, 1], [1, 1])

@@ -304,3 +304,27 @@ def test_depthwise_convolution_copies_end_inside_their_arrays(k, gradients):
         part = distdl.Partition((1, 1, 6, 3), (1, 1, 1, 3), h, h)
         past, by_cell = distdl.selftest_conv_row_reads(part, k, gradients)
         assert past <= 0 and by_cell <= 3 * 3
+
+
+def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
+    """Kernels are launched while their predecessors in the stream run; what those wrote is visible to a kernel only after its
+    own wait.  So every kernel launched that way begins with stream_enter(), under no condition, and nothing else lets
+    successors in."""
+    src = os.path.join(ROOT, "paper_2006_03108_b200", "csrc")
+    launched, bodies, triggers = set(), {}, 0
+    for name in sorted(os.listdir(src)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, name)).read())
+        launched.update(re.findall(r"launch_(?:clusters_)?in_stream\((\w+_kernel\w*|pool_\w+_fixed)\b", text))
+        triggers += text.count("griddepcontrol.launch_dependents")
+        for m in re.finditer(r"__global__ void (?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\(", text):
+            brace = text.index("{", m.end())
+            depth, end = 1, brace + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[end], 0)
+                end += 1
+            bodies[m.group(1)] = text[brace + 1:end - 1]
+    assert triggers == 1 and len(launched) >= 20
+    for kernel in sorted(launched):
+        body = bodies[kernel]
+        assert len(re.findall(r"^    stream_enter\(\);", body, re.M)) == 1, kernel
+        assert body.count("stream_enter") == 1 and body.count("griddepcontrol") == 0, kernel
