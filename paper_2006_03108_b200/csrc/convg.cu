@@ -539,6 +539,9 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
 // and workers, so the running sums stay in registers from tile to tile.  At the end of an item the block adds up its
 // splits in order and writes one row of K * K + 1 values per channel pair to the scratch table; a second small kernel adds
 // the rows of a pair in order.  The assignment of tiles to sums is static, so the result does not change from run to run.
+// The error of an fp32 sum grows with its length, so a running sum takes at most kGgSumTerms terms (one tile at least): longer
+// shares of tiles are several launches, each adding its sums onto the rows (0.6 to 1.3 % of the time, 8 us a launch; as a loop
+// inside the kernel the accumulators' second life costs the inner loop a tenth).
 //
 // What bounds it: the fp32 pipe.  A thread owns one input channel c, one kernel row a and all OC output channels of the
 // group, and walks along the rows of the tile four pixels at a time: K * OC sums as pairs (even pixels, odd pixels), one new
@@ -547,13 +550,14 @@ static distdl_status_t convg_impl(const distdl_partition *px, int64_t nco, int32
 // is left of the threads, and one more combination reads ones instead of x: its sums are db.  Lanes that own pixels
 // instead (all K * K sums of one or two channel pairs per lane) spend as many instructions on putting x pairs together and
 // on folding lanes as on FMAs.
-// Measured (B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.40 ms = 38 TFLOP/s (1.94 ms with one channel
+// Measured (B200): 16 -> 16 channels, 5 x 5, 4 x 1024 x 1024 on 2 x 2 workers 1.41 ms = 38 TFLOP/s (1.94 ms with one channel
 // pair per block, both its tiles staged again for every pair); 6 -> 16 channels, 256 images of 28 x 28 0.063 ms (1.61 ms).
 // Two steps per turn instead of moving the window: 1.63 ms (spills); 192 threads with 168 registers: 1.67 ms.
 // ---------------------------------------------------------------------------------------------
 constexpr int kGradRow = 64;            // floats per row of the scratch table (K * K + 1 <= 50 used)
 constexpr int kGgThreads = 256;
 constexpr int kGgSmem = 112 * 1024;     // two blocks per SM
+constexpr int kGgSumTerms = 2560;
 // output channels of a group: more would need more than the 128 registers of two blocks per SM
 constexpr int gg_max_oc(int k) { return k == 7 ? 4 : 8; }
 
@@ -575,6 +579,8 @@ struct ConvGGradParams {
     int32_t slices;                     // slices per pair of groups
     int32_t xc, splits;                 // input channels per block; splits of a tile's rows
     int32_t tiles;                      // tiles of one channel: workers, images, rows, columns
+    int32_t run;                        // tiles of a launch: a whole number of turns of the slices
+    int32_t first, last;                // those of this launch
     uint32_t zero;                      // 0, see fresh()
     float *partial;                     // [pairs][slices][kGradRow]
     GgShape t;
@@ -710,14 +716,14 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
         return true;
     };
 
-    int L = sl, buf = 0;
-    bool cur = L < G.tiles && stage((uint32_t)L, 0);
+    int L = G.first + sl, buf = 0;
+    bool cur = L < G.last && stage((uint32_t)L, 0);
     cp_async_commit();
-    while (L < G.tiles) {
+    while (L < G.last) {
         cp_async_wait_group<0>();
         __syncthreads();                // this tile has arrived, the other buffer has been read
         const int next = L + G.slices;
-        const bool nxt = next < G.tiles && stage((uint32_t)next, buf ^ 1);
+        const bool nxt = next < G.last && stage((uint32_t)next, buf ^ 1);
         cp_async_commit();
         if (cur && active) {
             const float *xt = is_ones ? smem + 2 * T.buf_floats : smem + buf * T.buf_floats + my_c * T.x_floats + my_a * T.pitch;
@@ -772,7 +778,7 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
         L = next;
         buf ^= 1;
     }
-    // add up: the two halves of a pair, then the splits in order; one row per channel pair
+    // add up: the two halves of a pair, then the splits in order, onto the launches before; one row per channel pair
     __syncthreads();
     if (active)
 #pragma unroll
@@ -794,7 +800,8 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
         float v = src[0];
         for (int s = 1; s < G.splits; ++s) v += src[s * combos];
         const size_t pair = (size_t)(G.y_start[ib] + o0 + k) * G.n_x + (G.x_start[jb] + c0 + ch);
-        G.partial[(pair * G.slices + sl) * kGradRow + (ones ? K * K : (cb - ch * K) * K + b)] = v;
+        float *sum = G.partial + (pair * G.slices + sl) * kGradRow + (ones ? K * K : (cb - ch * K) * K + b);
+        *sum = G.first ? *sum + v : v;
     }
 }
 
@@ -973,6 +980,10 @@ static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, 
     G->tiles = (int32_t)tiles;
     const int64_t slices = std::min<int64_t>(slots, tiles);
     G->slices = (int32_t)slices;
+    // launches with equal shares of a slice's tiles, none with more terms to a sum than the limit
+    const int64_t terms = (int64_t)((G->t.tn * G->t.th + G->splits - 1) / G->splits) * 2 * G->t.seg, share = (tiles + slices - 1) / slices;
+    const int64_t most = std::max<int64_t>(1, kGgSumTerms / terms), launches = (share + most - 1) / most;
+    G->run = (int32_t)std::min<int64_t>(tiles, (share + launches - 1) / launches * slices);
     G->slice_div = make_fast_div((uint32_t)slices);
     G->cgrp_div = make_fast_div((uint32_t)G->cgrp[pci]);
     G->tiles_x = make_fast_div((uint32_t)tiles_x);
@@ -989,7 +1000,7 @@ static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, 
 }
 
 template <int K, int OC>
-static distdl_status_t launch_convg_grad(const ConvGGradParams &G, const ConvGGradOut &O, int grid, int pairs, cudaStream_t s) {
+static distdl_status_t launch_convg_grad(ConvGGradParams &G, const ConvGGradOut &O, int grid, int pairs, cudaStream_t s) {
     static bool configured_on[kMaxDevicesPerProcess] = {false};
     int dev = 0;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
@@ -1002,15 +1013,19 @@ static distdl_status_t launch_convg_grad(const ConvGGradParams &G, const ConvGGr
             configured_on[dev] = true;
         }
     }
-    launch_in_stream(convg_grad_kernel<K, OC>, grid, kGgThreads, G.t.smem_bytes, s, G);
-    DISTDL_CUDA_CHECK(cudaGetLastError());
+    for (int64_t at = 0; at < G.tiles; at += G.run) {
+        G.first = (int32_t)at;
+        G.last = (int32_t)std::min<int64_t>(G.tiles, at + G.run);
+        launch_in_stream(convg_grad_kernel<K, OC>, grid, kGgThreads, G.t.smem_bytes, s, G);
+        DISTDL_CUDA_CHECK(cudaGetLastError());
+    }
     launch_in_stream(convg_grad_finish_kernel, pairs, 64 * kGradFoldGroups, 0, s, G, O, K * K);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
 
 template <int K>
-static distdl_status_t launch_convg_grad_channels(const ConvGGradParams &G, const ConvGGradOut &O, int oc, int grid, int pairs, cudaStream_t s) {
+static distdl_status_t launch_convg_grad_channels(ConvGGradParams &G, const ConvGGradOut &O, int oc, int grid, int pairs, cudaStream_t s) {
     constexpr int most = gg_max_oc(K);
     if (oc == 2) return launch_convg_grad<K, 2>(G, O, grid, pairs, s);
     if (oc == 4) return launch_convg_grad<K, 4>(G, O, grid, pairs, s);

@@ -30,6 +30,27 @@ def test_generalized_conv_tiles(case, integer):
     parity.test_generalized_conv_param_gradients(case, integer)
 
 
+@pytest.mark.parametrize("case", [(104, 112, 640, 5), (16, 16, 1600, 3), (24, 20, 900, 7)], ids=str)
+def test_generalized_conv_gradient_sums_stay_short(case):
+    """Sums over many pixels are added up in short runs.  dy = 1 + 2^-12 and x = 1: a run of up to 4096 terms is exact in fp32,
+    longer ones lose the 2^-12 of every further term; adding up the runs (pair halves, splits, folds, slices: fewer than 100
+    additions on a path) costs at most 100 * 2^-24."""
+    torch, distdl, dev = parity.torch, parity.distdl, parity.DEV
+    ci, co, n, k = case
+    h = k // 2
+    part = distdl.Partition((1, ci, n, n), (1, 1, 1, 1), (0, 0, h, h), (0, 0, h, h))
+    x = torch.ones(part.padded_shape(0), device=dev)
+    dy = torch.full((1, co, n, n), 1 + 2.0 ** -12, device=dev)
+    dw, db = torch.empty(co, ci, k, k, device=dev), torch.empty(co, device=dev)
+    ws = torch.empty(distdl.convg_adj_params_workspace(part, co, 1, k, k), dtype=torch.uint8, device=dev)
+    distdl.convg_adj_params(part, co, 1, [x], [dy], (k, k), [dw], [db], ws)
+    distdl.device_status()
+    cells = n - (torch.arange(k, device=dev, dtype=torch.float64) - h).abs()           # pixels that have the tap inside the tensor
+    want = (1 + 2.0 ** -12) * cells[:, None] * cells[None, :]
+    assert ((dw.double() - want).abs() <= 100 * 2.0 ** -24 * want).all()
+    assert ((db.double() - (1 + 2.0 ** -12) * n * n).abs() <= 100 * 2.0 ** -24 * n * n).all()
+
+
 # global NCHW, partition, kernel
 CONV_EDGES = [
     ((1, 1, 5, 1), (1, 1, 1, 1), 3),         # one column
