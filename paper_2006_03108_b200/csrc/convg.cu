@@ -866,7 +866,7 @@ static GgShape gg_shape(int K, int tn, int th, int seg, int xc, int oc) {
 // counts 2.5: the rate of a register outer product), staging 40 per unit and 2 or 12 more per channel.  Sizes are tried from
 // the largest down in steps of a fifth, shards cut into that many equal tiles, and what cannot win by its FMAs alone is passed
 // over: 3 to 7 us of host time (7 to 27 us with every size in turn).
-static GgShape gg_choose(int K, int xc, int splits, int oc, int max_bh, int max_bw, int batch, int workers, int slots) {
+static GgShape gg_choose(int K, int xc, int splits, int oc, int max_bh, int max_bw, int batch, int workers, int slots, double *tile_cost) {
     GgShape best;
     memset(&best, 0, sizeof(best));
     double best_cost = 0;
@@ -897,11 +897,16 @@ static GgShape gg_choose(int K, int xc, int splits, int oc, int max_bh, int max_
                 if (best.tn == 0 || cost < best_cost) {
                     best = t;
                     best_cost = cost;
+                    *tile_cost = cost / turns;
                 }
             }
         }
     }
     return best;
+}
+
+static int64_t gg_tiles(const GgShape &t, int64_t max_bh, int64_t max_bw, int64_t batch, int64_t workers) {
+    return (max_bw + 4 * t.seg - 1) / (4 * t.seg) * ((max_bh + t.th - 1) / t.th) * workers * ((batch + t.tn - 1) / t.tn);
 }
 
 // Geometry, groups and slices: shared by the workspace query and the launch.
@@ -970,13 +975,32 @@ static distdl_status_t convg_grad_plan(const distdl_partition *px, int64_t nco, 
     int dev = 0, sms = 148;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
     DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // as many slices as fill the resident blocks once; never more than tiles
-    const int64_t group_pairs = (int64_t)G->cgrp[pci] * G->ogrp[pco];
-    const int64_t slots = std::max<int64_t>(1, 2 * (int64_t)sms / group_pairs);
-    G->t = gg_choose(kh, xc, G->splits, oc, (int)max_bh, (int)max_bw, G->batch, ph * pw, slots);
-    const int64_t tiles_x = (max_bw + 4 * G->t.seg - 1) / (4 * G->t.seg), tiles_y = (max_bh + G->t.th - 1) / G->t.th;
-    const int64_t tiles = tiles_x * tiles_y * ph * pw * ((G->batch + G->t.tn - 1) / G->t.tn);
+    // Slices: as many as fill the resident blocks once -- or, where many groups leave that far from full or past it, the number
+    // (16 at most: it is the size of the scratch table) whose turns of the resident blocks take the least time; 15000: what a block
+    // spends besides its tiles.  5 x 5, 128 x 128: 80 -> 80 channels, four images, 943 us with the two slices that fit, now 687; 136 ->
+    // 144, two images (more groups than blocks), 1403 and 987.
+    const int64_t group_pairs = (int64_t)G->cgrp[pci] * G->ogrp[pco], resident = 2 * (int64_t)sms;
+    int64_t slots = std::max<int64_t>(1, resident / group_pairs);
+    double tile_cost = 0;
+    const auto choose = [&]() {
+        G->t = gg_choose(kh, xc, G->splits, oc, (int)max_bh, (int)max_bw, G->batch, ph * pw, (int)slots, &tile_cost);
+        return gg_tiles(G->t, max_bh, max_bw, G->batch, ph * pw);
+    };
+    int64_t tiles = choose();
+    if (slots < 16) {
+        const auto time = [&](int64_t n) {
+            return (double)((n * group_pairs + resident - 1) / resident) * ((double)((tiles + n - 1) / n) * tile_cost + 15000);
+        };
+        int64_t best_slots = slots;
+        for (int64_t n = 1; n <= std::min<int64_t>(16, tiles); ++n)
+            if (time(n) < 0.97 * time(best_slots)) best_slots = n;
+        if (best_slots != slots) {
+            slots = best_slots;
+            tiles = choose();
+        }
+    }
     if (tiles >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles or channel pairs", what);
+    const int64_t tiles_x = (max_bw + 4 * G->t.seg - 1) / (4 * G->t.seg), tiles_y = (max_bh + G->t.th - 1) / G->t.th;
     G->tiles = (int32_t)tiles;
     const int64_t slices = std::min<int64_t>(slots, tiles);
     G->slices = (int32_t)slices;

@@ -20,6 +20,7 @@ CONVG_EDGES = [
     (4, 2, 8, 301, 310, 1, 1, 1, 1, 3),      # tiles enough for several waves: eight pixels a thread, all of four pairs / one pair
     (300, 4, 7, 30, 39, 1, 1, 1, 1, 5),      # the same with tiles of several images; rows that end inside a thread's pixels
     (200, 4, 10, 29, 31, 1, 2, 1, 1, 7),     # the same, 7 x 7 and two blocks of channels
+    (2, 70, 66, 24, 33, 2, 2, 1, 1, 3),      # 90 pairs of channel groups: slices chosen by the turns they make
 ]
 
 
@@ -49,6 +50,16 @@ def test_generalized_conv_gradient_sums_stay_short(case):
     want = (1 + 2.0 ** -12) * cells[:, None] * cells[None, :]
     assert ((dw.double() - want).abs() <= 100 * 2.0 ** -24 * want).all()
     assert ((db.double() - (1 + 2.0 ** -12) * n * n).abs() <= 100 * 2.0 ** -24 * n * n).all()
+
+
+@pytest.mark.parametrize("case", [(2, 136, 144, 128, 5), (4, 80, 80, 128, 5), (4, 32, 40, 64, 7)], ids=str)
+def test_generalized_conv_gradient_slices_follow_the_device(case):
+    """Layers whose pairs of channel groups leave the device far from full, or its last turn far from full, are cut into more
+    slices (read off the scratch table: 256 bytes per channel pair and slice), but no more than 16."""
+    n, ci, co, side, k = case
+    part = parity.distdl.Partition((n, ci, side, side), (1, 1, 1, 1), (0, 0, k // 2, k // 2), (0, 0, k // 2, k // 2))
+    slices = parity.distdl.convg_adj_params_workspace(part, co, 1, k, k) / (256 * ci * co)
+    assert slices in range(3, 17)
 
 
 # global NCHW, partition, kernel
