@@ -82,23 +82,13 @@ __device__ __forceinline__ void dw_bulk_copy(uint32_t dst, const float *src, uin
 // (w, w) pairs of one channel, in floats, whole 16-byte units
 __host__ __device__ constexpr int dw_weight_floats(int K) { return (2 * K * K + 3) / 4 * 4; }
 
-// Cells of a strip's rows that one copy brings: columns [ja, ja + n) of the shard, the first of them at column `col` of the tile.
-struct DwSpan {
-    int ja, n, col;
-};
-__host__ __device__ inline DwSpan dw_span(int j0, int cols, int halo, int bw) {
-    const int ja = j0 > halo ? j0 - halo : 0, jb = j0 + cols + halo < bw ? j0 + cols + halo : bw;
-    return {ja, jb - ja, ja - (j0 - halo)};
-}
-// Floats that the bulk copy of n cells takes, from the boundary `lead` floats before the first of them.
-__host__ __device__ inline int dw_copy_floats(int lead, int n) { return (lead + n + 3) & ~3; }
-// Whether that copy would reach past the end of an array without ghosts.  (Beyond a bulk row of a padded array lie more than
-// three ghost cells.)  `first`: a cell of row i of a plane of bh x bw; `end`: of all planes of the shard.  Three cells or more
-// follow all rows but a plane's last when the rows have three; rows of one or two are asked for every row.
-__host__ __device__ inline bool dw_past_end(const float *first, int n, int i, int bh, int bw, const float *end) {
-    if (i != bh - 1 && bw >= 3) return false;
-    const int lead = (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3);
-    return first - lead + dw_copy_floats(lead, n) > end;
+// Rows of arrays without ghosts travel in whole 16-byte blocks.  Whether the last block of a row may reach past the end of the
+// array: of a plane's last row, and of any whose rows are shorter than the three cells that a block takes in beyond one (beyond a
+// bulk row of a padded array lie more than three ghost cells).
+__host__ __device__ inline bool dw_may_pass_end(int i, int bh, int bw) { return i == bh - 1 || bw < 3; }
+// Whether the block of cells [first, first + n) does.
+__host__ __device__ inline bool dw_past_end(const float *first, int n, const float *end) {
+    return first + ((n + 3 + (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3)) & ~3) - (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3) > end;
 }
 
 // One warp's work: plane, shard (r, c), first row and column, rows and columns of the segment.
@@ -177,7 +167,7 @@ struct DwRing {
     __device__ __forceinline__ int row_copy(const float *first, int n, int col, float *slot, uint32_t bar) {
         const int m = (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3);
         const int o = (m - col) & 3;
-        const uint32_t bytes = (uint32_t)dw_copy_floats(m, n) * 4u;
+        const uint32_t bytes = (uint32_t)((m + n + 3) & ~3) * 4u;
         mbar_expect_tx(bar, bytes);
         dw_bulk_copy(smem_u32(slot + o + col - m), first - m, bytes, bar);
         return o;
@@ -217,8 +207,7 @@ struct DwRing {
         const int d = g % C::D;
         const int bw = P.bw[t.c];
         const uint32_t bar = bars + 8 * d;
-        const DwSpan a = dw_span(t.j0, t.cols, C::PH, bw);
-        const int ja = a.ja, n = a.n, col = a.col;
+        const int ja = max(t.j0 - C::PH, 0), n = min(t.j0 + t.cols + C::PH, bw) - ja, col = ja - (t.j0 - C::PH);
         fence_proxy_async();
         if (lane < C::G) {
             const int i = t.i0 - C::PH + g * C::G + lane;
@@ -233,7 +222,8 @@ struct DwRing {
             int o = -1;
             if (!ok) {
                 mbar_expect_tx(bar, 0);
-            } else if (IO == 0 && dw_past_end(f, n, ii, P.bh[rr], bw, P.in[rr * P.pw + t.c] + (size_t)P.planes * (uint32_t)(P.bh[rr] * bw))) {
+            } else if (IO == 0 && dw_may_pass_end(ii, P.bh[rr], bw) &&
+                       dw_past_end(f, n, P.in[rr * P.pw + t.c] + (size_t)P.planes * (uint32_t)(P.bh[rr] * bw))) {
                 // a few rows of a shard at most: their lanes copy them element by element
                 mbar_expect_tx(bar, 0);
                 for (int e = 0; e < n; ++e) slot[col + e] = __ldg(f + e);
@@ -250,7 +240,8 @@ struct DwRing {
             float *slot = y + (d * C::G + l) * C::PITCHY;
             if (i >= t.i0 + t.rows) {
                 mbar_expect_tx(bar, 0);
-            } else if (dw_past_end(f, t.cols, i, P.bh[t.r], bw, P.dy[t.r * P.pw + t.c] + (size_t)P.planes * (uint32_t)(P.bh[t.r] * bw))) {
+            } else if (dw_may_pass_end(i, P.bh[t.r], bw) &&
+                       dw_past_end(f, t.cols, P.dy[t.r * P.pw + t.c] + (size_t)P.planes * (uint32_t)(P.bh[t.r] * bw))) {
                 mbar_expect_tx(bar, 0);
                 for (int e = 0; e < t.cols; ++e) slot[e] = __ldg(f + e);
             } else {
@@ -895,14 +886,14 @@ extern "C" distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition
         for (int64_t row = 0; row < (int64_t)P.planes * bh; ++row)
             for (int j0 = 0; j0 < bw; j0 += strip) {
                 const int cols = std::min(strip, bw - j0);
-                const DwSpan a = gradients ? DwSpan{j0, cols, 0} : dw_span(j0, cols, k / 2, bw);
-                const uintptr_t first = base + 4 * (uintptr_t)(row * bw + a.ja);
-                if (dw_past_end(reinterpret_cast<const float *>(first), a.n, (int)(row % bh), bh, bw, end)) {
+                const int halo = gradients ? 0 : k / 2, ja = std::max(j0 - halo, 0), n = std::min(j0 + cols + halo, bw) - ja;
+                const uintptr_t first = base + 4 * (uintptr_t)(row * bw + ja);
+                if (dw_may_pass_end((int)(row % bh), bh, bw) && dw_past_end(reinterpret_cast<const float *>(first), n, end)) {
                     ++*rows_by_cell;
                     continue;
                 }
                 const int lead = (int)((first >> 2) & 3);
-                *floats_past_end = std::max<int64_t>(*floats_past_end, row * bw + a.ja - lead + dw_copy_floats(lead, a.n) - cells);
+                *floats_past_end = std::max<int64_t>(*floats_past_end, row * bw + ja - lead + ((lead + n + 3) & ~3) - cells);
             }
     }
     return DISTDL_OK;
