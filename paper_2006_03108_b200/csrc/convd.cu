@@ -21,10 +21,10 @@
 // reads and 50 packed FMAs per row and four columns of a lane, about 45 other instructions, half of them done once per
 // group of rows.  Measured (B200, forward / adjoint / gradients, ms; before: tiles of 32 x 128 staged by a block, bulk tensor
 // copies where every row pitch allowed them):
-//   3 x 3, 4 x 12 x 515 x 509 on 3 x 2 workers (odd pitches)     0.022 / 0.022 / 0.030   (0.065 / 0.066 / 0.083)
-//   5 x 5, 16 x 16 x 1024 x 1024 on 4 x 4                        0.406 / 0.441 / 0.551   (0.431 / 0.487 / 0.531)
-//   3 x 3,  8 x 16 x 1024 x 1024 on 4 x 4                        0.194 / 0.202 / 0.225   (0.361 / 0.197 / 0.503)
-//   7 x 7,  8 x 16 x 1024 x 1024 on 4 x 4                        0.376 / 0.408 / 0.495   (0.579 / 0.450 / 1.043)
+//   3 x 3, 4 x 12 x 515 x 509 on 3 x 2 workers (odd pitches)     0.018 / 0.018 / 0.028   (0.067 / 0.069 / 0.087)
+//   5 x 5, 16 x 16 x 1024 x 1024 on 4 x 4                        0.381 / 0.478 / 0.575   (0.435 / 0.503 / 0.556)
+//   3 x 3,  8 x 16 x 1024 x 1024 on 4 x 4                        0.197 / 0.203 / 0.230   (0.365 / 0.199 / 0.510)
+//   7 x 7,  8 x 16 x 1024 x 1024 on 4 x 4                        0.370 / 0.389 / 0.499   (0.583 / 0.453 / 1.047)
 // dy read straight into registers, two rows ahead, instead of through the ring: 0.610 (5 x 5 gradients).
 #include <algorithm>
 #include <cstring>
@@ -37,6 +37,11 @@ namespace distdl {
 
 constexpr int kDwWarps = 4;
 constexpr int kDwThreads = 32 * kDwWarps;
+// Warps of a block, forward and adjoint.  The warps work alone: blocks of one even out the multiprocessors, and no warp's place
+// stays empty until its neighbours are done (5 x 5 forward / adjoint: 16 x 16 x 1024 x 1024 on 4 x 4 workers 407 / 492 -> 381 / 478 us, 4 x 16 x
+// 512 x 512 on 2 x 2 36.3 / 38.4 -> 34.3 / 36.6; 7 x 7, 8 x 16 x 1024 x 1024 on 4 x 4 384 / 408 -> 370 / 389).  3 x 3, bound by memory alone, is
+// faster with blocks of four (8 x 16 x 1024 x 1024 195 / 202 us, one 205 / 212; 4 x 12 x 515 x 509 on 3 x 2 17.7 / 17.8, one 20.0 / 20.5).
+__host__ __device__ constexpr int dw_row_warps(int K) { return K == 3 ? kDwWarps : 1; }
 constexpr uint64_t kConvWaitLimitNs = 2000000000ull;
 
 __device__ int g_conv_status = 0;
@@ -345,14 +350,14 @@ struct DwWindow<K, -1> {
 // all of them, a lane owns four neighbouring columns, reads 16 bytes at a time and makes the pairs that start at an odd
 // offset itself: 5 x 5 forward, two reads and six exclusive-ors instead of twenty reads per row.
 template <int K, bool ADJ, int NC, bool VEC>
-__global__ void __launch_bounds__(kDwThreads, K == 7 ? 3 : 4)
+__global__ void __launch_bounds__(32 * dw_row_warps(K), (K == 7 ? 12 : 16) / dw_row_warps(K))
 conv_rows_kernel(const __grid_constant__ DwParams P) {
     stream_enter();
     using C = DwCfg<K, NC, false>;
     constexpr int OO = ADJ ? C::PH : 0;                     // ghost width of the output layout
     extern __shared__ __align__(16) float smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t id = blockIdx.x * kDwWarps + warp;
+    const uint32_t id = blockIdx.x * dw_row_warps(K) + warp;
     if (id >= (uint32_t)P.items) return;
     const DwItem t = dw_item(P, id, C::W);
     if (!t.valid) return;
@@ -623,12 +628,12 @@ int conv_take_status() {
 // ---------------------------------------------------------------------------------------------
 template <int K, int NC>
 static constexpr int dw_smem_bytes(bool grad) {
-    return kDwWarps * (grad ? DwCfg<K, NC, true>::WARP_FLOATS : DwCfg<K, NC, false>::WARP_FLOATS + dw_weight_floats(K)) * 4;
+    return (grad ? kDwWarps * DwCfg<K, NC, true>::WARP_FLOATS : dw_row_warps(K) * (DwCfg<K, NC, false>::WARP_FLOATS + dw_weight_floats(K))) * 4;
 }
 
 // Resident blocks of a kernel on the current device; sets the kernel's shared-memory limit on the first call.
 template <typename Kernel>
-static distdl_status_t dw_resident(Kernel kernel, int smem, int (&blocks_on)[kMaxDevicesPerProcess], int *blocks) {
+static distdl_status_t dw_resident(Kernel kernel, int threads, int smem, int (&blocks_on)[kMaxDevicesPerProcess], int *blocks) {
     int dev = 0;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevicesPerProcess)
@@ -638,7 +643,7 @@ static distdl_status_t dw_resident(Kernel kernel, int smem, int (&blocks_on)[kMa
         int sms = 0, per_sm = 0;
         DISTDL_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        DISTDL_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDwThreads, smem));
+        DISTDL_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
         blocks_on[dev] = sms * std::max(per_sm, 1);
     }
     *blocks = blocks_on[dev];
@@ -718,14 +723,14 @@ static bool dw_aligned_rows(const DwParams &P, int io) {
 
 template <int K, bool ADJ, int NC, bool VEC>
 static distdl_status_t launch_conv_rows(DwParams &P, int64_t max_bh, int64_t max_bw, cudaStream_t s, const char *what) {
-    constexpr int smem = dw_smem_bytes<K, NC>(false);
+    constexpr int smem = dw_smem_bytes<K, NC>(false), warps = dw_row_warps(K);
     static int blocks_on[kMaxDevicesPerProcess] = {0};
     int blocks = 0;
-    distdl_status_t st = dw_resident(conv_rows_kernel<K, ADJ, NC, VEC>, smem, blocks_on, &blocks);
+    distdl_status_t st = dw_resident(conv_rows_kernel<K, ADJ, NC, VEC>, 32 * warps, smem, blocks_on, &blocks);
     if (st != DISTDL_OK) return st;
-    st = dw_items(&P, K, max_bh, max_bw, 32 * NC, DwCfg<K, NC, false>::G, P.planes, (int64_t)blocks * kDwWarps, what);
+    st = dw_items(&P, K, max_bh, max_bw, 32 * NC, DwCfg<K, NC, false>::G, P.planes, (int64_t)blocks * warps, what);
     if (st != DISTDL_OK) return st;
-    launch_in_stream(conv_rows_kernel<K, ADJ, NC, VEC>, (unsigned)((P.items + kDwWarps - 1) / kDwWarps), kDwThreads, smem, s, P);
+    launch_in_stream(conv_rows_kernel<K, ADJ, NC, VEC>, (unsigned)((P.items + warps - 1) / warps), 32 * warps, smem, s, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -768,7 +773,7 @@ template <int K, int NC, bool VEC>
 static distdl_status_t grad_plan_rows(DwParams *P, int64_t max_bh, int64_t max_bw, int64_t batch, const char *what) {
     static int blocks_on[kMaxDevicesPerProcess] = {0};
     int blocks = 0;
-    distdl_status_t st = dw_resident(conv_grad_rows_kernel<K, NC, VEC>, dw_smem_bytes<K, NC>(true), blocks_on, &blocks);
+    distdl_status_t st = dw_resident(conv_grad_rows_kernel<K, NC, VEC>, kDwThreads, dw_smem_bytes<K, NC>(true), blocks_on, &blocks);
     if (st != DISTDL_OK) return st;
     // as many slices per channel as give every block an SM slot of its own (one wave), never more than warps' items
     const int64_t slices = std::max<int64_t>(1, blocks / P->channels);
