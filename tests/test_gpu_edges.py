@@ -88,6 +88,22 @@ def test_depthwise_conv_strips(case):
     parity.test_conv_param_gradients(case, False)
 
 
+def test_depthwise_conv_host_time_does_not_grow_with_the_image():
+    """The cut into row segments is chosen at every call: on shards of 65536 rows in the time of 1024 (a query of the scratch size,
+    which chooses it too; best of 30)."""
+    import time
+
+    def best(rows):
+        part = parity.distdl.Partition((1, 1, rows, 64), (1, 1, 1, 1), (0, 0, 2, 2), (0, 0, 2, 2))
+        times = []
+        for _ in range(30):
+            t = time.perf_counter()
+            parity.distdl.conv_adj_params_workspace(part, 5, 5)
+            times.append(time.perf_counter() - t)
+        return min(times)
+    assert best(65536) < best(1024) + 15e-6
+
+
 # Rows copied chunk by chunk: at least 96 elements, chunks of up to 512, tiles of whole rows
 REPART_EDGES = [
     ((61, 1203), (4, 1), (1, 3)),            # pieces of 401
