@@ -88,6 +88,27 @@ def test_depthwise_conv_strips(case):
     parity.test_conv_param_gradients(case, False)
 
 
+@pytest.mark.parametrize("width,k", [(64, 3), (128, 3), (128, 5)])
+def test_depthwise_conv_gradient_of_an_infinite_cell(width, k):
+    """dy = 1 and one infinite cell per channel: the taps that meet the cell inside the tensor are infinite, the others finite, and
+    none is NaN, wherever the cell lies among the rows that a warp takes together (3 x 3, and 5 x 5 on 16-byte rows)."""
+    torch, distdl, dev = parity.torch, parity.distdl, parity.DEV
+    rows, h = 150, k // 2
+    at = [0, 1, 2, 3, *range(20, 60), 74, 75, 146, 147, 148, 149]
+    part = distdl.Partition((1, len(at), rows, width), (1, 1, 1, 1), (0, 0, h, h), (0, 0, h, h))
+    x = torch.ones(part.padded_shape(0), device=dev)
+    for c, r in enumerate(at):
+        x[0, c, h + r, h + 30] = float("inf")
+    dy = torch.ones(1, len(at), rows, width, device=dev)
+    dw, db = torch.empty(len(at), k, k, device=dev), torch.empty(len(at), device=dev)
+    ws = torch.empty(distdl.conv_adj_params_workspace(part, k, k), dtype=torch.uint8, device=dev)
+    distdl.conv_adj_params(part, [x], [dy], (k, k), dw, db, ws)
+    distdl.device_status()
+    meets = torch.tensor([[0 <= r + h - a < rows for a in range(k)] for r in at], device=dev)
+    assert torch.equal(torch.isinf(dw), meets[:, :, None].expand(-1, -1, k)) and not torch.isnan(dw).any()
+    assert torch.equal(db, torch.full_like(db, rows * width))
+
+
 def test_depthwise_conv_host_time_does_not_grow_with_the_image():
     """The cut into row segments is chosen at every call: on shards of 65536 rows in the time of 1024 (a query of the scratch size,
     which chooses it too; best of 30)."""
