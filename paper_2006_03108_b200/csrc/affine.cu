@@ -1259,8 +1259,11 @@ static distdl_status_t affine_params_impl(int64_t nb, int64_t nfi, int64_t nfo, 
         configured = true;
     }
     const int64_t slots = sms > 0 ? sms : 1;
-    // what a tile moves between L2 and its SM bounds it: 128 KB of operands and 64 KB out, or 192 KB and 128 KB (batch 256)
-    const bool wide = (wide_tiles + slots - 1) / slots * (192 + 128) < (tiles + slots - 1) / slots * (128 + 64);
+    // What a tile moves between L2 and its SM bounds it: per 64 samples 32 KB of operands, or 48 for twice the columns, and 64 or 128 KB
+    // out.  (8192 x 3200, batch 64, 11 turns of narrow tiles or 6 of wide ones: 20.0 and 21.4 us; 4096 x 2432, batch 4096, 5 or 3 turns: 95.5
+    // and 83; 4096 x 4736, batch 1024, 8 or 5: 50.4 and 44.9.)
+    const int64_t kblocks = (nb + kBlockK - 1) / kBlockK;
+    const bool wide = (wide_tiles + slots - 1) / slots * (48 * kblocks + 128) < (tiles + slots - 1) / slots * (32 * kblocks + 64);
     P.tiles_n = (int32_t)(wide ? (bfi + 255) / 256 : (bfi + 127) / 128);
     P.total_tiles = (int32_t)(wide ? wide_tiles : tiles);
     P.pfo = pfo;

@@ -178,6 +178,15 @@ def test_affine_wide_gradient_tiles(case, integer):
     parity.test_affine_param_gradients(case, integer)
 
 
+@pytest.mark.parametrize("case", [(33, 8, 1040, 2, 1),       # more 64-column groups of db than tiles, the last of eight columns
+                                  (9, 16, 72, 1, 1),         # fewer samples than two per warp of db
+                                  (300, 1408, 8192, 1, 1)],  # 5 turns of narrow or 3 of wide tiles: wide with five k-blocks, not with four
+                         ids=str)
+@pytest.mark.parametrize("integer", [True, False], ids=["int", "normal"])
+def test_affine_bias_gradient_beside_the_tiles(case, integer):
+    parity.test_affine_param_gradients(case, integer)
+
+
 # global shape, partition, kernel, stride, padding
 POOL_EDGES = [
     ((1, 1, 7, 5), (1, 1, 1, 1), (3, 3), (1, 1), ((1, 1), (1, 1))),         # every window of a border column is clipped
