@@ -146,7 +146,6 @@ struct HaloPlanHost {
 // widths 1: 6.7 / 9.8 -> 5.1 / 7.8 us; max pooling of 8 x 8 x 512 x 512 on 2 x 2 workers with its H / H*: 32.1 / 39.5 -> 30.1 / 33.4 us;
 // 3226 x 101 from columns to rows: 5.4 -> 4.0 us.  Boxes not counted: 88 x 49 x 58 on 4 x 3 x 4, widths 3, 6.4 / 9.9 instead of 6.0 / 8.4 us).
 constexpr int64_t kTileUnits = 4096;
-constexpr int64_t kPlanBlocks = 8 * 148;
 void cut_tiles(HaloPlanHost *plan, bool fine);
 
 struct HaloPlanDevice {

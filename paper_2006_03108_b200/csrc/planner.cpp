@@ -85,11 +85,21 @@ extern "C" distdl_status_t distdl_halo_widths_1d(int64_t n, int32_t p, int32_t k
 // ---------------------------------------------------------------------------------------------
 // Box construction
 // ---------------------------------------------------------------------------------------------
+// Blocks that fill the current device (a B200 where there is none).
+static int64_t plan_blocks() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        sms = 148;
+    }
+    return 8 * (int64_t)sms;
+}
+
 void distdl::cut_tiles(HaloPlanHost *plan, bool fine) {
     constexpr int64_t kTileThreads = 32 * kHaloWarps;
     int64_t total = 0;
     for (const HaloPlanHost::Cut &c : plan->cuts) total += c.units;
-    const int64_t share = total / std::max<int64_t>(kPlanBlocks / 8, kPlanBlocks - (int64_t)plan->cuts.size()) + 1;
+    const int64_t blocks = plan_blocks(), share = total / std::max<int64_t>(blocks / 8, blocks - (int64_t)plan->cuts.size()) + 1;
     const int64_t whole = std::max<int64_t>(1, (share + kTileThreads - 1) / kTileThreads) * kTileThreads;
     const int64_t size = fine ? std::min(kTileUnits, whole) : kTileUnits;
     plan->tiles.clear();

@@ -261,21 +261,21 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
                             where = a * KW + row[a][u].b;
                         }
                 } else {
-                bool have = false;
+                    bool have = false;
 #pragma unroll
-                for (int a = 0; a < KH; ++a) {
-                    if (gi + a < 0 || gi + a >= P.hg || lo[u] >= hi[u]) continue;
-                    const PoolRow<KW> &r = row[a][u];
-                    if (!have) {
-                        const bool nan = r.x[0] != r.x[0];
-                        best = nan ? r.x[0] : r.m;
-                        where = a * KW + (nan ? lo[u] : r.b);
-                        have = true;
-                    } else if (r.m > best) {
-                        best = r.m;
-                        where = a * KW + r.b;
+                    for (int a = 0; a < KH; ++a) {
+                        if (gi + a < 0 || gi + a >= P.hg || lo[u] >= hi[u]) continue;
+                        const PoolRow<KW> &r = row[a][u];
+                        if (!have) {
+                            const bool nan = r.x[0] != r.x[0];
+                            best = nan ? r.x[0] : r.m;
+                            where = a * KW + (nan ? lo[u] : r.b);
+                            have = true;
+                        } else if (r.m > best) {
+                            best = r.m;
+                            where = a * KW + r.b;
+                        }
                     }
-                }
                 }
             }
             if (on[u]) {

@@ -1,5 +1,5 @@
 // Host helper to build TMA tensor maps without linking against the driver library, and the
-// device-side mbarrier / bulk-tensor-copy wrappers shared by the affine and convolution kernels.
+// device-side mbarrier / bulk-tensor-copy wrappers shared by the affine and depthwise convolution kernels.
 #pragma once
 
 #include <cuda.h>
@@ -55,12 +55,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1, int32_t c2,
-                                            uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
 }
 #endif
 
