@@ -125,15 +125,18 @@ def test_depthwise_conv_host_time_does_not_grow_with_the_image():
     assert best(65536) < best(1024) + 15e-6
 
 
-# Rows copied chunk by chunk: at least 96 elements, chunks of up to 512, tiles of whole rows
+# Rows copied chunk by chunk: at least 384 elements, chunks of up to 512, tiles of whole rows in boxes of more than 16384
 REPART_EDGES = [
     ((61, 1203), (4, 1), (1, 3)),            # pieces of 401
-    ((7, 95 * 3 + 1), (7, 1), (1, 3)),       # pieces of 96 and 95: one each side of the rule
+    ((7, 383 * 3 + 1), (7, 1), (1, 3)),      # pieces of 384 and 383: one each side of the rule; tiles of 256 cut inside a row
+    ((200, 383 * 3 + 1), (2, 1), (1, 3)),    # the same in boxes of tiles of whole rows
+    ((7, 95 * 3 + 1), (7, 1), (1, 3)),       # short rows: pieces of 96 and 95
     ((300, 1537), (2, 1), (1, 3)),           # pieces of 513 and 512: two chunks and one; several tiles per box
     ((3, 30001), (3, 1), (1, 2)),            # pieces longer than a tile
 ]
 HALO_EDGES = [
-    ((40, 403), (2, 2), 1, 1),               # ghost rows of 201 / 202 cells
+    ((40, 403), (2, 2), 1, 1),               # ghost rows of 201 / 202 cells: unit by unit
+    ((40, 767), (2, 2), 1, 1),               # of 384 and 383: one each side of the rule
     ((9, 10, 311), (2, 2, 1), (1, 2, 1), (2, 1, 1)),
     ((5, 40001), (2, 1), (1, 0), (1, 0)),
     ((9, 10, 385), (2, 2, 1), (1, 2, 1), (2, 1, 1)),     # rows just long enough to be copied by warps
@@ -146,6 +149,24 @@ HALO_EDGES = [
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_repartition_rows(case, dtype):
     parity.test_repartition_fwd_and_adj_bit_exact(case, dtype)
+
+
+@pytest.mark.parametrize("case", REPART_EDGES, ids=[str(c) for c in REPART_EDGES])
+def test_repartition_rows_fp64(case):
+    torch, distdl, dev = parity.torch, parity.distdl, parity.DEV
+    (rows, cols), src, dst = case
+    whole = torch.rand(rows, cols, device=dev, dtype=torch.float64)
+    rep = distdl.Repartition((rows, cols), src, dst, distdl.F64)
+
+    def blocks(shapes, axis):
+        return [b.clone(memory_format=torch.contiguous_format) for b in torch.split(whole, [s[axis] for s in shapes], axis)]
+    rows_of = blocks([rep.shard_shape(w) for w in range(rep.num_src)], 0)
+    cols_of = blocks([rep.shard_shape(w, destination=True) for w in range(rep.num_dst)], 1)
+    out, back = [torch.empty_like(c) for c in cols_of], [torch.empty_like(r) for r in rows_of]
+    distdl.repartition_fwd(rep, rows_of, out)
+    distdl.repartition_adj(rep, cols_of, back)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(out, cols_of)) and all(torch.equal(a, b) for a, b in zip(back, rows_of))
 
 
 @pytest.mark.parametrize("case", HALO_EDGES, ids=[str(c) for c in HALO_EDGES])

@@ -455,7 +455,7 @@ CONV_CASES = [
     ((1, 3, 140, 264), (1, 1, 2, 2), 5),     # 16-byte aligned rows
     ((1, 2, 130, 520), (1, 1, 1, 2), 3),
     ((1, 1, 64, 1040), (1, 1, 1, 4), 7),
-    ((1, 2, 300, 520), (1, 1, 2, 2), 5),     # three tile columns per shard, vertical neighbours, TMA path
+    ((1, 2, 300, 520), (1, 1, 2, 2), 5),     # three strips per shard, vertical neighbours, 16-byte rows
     ((1, 1, 200, 1032), (1, 1, 3, 2), 7),
     ((1, 1, 100, 780), (1, 1, 2, 3), 3),
     ((1, 2, 70, 260), (1, 1, 2, 2), 3),      # padded rows of whole 16-byte units, bulk rows not (K = 3)
@@ -465,9 +465,8 @@ CONV_CASES = [
     ((1, 2, 70, 272), (1, 1, 2, 2), 5),      # bulk widths of whole groups of eight columns (136), two tile columns of 128 + 8
     ((1, 2, 70, 272), (1, 1, 2, 2), 3),      # the same for the adjoint of K = 3 (rows 8-byte aligned)
     ((1, 1, 70, 528), (1, 1, 2, 2), 7),      # and of K = 7 (264 columns per worker)
-    ((1, 41, 160, 384), (1, 1, 1, 3), 5),    # 615 tiles: more than the persistent grid holds (4 x 148 blocks), so blocks take a
-                                             # second turn with swapped neighbours, and the odd last tile has no partner
-    ((1, 41, 160, 384), (1, 1, 1, 3), 3),    # the same through the kernel without bulk tensor copies (forward)
+    ((1, 41, 160, 384), (1, 1, 1, 3), 5),    # many planes, strips of exactly 128 columns, 16-byte rows
+    ((1, 41, 160, 384), (1, 1, 1, 3), 3),    # the same with padded rows (130) off 16-byte boundaries
 ]
 
 
