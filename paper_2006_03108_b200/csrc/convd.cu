@@ -21,10 +21,10 @@
 // reads and 50 packed FMAs per row and four columns of a lane, about 45 other instructions, half of them done once per
 // group of rows.  Measured (B200, forward / adjoint / gradients, ms; before: tiles of 32 x 128 staged by a block, bulk tensor
 // copies where every row pitch allowed them):
-//   3 x 3, 4 x 12 x 515 x 509 on 3 x 2 workers (odd pitches)     0.018 / 0.018 / 0.028   (0.067 / 0.069 / 0.087)
-//   5 x 5, 16 x 16 x 1024 x 1024 on 4 x 4                        0.381 / 0.478 / 0.575   (0.435 / 0.503 / 0.556)
-//   3 x 3,  8 x 16 x 1024 x 1024 on 4 x 4                        0.197 / 0.203 / 0.230   (0.365 / 0.199 / 0.510)
-//   7 x 7,  8 x 16 x 1024 x 1024 on 4 x 4                        0.370 / 0.389 / 0.499   (0.583 / 0.453 / 1.047)
+//   3 x 3, 4 x 12 x 515 x 509 on 3 x 2 workers (odd pitches)     0.018 / 0.018 / 0.025   (0.067 / 0.069 / 0.087)
+//   5 x 5, 16 x 16 x 1024 x 1024 on 4 x 4                        0.381 / 0.473 / 0.562   (0.435 / 0.503 / 0.556)
+//   3 x 3,  8 x 16 x 1024 x 1024 on 4 x 4                        0.197 / 0.203 / 0.190   (0.365 / 0.199 / 0.510)
+//   7 x 7,  8 x 16 x 1024 x 1024 on 4 x 4                        0.365 / 0.388 / 0.476   (0.583 / 0.453 / 1.047)
 // dy read straight into registers, two rows ahead, instead of through the ring: 0.610 (5 x 5 gradients).
 #include <algorithm>
 #include <cstring>
