@@ -587,7 +587,9 @@ struct ConvGGradParams {
     FastDiv slice_div, cgrp_div, tiles_x, pw_div, tiles_y, ph_div, units, rows, seg, th;
 };
 
-template <int K, int OC>
+// FIRST, MORE: whether this may be the launch of an item's first tiles, and one of those after it.  Compiled apart for 5 x 5 and 7 x 7 (5 x 5,
+// 2 -> 6 channels, 501 x 508: 18.7 us, as one kernel 19.3); 3 x 3 is faster as one (8 -> 6, 8 x 509 x 513: 119.7 us, apart 122).
+template <int K, int OC, bool FIRST, bool MORE>
 __global__ void __launch_bounds__(kGgThreads, 2)
 convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
     stream_enter();
@@ -716,7 +718,7 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
         return true;
     };
 
-    int L = G.first + sl, buf = 0;
+    int L = (MORE ? G.first : 0) + sl, buf = 0;
     bool cur = L < G.last && stage((uint32_t)L, 0);
     cp_async_commit();
     while (L < G.last) {
@@ -801,7 +803,7 @@ convg_grad_kernel(const __grid_constant__ ConvGGradParams G) {
         for (int s = 1; s < G.splits; ++s) v += src[s * combos];
         const size_t pair = (size_t)(G.y_start[ib] + o0 + k) * G.n_x + (G.x_start[jb] + c0 + ch);
         float *sum = G.partial + (pair * G.slices + sl) * kGradRow + (ones ? K * K : (cb - ch * K) * K + b);
-        *sum = G.first ? *sum + v : v;
+        *sum = MORE && (!FIRST || G.first) ? *sum + v : v;
     }
 }
 
@@ -1033,14 +1035,16 @@ static distdl_status_t launch_convg_grad(ConvGGradParams &G, const ConvGGradOut 
     {
         std::lock_guard<std::mutex> setup_lock(setup_mutex());
         if (!configured_on[dev]) {
-            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_grad_kernel<K, OC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmem));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_grad_kernel<K, OC, true, K == 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmem));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(convg_grad_kernel<K, OC, K == 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmem));
             configured_on[dev] = true;
         }
     }
     for (int64_t at = 0; at < G.tiles; at += G.run) {
         G.first = (int32_t)at;
         G.last = (int32_t)std::min<int64_t>(G.tiles, at + G.run);
-        launch_in_stream(convg_grad_kernel<K, OC>, grid, kGgThreads, G.t.smem_bytes, s, G);
+        if (at == 0) launch_in_stream(convg_grad_kernel<K, OC, true, K == 3>, grid, kGgThreads, G.t.smem_bytes, s, G);
+        else launch_in_stream(convg_grad_kernel<K, OC, K == 3, true>, grid, kGgThreads, G.t.smem_bytes, s, G);
         DISTDL_CUDA_CHECK(cudaGetLastError());
     }
     launch_in_stream(convg_grad_finish_kernel, pairs, 64 * kGradFoldGroups, 0, s, G, O, K * K);
