@@ -856,12 +856,20 @@ __device__ __forceinline__ void affine_db_columns(const AffineDwParams &P, int w
         float s0 = 0.f, s1 = 0.f;
         if (col0 + 2 * lane < P.bfo) {
             const uint16_t *src = P.dy[i] + col0 + 2 * lane;
-#pragma unroll 32
-            for (int b = b0; b < b1; ++b) {
-                const uint32_t two = __ldg(reinterpret_cast<const uint32_t *>(src + (size_t)b * P.bfo));
-                s0 += __uint_as_float(two << 16);
-                s1 += __uint_as_float(two & 0xffff0000u);
-            }
+            const auto rows = [&](int b, bool all) {        // rows b .. b + 31, those that there are
+                uint32_t two[32];
+#pragma unroll
+                for (int u = 0; u < 32; ++u)
+                    two[u] = all || b + u < b1 ? __ldg(reinterpret_cast<const uint32_t *>(src + (size_t)(b + u) * P.bfo)) : 0u;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) {              // rows past the end are +0, which changes no sum that began with +0
+                    s0 += __uint_as_float(two[u] << 16);
+                    s1 += __uint_as_float(two[u] & 0xffff0000u);
+                }
+            };
+            int b = b0;
+            for (; b + 32 <= b1; b += 32) rows(b, true);
+            if (b < b1) rows(b, false);
         }
         part[warp][2 * lane] = s0;
         part[warp][2 * lane + 1] = s1;
