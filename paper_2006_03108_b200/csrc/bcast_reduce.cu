@@ -13,7 +13,7 @@ namespace distdl {
 
 constexpr int kMaxFan = 16;         // destinations (B) or sources (R) handled by one launch
 constexpr int kStreamThreads = 256;
-constexpr int kUnroll = 4;          // 16-byte vectors per thread per step
+constexpr int kUnroll = 4;          // vectors in flight per thread in a large broadcast
 
 struct FanPointers {
     void *p[kMaxFan];
@@ -34,32 +34,6 @@ __device__ __forceinline__ uint4 ld_stream_coherent(const uint4 *p) {
 }
 __device__ __forceinline__ void st_stream(uint4 *p, uint4 v) {
     asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-// dst[j][i] = src[i] for j < k; nvec 16-byte vectors, then `tail` trailing bytes.
-__global__ void __launch_bounds__(kStreamThreads)
-broadcast_kernel(const uint4 *__restrict__ src, const __grid_constant__ FanPointers dst, int k, size_t nvec, int tail) {
-    stream_enter();
-    const size_t stride = (size_t)gridDim.x * kStreamThreads;
-    size_t i = (size_t)blockIdx.x * kStreamThreads + threadIdx.x;
-    for (; i + (kUnroll - 1) * stride < nvec; i += kUnroll * stride) {
-        uint4 v[kUnroll];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) v[u] = ld_stream(src + i + u * stride);
-        for (int j = 0; j < k; ++j) {
-            uint4 *d = reinterpret_cast<uint4 *>(dst.p[j]);
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) st_stream(d + i + u * stride, v[u]);
-        }
-    }
-    for (; i < nvec; i += stride) {
-        const uint4 v = ld_stream(src + i);
-        for (int j = 0; j < k; ++j) st_stream(reinterpret_cast<uint4 *>(dst.p[j]) + i, v);
-    }
-    if (blockIdx.x == 0 && (int)threadIdx.x < tail) {
-        const unsigned char b = reinterpret_cast<const unsigned char *>(src + nvec)[threadIdx.x];
-        for (int j = 0; j < k; ++j) (reinterpret_cast<unsigned char *>(reinterpret_cast<uint4 *>(dst.p[j]) + nvec))[threadIdx.x] = b;
-    }
 }
 
 // One addition per element of a 16-byte vector, each the exact sum rounded once to the type.
@@ -161,27 +135,38 @@ __device__ __forceinline__ void st_stream32(Vec32 *p, const Vec32 &r) {
 }
 inline bool aligned32(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
-// 32-byte form of the broadcast: nvec32 vectors; the caller handles what is left with the 16-byte kernel.
-constexpr int kUnroll32 = 4;
+__device__ __forceinline__ uint4 ld_vec(const uint4 *p) { return ld_stream(p); }
+__device__ __forceinline__ Vec32 ld_vec(const Vec32 *p) { return ld_stream32(p); }
+__device__ __forceinline__ void st_vec(uint4 *p, const uint4 &v) { st_stream(p, v); }
+__device__ __forceinline__ void st_vec(Vec32 *p, const Vec32 &v) { st_stream32(p, v); }
+
+// dst[j][i] = src[i] for j < k; nvec vectors, U of them in flight per thread, then `tail` trailing bytes, fewer than a vector.
+template <typename V, int U>
 __global__ void __launch_bounds__(kStreamThreads)
-broadcast_kernel32(const Vec32 *__restrict__ src, const __grid_constant__ FanPointers dst, int k, size_t nvec32) {
+broadcast_kernel(const V *__restrict__ src, const __grid_constant__ FanPointers dst, int k, size_t nvec, int tail) {
     stream_enter();
+    // read at once, written after the vectors: all of it first costs a wait for memory (3005555 elements to four copies 9.9 -> 11.0 us)
+    const bool odd = blockIdx.x == 0 && (int)threadIdx.x < tail;
+    const unsigned char last = odd ? reinterpret_cast<const unsigned char *>(src + nvec)[threadIdx.x] : 0;
     const size_t stride = (size_t)gridDim.x * kStreamThreads;
     size_t i = (size_t)blockIdx.x * kStreamThreads + threadIdx.x;
-    for (; i + (kUnroll32 - 1) * stride < nvec32; i += kUnroll32 * stride) {
-        Vec32 v[kUnroll32];
+    for (; i + (U - 1) * stride < nvec; i += U * stride) {
+        V v[U];
 #pragma unroll
-        for (int u = 0; u < kUnroll32; ++u) v[u] = ld_stream32(src + i + u * stride);
+        for (int u = 0; u < U; ++u) v[u] = ld_vec(src + i + u * stride);
         for (int j = 0; j < k; ++j) {
-            Vec32 *d = reinterpret_cast<Vec32 *>(dst.p[j]);
+            V *d = reinterpret_cast<V *>(dst.p[j]);
 #pragma unroll
-            for (int u = 0; u < kUnroll32; ++u) st_stream32(d + i + u * stride, v[u]);
+            for (int u = 0; u < U; ++u) st_vec(d + i + u * stride, v[u]);
         }
     }
-    for (; i < nvec32; i += stride) {
-        const Vec32 v = ld_stream32(src + i);
-        for (int j = 0; j < k; ++j) st_stream32(reinterpret_cast<Vec32 *>(dst.p[j]) + i, v);
-    }
+    if (U > 1)
+        for (; i < nvec; i += stride) {
+            const V v = ld_vec(src + i);
+            for (int j = 0; j < k; ++j) st_vec(reinterpret_cast<V *>(dst.p[j]) + i, v);
+        }
+    if (odd)
+        for (int j = 0; j < k; ++j) (reinterpret_cast<unsigned char *>(reinterpret_cast<V *>(dst.p[j]) + nvec))[threadIdx.x] = last;
 }
 
 static int stream_grid(size_t nvec, int per_thread) {
@@ -191,6 +176,19 @@ static int stream_grid(size_t nvec, int per_thread) {
     const size_t want = (nvec + (size_t)kStreamThreads * per_thread - 1) / ((size_t)kStreamThreads * per_thread);
     const size_t cap = (size_t)sms * 8;   // 8 resident blocks of 256 threads per SM
     return (int)std::max<size_t>(1, std::min(want, cap));
+}
+
+// One vector per thread as long as the resident threads hold them all, kUnroll beyond that.  Four to a thread whatever the size left three
+// blocks for 10,000 elements (to four copies 3.7 -> 1.6 us; 100,000 to eight 6.8 -> 2.2), and a thread per vector beyond them costs the
+// loads in flight (3 M elements to eight 17.7 us with four, 21.3 with one).  Runs of consecutive vectors to a block instead of vectors a whole
+// grid apart: faster where the copies do not fit L2 (16.8 M elements to two 33.8 -> 33.2 us), slower with the sum behind it where
+// they do (3 M to four 21.6 -> 22.9 us for the pair): left as it was.
+template <typename V>
+static void launch_broadcast(const void *src, const FanPointers &dst, int k, size_t bytes, cudaStream_t s) {
+    const size_t nvec = bytes / sizeof(V);
+    const int tail = (int)(bytes % sizeof(V)), grid = stream_grid(nvec, 1);
+    if ((size_t)grid * kStreamThreads >= nvec) launch_in_stream(broadcast_kernel<V, 1>, grid, kStreamThreads, 0, s, (const V *)src, dst, k, nvec, tail);
+    else launch_in_stream(broadcast_kernel<V, kUnroll>, stream_grid(nvec, kUnroll), kStreamThreads, 0, s, (const V *)src, dst, k, nvec, tail);
 }
 
 static distdl_status_t broadcast_impl(const void *src, void *const *dst, int32_t k, int64_t n, distdl_dtype_t t,
@@ -206,9 +204,6 @@ static distdl_status_t broadcast_impl(const void *src, void *const *dst, int32_t
     }
     if (n == 0) return DISTDL_OK;
     const size_t bytes = (size_t)n * elem_size(t);
-    const size_t nvec = bytes / 16;
-    const int tail = (int)(bytes % 16);
-    const int grid = stream_grid(nvec, kUnroll);
     // destinations in groups of kMaxFan; a destination equal to the source is the in-place form
     FanPointers fp;
     int filled = 0;
@@ -216,24 +211,11 @@ static distdl_status_t broadcast_impl(const void *src, void *const *dst, int32_t
         if (j < k && dst[j] != src) fp.p[filled++] = dst[j];
         if (filled == kMaxFan || (j == k && filled > 0)) {
             for (int r = filled; r < kMaxFan; ++r) fp.p[r] = nullptr;
-            bool wide = aligned32(src) && bytes >= 32;
+            bool wide = aligned32(src);
             for (int r = 0; r < filled; ++r) wide = wide && aligned32(fp.p[r]);
-            if (wide) {
-                // 256-bit accesses for the body, the 16-byte kernel for what is left (under 32 bytes)
-                const size_t nvec32 = bytes / 32;
-                launch_in_stream(broadcast_kernel32, stream_grid(nvec32, kUnroll32), kStreamThreads, 0, (cudaStream_t)stream, (const Vec32 *)src, fp, filled, nvec32);
-                DISTDL_CUDA_CHECK(cudaGetLastError());
-                const size_t done = nvec32 * 32;
-                if (done < bytes) {
-                    FanPointers rest;
-                    for (int r = 0; r < kMaxFan; ++r) rest.p[r] = fp.p[r] ? (char *)fp.p[r] + done : nullptr;
-                    launch_in_stream(broadcast_kernel, 1, kStreamThreads, 0, (cudaStream_t)stream, (const uint4 *)((const char *)src + done), rest, filled, (bytes - done) / 16, tail);
-                    DISTDL_CUDA_CHECK(cudaGetLastError());
-                }
-            } else {
-                launch_in_stream(broadcast_kernel, grid, kStreamThreads, 0, (cudaStream_t)stream, (const uint4 *)src, fp, filled, nvec, tail);
-                DISTDL_CUDA_CHECK(cudaGetLastError());
-            }
+            if (wide) launch_broadcast<Vec32>(src, fp, filled, bytes, (cudaStream_t)stream);
+            else launch_broadcast<uint4>(src, fp, filled, bytes, (cudaStream_t)stream);
+            DISTDL_CUDA_CHECK(cudaGetLastError());
             filled = 0;
         }
     }

@@ -62,6 +62,21 @@ def test_generalized_conv_gradient_slices_follow_the_device(case):
     assert slices in range(3, 17)
 
 
+@pytest.mark.parametrize("vector", [16, 32])
+@pytest.mark.parametrize("more", [-1, 0, 1, 5, 4097, 70011])
+def test_broadcast_around_one_vector_per_resident_thread(vector, more):
+    """bfloat16 elements that end anywhere inside a vector, one vector per resident thread (2048 a multiprocessor) and a few less or
+    more; the cells around every copy stay untouched."""
+    torch = parity.torch
+    n = torch.cuda.get_device_properties(0).multi_processor_count * 2048 * vector // 2 + more
+    at = 64 if vector == 32 else 8
+    src = torch.randint(-2 ** 15, 2 ** 15, (n + at,), device=parity.DEV, dtype=torch.int16)
+    bufs = [torch.full((n + at + 64,), 7, device=parity.DEV, dtype=torch.int16) for _ in range(3)]
+    parity.distdl.broadcast_fwd(src[at:].view(torch.bfloat16), [b[at:at + n].view(torch.bfloat16) for b in bufs])
+    for b in bufs:
+        assert torch.equal(b[at:at + n], src[at:]) and (b[:at] == 7).all() and (b[at + n:] == 7).all()
+
+
 # global NCHW, partition, kernel
 CONV_EDGES = [
     ((1, 1, 5, 1), (1, 1, 1, 1), 3),         # one column
