@@ -289,6 +289,8 @@ distdl_status_t upload_plan_pair(const HaloPlanHost &a, const HaloPlanHost &b, H
                                  size_t extra_bytes = 0, void **extra_dev = nullptr);
 // Builds the forward (H) and adjoint (H*) box/tile lists of a partition (host only).
 distdl_status_t build_halo_plans(distdl_partition *p, bool forward_only = false);
+// What H and H* ask of the shards that they work on in place: none missing, on 16-byte boundaries, no two overlapping.
+distdl_status_t halo_check_shards(const distdl_partition *p, void *const *shards, const char *what);
 // Fills p->fast (row plan) where the geometry allows it.
 void build_fast_plan(distdl_partition *p);
 // Geometry and halo plans only, no device memory.

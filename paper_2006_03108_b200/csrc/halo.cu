@@ -817,18 +817,22 @@ static distdl_status_t check_disjoint(const distdl_partition *p, const void *con
     return DISTDL_OK;
 }
 
-static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &plan, void *const *shards,
-                              void *stream, bool adjoint, const char *what) {
-    clear_error();
+distdl_status_t halo_check_shards(const distdl_partition *p, void *const *shards, const char *what) {
     if (!p || !shards) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
     if (!p->device_block) return fail(DISTDL_ERR_CUDA, "%s: the partition was created without a CUDA device", what);
-    ShardPointers sh;
     for (int32_t w = 0; w < p->num_workers; ++w) {
         if (!shards[w]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shards[%d] is NULL", what, w);
         if (!aligned16(shards[w])) return fail(DISTDL_ERR_ALIGNMENT, "%s: shards[%d] is not 16-byte aligned", what, w);
-        sh.p[w] = shards[w];
     }
-    if (const distdl_status_t st = check_disjoint(p, shards, what)) return st;
+    return check_disjoint(p, shards, what);
+}
+
+static distdl_status_t launch(const distdl_partition *p, const HaloPlanDevice &plan, void *const *shards,
+                              void *stream, bool adjoint, const char *what) {
+    clear_error();
+    if (const distdl_status_t st = halo_check_shards(p, shards, what)) return st;
+    ShardPointers sh;
+    for (int32_t w = 0; w < p->num_workers; ++w) sh.p[w] = shards[w];
     for (int32_t w = p->num_workers; w < DISTDL_MAX_WORKERS; ++w) sh.p[w] = nullptr;
     if (plan.num_tiles == 0) return DISTDL_OK;
     // DISTDL_HALO_PLAN=box in the environment sends every call through the general box plan (for comparisons)

@@ -9,6 +9,7 @@
 // then H*.  The local adjoint is evaluated in gather form -- a cell sums over the outputs whose
 // window holds it, in ascending output order -- so overlapping windows need no atomics.
 #include <algorithm>
+#include <climits>
 #include <cstring>
 #include <vector>
 
@@ -27,11 +28,14 @@ struct PoolShard {
     int32_t oh, ow;        // this worker's block of the output
     int32_t i0, j0;        // padded-local index of the first input of output (0, 0)
     int32_t g0h, g0w;      // global index of padded-local index 0
+    int32_t hlh, hlw;      // low ghost rows / columns
+    int32_t bh, bw;        // bulk rows / columns
 };
 
 struct PoolParams {
     PoolShard s[kPoolMaxWorkers];
     int32_t planes, kh, kw, sh, sw, hg, wg, mode;
+    int32_t wrows, wcols;  // rows and columns of workers
 };
 
 // One thread per output.  blockIdx.y = worker, blockIdx.x = (plane, row tile, column tile).
@@ -116,14 +120,15 @@ pool_adj_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) 
 // what overlapping windows share stays in registers, the loads of the next step are issued before this step's arithmetic,
 // and neighbouring lanes touch neighbouring addresses.  Same results as the general kernels above.
 //
-// What bounds them: device memory, instruction issue close behind.  Measured (B200, with the H / H* around them, forward /
-// adjoint, us; before: four outputs or groups of one row per thread, nothing shared between rows; 3 x 3 / 1: the general kernels):
-//   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    358 / 421   (368 / 538)
-//   2 x 2 / 2 max, the same                                   260 / 252   (259 / 313)
-//   3 x 3 / 1 max,  8 x 16 x 1024 x 1024                      457 / 651   (1653 / 2687)
-// The adjoint's cells of a row put together by shuffles, so that a store is 32 cells and not every other one of 64: 3 x 3 / 2
-// 434 -> 500.  A maximum is taken per input row first (value, first
-// position); a NaN counts as the scan in window order counts it: it wins only as the window's first cell.
+// What bounds them: device memory, instruction issue close behind.  Measured (B200, with H / H*, forward / adjoint, us; before: H* as a
+// kernel of its own behind the local adjoint):
+//   3 x 3 / 2 max, 16 x 16 x 1024 x 1024 on 4 x 4 workers    354 / 350   (354 / 417)
+//   3 x 3 / 1 avg, 12 x 13 x 802 x 239 on 1 x 2               108 / 101   (108 / 127)
+//   3 x 3 / 1 max, 2 x 7 x 752 x 84 on 3 x 4                  18.8 / 14.6  (18.8 / 15.7)
+//   3 x 3 / 2 avg, 3 x 1 x 91 x 337 on 1 x 3                  3.9 / 3.1    (3.9 / 3.9)
+// H in the forward kernel as well: ghosts copied by the warps that read them 349 of 357 us, but 3.9 -> 5.4 us for the last of these; read
+// where they lie and written beside that 407 us: the forward's loop has no instructions to spare.  A maximum is taken per input row first
+// (value, first position); a NaN counts as the scan in window order counts it: it wins only as the window's first cell.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPoolCols = 2;           // columns per lane, 32 apart
 
@@ -292,8 +297,243 @@ pool_fwd_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
     }
 }
 
-// Adjoint: a lane owns the SH x SW cells {i0 + SH * gi + r, j0 + SW * gj + c} of a group and marches down gi.  The outputs whose
-// window holds cell (r, c) of the group are (gi - t, gj - v) with window positions a = r + t * SH < KH, b = c + v * SW < KW, all
+// Cells of one row: lane l of a strip holds cells SW * (l + 32 u) + c.  Two to a lane are stored as 8-byte pairs; in rows that start off an
+// 8-byte boundary (every other one at an odd pitch) a pair is a lane's second cell and the next lane's first (3 x 3 / 2 max, 16 x 16 x 1024 x
+// 1024: 367 -> 359 us).
+template <int SW, int NU>
+__device__ __forceinline__ void pool_store_row(float *out, const float (&v)[NU][SW], int cols, int lane) {
+    if (SW == 2 && cols == 64 * NU) {
+        float *o = out + 2 * lane;
+        if ((reinterpret_cast<uintptr_t>(out) & 7u) == 0) {
+#pragma unroll
+            for (int u = 0; u < NU; ++u) *reinterpret_cast<float2 *>(o + 64 * u) = make_float2(v[u][0], v[u][SW - 1]);
+        } else {
+            float next[NU];
+#pragma unroll
+            for (int u = 0; u < NU; ++u) next[u] = __shfl_sync(0xffffffffu, v[u][0], (lane + 1) & 31);
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                const float n = lane < 31 ? next[u] : next[u + 1 < NU ? u + 1 : u];
+                if (u + 1 < NU || lane < 31) *reinterpret_cast<float2 *>(o + 64 * u + 1) = make_float2(v[u][SW - 1], n);
+            }
+            if (lane == 0) out[0] = v[0][0];
+            if (lane == 31) o[64 * (NU - 1) + 1] = v[NU - 1][SW - 1];
+        }
+        return;
+    }
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int c = 0; c < SW; ++c)
+            if (SW * (lane + 32 * u) + c < cols) out[SW * (lane + 32 * u) + c] = v[u][c];
+}
+
+// Adjoint with H* in it: every bulk cell sums over all outputs whose window holds it, the neighbours' among them, in ascending order, and
+// the ghosts are cleared.  A lane owns groups of SH x SW bulk cells and marches down the rows of outputs; an output row is added to the KH
+// rows of cells that its windows hold, whose sums move up by SH rows as the first of them are done.  The first column of a group is
+// column DW of the windows that begin every SW columns, so the columns of a shard fill its strips whatever its ghosts (256 columns behind
+// a ghost one: two strips of 64 groups, three when the groups begin with the windows).
+// The outputs whose window holds cell column c of a group are J - v with window column b = c + DW + (v - EW) * SW < KW, known at compile
+// time.  Rows of outputs above and below are read where they lie, the one column of outputs left and right of the shard that is met is
+// fetched once by the lanes, a row each, and handed out by shuffles.
+// NU columns of groups a lane: one where the shards are no wider than 32 groups (max 2 x 7 x 752 x 84 on 3 x 4 workers 20.2 -> 14.6 us), two
+// otherwise (one for all: 350 -> 460 us at 16 x 16 x 1024 x 1024).  The next row is fetched before this one is added up, and four blocks fit a
+// multiprocessor: with the fetch behind the sums 359 us, with three blocks 405, with five 375.
+template <int KH, int KW, int SH, int SW, int MODE, int DW, int NU>
+__device__ __forceinline__ void pool_adj_strip(const PoolParams &P, int w, int plane, int first_row, int rows, int col0, int lane) {
+    constexpr int EW = DW > 0 ? 1 : 0, NI = (KH + SH - 1) / SH, NJ = (KW - 1 - DW) / SW + EW + 1;
+    const PoolShard &S = P.s[w];
+    const int wr = w / P.wcols, wc = w - wr * P.wcols;
+    const int gi0 = div_floor(S.hlh - S.i0, SH) + first_row, bulk_end = S.hlh + S.bh;
+    if (S.i0 + gi0 * SH >= bulk_end || col0 * SW >= S.bw) return;
+    const int i_begin = gi0 - (NI - 1), i_end = min(gi0 + rows, div_floor(bulk_end - 1 - S.i0, SH) + 1);   // output rows
+    const int j0 = col0 + lane + div_floor(S.hlw - S.j0, SW) + EW;                     // newest output column of the lane's first group
+    const int cols = min(S.bw - col0 * SW, 32 * NU * SW);                       // cells of this strip
+    // row i of the outputs of this worker column (of the worker column beside: dc): worker and row there, false if there is none
+    auto owner = [&](int i, int &dr, int &il) {
+        dr = i < 0 ? -1 : i >= S.oh ? 1 : 0;
+        if ((unsigned)(wr + dr) >= (unsigned)P.wrows) return false;
+        const int oh = P.s[w + dr * P.wcols].oh;
+        il = dr < 0 ? i + oh : dr ? i - S.oh : i;
+        return (unsigned)il < (unsigned)oh;
+    };
+    // outputs -1 and ow of row i_begin + lane
+    const bool has_left = wc > 0 && col0 == 0 && j0 - lane - (NJ - 1) < 0, has_right = wc + 1 < P.wcols && col0 * SW + cols == S.bw;
+    float sg[2] = {0.f, 0.f};
+    int sc[2] = {-1, -1};
+    if (has_left || has_right) {
+        int dr, il;
+        if (i_begin + lane < i_end && owner(i_begin + lane, dr, il)) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (!(k ? has_right : has_left)) continue;
+                const PoolShard &N = P.s[w + dr * P.wcols + 2 * k - 1];
+                const size_t o = ((size_t)plane * N.oh + il) * N.ow + (k ? 0 : N.ow - 1);
+                sg[k] = __ldg(N.in + o);
+                if (MODE == DISTDL_POOL_MAX) sc[k] = __ldg(N.arg + o);
+            }
+        }
+    }
+    bool jok[NU][NJ], whole = true;
+#pragma unroll
+    for (int u = 0; u < NU; ++u)
+#pragma unroll
+        for (int v = 0; v < NJ; ++v) {
+            jok[u][v] = (unsigned)(j0 + 32 * u - v) < (unsigned)S.ow;
+            whole = whole && jok[u][v];
+        }
+    whole = __all_sync(0xffffffffu, whole);
+    const float *dy = S.in;
+    const int32_t *arg = S.arg;
+    bool row_ok = false;
+    int at = i_begin, seek_at = i_begin;                   // output row to load next; row where the pointers move to another shard
+    float gn[NU][NJ];
+    int cn[NU][NJ];                                        // MAX: recorded position, -1 for an absent output
+    auto load = [&]() {
+        if (at == seek_at) {
+            int dr, il = 0;
+            row_ok = owner(at, dr, il);
+            const PoolShard &N = P.s[row_ok ? w + dr * P.wcols : w];
+            // above: down to row 0 (from a row above the shard above, which no window of this one's cells needs: to that shard)
+            seek_at = dr < 0 ? (!row_ok && il < 0 ? at - il : 0) : dr == 0 ? S.oh : row_ok ? S.oh + N.oh : INT_MAX;
+            const size_t o = ((size_t)plane * N.oh + il) * N.ow + j0;
+            dy = N.in + o;
+            if (MODE == DISTDL_POOL_MAX) arg = N.arg + o;
+        }
+        if (whole && row_ok) {
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+#pragma unroll
+                for (int v = 0; v < NJ; ++v) {
+                    gn[u][v] = __ldg(dy + (32 * u - v));
+                    if (MODE == DISTDL_POOL_MAX) cn[u][v] = __ldg(arg + (32 * u - v));
+                }
+        } else {
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+#pragma unroll
+                for (int v = 0; v < NJ; ++v) {
+                    const bool on = row_ok && jok[u][v];
+                    gn[u][v] = on ? __ldg(dy + (32 * u - v)) : 0.f;
+                    if (MODE == DISTDL_POOL_MAX) cn[u][v] = on ? __ldg(arg + (32 * u - v)) : -1;
+                }
+        }
+        dy += S.ow;
+        if (MODE == DISTDL_POOL_MAX) arg += S.ow;
+        ++at;
+    };
+    load();
+    constexpr int SLOTS = KH > SH ? KH : SH;
+    float acc[SLOTS][NU][SW];
+#pragma unroll
+    for (int a = 0; a < SLOTS; ++a)
+#pragma unroll
+        for (int u = 0; u < NU; ++u)
+#pragma unroll
+            for (int c = 0; c < SW; ++c) acc[a][u][c] = 0.f;
+    // the ghost cell of every row that this lane clears: lanes 0 on left of the strip, lanes 16 on right of it
+    const bool left = col0 == 0 && S.hlw > 0, right = col0 * SW + cols == S.bw && S.hlw + S.bw < S.pw;
+    const bool clears = lane < 16 ? left && lane < S.hlw : right && lane - 16 < S.pw - S.hlw - S.bw;
+    const int clear_at = lane < 16 ? lane - S.hlw : cols + lane - 16;
+    float *shard = S.out + (size_t)plane * S.ph * S.pw;
+    float *out = shard + (size_t)(S.i0 + gi0 * SH) * S.pw + (S.hlw + col0 * SW);       // first cell of the strip
+#pragma unroll 1
+    for (int i = i_begin; i < i_end; ++i) {
+        float g[NU][NJ];
+        int code[NU][NJ];
+#pragma unroll
+        for (int u = 0; u < NU; ++u)
+#pragma unroll
+            for (int v = 0; v < NJ; ++v) {
+                g[u][v] = gn[u][v];
+                code[u][v] = cn[u][v];
+            }
+        if (i + 1 < i_end) load();
+        if (has_left) {
+            const float x = __shfl_sync(0xffffffffu, sg[0], i - i_begin);
+            const int c = MODE == DISTDL_POOL_MAX ? __shfl_sync(0xffffffffu, sc[0], i - i_begin) : 0;
+#pragma unroll
+            for (int v = 1; v < NJ; ++v)
+                if (j0 - v == -1) {
+                    g[0][v] = x;
+                    code[0][v] = c;
+                }
+        }
+        if (has_right) {
+            const float x = __shfl_sync(0xffffffffu, sg[1], i - i_begin);
+            const int c = MODE == DISTDL_POOL_MAX ? __shfl_sync(0xffffffffu, sc[1], i - i_begin) : 0;
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+#pragma unroll
+                for (int v = 0; v < NJ; ++v)
+                    if (j0 + 32 * u - v == S.ow) {
+                        g[u][v] = x;
+                        code[u][v] = c;
+                    }
+        }
+#pragma unroll
+        for (int a = 0; a < KH; ++a)
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+#pragma unroll
+                for (int c = 0; c < SW; ++c)
+#pragma unroll
+                    for (int v = NJ - 1; v >= 0; --v) {
+                        const int b = c + DW + (v - EW) * SW;
+                        if (b < 0 || b >= KW) continue;                                // compile-time
+                        if (MODE == DISTDL_POOL_AVG || code[u][v] == a * KW + b) acc[a][u][c] = __fadd_rn(acc[a][u][c], g[u][v]);
+                    }
+        if (i >= gi0) {
+#pragma unroll
+            for (int r = 0; r < SH; ++r) {
+                const int p = S.i0 + i * SH + r;
+                if (p >= S.hlh && p < bulk_end) {
+                    if (MODE == DISTDL_POOL_AVG)
+#pragma unroll
+                        for (int u = 0; u < NU; ++u)
+#pragma unroll
+                            for (int c = 0; c < SW; ++c) acc[r][u][c] = __fmul_rn(acc[r][u][c], 1.0f / (float)(KH * KW));
+                    pool_store_row<SW, NU>(out, acc[r], cols, lane);
+                    if (clears) out[clear_at] = 0.f;
+                }
+                out += S.pw;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < SLOTS; ++a)
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+#pragma unroll
+                for (int c = 0; c < SW; ++c) acc[a][u][c] = a + SH < SLOTS ? acc[a + SH < SLOTS ? a + SH : a][u][c] : 0.f;
+    }
+    // ghost rows above and below this strip
+    const int qa = left ? 0 : S.hlw + col0 * SW, qb = right ? S.pw : S.hlw + col0 * SW + cols;
+    if (first_row == 0)
+        for (int p = 0; p < S.hlh; ++p)
+            for (int q = qa + lane; q < qb; q += 32) shard[(size_t)p * S.pw + q] = 0.f;
+    if (S.i0 + (gi0 + rows) * SH >= bulk_end)
+        for (int p = bulk_end; p < S.ph; ++p)
+            for (int q = qa + lane; q < qb; q += 32) shard[(size_t)p * S.pw + q] = 0.f;
+}
+
+template <int KH, int KW, int SH, int SW, int MODE, int NU>
+__global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY, 4)
+pool_adj_fused(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {
+    stream_enter();
+    const PoolShard &S = P.s[blockIdx.y];
+    int rest = blockIdx.x;
+    const int tx = rest % tiles_x;
+    rest /= tiles_x;
+    const int ty = rest % tiles_y;
+    const int plane = rest / tiles_y;
+    const int first_row = (ty * kPoolThreadsY + (int)threadIdx.y) * rows, col0 = tx * (32 * NU);
+    const int shift = S.hlw - S.j0 - SW * div_floor(S.hlw - S.j0, SW);
+    if (SW == 1 || shift == 0) pool_adj_strip<KH, KW, SH, SW, MODE, 0, NU>(P, blockIdx.y, plane, first_row, rows, col0, threadIdx.x);
+    else pool_adj_strip<KH, KW, SH, SW, MODE, SW - 1, NU>(P, blockIdx.y, plane, first_row, rows, col0, threadIdx.x);
+}
+
+// Adjoint of the local layer alone (H* follows), where a shard meets more than a column of a neighbour's outputs: a lane owns the SH x SW
+// cells {i0 + SH * gi + r, j0 + SW * gj + c} of a group and marches down gi.  The outputs whose window holds cell (r, c) of the group are (gi - t, gj - v) with window positions a = r + t * SH < KH, b = c + v * SW < KW, all
 // known at compile time; the outputs (gi - t, .) of the rows above stay in registers, and every cell picks its terms
 // (ascending output order = descending t, v).
 template <int KH, int KW, int SH, int SW, int MODE>
@@ -390,15 +630,17 @@ pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
 }
 
 template <int KH, int KW, int SH, int SW>
-static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int tiles_x, int tiles_y, int rows, bool adjoint, cudaStream_t s) {
-    if (!adjoint) {
-        if (P.mode == DISTDL_POOL_AVG) launch_in_stream(pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
-        else launch_in_stream(pool_fwd_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
-    } else {
-        if (P.mode == DISTDL_POOL_AVG) launch_in_stream(pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_AVG>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
-        else launch_in_stream(pool_adj_fixed<KH, KW, SH, SW, DISTDL_POOL_MAX>, grid, block, 0, s, P, tiles_x, tiles_y, rows);
-    }
+static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int tiles_x, int tiles_y, int rows, bool adjoint, bool fused, int nu, cudaStream_t s) {
+    const auto run = [&](auto kernel) { launch_in_stream(kernel, grid, block, 0, s, P, tiles_x, tiles_y, rows); };
+    constexpr int AVG = DISTDL_POOL_AVG, MAX = DISTDL_POOL_MAX;
+    const bool avg = P.mode == AVG;
+    if (!adjoint) avg ? run(pool_fwd_fixed<KH, KW, SH, SW, AVG>) : run(pool_fwd_fixed<KH, KW, SH, SW, MAX>);
+    else if (fused && nu == 1) avg ? run(pool_adj_fused<KH, KW, SH, SW, AVG, 1>) : run(pool_adj_fused<KH, KW, SH, SW, MAX, 1>);
+    else if (fused) avg ? run(pool_adj_fused<KH, KW, SH, SW, AVG, 2>) : run(pool_adj_fused<KH, KW, SH, SW, MAX, 2>);
+    else avg ? run(pool_adj_fixed<KH, KW, SH, SW, AVG>) : run(pool_adj_fixed<KH, KW, SH, SW, MAX>);
 }
+
+static int pool_floor(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 struct PoolDim {
     std::vector<int64_t> out_start, out_size;
@@ -466,7 +708,14 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
     P.hg = (int32_t)p->global_shape[2];
     P.wg = (int32_t)p->global_shape[3];
     P.mode = mode;
+    P.wrows = p->pshape[2];
+    P.wcols = p->pshape[3];
     int64_t max_rows = 0, max_cols = 0;
+    // The adjoint with H* in it: where there is an H* (a ghost anywhere).  Max pooling on windows that do not overlap has one term a cell and
+    // half the registers without it, and is faster so once the launch no longer counts (2 x 2 / 2, pairs: 12 x 7 x 333 x 129 on 3 x 2 workers
+    // 22.2 -> 18.7 us; 8 x 16 x 514 x 514 on 4 x 4 101 -> 109; average pooling 93 -> 93 there, 16 x 16 x 1000 x 1000 on 3 x 3 615 -> 532).
+    bool fused = adjoint && p->adj_dev.num_tiles > 0 &&
+                 (mode == DISTDL_POOL_AVG || sh < kh || sw < kw || (int64_t)P.planes * P.hg * P.wg < ((int64_t)8 << 20));
     for (int32_t w = 0; w < p->num_workers; ++w) {
         const int32_t r = w / p->pshape[3], c = w % p->pshape[3];
         if (!in[w] || !out[w]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shard pointer %d is NULL", what, w);
@@ -481,6 +730,10 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         S.ow = (int32_t)dw.out_size[c];
         S.g0h = (int32_t)(p->start[2][r] - p->hlo[2][r]);
         S.g0w = (int32_t)(p->start[3][c] - p->hlo[3][c]);
+        S.hlh = p->hlo[2][r];
+        S.hlw = p->hlo[3][c];
+        S.bh = (int32_t)p->size[2][r];
+        S.bw = (int32_t)p->size[3][c];
         S.i0 = (int32_t)(dh.out_start[r] * sh - plh - S.g0h);
         S.j0 = (int32_t)(dw.out_start[c] * sw - plw - S.g0w);
         if (S.oh > 0 && (S.i0 < 0 || S.i0 + (int64_t)(S.oh - 1) * sh + kh > S.ph))
@@ -489,18 +742,34 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
             return fail(DISTDL_ERR_SHAPE, "%s: worker column %d does not hold the inputs of its outputs", what, c);
         max_rows = std::max<int64_t>(max_rows, adjoint ? S.ph : S.oh);
         max_cols = std::max<int64_t>(max_cols, adjoint ? S.pw : S.ow);
+        // it hands one column of the neighbours' outputs on either side from lane to lane, and a lane clears one ghost cell a row
+        fused = fused && S.oh >= 1 && S.ow >= kw && S.hlw <= 16 && S.pw - S.hlw - S.bw <= 16 &&
+                (c == 0 || pool_floor(S.hlw - S.j0 - kw + sw, sw) >= -1) && (c + 1 == p->pshape[3] || pool_floor(S.hlw + S.bw - 1 - S.j0, sw) <= S.ow);
     }
+    // H and H* work on the padded shards: what they ask of them holds for the layer as well
+    st = halo_check_shards(p, adjoint ? out : const_cast<void *const *>(reinterpret_cast<const void *const *>(in)), what);
+    if (st != DISTDL_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    // the compile-time variants: 64 columns and up to 16 rows per warp, fewer where eight warps would leave some without a row
+    // the compile-time variants: 64 (or 32) columns and up to 16 rows (20 of the fused adjoint) per warp, fewer where eight warps would leave some without a row
     // or an SM would have fewer than 16 warps
     const int fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
                     : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
-    if (fixed && adjoint) {
-        // the compile-time adjoint walks groups of sh x sw cells; the group lattice starts up to one group before cell 0
+    fused = fused && fixed;
+    if (fixed && adjoint && !fused) {
+        // groups of sh x sw cells; the group lattice starts up to one group before cell 0
         max_rows = max_rows / sh + 2;
         max_cols = max_cols / sw + 2;
+    } else if (fixed && adjoint) {
+        // the compile-time adjoint walks groups of sh x sw bulk cells, the first row of groups may begin above the bulk
+        max_rows = max_cols = 0;
+        for (int32_t w = 0; w < p->num_workers; ++w) {
+            const PoolShard &S = P.s[w];
+            max_rows = std::max<int64_t>(max_rows, pool_floor(S.hlh + S.bh - 1 - S.i0, sh) - pool_floor(S.hlh - S.i0, sh) + 1);
+            max_cols = std::max<int64_t>(max_cols, (S.bw + sw - 1) / sw);
+        }
     }
-    const int cols = fixed ? 32 * kPoolCols : kPoolThreadsX;
+    const int nu = fused && max_cols <= 32 ? 1 : kPoolCols;      // columns per lane
+    const int cols = fixed ? 32 * nu : kPoolThreadsX;
     const int tiles_x = (int)((max_cols + cols - 1) / cols);
     int rows = 1;
     if (fixed) {
@@ -508,7 +777,7 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
         DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const int64_t all = (int64_t)p->num_workers * P.planes * tiles_x * max_rows;      // rows of 64 columns
-        rows = (int)std::min<int64_t>(16, std::max<int64_t>(2, std::min((max_rows + kPoolThreadsY - 1) / kPoolThreadsY, all / (16 * sms))));
+        rows = (int)std::min<int64_t>(fused ? 20 : 16, std::max<int64_t>(2, std::min((max_rows + kPoolThreadsY - 1) / kPoolThreadsY, all / (16 * sms))));
     }
     const int tiles_y = (int)((max_rows + kPoolThreadsY * rows - 1) / (kPoolThreadsY * rows));
     if (fixed) rows = (int)((max_rows + kPoolThreadsY * tiles_y - 1) / (kPoolThreadsY * tiles_y));      // equal shares
@@ -521,14 +790,14 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         if (st != DISTDL_OK) return st;
     }
     if (blocks > 0) {
-        if (fixed == 1) launch_pool_fixed<2, 2, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
-        else if (fixed == 2) launch_pool_fixed<3, 3, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
-        else if (fixed == 3) launch_pool_fixed<3, 3, 1, 1>(P, grid, block, tiles_x, tiles_y, rows, adjoint, s);
+        if (fixed == 1) launch_pool_fixed<2, 2, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, fused, nu, s);
+        else if (fixed == 2) launch_pool_fixed<3, 3, 2, 2>(P, grid, block, tiles_x, tiles_y, rows, adjoint, fused, nu, s);
+        else if (fixed == 3) launch_pool_fixed<3, 3, 1, 1>(P, grid, block, tiles_x, tiles_y, rows, adjoint, fused, nu, s);
         else if (!adjoint) launch_in_stream(pool_fwd_kernel, grid, block, 0, s, P, tiles_x, tiles_y);
         else launch_in_stream(pool_adj_kernel, grid, block, 0, s, P, tiles_x, tiles_y);
     }
     DISTDL_CUDA_CHECK(cudaGetLastError());
-    if (!adjoint) return DISTDL_OK;
+    if (!adjoint || fused) return DISTDL_OK;
     return distdl_halo_adj(p, out, stream);
 }
 

@@ -232,6 +232,14 @@ POOL_EDGES = [
     ((1, 3, 9, 260), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),       # 65 outputs: one column past a warp's 64
     ((40, 9, 66, 61), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),      # several rows a warp, every warp at both ends of the rows
     ((90, 16, 75, 33), (1, 1, 1, 1), (3, 3), (1, 1), ((1, 1), (1, 1))),     # 75 rows in equal shares of 16 warps
+    ((1, 2, 100, 84), (1, 1, 2, 4), (3, 3), (1, 1), ((1, 1), (1, 1))),      # shards of 21 columns: one column a lane, outputs met on both sides
+    ((1, 1, 20, 64), (1, 1, 1, 2), (3, 3), (1, 1), ((1, 1), (1, 1))),       # of 32
+    ((1, 1, 20, 66), (1, 1, 2, 2), (3, 3), (1, 1), ((1, 1), (1, 1))),       # of 33: two columns a lane
+    ((1, 2, 30, 512), (1, 1, 2, 4), (3, 3), (2, 2), ((1, 1), (1, 1))),      # whole strips, every other row off an 8-byte boundary
+    ((1, 1, 61, 259), (1, 1, 3, 2), (2, 2), (2, 2), ((0, 0), (0, 0))),      # windows cut by shards' ends
+    ((1, 1, 30, 31), (1, 1, 4, 4), (3, 3), (1, 1), ((0, 0), (0, 0))),       # two columns of a neighbour's outputs: the local adjoint, then H*
+    ((1, 1, 6, 7), (1, 1, 3, 3), (3, 3), (2, 2), ((1, 1), (1, 1))),         # one output a shard: the same
+    ((8, 60, 264, 36), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),     # 17 rows of groups a warp
 ]
 
 
