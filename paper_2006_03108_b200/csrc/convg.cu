@@ -73,7 +73,6 @@ constexpr int cg_blocks(int px) { return px == 8 ? 3 : 4; }
 template <int K, bool ADJ, int CP, int PX>
 __global__ void __launch_bounds__(kCgThreads, cg_blocks(PX))
 convg_kernel(const __grid_constant__ ConvGParams G) {
-    stream_enter();
     constexpr int PH = K / 2, CT = 2 * CP;
     constexpr int NF = ((PX + K - 1 + 3) / 4) * 4;         // floats of a thread's window per row
     constexpr int WF = ((K * K * CT + 3) / 4) * 4;
@@ -95,12 +94,12 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
     const int n0 = (int)id * T.tn;
     const int bh = G.bh[r], bw = G.bw[c];
     const int i0 = ty * T.th, j0 = tx * PX * T.seg;
-    if (i0 >= bh || j0 >= bw) return;                      // shards smaller than the largest
+    const bool live = i0 < bh && j0 < bw;                  // shards smaller than the largest
     const int ob = G.grp_block[g], o0 = G.grp_first[g], oc = G.grp_count[g];
     const int spatial = G.ph * G.pw;
 
-    // where every staged cell comes from (each thread reads back its own entries only)
-    for (int e = tid; e < T.entries; e += kCgThreads) {
+    // where every staged cell comes from (each thread reads back its own entries only): while the kernel before this one ends
+    for (int e = tid; live && e < T.entries; e += kCgThreads) {
         uint32_t q = (uint32_t)e;
         const int s = (int)fast_rem(G.cols, q);
         const int ry = (int)fast_rem(G.rows, q);
@@ -143,22 +142,41 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
     }
     if (oc < CT)
         for (int idx = tid; idx < 2 * WF; idx += kCgThreads) wbuf[idx] = 0.f;
+    stream_enter();
+    if (!live) return;
 
-    // first cell (bulk row 0, column 0) of the channel's plane in every neighbour, per image
+    // First cell (bulk row 0, column 0) of the channel's plane in every neighbour, per image.  Channels come one after another: with four
+    // pixels a thread its pointer and its weights' offsets are worked out at the first channel of a block and moved on from there (1 x 14
+    // x 61 x 68, 3 x 3, forward / adjoint / gradients 33.6 -> 30.4 us, 29.0 with the table above ahead of the wait as well); with eight there is
+    // no register for it (16 -> 16 channels at 1024 x 1024: 1.10 -> 1.12 ms).
+    constexpr bool KEEP = PX == 4;
+    const float *plane_p = nullptr;
+    uint32_t plane_step = 0;
     auto set_pointers = [&](int ib, int cl, int b) {
         for (int t = tid; t < 9 * T.tn; t += kCgThreads) {
+            if (KEEP && cl > 0 && t == tid) {
+                plane_p += plane_step;
+                ptrs[b * 9 * T.tn + t] = plane_p;
+                continue;
+            }
             uint32_t q = (uint32_t)t;
             const int tn = (int)fast_rem(G.tn, q);
             const int rr = r + (int)q / 3 - 1, cc = c + (int)q % 3 - 1;
             const float *p = nullptr;
             if (rr >= 0 && rr < G.ph && cc >= 0 && cc < G.pw) {
                 const uint32_t pitch = (uint32_t)(G.bw[cc] + 2 * io);
-                p = G.in[ib * spatial + rr * G.pw + cc] +
-                    (size_t)((n0 + tn) * G.cnt_in[ib] + cl) * ((uint32_t)(G.bh[rr] + 2 * io) * pitch) + (io * pitch + io);
+                const uint32_t step = (uint32_t)(G.bh[rr] + 2 * io) * pitch;
+                p = G.in[ib * spatial + rr * G.pw + cc] + (size_t)((n0 + tn) * G.cnt_in[ib] + cl) * step + (io * pitch + io);
+                if (KEEP && t == tid) plane_step = step;
             }
+            if (KEEP && t == tid) plane_p = p;
             ptrs[b * 9 * T.tn + t] = p;
         }
     };
+    // this thread's weights of a channel: their offsets in the block, and the channel's first
+    constexpr int NW = (K * K * CT + kCgThreads - 1) / kCgThreads;
+    int w_off[NW], w_step = 0;
+    const float *w_p = nullptr;
     const uint32_t tiles_s = (uint32_t)__cvta_generic_to_shared(tiles), wbuf_s = (uint32_t)__cvta_generic_to_shared(wbuf);
     auto stage = [&](int ib, int cl, int b) {
         const uint32_t dst0 = tiles_s + (uint32_t)(b * T.tile_floats) * 4u;
@@ -167,15 +185,30 @@ convg_kernel(const __grid_constant__ ConvGParams G) {
             const uint2 t = table[e];
             if (t.x != 0xffffffffu) cp_async4_to(dst0 + (t.y & 0xffffu) * 4u, pt[t.y >> 16] + t.x);
         }
-        const float *blk = ADJ ? G.w[ib * G.pci + ob] : G.w[ob * G.pci + ib];
         const int s_out = ADJ ? K * K : G.cnt_in[ib] * K * K, s_in = ADJ ? G.cnt_out[ob] * K * K : K * K;
-        const float *wsrc = blk + (size_t)o0 * s_out + (size_t)cl * s_in;
+        const float *first = (ADJ ? G.w[ib * G.pci + ob] : G.w[ob * G.pci + ib]) + (size_t)o0 * s_out;
+        if constexpr (KEEP) {
+            if (cl == 0) {
+                w_p = first;
+                w_step = s_in;
 #pragma unroll
-        for (int k = 0; k < (K * K * CT + kCgThreads - 1) / kCgThreads; ++k) {
-            const int idx = tid + k * kCgThreads;
-            const int tap = idx / CT, o = idx - tap * CT;
-            if (idx < K * K * CT && o < oc)
-                cp_async4_to(wbuf_s + (uint32_t)(b * WF + idx) * 4u, wsrc + (size_t)o * s_out + (ADJ ? K * K - 1 - tap : tap));   // adjoint: rotated
+                for (int k = 0; k < NW; ++k) {
+                    const int idx = tid + k * kCgThreads, tap = idx / CT, o = idx - tap * CT;
+                    w_off[k] = idx < K * K * CT && o < oc ? o * s_out + (ADJ ? K * K - 1 - tap : tap) : -1;      // adjoint: rotated
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NW; ++k)
+                if (w_off[k] >= 0) cp_async4_to(wbuf_s + (uint32_t)(b * WF + tid + k * kCgThreads) * 4u, w_p + w_off[k]);
+            w_p += w_step;
+        } else {
+            const float *wsrc = first + (size_t)cl * s_in;
+#pragma unroll
+            for (int k = 0; k < NW; ++k) {
+                const int idx = tid + k * kCgThreads, tap = idx / CT, o = idx - tap * CT;
+                if (idx < K * K * CT && o < oc)
+                    cp_async4_to(wbuf_s + (uint32_t)(b * WF + idx) * 4u, wsrc + (size_t)o * s_out + (ADJ ? K * K - 1 - tap : tap));
+            }
         }
     };
     auto advance = [&](int &ib, int &cl) {
