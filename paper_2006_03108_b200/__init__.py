@@ -1,7 +1,7 @@
 """Thin Python binding of the C-ABI library (include/distdl.h).
 
-Argument marshalling only: tensors are turned into device pointers and sizes, every step of
-every operator runs in the CUDA kernels of libdistdl.so.  There is no CPU or PyTorch fallback:
+Argument marshalling only: tensors are turned into device pointers and sizes (for the operators in _binding.so,
+csrc/binding.cpp), every step of every operator runs in the CUDA kernels of libdistdl.so.  There is no CPU or PyTorch fallback:
 if the library is missing or a call fails, an exception is raised.
 
 PyTorch is used by callers for device memory and streams; this module only reads
@@ -9,6 +9,7 @@ PyTorch is used by callers for device memory and streams; this module only reads
 """
 
 import ctypes
+import importlib
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -142,15 +143,40 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+_calls = None
+
+
+def _load():
+    """The operators' calls (once)."""
+    global _calls
+    if _calls is None:
+        lib()
+        calls = importlib.import_module(__name__ + "._binding")
+
+        def device():
+            import torch
+            d = torch.cuda.current_device()                  # sets CUDA up in PyTorch
+            calls.set_stream_lookup(getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device),
+                                    getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda d: torch.cuda.current_stream(d).cuda_stream))
+            return d
+
+        calls.set_stream_lookup(device, device)              # until the first call on the current stream
+        _calls = calls
+    return _calls
+
+
+_dtype_codes = {}
+
+
 def _dtype_code(t):
-    import torch
-    if t.dtype == torch.float32:
-        return F32
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float64:
-        return F64
-    raise TypeError("unsupported dtype %s" % t.dtype)
+    code = _dtype_codes.get(t.dtype)
+    if code is None:
+        import torch
+        _dtype_codes.update({torch.float32: F32, torch.bfloat16: BF16, torch.float64: F64})
+        code = _dtype_codes.get(t.dtype)
+        if code is None:
+            raise TypeError("unsupported dtype %s" % t.dtype)
+    return code
 
 
 class Partition:
@@ -256,23 +282,19 @@ def halo_widths_1d(n, p, kernel, stride=1, dilation=1, pad_lo=0, pad_hi=0):
 
 
 def broadcast_fwd(src, dsts, stream=None):
-    _check(lib().distdl_broadcast_fwd(_ptr(src), _ptr_array(dsts), len(dsts), src.numel(), _dtype_code(src),
-                                      _stream(stream)))
+    _check((_calls or _load()).broadcast_fwd(src, dsts, len(dsts), src.numel(), _dtype_code(src), stream))
 
 
 def sumreduce_adj(dy, dxs, stream=None):
-    _check(lib().distdl_sumreduce_adj(_ptr(dy), _ptr_array(dxs), len(dxs), dy.numel(), _dtype_code(dy),
-                                      _stream(stream)))
+    _check((_calls or _load()).sumreduce_adj(dy, dxs, len(dxs), dy.numel(), _dtype_code(dy), stream))
 
 
 def sumreduce_fwd(srcs, dst, stream=None):
-    _check(lib().distdl_sumreduce_fwd(_ptr_array(srcs), _ptr(dst), len(srcs), dst.numel(), _dtype_code(dst),
-                                      _stream(stream)))
+    _check((_calls or _load()).sumreduce_fwd(srcs, dst, len(srcs), dst.numel(), _dtype_code(dst), stream))
 
 
 def broadcast_adj(dys, dx, stream=None):
-    _check(lib().distdl_broadcast_adj(_ptr_array(dys), _ptr(dx), len(dys), dx.numel(), _dtype_code(dx),
-                                      _stream(stream)))
+    _check((_calls or _load()).broadcast_adj(dys, dx, len(dys), dx.numel(), _dtype_code(dx), stream))
 
 
 def _partition_pair(src_pshape, dst_pshape, small):
@@ -300,11 +322,11 @@ def partition_broadcast_adj(src_pshape, dst_pshape, dy, dx, stream=None):
 
 
 def halo_fwd(part, shards, stream=None):
-    _check(lib().distdl_halo_fwd(part.handle, _ptr_array(shards), _stream(stream)))
+    _check((_calls or _load()).halo_fwd(part.handle.value, shards, stream))
 
 
 def halo_adj(part, shards, stream=None):
-    _check(lib().distdl_halo_adj(part.handle, _ptr_array(shards), _stream(stream)))
+    _check((_calls or _load()).halo_adj(part.handle.value, shards, stream))
 
 
 def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dtype=F32, stream=None):
@@ -320,47 +342,42 @@ def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dt
 
 
 def conv_fwd(part, x, w, bias, y, stream=None):
-    kh, kw = int(w.shape[-2]), int(w.shape[-1])
-    _check(lib().distdl_conv_fwd(part.handle, _ptr_array(x), _ptr(w), _ptr(bias), kh, kw, _ptr_array(y),
-                                 _stream(stream)))
+    kh, kw = w.shape[-2:]
+    _check((_calls or _load()).conv_fwd(part.handle.value, x, w, bias, kh, kw, y, stream))
 
 
 def conv_adj(part, dy, w, dx, stream=None):
-    kh, kw = int(w.shape[-2]), int(w.shape[-1])
-    _check(lib().distdl_conv_adj(part.handle, _ptr_array(dy), _ptr(w), kh, kw, _ptr_array(dx), _stream(stream)))
+    kh, kw = w.shape[-2:]
+    _check((_calls or _load()).conv_adj(part.handle.value, dy, w, kh, kw, dx, stream))
 
 
 def _taps(w):
     """Host array of the 3 x (2R+1) taps (any nested sequence or numpy array) and the radius."""
-    rows = [[float(v) for v in row] for row in w]
-    if len(rows) != 3 or len(set(len(r) for r in rows)) != 1 or len(rows[0]) % 2 != 1:
+    taps = (_calls or _load()).taps(w)
+    if taps is None:
         raise ValueError("taps must have shape [3][2R+1]")
-    n = len(rows[0])
-    return (ctypes.c_float * (3 * n))(*[v for row in rows for v in row]), n // 2
+    return taps
 
 
 def stencil3d_fwd(part, x, w, y, stream=None):
-    arr, radius = _taps(w)
-    _check(lib().distdl_stencil3d_fwd(part.handle, _ptr_array(x), arr, radius, _ptr_array(y), _stream(stream)))
+    taps, radius = _taps(w)
+    _check(_calls.stencil3d_fwd(part.handle.value, x, taps, radius, y, stream))
 
 
 def stencil3d_adj(part, dy, w, dx, stream=None):
-    arr, radius = _taps(w)
-    _check(lib().distdl_stencil3d_adj(part.handle, _ptr_array(dy), arr, radius, _ptr_array(dx), _stream(stream)))
+    taps, radius = _taps(w)
+    _check(_calls.stencil3d_adj(part.handle.value, dy, taps, radius, dx, stream))
 
 
 def convg_fwd(px, nco, pco, x, w, bias, y, stream=None):
     """Channel-partitioned convolution layer; w: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j."""
-    kh, kw = int(w[0].shape[-2]), int(w[0].shape[-1])
-    b = None if bias is None else _ptr_array(bias)
-    _check(lib().distdl_convg_fwd(px.handle, nco, pco, _ptr_array(x), _ptr_array(w), b, kh, kw, _ptr_array(y),
-                                  _stream(stream)))
+    kh, kw = w[0].shape[-2:]
+    _check((_calls or _load()).convg_fwd(px.handle.value, nco, pco, x, w, bias, kh, kw, y, stream))
 
 
 def convg_adj(px, nco, pco, dy, w, dx, stream=None):
-    kh, kw = int(w[0].shape[-2]), int(w[0].shape[-1])
-    _check(lib().distdl_convg_adj(px.handle, nco, pco, _ptr_array(dy), _ptr_array(w), kh, kw, _ptr_array(dx),
-                                  _stream(stream)))
+    kh, kw = w[0].shape[-2:]
+    _check((_calls or _load()).convg_adj(px.handle.value, nco, pco, dy, w, kh, kw, dx, stream))
 
 
 def convg_adj_params_workspace(px, nco, pco, kh, kw):
@@ -371,10 +388,8 @@ def convg_adj_params_workspace(px, nco, pco, kh, kw):
 
 def convg_adj_params(px, nco, pco, x, dy, kernel, dw, db, workspace, stream=None):
     """dw: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j; db: list of [nco_i] or None."""
-    b = None if db is None else _ptr_array(db)
-    _check(lib().distdl_convg_adj_params(px.handle, nco, pco, _ptr_array(x), _ptr_array(dy), kernel[0], kernel[1],
-                                         _ptr_array(dw), b, _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream)))
+    _check((_calls or _load()).convg_adj_params(px.handle.value, nco, pco, x, dy, kernel[0], kernel[1], dw, db, workspace,
+                                                workspace.numel() * workspace.element_size(), stream))
 
 
 class Repartition:
@@ -414,15 +429,15 @@ class Repartition:
 
 
 def repartition_fwd(rep, src, dst, stream=None):
-    _check(lib().distdl_repartition_fwd(rep.handle, _ptr_array(src), _ptr_array(dst), _stream(stream)))
+    _check((_calls or _load()).repartition_fwd(rep.handle.value, src, dst, stream))
 
 
 def repartition_adj(rep, dy, dx, stream=None):
-    _check(lib().distdl_repartition_adj(rep.handle, _ptr_array(dy), _ptr_array(dx), _stream(stream)))
+    _check((_calls or _load()).repartition_adj(rep.handle.value, dy, dx, stream))
 
 
 def allreduce(bufs, stream=None):
-    _check(lib().distdl_allreduce(_ptr_array(bufs), len(bufs), bufs[0].numel(), _dtype_code(bufs[0]), _stream(stream)))
+    _check((_calls or _load()).allreduce(bufs, len(bufs), bufs[0].numel(), _dtype_code(bufs[0]), stream))
 
 
 POOL_AVG, POOL_MAX = 0, 1
@@ -430,33 +445,26 @@ POOL_AVG, POOL_MAX = 0, 1
 
 def pool_fwd(part, x, kernel, stride, pad, mode, y, argmax=None, stream=None):
     """kernel = (kh, kw), stride = (sh, sw), pad = ((lo_h, hi_h), (lo_w, hi_w)); x is updated in place by H."""
-    a = None if argmax is None else _ptr_array(argmax)
-    _check(lib().distdl_pool_fwd(part.handle, _ptr_array(x), kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
-                                 pad[0][1], pad[1][0], pad[1][1], mode, _ptr_array(y), a, _stream(stream)))
+    _check((_calls or _load()).pool_fwd(part.handle.value, x, kernel[0], kernel[1], stride[0], stride[1], pad[0][0], pad[0][1],
+                                        pad[1][0], pad[1][1], mode, y, argmax, stream))
 
 
 def pool_adj(part, dy, argmax, kernel, stride, pad, mode, dx, stream=None):
-    a = None if argmax is None else _ptr_array(argmax)
-    _check(lib().distdl_pool_adj(part.handle, _ptr_array(dy), a, kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
-                                 pad[0][1], pad[1][0], pad[1][1], mode, _ptr_array(dx), _stream(stream)))
+    _check((_calls or _load()).pool_adj(part.handle.value, dy, argmax, kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
+                                        pad[0][1], pad[1][0], pad[1][1], mode, dx, stream))
 
 
 def affine_fwd(nb, nfi, nfo, pfo, pfi, x, w, bias, y, stream=None):
-    b = None if bias is None else _ptr_array(bias)
-    _check(lib().distdl_affine_fwd(nb, nfi, nfo, pfo, pfi, _ptr_array(x), _ptr_array(w), b, _ptr_array(y),
-                                   _stream(stream)))
+    _check((_calls or _load()).affine_fwd(nb, nfi, nfo, pfo, pfi, x, w, bias, y, stream))
 
 
 def affine_adj(nb, nfi, nfo, pfo, pfi, dy, w, dx, stream=None):
-    _check(lib().distdl_affine_adj(nb, nfi, nfo, pfo, pfi, _ptr_array(dy), _ptr_array(w), _ptr_array(dx),
-                                   _stream(stream)))
+    _check((_calls or _load()).affine_adj(nb, nfi, nfo, pfo, pfi, dy, w, dx, stream))
 
 
 def affine_adj_params(nb, nfi, nfo, pfo, pfi, dy, x, dw, db=None, stream=None):
     """dW blocks (worker order i * pfi + j) and, if given, the db blocks of the adjoint affine algorithm."""
-    b = None if db is None else _ptr_array(db)
-    _check(lib().distdl_affine_adj_params(nb, nfi, nfo, pfo, pfi, _ptr_array(dy), _ptr_array(x), _ptr_array(dw), b,
-                                          _stream(stream)))
+    _check((_calls or _load()).affine_adj_params(nb, nfi, nfo, pfo, pfi, dy, x, dw, db, stream))
 
 
 def conv_adj_params_workspace(part, kh, kw):
@@ -468,9 +476,8 @@ def conv_adj_params_workspace(part, kh, kw):
 
 def conv_adj_params(part, x, dy, kernel, dw, db, workspace, stream=None):
     """dw [C, kh, kw] and db [C] (or None) of the adjoint convolution algorithm; workspace: a uint8 tensor."""
-    _check(lib().distdl_conv_adj_params(part.handle, _ptr_array(x), _ptr_array(dy), kernel[0], kernel[1], _ptr(dw),
-                                        _ptr(db), _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                        _stream(stream)))
+    _check((_calls or _load()).conv_adj_params(part.handle.value, x, dy, kernel[0], kernel[1], dw, db, workspace,
+                                               workspace.numel() * workspace.element_size(), stream))
 
 
 def device_status(stream=None):

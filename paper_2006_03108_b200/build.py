@@ -6,11 +6,13 @@ Usage: python -m paper_2006_03108_b200.build   (or build.build() from Python)
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdistdl.so")
+BINDING = os.path.join(HERE, "_binding.so")          # the calls from Python, a CPython extension
 
 SOURCES = ["planner.cpp", "partition.cu", "bcast_reduce.cu", "halo.cu", "convd.cu", "convg.cu", "pool.cu", "stencil3d.cu", "affine.cu"]
 
@@ -35,6 +37,7 @@ def build(force=False, verbose=False):
     deps = srcs + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     deps.append(os.path.join(ROOT, "include", "distdl.h"))
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest(deps):
+        build_binding()
         return LIB
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
@@ -59,7 +62,16 @@ def build(force=False, verbose=False):
         raise RuntimeError("nvcc failed; see the log above")
     cmd = [nvcc, "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"]
     subprocess.check_call(cmd)
+    build_binding(force)
     return LIB
+
+
+def build_binding(force=False):
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest([src, os.path.join(ROOT, "include", "distdl.h")]):
+        return
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-Wall", "-I", sysconfig.get_paths()["include"],
+                           "-I", os.path.join(ROOT, "include"), src, "-o", BINDING, "-L", HERE, "-l:libdistdl.so", "-Wl,-rpath,$ORIGIN"])
 
 
 if __name__ == "__main__":

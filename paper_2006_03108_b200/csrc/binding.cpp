@@ -1,0 +1,185 @@
+// Calls of the C ABI from Python: shards to arrays of pointers, the current stream, the call without the interpreter's lock.
+//
+// What bounds a small call is the host: H of 256 x 256 on 2 x 2 workers is 2 us on the device.  Through ctypes an array of pointers cost 0.24 us a
+// shard and a call 0.6 us before the library was entered; here a shard is one method call (0.08 us) and the arguments of a call are converted by
+// their types in the C prototype, so that the two cannot disagree.  Back to back (B200): H and H* of 256 x 256 9.1 -> 5.5 us, repartition of
+// 280 x 333 and back 11.9 -> 5.7.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <stdint.h>
+
+#include <tuple>
+#include <utility>
+#include <vector>
+
+#include "distdl.h"
+
+namespace {
+
+PyObject *g_data_ptr, *g_cuda_stream;                 // attribute names
+PyObject *g_device, *g_raw_stream;                    // PyTorch's current device, and the handle of a device's current stream
+
+bool pointer_of(PyObject *number, void **out) {       // takes the reference
+    if (!number) return false;
+    *out = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(number);
+    Py_DECREF(number);
+    return !PyErr_Occurred();
+}
+
+// Device (or host) address of a tensor, or of a raw int; None: NULL.
+bool address(PyObject *o, void **out) {
+    *out = nullptr;
+    if (o == Py_None) return true;
+    return pointer_of(PyLong_Check(o) ? Py_NewRef(o) : PyObject_CallMethodNoArgs(o, g_data_ptr), out);
+}
+
+// Handle of a stream: an int, or an object with `cuda_stream`; None: PyTorch's current stream of the current device.
+bool stream_handle(PyObject *o, void **out) {
+    if (o != Py_None) return pointer_of(PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttr(o, g_cuda_stream), out);
+    // the first lookup of the device puts others in the place of both
+    PyObject *lookup = Py_NewRef(g_device), *device = PyObject_CallNoArgs(lookup);
+    Py_DECREF(lookup);
+    if (!device) return false;
+    lookup = Py_NewRef(g_raw_stream);
+    PyObject *stream = PyObject_CallOneArg(lookup, device);
+    Py_DECREF(lookup);
+    Py_DECREF(device);
+    return pointer_of(stream, out);
+}
+
+template <typename T>
+struct Arg {                                          // whole numbers
+    T value;
+    bool read(PyObject *o, bool) {
+        value = (T)PyLong_AsUnsignedLongLongMask(o);
+        return !PyErr_Occurred();
+    }
+    T get() { return value; }
+};
+
+template <typename T>
+struct Arg<T *> {                                     // handles, buffers, the stream
+    void *value;
+    bool read(PyObject *o, bool is_stream) { return is_stream ? stream_handle(o, &value) : address(o, &value); }
+    T *get() { return static_cast<T *>(value); }
+};
+
+template <>
+struct Arg<const float *> {                           // what taps() returns
+    const float *value;
+    bool read(PyObject *o, bool) {
+        value = reinterpret_cast<const float *>(PyBytes_AsString(o));
+        return value != nullptr;
+    }
+    const float *get() { return value; }
+};
+
+struct Pointers {                                     // shards; None: no array.  Ones that are not there are NULL
+    void *few[64] = {};
+    std::vector<void *> many;
+    void **p = nullptr;
+    bool read(PyObject *o, bool) {
+        if (o == Py_None) return true;
+        PyObject *s = PySequence_Fast(o, "a sequence of shards is needed");
+        if (!s) return false;
+        const Py_ssize_t n = PySequence_Fast_GET_SIZE(s);
+        if (n > 64) many.resize((size_t)(n > DISTDL_MAX_WORKERS ? n : DISTDL_MAX_WORKERS));
+        p = n > 64 ? many.data() : few;
+        bool ok = true;
+        for (Py_ssize_t i = 0; ok && i < n && i < PySequence_Fast_GET_SIZE(s); ++i) {      // another thread may change a list meanwhile
+            PyObject *shard = Py_NewRef(PySequence_Fast_GET_ITEM(s, i));
+            ok = address(shard, p + i);
+            Py_DECREF(shard);
+        }
+        Py_DECREF(s);
+        return ok;
+    }
+};
+template <>
+struct Arg<void *const *> : Pointers {
+    void *const *get() { return p; }
+};
+template <>
+struct Arg<const void *const *> : Pointers {
+    const void *const *get() { return p; }
+};
+
+// The stream is every function's last argument.
+template <auto Function>
+struct Call;
+template <typename... A, distdl_status_t (*Function)(A...)>
+struct Call<Function> {
+    template <size_t... I>
+    static PyObject *run(PyObject *const *args, std::index_sequence<I...>) {
+        std::tuple<Arg<A>...> a;
+        if (!(std::get<I>(a).read(args[I], I + 1 == sizeof...(A)) && ...)) return nullptr;
+        distdl_status_t status;
+        Py_BEGIN_ALLOW_THREADS
+        status = Function(std::get<I>(a).get()...);
+        Py_END_ALLOW_THREADS
+        return PyLong_FromLong((long)status);
+    }
+    static PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n) {
+        if (n != (Py_ssize_t)sizeof...(A)) return PyErr_Format(PyExc_TypeError, "%zd arguments, %zd needed", n, (Py_ssize_t)sizeof...(A));
+        return run(args, std::index_sequence_for<A...>{});
+    }
+};
+
+// taps(w) -> (bytes of 3 x (2R+1) floats, R) of any nested sequence of numbers, or None if it has another shape
+PyObject *taps(PyObject *, PyObject *w) {
+    PyObject *rows = PySequence_Fast(w, "taps must have shape [3][2R+1]");
+    if (!rows) return nullptr;
+    std::vector<float> v;
+    Py_ssize_t width = -1;
+    bool shaped = PySequence_Fast_GET_SIZE(rows) == 3, failed = false;
+    for (Py_ssize_t r = 0; !failed && r < PySequence_Fast_GET_SIZE(rows); ++r) {
+        PyObject *row = PySequence_Fast(PySequence_Fast_GET_ITEM(rows, r), "taps must have shape [3][2R+1]");
+        failed = !row;
+        const Py_ssize_t n = row ? PySequence_Fast_GET_SIZE(row) : 0;
+        shaped = shaped && n % 2 == 1 && (width < 0 || n == width);
+        width = n;
+        for (Py_ssize_t k = 0; !failed && k < n; ++k) {
+            PyObject *f = PyNumber_Float(PySequence_Fast_GET_ITEM(row, k));
+            failed = !f;
+            if (f) v.push_back((float)PyFloat_AS_DOUBLE(f));
+            Py_XDECREF(f);
+        }
+        Py_XDECREF(row);
+    }
+    Py_DECREF(rows);
+    if (failed) return nullptr;
+    if (!shaped) Py_RETURN_NONE;
+    return Py_BuildValue("y#n", (const char *)v.data(), (Py_ssize_t)(v.size() * sizeof(float)), width / 2);
+}
+
+PyObject *set_stream_lookup(PyObject *, PyObject *const *args, Py_ssize_t n) {
+    if (n != 2) return PyErr_Format(PyExc_TypeError, "two functions are needed");
+    Py_XSETREF(g_device, Py_NewRef(args[0]));
+    Py_XSETREF(g_raw_stream, Py_NewRef(args[1]));
+    Py_RETURN_NONE;
+}
+
+#define FUNCTION(name) {#name, (PyCFunction)(void (*)(void))Call<distdl_##name>::entry, METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {
+    FUNCTION(broadcast_fwd), FUNCTION(broadcast_adj), FUNCTION(sumreduce_fwd), FUNCTION(sumreduce_adj), FUNCTION(allreduce),
+    FUNCTION(halo_fwd), FUNCTION(halo_adj), FUNCTION(repartition_fwd), FUNCTION(repartition_adj),
+    FUNCTION(conv_fwd), FUNCTION(conv_adj), FUNCTION(conv_adj_params), FUNCTION(convg_fwd), FUNCTION(convg_adj), FUNCTION(convg_adj_params),
+    FUNCTION(stencil3d_fwd), FUNCTION(stencil3d_adj), FUNCTION(pool_fwd), FUNCTION(pool_adj),
+    FUNCTION(affine_fwd), FUNCTION(affine_adj), FUNCTION(affine_adj_params),
+    {"taps", taps, METH_O, nullptr},
+    {"set_stream_lookup", (PyCFunction)(void (*)(void))set_stream_lookup, METH_FASTCALL, nullptr},
+    {nullptr, nullptr, 0, nullptr},
+};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__binding(void) {
+    g_data_ptr = PyUnicode_InternFromString("data_ptr");
+    g_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+    g_device = Py_NewRef(Py_None);
+    g_raw_stream = Py_NewRef(Py_None);
+    return PyModule_Create(&module);
+}

@@ -327,3 +327,24 @@ def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
     for kernel, body in sorted(bodies.items()):
         assert len(re.findall(r"^    stream_enter\(\);", body, re.M)) == 1, kernel
         assert body.count("stream_enter") == 1 and body.count("griddepcontrol") == 0, kernel
+
+
+def test_calls_check_their_arguments_before_the_library_sees_them():
+    """Shards missing from a list are NULL (an error), not whatever lies behind it; wrong types are exceptions."""
+    part = distdl.Partition((8, 8), (2, 2), (1, 1), (1, 1))
+    y, few = [256] * 4, [256, 512]
+    conv = distdl.Partition((1, 1, 8, 8), (1, 1, 2, 2), (0, 0, 1, 1), (0, 0, 1, 1))
+    w = np.zeros((1, 3, 3))
+    w_ptr = type("W", (), {"shape": w.shape, "data_ptr": lambda self: 1024})()
+    for shards in (few, tuple(few), [None] * 4, []):
+        with pytest.raises(distdl.DistdlError) as e:
+            distdl.conv_fwd(conv, shards, w_ptr, None, y, stream=0)
+        assert e.value.status == 1
+    with pytest.raises(AttributeError):
+        distdl.halo_fwd(part, ["shard"] * 4, stream=0)
+    with pytest.raises(TypeError):
+        distdl.pool_fwd(conv, y, (3.5, 3), (1, 1), ((1, 1), (1, 1)), distdl.POOL_MAX, y, stream=0)
+    with pytest.raises(ValueError):
+        distdl.stencil3d_fwd(part, y, [[1, 2, 3], [1, 2, 3], [1, 2]], y, stream=0)
+    raw, radius = distdl._taps(np.arange(9).reshape(3, 3))
+    assert radius == 1 and np.array_equal(np.frombuffer(raw, np.float32), np.arange(9, dtype=np.float32))
