@@ -727,7 +727,14 @@ static distdl_status_t dw_geometry(const distdl_partition *p, int32_t kh, int32_
 
 // Strips of 64 columns instead of 128 where they leave fewer lanes without a column (a narrow strip pays about a sixth more
 // per column for what is done once per row).
-static bool dw_narrow(int64_t max_bw) { return 2 * ((max_bw + 63) / 64) * 7 < 4 * ((max_bw + 127) / 128) * 6; }
+// Nor where wide strips, in segments of eight rows, leave a scheduler of the device with one warp at most: it goes at the pace of one warp's
+// instructions, and half the columns are half of them (forward, adjoint and gradients, 7 x 7, 1 x 10 x 375 x 111: 33.7 -> 26.1 us; 5 x 5, 1 x 3
+// x 33 x 169 on 1 x 2 workers 26.0 -> 22.0, 2 x 1 x 217 x 753 on 4 x 3 24.7 -> 22.1).
+constexpr int64_t kDwFewItems = 592;       // schedulers of a B200
+static bool dw_narrow(const DwParams &P, int64_t max_bh, int64_t max_bw) {
+    if (2 * ((max_bw + 63) / 64) * 7 < 4 * ((max_bw + 127) / 128) * 6) return true;
+    return ((max_bw + 127) / 128) * ((max_bh + 7) / 8) * P.ph * P.pw * P.planes <= kDwFewItems;
+}
 
 // Rows per segment: the smallest estimated time, turns of the resident warps times rows an item reads (its halo, whole
 // groups and about a dozen rows' worth of start-up included), and of equal ones the longest segments.  For a number of turns the most segments that
@@ -792,7 +799,7 @@ static distdl_status_t launch_conv_rows(DwParams &P, int64_t max_bh, int64_t max
 
 template <int K, bool ADJ>
 static distdl_status_t launch_conv(DwParams &P, int64_t max_bh, int64_t max_bw, cudaStream_t s, const char *what) {
-    if (dw_narrow(max_bw)) return launch_conv_rows<K, ADJ, 2, false>(P, max_bh, max_bw, s, what);
+    if (dw_narrow(P, max_bh, max_bw)) return launch_conv_rows<K, ADJ, 2, false>(P, max_bh, max_bw, s, what);
     return dw_aligned_rows(P, ADJ ? 0 : K / 2) ? launch_conv_rows<K, ADJ, 4, true>(P, max_bh, max_bw, s, what)
                                                : launch_conv_rows<K, ADJ, 4, false>(P, max_bh, max_bw, s, what);
 }
@@ -849,7 +856,7 @@ static distdl_status_t grad_plan(const distdl_partition *p, int32_t kh, int32_t 
     const distdl_status_t st = dw_geometry(p, kh, kw, what, P, &max_bh, &max_bw);
     if (st != DISTDL_OK) return st;
     const int64_t n = p->global_shape[0];
-    *kind = dw_narrow(max_bw) ? kDwNarrow : kh == 5 && dw_aligned_rows(*P, 0) ? kDwVector : kDwWide;
+    *kind = dw_narrow(*P, max_bh, max_bw) ? kDwNarrow : kh == 5 && dw_aligned_rows(*P, 0) ? kDwVector : kDwWide;
     if (*kind == kDwNarrow)
         return kh == 3 ? grad_plan_rows<3, 2, false>(P, max_bh, max_bw, n, what) : kh == 5 ? grad_plan_rows<5, 2, false>(P, max_bh, max_bw, n, what)
                                                                                            : grad_plan_rows<7, 2, false>(P, max_bh, max_bw, n, what);
@@ -937,7 +944,7 @@ extern "C" distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition
     const distdl_status_t st = dw_geometry(p, k, k, "selftest_conv_row_reads", &P, &max_bh, &max_bw);
     if (st != DISTDL_OK) return st;
     *floats_past_end = *rows_by_cell = 0;
-    const int strip = dw_narrow(max_bw) ? 64 : 128;
+    const int strip = dw_narrow(P, max_bh, max_bw) ? 64 : 128;
     const uintptr_t base = 256;                                 // never read: addresses only
     for (int32_t w = 0; w < p->num_workers; ++w) {
         const int bh = P.bh[w / P.pw], bw = P.bw[w % P.pw];

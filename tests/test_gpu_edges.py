@@ -93,6 +93,8 @@ CONV_EDGES = [
     ((1, 1, 30, 408), (1, 1, 1, 3), 7),      # the other way round (142 / 136)
     ((1, 1, 700, 70), (1, 1, 2, 1), 3),      # several row segments per shard
     ((5, 3, 19, 45), (1, 1, 3, 2), 5),       # shards of 7, 6, 6 rows and 23, 22 columns
+    ((37, 16, 8, 128), (1, 1, 1, 1), 5),     # strips of 64 columns: as many of 128 as the device has schedulers
+    ((37, 16, 9, 128), (1, 1, 1, 1), 5),     # strips of 128: twice as many segments
 ]
 
 
