@@ -10,7 +10,7 @@
 // the same star with every 1-D kernel reversed, evaluated in gather form on the bulk-shaped dy,
 // written into the bulk of the padded dx shards whose ghosts are cleared as H* leaves them.
 //
-// Blocking: a block (four warps) owns 8 rows x 128 columns of one shard and marches through a chunk
+// Blocking: a block (four warps) owns 16 rows x 64 columns (or 8 x 128) of one shard and marches through a chunk
 // of planes.  A thread owns 4 consecutive columns of two consecutive rows and keeps the running sums of the
 // 2R+1 outputs around the current plane in registers: a cell of plane p is tap 2R - i of output p - R + i, and the
 // sum moves from slot i + 1 to slot i as the destination of that very FMA (a queue of the 2R+1 input planes instead costs
@@ -22,10 +22,13 @@
 // 16-byte boundaries (R < 4 on the padded side) are copied four bytes a lane, a warp's cells next to one another.
 // Issue bounds it, not memory: 116 of ~300 instructions a plane are the warp's FMA (25 taps on eight cells, pairs
 // packed but for the odd column shifts), and a fourth block per multiprocessor makes it 301 us from 233.  At 512^3, R = 4,
-// forward 308 -> 233 us, adjoint 365 -> 264 us, where reading and writing the bulk once takes 164 us and 170 us.  The rest
+// forward 308 -> 233 us, adjoint 365 -> 264 us, where reading and writing the bulk once takes 164 us and 170 us (those with tiles of 8 x 128; 16 x 64
+// forward and adjoint 565 -> 540 us together, shards that 128 columns do not fit: 296 x 226 x 96 on 1 x 1 x 2 workers 102 -> 43, 201 x 238 x 44 on
+// 1 x 2 x 4 195 -> 103, 151 x 307 x 238 on 3 x 3 x 4, R = 2, 140 -> 85).  The rest
 // of the radii and sizes gain by the rule for the chunks as well (200^3, R = 2: 61 -> 32 and 78 -> 31 us; 64^3, R = 4: 40 -> 6.4 us).
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "common.h"
 #include "conv_common.h"
@@ -37,10 +40,11 @@ constexpr int kStMaxPerDim = 8;
 constexpr int kStMaxR = 4;
 constexpr int kStRpt = 2;             // consecutive rows per thread
 constexpr int kStThreads = 128;
-constexpr int kStRows = kStRpt * (kStThreads / 32);   // rows of a tile: 8
-constexpr int kStCols = 128;          // columns of a tile = 32 lanes x 4
+// Tile of LANES threads a row: 16 rows x 64 columns or 8 x 128
+__host__ __device__ constexpr int st_rows(int lanes) { return kStRpt * (kStThreads / lanes); }
+__host__ __device__ constexpr int st_cols(int lanes) { return 4 * lanes; }
 constexpr int kStLead = 4;            // shared-memory column of the tile's first column (keeps rows 16-byte aligned)
-constexpr int kStPitch = kStLead + kStCols + 4;   // 136 floats
+__host__ __device__ constexpr int st_pitch(int lanes) { return kStLead + st_cols(lanes) + 4; }
 constexpr int kStDepth = 5;           // planes in the ring (4 and 6 measure the same within 2 %)
 // Blocks per multiprocessor.  With 16-byte copies a fourth block of the wide stars costs more in registers (128 instead of 168: moves and
 // spills) than it hides; scalar copies have latency left for it (22 x 126 x 103 shards, R = 4, 576 blocks: 56 -> 48 and 74 -> 58 us; a
@@ -93,8 +97,8 @@ __device__ __forceinline__ void st_copy4(uint32_t dst, const float *src, uint32_
                  ::"r"(dst), "l"(src), "r"(bytes), "r"((uint32_t)on) : "memory");
 }
 
-template <int R>
-constexpr int st_smem_bytes() { return kStDepth * (kStRows + 2 * R) * kStPitch * 4; }
+template <int R, int LANES>
+constexpr int st_smem_bytes() { return kStDepth * (st_rows(LANES) + 2 * R) * st_pitch(LANES) * 4; }
 
 // Ghost shell of an output shard but for the row ends, which the threads that write the rows clear: the ghost planes below and
 // above, and the ghost rows of each bulk plane, which lie next to those of the plane before it in memory.  All of them are
@@ -114,16 +118,20 @@ __device__ __forceinline__ void st_clear(float *out, int bz, int opy, int opx, i
     zero((bz + oo) * plane + lo, (bz + oo) * plane + hi);
 }
 
-template <int R, bool VEC>
+template <int R, bool VEC, int LANES>
 __global__ void __launch_bounds__(kStThreads, kStBlocks<R, VEC>)
 stencil3d_kernel(const __grid_constant__ StencilParams P) {
     stream_enter();
+    constexpr int kStRows = st_rows(LANES), kStCols = st_cols(LANES), kStPitch = st_pitch(LANES);
     extern __shared__ __align__(16) float ring[];          // planes of kStRows + 2 R rows
     constexpr int kPlane = (kStRows + 2 * R) * kStPitch;
     constexpr int N = 2 * R + 1;
-    constexpr int kWarps = kStThreads / 32;
-    constexpr int HR = (2 * R + kWarps - 1) / kWarps;     // extra rows a warp fetches per plane
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // Copies: 16 bytes a thread, the LANES threads of a row together, or (4 bytes a thread) 32 columns of a row at a time, a warp together
+    constexpr int CL = VEC ? LANES : 32, CE = VEC ? 1 : kStCols / 32;      // threads that copy a row, copies of each
+    constexpr int CG = kStThreads / CL, CR = kStRows / CG;                // groups of such threads, rows of a tile that each copies
+    constexpr int HR = (2 * R + CG - 1) / CG;                              // extra rows that each copies per plane
+    const int group = threadIdx.x / LANES, lane = threadIdx.x % LANES;
+    const int cgroup = threadIdx.x / CL, clane = threadIdx.x % CL;
     // block -> (shard, plane chunk, row tile, column tile), column tile fastest
     int rest = blockIdx.x;
     const int tx = rest % P.tiles_x;
@@ -143,7 +151,7 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
     const int io = P.in_off;
     const int ipx = bx + 2 * io;                       // input row pitch of every shard in this worker column
 
-    const int rw = kStRpt * warp;                      // first of this warp's rows inside the tile
+    const int rw = kStRpt * group;                     // first of this thread's rows inside the tile
     const int x = x0 + 4 * lane;
     const bool col_ok = x < bx;
     bool row_ok[kStRpt];
@@ -154,22 +162,26 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
     // plane, the step (the plane stride of the owning shard, in elements: a shard holds fewer than 2^31 of them) and the bytes
     // to read (0: zeros, and the pointer stands still)
     // the columns that this thread copies of a row: its own four, or where rows are not aligned every 32nd
-    const int xc = VEC ? x : x0 + lane;
-    bool col_in[4];
+    const int xc = VEC ? x : x0 + clane, rc = CR == kStRpt ? rw : CR * cgroup;        // and the first of the rows
+    // which of them lie inside the shard: flags where the store's can serve for the rows, counts otherwise (registers)
+    const int cols_in = bx - xc, rows_in = by - y0 - rc;
+    bool col_flag[CE];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) col_in[e] = VEC ? col_ok : xc + 32 * e < bx;
+    for (int e = 0; e < CE; ++e) col_flag[e] = VEC ? col_ok : xc + 32 * e < bx;
+    auto row_in = [&](int r) { return CR == kStRpt ? row_ok[r < kStRpt ? r : 0] : r < rows_in; };
+    auto col_in = [&](int e) { return CR == kStRpt ? col_flag[e] : 32 * e < cols_in; };
     auto copy4 = [&](uint32_t dst, const float *src, uint32_t bytes, bool on) {
         if (VEC) {
             st_copy16(dst, src, bytes, on && col_ok);
         } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) st_copy4(dst + 128 * e, src + 32 * e, bytes, on && col_in[e]);
+            for (int e = 0; e < CE; ++e) st_copy4(dst + 128 * e, src + 32 * e, bytes, on && col_in(e));
         }
     };
     constexpr uint32_t kBytes = VEC ? 16 : 4;
-    const uint32_t copy_dst = (uint32_t)((kStLead + (VEC ? 4 : 1) * lane) * 4);
+    const uint32_t copy_dst = (uint32_t)((kStLead + (VEC ? 4 : 1) * clane) * 4);
     const uint32_t ipy = (uint32_t)(by + 2 * io);
-    const uint32_t own_off = (uint32_t)(y0 + rw + io) * (uint32_t)ipx + (uint32_t)(xc + io);   // row 0 of the thread
+    const uint32_t own_off = (uint32_t)(y0 + rc + io) * (uint32_t)ipx + (uint32_t)(xc + io);   // first row it copies
     const uint32_t own_stride = ipy * (uint32_t)ipx;                   // the same in the shards below and above
     const float *own_p = P.in[shard];
     uint32_t own_bytes = 0;
@@ -185,22 +197,22 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
             n = sz + 1 < P.pz ? P.bz[sz + 1] : 0;
             zp -= bz;
         }
-        own_bytes = s3 >= 0 && col_in[0] && (unsigned)zp < (unsigned)n ? kBytes : 0u;
+        own_bytes = s3 >= 0 && col_in(0) && (unsigned)zp < (unsigned)n ? kBytes : 0u;
         own_p = own_bytes ? P.in[s3] + ((uint32_t)(zp + io) * own_stride + own_off) : P.in[shard];
     };
-    // extra rows of the current plane: row h of the 2R (R above the tile, R below) goes to warp h % kWarps
+    // extra rows of the current plane: row h of the 2R (R above the tile, R below) goes to group h % CG
     const float *hrow_p[HR];
     uint32_t hrow_step[HR], hrow_bytes[HR], hrow_dst[HR];
 #pragma unroll
     for (int i = 0; i < HR; ++i) {
-        const int h = warp + kWarps * i;
+        const int h = cgroup + CG * i;
         hrow_p[i] = P.in[shard];
         hrow_step[i] = hrow_bytes[i] = 0;
         // its row in the shared-memory plane: the rows below follow the tile's last one
         hrow_dst[i] = (uint32_t)(((h < R ? h : th + h) * kStPitch) * 4) + copy_dst;
         const int hy = h < R ? y0 - R + h : y0 + th + (h - R);
         int so, yo;
-        if (h < 2 * R && col_in[0] && st_owner(P.by, P.py, sy, hy, so, yo)) {
+        if (h < 2 * R && col_in(0) && st_owner(P.by, P.py, sy, hy, so, yo)) {
             hrow_bytes[i] = kBytes;
             hrow_step[i] = (uint32_t)(P.by[so] + 2 * io) * (uint32_t)ipx;
             hrow_p[i] = P.in[(sz * P.py + so) * P.px + sx] + (uint32_t)(z0 + io) * hrow_step[i] +
@@ -224,19 +236,19 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
         }
     }
     const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-    const uint32_t own_dst = ring_s + (uint32_t)((R + rw) * kStPitch * 4) + copy_dst;
+    const uint32_t own_dst = ring_s + (uint32_t)((R + rc) * kStPitch * 4) + copy_dst;
     own_at(z0 - R);
     // plane zp into the slot `at` bytes into the ring: own cells, and if it is to be the current one a vector of each extra row and
     // one extra-column cell; cells beyond the bulk are written by the extra-row / extra-column threads only
     auto issue = [&](int zp, uint32_t at) {
 #pragma unroll
-        for (int r = 0; r < kStRpt; ++r) copy4(own_dst + at + (uint32_t)(r * kStPitch * 4), own_p + r * ipx, own_bytes, row_ok[r]);
+        for (int r = 0; r < CR; ++r) copy4(own_dst + at + (uint32_t)(r * kStPitch * 4), own_p + r * ipx, own_bytes, row_in(r));
         if (zp + 1 == 0 || zp + 1 == bz) own_at(zp + 1);
         else own_p += own_bytes ? own_stride : 0u;
         if (zp >= z0 && zp < z1) {
 #pragma unroll
             for (int i = 0; i < HR; ++i) {
-                copy4(ring_s + at + hrow_dst[i], hrow_p[i], hrow_bytes[i], (2 * R) % kWarps == 0 || warp + kWarps * i < 2 * R);
+                copy4(ring_s + at + hrow_dst[i], hrow_p[i], hrow_bytes[i], (2 * R) % CG == 0 || cgroup + CG * i < 2 * R);
                 hrow_p[i] += hrow_step[i];
             }
             st_copy4(ring_s + at + hcol_dst, hcol_p, hcol_bytes, hc_active);
@@ -379,9 +391,9 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
     }
 }
 
-template <int R>
+template <int R, int LANES>
 static distdl_status_t launch_stencil(const StencilParams &P, unsigned grid, bool vec, cudaStream_t s) {
-    constexpr int smem = st_smem_bytes<R>();
+    constexpr int smem = st_smem_bytes<R, LANES>();
     static bool configured_on[kMaxDevicesPerProcess] = {false};
     int dev = 0;
     DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
@@ -390,13 +402,13 @@ static distdl_status_t launch_stencil(const StencilParams &P, unsigned grid, boo
     {
         std::lock_guard<std::mutex> setup_lock(setup_mutex());
         if (!configured_on[dev]) {
-            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, true, LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+            DISTDL_CUDA_CHECK(cudaFuncSetAttribute(stencil3d_kernel<R, false, LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
             configured_on[dev] = true;
         }
     }
-    if (vec) launch_in_stream(stencil3d_kernel<R, true>, grid, kStThreads, smem, s, P);
-    else launch_in_stream(stencil3d_kernel<R, false>, grid, kStThreads, smem, s, P);
+    if (vec) launch_in_stream(stencil3d_kernel<R, true, LANES>, grid, kStThreads, smem, s, P);
+    else launch_in_stream(stencil3d_kernel<R, false, LANES>, grid, kStThreads, smem, s, P);
     DISTDL_CUDA_CHECK(cudaGetLastError());
     return DISTDL_OK;
 }
@@ -446,8 +458,17 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
     P.in_off = adj ? 0 : radius;
     P.out_off = adj ? radius : 0;
     P.clear_ghosts = adj ? 1 : 0;
-    P.tiles_x = (int32_t)((mx + kStCols - 1) / kStCols);
-    P.tiles_y = (int32_t)((my + kStRows - 1) / kStRows);
+    // 16-byte accesses: every row of the layout starts on a 16-byte boundary and holds whole vectors
+    bool whole = true;
+    for (int32_t c = 0; c < p->pshape[2]; ++c) whole = whole && (P.bx[c] % 4) == 0;
+    const bool vec = whole && P.in_off % 4 == 0;
+    P.vec_out = whole && P.out_off % 4 == 0;
+    // 16 rows x 64 columns where that makes fewer tiles, or as many with 16-byte copies: fewer rows and vectors around a tile (512^3, R = 4, pair 565 ->
+    // 540 us); with 4-byte copies and as many tiles the longer rows win (66 x 305 x 202 on 3 x 4 x 1 workers, R = 1: 33.3 against 31.9 us).
+    const auto tiles = [&](int lanes) { return ((mx + st_cols(lanes) - 1) / st_cols(lanes)) * ((my + st_rows(lanes) - 1) / st_rows(lanes)); };
+    const int lanes = tiles(16) < tiles(32) || (tiles(16) == tiles(32) && vec) ? 16 : 32;
+    P.tiles_x = (int32_t)((mx + st_cols(lanes) - 1) / st_cols(lanes));
+    P.tiles_y = (int32_t)((my + st_rows(lanes) - 1) / st_rows(lanes));
     for (int d = 0; d < 3; ++d)
         for (int k = 0; k <= 2 * radius; ++k) P.w[d][k] = adj ? w[d * (2 * radius + 1) + (2 * radius - k)] : w[d * (2 * radius + 1) + k];
     P.w[0][radius] = (float)((double)P.w[0][radius] + (double)P.w[1][radius] + (double)P.w[2][radius]);
@@ -457,11 +478,6 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
             memcpy(&bits, &P.w[d][k], 4);
             P.w2[d][k] = (uint64_t)bits << 32 | bits;
         }
-    // 16-byte accesses: every row of the layout starts on a 16-byte boundary and holds whole vectors
-    bool whole = true;
-    for (int32_t c = 0; c < p->pshape[2]; ++c) whole = whole && (P.bx[c] % 4) == 0;
-    const bool vec = whole && P.in_off % 4 == 0;
-    P.vec_out = whole && P.out_off % 4 == 0;
     for (int32_t wk = 0; wk < p->num_workers; ++wk) {
         if (!in[wk] || !out[wk]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shard pointer %d is NULL", what, wk);
         if (!aligned16(in[wk]) || !aligned16(out[wk])) return fail(DISTDL_ERR_ALIGNMENT, "%s: shard %d is not 16-byte aligned", what, wk);
@@ -477,11 +493,15 @@ static distdl_status_t stencil_impl(const distdl_partition *p, const void *const
     const int64_t blocks = (int64_t)p->num_workers * P.chunks_z * P.tiles_y * P.tiles_x;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     cudaStream_t s = (cudaStream_t)stream;
+    const auto run = [&](auto r) {
+        constexpr int R = decltype(r)::value;
+        return lanes == 16 ? launch_stencil<R, 16>(P, (unsigned)blocks, vec, s) : launch_stencil<R, 32>(P, (unsigned)blocks, vec, s);
+    };
     switch (radius) {
-        case 1: return launch_stencil<1>(P, (unsigned)blocks, vec, s);
-        case 2: return launch_stencil<2>(P, (unsigned)blocks, vec, s);
-        case 3: return launch_stencil<3>(P, (unsigned)blocks, vec, s);
-        default: return launch_stencil<4>(P, (unsigned)blocks, vec, s);
+        case 1: return run(std::integral_constant<int, 1>{});
+        case 2: return run(std::integral_constant<int, 2>{});
+        case 3: return run(std::integral_constant<int, 3>{});
+        default: return run(std::integral_constant<int, 4>{});
     }
 }
 

@@ -285,6 +285,11 @@ STENCIL_EDGES = [
     ((301, 8, 12), (1, 1, 1), 3),            # many chunks of planes, the last one short
     ((10, 17, 258), (2, 2, 2), 4),           # rows 9 and 8, columns 129: shards with different numbers of tiles share the clearing
     ((13, 9, 260), (3, 1, 2), 4),            # planes 5, 4, 4: neighbours exactly as deep as the radius
+    ((7, 17, 64), (1, 1, 1), 4),             # tiles of 16 rows x 64 columns, the second of one row
+    ((9, 33, 61), (1, 2, 1), 3),             # the same with 4-byte copies, rows 17 and 16
+    ((8, 16, 193), (1, 1, 1), 1),            # one column in the last of four tiles
+    ((6, 8, 128), (1, 1, 1), 4),             # one tile of 8 rows x 128 columns, two of the others
+    ((6, 24, 65), (1, 1, 1), 2),             # 4-byte copies, fewer tiles of 8 x 128
 ]
 
 
