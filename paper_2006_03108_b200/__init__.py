@@ -95,6 +95,7 @@ def lib():
     L.distdl_selftest_wait_timeout.argtypes = [c_i64, vp]
     L.distdl_selftest_row_plan.argtypes = [vp, c_i32, pi32, c_i32, pi32, c_i32, pi32]
     L.distdl_selftest_conv_row_reads.argtypes = [vp, c_i32, c_i32, pi64, pi64]
+    L.distdl_selftest_pool_adj_terms.argtypes = [vp] + [c_i32] * 7 + [pi32, pi32, c_i32]
     _lib = L
     return L
 
@@ -507,3 +508,13 @@ def selftest_conv_row_reads(part, k, gradients=False):
     past, cells = ctypes.c_int64(0), ctypes.c_int64(0)
     _check(lib().distdl_selftest_conv_row_reads(part.handle, int(k), 1 if gradients else 0, ctypes.byref(past), ctypes.byref(cells)))
     return past.value, cells.value
+
+
+def selftest_pool_adj_terms(part, kernel, stride, pad, mode, worker, dim):
+    """For every row (dim 0) or column (dim 1) of a worker's bulk the outputs that the pooling adjoint with H* in it adds to it, one per row or
+    column of the window, -1: none (include/distdl_selftest.h); None if the layer runs as two kernels."""
+    cells = part.shard_extents(worker)[1][2 + dim]
+    terms, fused = (ctypes.c_int32 * (kernel * cells))(), ctypes.c_int32(0)
+    _check(lib().distdl_selftest_pool_adj_terms(part.handle, kernel, stride, pad[0], pad[1], mode, worker, dim, ctypes.byref(fused), terms,
+                                                kernel * cells))
+    return [list(terms[kernel * q:kernel * q + kernel]) for q in range(cells)] if fused.value else None

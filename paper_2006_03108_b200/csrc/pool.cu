@@ -38,6 +38,8 @@ struct PoolParams {
     int32_t wrows, wcols;  // rows and columns of workers
 };
 
+__host__ __device__ __forceinline__ int div_floor(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
+
 // One thread per output.  blockIdx.y = worker, blockIdx.x = (plane, row tile, column tile).
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_fwd_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) {
@@ -79,8 +81,6 @@ pool_fwd_kernel(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y) 
         if (S.arg) S.arg[o] = where < 0 ? 0 : where;
     }
 }
-
-__device__ __forceinline__ int div_floor(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 // One thread per cell of the padded dx.  A cell (p, q) lies in the window of output (i, j) iff
 // 0 <= p - i0 - i*sh < kh and likewise for the columns.
@@ -328,6 +328,54 @@ __device__ __forceinline__ void pool_store_row(float *out, const float (&v)[NU][
             if (SW * (lane + 32 * u) + c < cols) out[SW * (lane + 32 * u) + c] = v[u][c];
 }
 
+// Which columns of outputs the cells of a strip of the adjoint with H* in it meet: what the kernel computes with and what
+// distdl_selftest_pool_adj_terms() replays.  A lane holds groups lane + 32 u of SW cells; the outputs that one meets are newest + 32 u - v.
+template <int KW, int SW, int DW, int NU>
+struct PoolStrip {
+    static constexpr int EW = DW > 0 ? 1 : 0, NJ = (KW - 1 - DW) / SW + EW + 1;
+    int newest;            // newest output column of the lane's first group
+    int cols;              // cells of the strip
+    bool left, right;      // the last column of the outputs on the left is met, the first column of those on the right
+    __host__ __device__ __forceinline__ PoolStrip(const PoolShard &S, int wc, int wcols, int col0, int lane) {
+        newest = col0 + lane + div_floor(S.hlw - S.j0, SW) + EW;
+        cols = min(S.bw - col0 * SW, 32 * NU * SW);
+        left = wc > 0 && col0 == 0 && newest - lane - (NJ - 1) < 0;
+        right = wc + 1 < wcols && col0 * SW + cols == S.bw;
+    }
+    // window column under which output v of a group holds the group's cell c (outside 0 .. KW - 1: it does not)
+    static constexpr __host__ __device__ __forceinline__ int window(int c, int v) { return c + DW + (v - EW) * SW; }
+    // (x, at) in the place of the output on the left (right) of the shard's own.  The one on the left can be the newest of the first group
+    // where windows do not overlap: a shard that begins with a whole window of its neighbour's.
+    template <typename T>
+    static __host__ __device__ __forceinline__ void put_left(T (&g)[NU][NJ], int (&code)[NU][NJ], T x, int at, int newest) {
+#pragma unroll
+        for (int v = KW > SW ? 1 : 0; v < NJ; ++v)
+            if (newest - v == -1) {
+                g[0][v] = x;
+                code[0][v] = at;
+            }
+    }
+    template <typename T>
+    static __host__ __device__ __forceinline__ void put_right(T (&g)[NU][NJ], int (&code)[NU][NJ], T x, int at, int newest, int ow) {
+#pragma unroll
+        for (int u = 0; u < NU; ++u)
+#pragma unroll
+            for (int v = 0; v < NJ; ++v)
+                if (newest + 32 * u - v == ow) {
+                    g[u][v] = x;
+                    code[u][v] = at;
+                }
+    }
+};
+// Row i of the outputs, counted from the own of worker w (shard S, in worker row wr): row il of the worker dr rows of workers below; false if there is none.
+__host__ __device__ __forceinline__ bool pool_row_owner(const PoolParams &P, const PoolShard &S, int w, int wr, int i, int &dr, int &il) {
+    dr = i < 0 ? -1 : i >= S.oh ? 1 : 0;
+    if ((unsigned)(wr + dr) >= (unsigned)P.wrows) return false;
+    const int oh = P.s[w + dr * P.wcols].oh;
+    il = dr < 0 ? i + oh : dr ? i - S.oh : i;
+    return (unsigned)il < (unsigned)oh;
+}
+
 // Adjoint with H* in it: every bulk cell sums over all outputs whose window holds it, the neighbours' among them, in ascending order, and
 // the ghosts are cleared.  A lane owns groups of SH x SW bulk cells and marches down the rows of outputs; an output row is added to the KH
 // rows of cells that its windows hold, whose sums move up by SH rows as the first of them are done.  The first column of a group is
@@ -341,29 +389,22 @@ __device__ __forceinline__ void pool_store_row(float *out, const float (&v)[NU][
 // multiprocessor: with the fetch behind the sums 359 us, with three blocks 405, with five 375.
 template <int KH, int KW, int SH, int SW, int MODE, int DW, int NU>
 __device__ __forceinline__ void pool_adj_strip(const PoolParams &P, int w, int plane, int first_row, int rows, int col0, int lane) {
-    constexpr int EW = DW > 0 ? 1 : 0, NI = (KH + SH - 1) / SH, NJ = (KW - 1 - DW) / SW + EW + 1;
+    using Strip = PoolStrip<KW, SW, DW, NU>;
+    constexpr int NI = (KH + SH - 1) / SH, NJ = Strip::NJ;
     const PoolShard &S = P.s[w];
     const int wr = w / P.wcols, wc = w - wr * P.wcols;
     const int gi0 = div_floor(S.hlh - S.i0, SH) + first_row, bulk_end = S.hlh + S.bh;
     if (S.i0 + gi0 * SH >= bulk_end || col0 * SW >= S.bw) return;
     const int i_begin = gi0 - (NI - 1), i_end = min(gi0 + rows, div_floor(bulk_end - 1 - S.i0, SH) + 1);   // output rows
-    const int j0 = col0 + lane + div_floor(S.hlw - S.j0, SW) + EW;                     // newest output column of the lane's first group
-    const int cols = min(S.bw - col0 * SW, 32 * NU * SW);                       // cells of this strip
-    // row i of the outputs of this worker column (of the worker column beside: dc): worker and row there, false if there is none
-    auto owner = [&](int i, int &dr, int &il) {
-        dr = i < 0 ? -1 : i >= S.oh ? 1 : 0;
-        if ((unsigned)(wr + dr) >= (unsigned)P.wrows) return false;
-        const int oh = P.s[w + dr * P.wcols].oh;
-        il = dr < 0 ? i + oh : dr ? i - S.oh : i;
-        return (unsigned)il < (unsigned)oh;
-    };
+    const Strip strip(S, wc, P.wcols, col0, lane);
+    const int j0 = strip.newest, cols = strip.cols;
     // outputs -1 and ow of row i_begin + lane
-    const bool has_left = wc > 0 && col0 == 0 && j0 - lane - (NJ - 1) < 0, has_right = wc + 1 < P.wcols && col0 * SW + cols == S.bw;
+    const bool has_left = strip.left, has_right = strip.right;
     float sg[2] = {0.f, 0.f};
     int sc[2] = {-1, -1};
     if (has_left || has_right) {
         int dr, il;
-        if (i_begin + lane < i_end && owner(i_begin + lane, dr, il)) {
+        if (i_begin + lane < i_end && pool_row_owner(P, S, w, wr, i_begin + lane, dr, il)) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 if (!(k ? has_right : has_left)) continue;
@@ -392,7 +433,7 @@ __device__ __forceinline__ void pool_adj_strip(const PoolParams &P, int w, int p
     auto load = [&]() {
         if (at == seek_at) {
             int dr, il = 0;
-            row_ok = owner(at, dr, il);
+            row_ok = pool_row_owner(P, S, w, wr, at, dr, il);
             const PoolShard &N = P.s[row_ok ? w + dr * P.wcols : w];
             // above: down to row 0 (from a row above the shard above, which no window of this one's cells needs: to that shard)
             seek_at = dr < 0 ? (!row_ok && il < 0 ? at - il : 0) : dr == 0 ? S.oh : row_ok ? S.oh + N.oh : INT_MAX;
@@ -452,24 +493,12 @@ __device__ __forceinline__ void pool_adj_strip(const PoolParams &P, int w, int p
         if (has_left) {
             const float x = __shfl_sync(0xffffffffu, sg[0], i - i_begin);
             const int c = MODE == DISTDL_POOL_MAX ? __shfl_sync(0xffffffffu, sc[0], i - i_begin) : 0;
-#pragma unroll
-            for (int v = 1; v < NJ; ++v)
-                if (j0 - v == -1) {
-                    g[0][v] = x;
-                    code[0][v] = c;
-                }
+            Strip::put_left(g, code, x, c, j0);
         }
         if (has_right) {
             const float x = __shfl_sync(0xffffffffu, sg[1], i - i_begin);
             const int c = MODE == DISTDL_POOL_MAX ? __shfl_sync(0xffffffffu, sc[1], i - i_begin) : 0;
-#pragma unroll
-            for (int u = 0; u < NU; ++u)
-#pragma unroll
-                for (int v = 0; v < NJ; ++v)
-                    if (j0 + 32 * u - v == S.ow) {
-                        g[u][v] = x;
-                        code[u][v] = c;
-                    }
+            Strip::put_right(g, code, x, c, j0, S.ow);
         }
 #pragma unroll
         for (int a = 0; a < KH; ++a)
@@ -479,7 +508,7 @@ __device__ __forceinline__ void pool_adj_strip(const PoolParams &P, int w, int p
                 for (int c = 0; c < SW; ++c)
 #pragma unroll
                     for (int v = NJ - 1; v >= 0; --v) {
-                        const int b = c + DW + (v - EW) * SW;
+                        const int b = Strip::window(c, v);
                         if (b < 0 || b >= KW) continue;                                // compile-time
                         if (MODE == DISTDL_POOL_AVG || code[u][v] == a * KW + b) acc[a][u][c] = __fadd_rn(acc[a][u][c], g[u][v]);
                     }
@@ -640,8 +669,6 @@ static void launch_pool_fixed(const PoolParams &P, dim3 grid, dim3 block, int ti
     else avg ? run(pool_adj_fixed<KH, KW, SH, SW, AVG>) : run(pool_adj_fixed<KH, KW, SH, SW, MAX>);
 }
 
-static int pool_floor(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-
 struct PoolDim {
     std::vector<int64_t> out_start, out_size;
     std::vector<int32_t> hlo, hhi;
@@ -667,11 +694,17 @@ static distdl_status_t pool_dim(int64_t n, int32_t p, int32_t k, int32_t s, int3
     return DISTDL_OK;
 }
 
-static distdl_status_t pool_impl(const distdl_partition *p, const void *const *in, void *const *out, void *const *arg,
-                                 int32_t kh, int32_t kw, int32_t sh, int32_t sw, int32_t plh, int32_t phh, int32_t plw,
-                                 int32_t phw, int32_t mode, void *stream, bool adjoint, const char *what) {
-    clear_error();
-    if (!p || !in || !out) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
+// A layer's geometry and kernel; the shards' addresses are filled in by the call.
+struct PoolPlan {
+    PoolParams P;
+    int fixed;                       // which of the compile-time variants, 0: the general kernels
+    bool fused;                      // adjoint with H* in it
+    int nu;                          // columns (fused: of groups) per lane
+    int64_t max_rows, max_cols;      // of the items that threads (general), lanes (fixed) and groups (adjoint, fixed) walk
+};
+
+static distdl_status_t pool_plan(const distdl_partition *p, int32_t kh, int32_t kw, int32_t sh, int32_t sw, int32_t plh, int32_t phh,
+                                 int32_t plw, int32_t phw, int32_t mode, bool adjoint, const char *what, PoolPlan &plan) {
     if (p->rank != 4 || p->dtype != DISTDL_F32) return fail(DISTDL_ERR_SHAPE, "%s: needs a rank-4 F32 partition", what);
     if (p->any_periodic()) return fail(DISTDL_ERR_UNSUPPORTED, "%s: periodic partitions are not supported by the fused layers", what);
     if (p->pshape[0] != 1 || p->pshape[1] != 1)
@@ -681,7 +714,6 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
     if (kh < 1 || kw < 1 || sh < 1 || sw < 1 || plh < 0 || phh < 0 || plw < 0 || phw < 0)
         return fail(DISTDL_ERR_INVALID_ARG, "%s: bad kernel, stride or padding", what);
     if (kh > 16 || kw > 16) return fail(DISTDL_ERR_UNSUPPORTED, "%s: kernels beyond 16 x 16", what);
-    if (mode == DISTDL_POOL_MAX && adjoint && !arg) return fail(DISTDL_ERR_INVALID_ARG, "%s: max pooling needs argmax", what);
     PoolDim dh, dw;
     distdl_status_t st = pool_dim(p->global_shape[2], p->pshape[2], kh, sh, plh, phh, dh, what);
     if (st != DISTDL_OK) return st;
@@ -698,7 +730,7 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
     for (int k = 0; k < 2; ++k)
         if (p->hlo[k][0] != 0 || p->hhi[k][0] != 0) return fail(DISTDL_ERR_SHAPE, "%s: ghosts along batch or channels", what);
 
-    PoolParams P;
+    PoolParams &P = plan.P;
     memset(&P, 0, sizeof(P));
     P.planes = (int32_t)(p->global_shape[0] * p->global_shape[1]);
     P.kh = kh;
@@ -710,20 +742,19 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
     P.mode = mode;
     P.wrows = p->pshape[2];
     P.wcols = p->pshape[3];
-    int64_t max_rows = 0, max_cols = 0;
+    int64_t &max_rows = plan.max_rows, &max_cols = plan.max_cols;
+    max_rows = max_cols = 0;
+    // the compile-time variants
+    const int fixed = plan.fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
+                                 : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
     // The adjoint with H* in it: where there is an H* (a ghost anywhere).  Max pooling on windows that do not overlap has one term a cell and
     // half the registers without it, and is faster so once the launch no longer counts (2 x 2 / 2, pairs: 12 x 7 x 333 x 129 on 3 x 2 workers
     // 22.2 -> 18.7 us; 8 x 16 x 514 x 514 on 4 x 4 101 -> 109; average pooling 93 -> 93 there, 16 x 16 x 1000 x 1000 on 3 x 3 615 -> 532).
-    bool fused = adjoint && p->adj_dev.num_tiles > 0 &&
+    bool fused = fixed && adjoint && !p->adj_host.tiles.empty() &&
                  (mode == DISTDL_POOL_AVG || sh < kh || sw < kw || (int64_t)P.planes * P.hg * P.wg < ((int64_t)8 << 20));
     for (int32_t w = 0; w < p->num_workers; ++w) {
         const int32_t r = w / p->pshape[3], c = w % p->pshape[3];
-        if (!in[w] || !out[w]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shard pointer %d is NULL", what, w);
         PoolShard &S = P.s[w];
-        S.in = (const float *)in[w];
-        S.out = (float *)out[w];
-        S.arg = arg ? (int32_t *)arg[w] : nullptr;
-        if (mode == DISTDL_POOL_MAX && adjoint && !S.arg) return fail(DISTDL_ERR_INVALID_ARG, "%s: argmax[%d] is NULL", what, w);
         S.ph = (int32_t)p->padded_extent(2, r);
         S.pw = (int32_t)p->padded_extent(3, c);
         S.oh = (int32_t)dh.out_size[r];
@@ -744,17 +775,8 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         max_cols = std::max<int64_t>(max_cols, adjoint ? S.pw : S.ow);
         // it hands one column of the neighbours' outputs on either side from lane to lane, and a lane clears one ghost cell a row
         fused = fused && S.oh >= 1 && S.ow >= kw && S.hlw <= 16 && S.pw - S.hlw - S.bw <= 16 &&
-                (c == 0 || pool_floor(S.hlw - S.j0 - kw + sw, sw) >= -1) && (c + 1 == p->pshape[3] || pool_floor(S.hlw + S.bw - 1 - S.j0, sw) <= S.ow);
+                (c == 0 || div_floor(S.hlw - S.j0 - kw + sw, sw) >= -1) && (c + 1 == p->pshape[3] || div_floor(S.hlw + S.bw - 1 - S.j0, sw) <= S.ow);
     }
-    // H and H* work on the padded shards: what they ask of them holds for the layer as well
-    st = halo_check_shards(p, adjoint ? out : const_cast<void *const *>(reinterpret_cast<const void *const *>(in)), what);
-    if (st != DISTDL_OK) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    // the compile-time variants: 64 (or 32) columns and up to 16 rows (20 of the fused adjoint) per warp, fewer where eight warps would leave some without a row
-    // or an SM would have fewer than 16 warps
-    const int fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
-                    : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
-    fused = fused && fixed;
     if (fixed && adjoint && !fused) {
         // groups of sh x sw cells; the group lattice starts up to one group before cell 0
         max_rows = max_rows / sh + 2;
@@ -764,11 +786,73 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
         max_rows = max_cols = 0;
         for (int32_t w = 0; w < p->num_workers; ++w) {
             const PoolShard &S = P.s[w];
-            max_rows = std::max<int64_t>(max_rows, pool_floor(S.hlh + S.bh - 1 - S.i0, sh) - pool_floor(S.hlh - S.i0, sh) + 1);
+            max_rows = std::max<int64_t>(max_rows, div_floor(S.hlh + S.bh - 1 - S.i0, sh) - div_floor(S.hlh - S.i0, sh) + 1);
             max_cols = std::max<int64_t>(max_cols, (S.bw + sw - 1) / sw);
         }
     }
-    const int nu = fused && max_cols <= 32 ? 1 : kPoolCols;      // columns per lane
+    plan.fused = fused;
+    plan.nu = fused && max_cols <= 32 ? 1 : kPoolCols;
+    return DISTDL_OK;
+}
+
+// terms[k * q + b]: output column (counted from the shard's own) that the adjoint with H* in it adds to bulk column q as window column b.
+template <int KW, int SW, int DW, int NU>
+static void pool_column_terms(const PoolShard &S, int wc, int wcols, int32_t *terms) {
+    using Strip = PoolStrip<KW, SW, DW, NU>;
+    constexpr int kNone = INT_MIN;
+    for (int col0 = 0; col0 * SW < S.bw; col0 += 32 * NU) {
+        for (int lane = 0; lane < 32; ++lane) {
+            const Strip strip(S, wc, wcols, col0, lane);
+            const int newest = strip.newest;
+            int g[NU][Strip::NJ], code[NU][Strip::NJ];
+            for (int u = 0; u < NU; ++u)
+                for (int v = 0; v < Strip::NJ; ++v) g[u][v] = (unsigned)(newest + 32 * u - v) < (unsigned)S.ow ? newest + 32 * u - v : kNone;
+            if (strip.left) Strip::put_left(g, code, -1, 0, newest);
+            if (strip.right) Strip::put_right(g, code, S.ow, 0, newest, S.ow);
+            for (int u = 0; u < NU; ++u)
+                for (int c = 0; c < SW; ++c)
+                    for (int v = 0; v < Strip::NJ; ++v) {
+                        const int cell = SW * (lane + 32 * u) + c, b = Strip::window(c, v);
+                        if (cell < strip.cols && b >= 0 && b < KW) terms[KW * (SW * col0 + cell) + b] = g[u][v];
+                    }
+        }
+    }
+}
+template <int KW, int SW>
+static void pool_column_terms(const PoolShard &S, int wc, int wcols, int nu, int32_t *terms) {
+    if (SW == 1 || (S.hlw - S.j0 - SW * div_floor(S.hlw - S.j0, SW)) == 0)
+        nu == 1 ? pool_column_terms<KW, SW, 0, 1>(S, wc, wcols, terms) : pool_column_terms<KW, SW, 0, 2>(S, wc, wcols, terms);
+    else
+        nu == 1 ? pool_column_terms<KW, SW, SW - 1, 1>(S, wc, wcols, terms) : pool_column_terms<KW, SW, SW - 1, 2>(S, wc, wcols, terms);
+}
+
+static distdl_status_t pool_impl(const distdl_partition *p, const void *const *in, void *const *out, void *const *arg,
+                                 int32_t kh, int32_t kw, int32_t sh, int32_t sw, int32_t plh, int32_t phh, int32_t plw,
+                                 int32_t phw, int32_t mode, void *stream, bool adjoint, const char *what) {
+    clear_error();
+    if (!p || !in || !out) return fail(DISTDL_ERR_INVALID_ARG, "%s: NULL argument", what);
+    PoolPlan plan;
+    distdl_status_t st = pool_plan(p, kh, kw, sh, sw, plh, phh, plw, phw, mode, adjoint, what, plan);
+    if (st != DISTDL_OK) return st;
+    if (mode == DISTDL_POOL_MAX && adjoint && !arg) return fail(DISTDL_ERR_INVALID_ARG, "%s: max pooling needs argmax", what);
+    PoolParams &P = plan.P;
+    for (int32_t w = 0; w < p->num_workers; ++w) {
+        PoolShard &S = P.s[w];
+        if (!in[w] || !out[w]) return fail(DISTDL_ERR_INVALID_ARG, "%s: shard pointer %d is NULL", what, w);
+        S.in = (const float *)in[w];
+        S.out = (float *)out[w];
+        S.arg = arg ? (int32_t *)arg[w] : nullptr;
+        if (mode == DISTDL_POOL_MAX && adjoint && !S.arg) return fail(DISTDL_ERR_INVALID_ARG, "%s: argmax[%d] is NULL", what, w);
+    }
+    // H and H* work on the padded shards: what they ask of them holds for the layer as well
+    st = halo_check_shards(p, adjoint ? out : const_cast<void *const *>(reinterpret_cast<const void *const *>(in)), what);
+    if (st != DISTDL_OK) return st;
+    cudaStream_t s = (cudaStream_t)stream;
+    const int fixed = plan.fixed, nu = plan.nu;
+    const bool fused = plan.fused;
+    const int64_t max_rows = plan.max_rows, max_cols = plan.max_cols;
+    // the compile-time variants: 64 (or 32) columns and up to 16 rows (20 of the fused adjoint) per warp, fewer where eight warps would leave some without a row
+    // or an SM would have fewer than 16 warps
     const int cols = fixed ? 32 * nu : kPoolThreadsX;
     const int tiles_x = (int)((max_cols + cols - 1) / cols);
     int rows = 1;
@@ -818,4 +902,43 @@ extern "C" distdl_status_t distdl_pool_adj(const distdl_partition_t *p, const vo
     // the positions are only read here; pool_impl shares one pointer type with the forward call
     return distdl::pool_impl(p, dy, dx, (void *const *)argmax, kh, kw, sh, sw, pad_h_lo, pad_h_hi, pad_w_lo, pad_w_hi, mode,
                              stream, true, "pool_adj");
+}
+
+// Which outputs the adjoint with H* in it adds to the rows (dim 0) or columns (dim 1) of a worker's bulk, by the rules of the kernel.
+extern "C" distdl_status_t distdl_selftest_pool_adj_terms(const distdl_partition_t *p, int32_t k, int32_t stride, int32_t pad_lo, int32_t pad_hi,
+                                                          int32_t mode, int32_t worker, int32_t dim, int32_t *fused, int32_t *terms, int32_t num_terms) {
+    using namespace distdl;
+    clear_error();
+    const char *what = "selftest_pool_adj_terms";
+    if (!p || !fused || !terms || worker < 0 || worker >= p->num_workers || dim < 0 || dim > 1) return fail(DISTDL_ERR_INVALID_ARG, "%s: bad argument", what);
+    PoolPlan plan;
+    const distdl_status_t st = pool_plan(p, k, k, stride, stride, pad_lo, pad_hi, pad_lo, pad_hi, mode, true, what, plan);
+    if (st != DISTDL_OK) return st;
+    *fused = plan.fused ? 1 : 0;
+    if (!plan.fused) return DISTDL_OK;
+    const PoolParams &P = plan.P;
+    const PoolShard &S = P.s[worker];
+    const int wr = worker / P.wcols, wc = worker % P.wcols, cells = dim ? S.bw : S.bh;
+    if (num_terms < k * cells) return fail(DISTDL_ERR_INVALID_ARG, "%s: need %d terms", what, k * cells);
+    for (int i = 0; i < k * cells; ++i) terms[i] = -1;
+    std::vector<int32_t> own(dim ? k * cells : 0, INT_MIN);
+    if (dim) {
+        if (plan.fixed == 1) pool_column_terms<2, 2>(S, wc, P.wcols, plan.nu, own.data());
+        else if (plan.fixed == 2) pool_column_terms<3, 2>(S, wc, P.wcols, plan.nu, own.data());
+        else pool_column_terms<3, 1>(S, wc, P.wcols, plan.nu, own.data());
+    }
+    std::vector<int32_t> first(dim ? P.wcols : P.wrows, 0);          // outputs of the workers before each
+    for (size_t w = 1; w < first.size(); ++w) first[w] = first[w - 1] + (dim ? P.s[w - 1].ow : P.s[(w - 1) * P.wcols].oh);
+    if (dim) {
+        for (int i = 0; i < k * cells; ++i)
+            if (own[i] != INT_MIN) terms[i] = first[wc] + own[i];
+    } else {
+        // cell row p is a = p - i0 - i * stride rows into the windows of output row i
+        for (int q = 0; q < cells; ++q)
+            for (int a = (S.hlh + q - S.i0) - stride * div_floor(S.hlh + q - S.i0, stride); a < k; a += stride) {
+                int dr, il;
+                if (pool_row_owner(P, S, worker, wr, div_floor(S.hlh + q - S.i0 - a, stride), dr, il)) terms[k * q + a] = first[wr + dr] + il;
+            }
+    }
+    return DISTDL_OK;
 }

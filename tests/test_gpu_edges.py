@@ -242,6 +242,11 @@ POOL_EDGES = [
     ((1, 1, 30, 31), (1, 1, 4, 4), (3, 3), (1, 1), ((0, 0), (0, 0))),       # two columns of a neighbour's outputs: the local adjoint, then H*
     ((1, 1, 6, 7), (1, 1, 3, 3), (3, 3), (2, 2), ((1, 1), (1, 1))),         # one output a shard: the same
     ((8, 60, 264, 36), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),     # 17 rows of groups a warp
+    ((1, 2, 20, 20), (1, 1, 2, 4), (2, 2), (2, 2), ((0, 0), (0, 0))),       # a shard that begins with a whole window of the worker on its left
+    ((1, 1, 12, 1020), (1, 1, 1, 4), (2, 2), (2, 2), ((0, 0), (0, 0))),     # the same, two groups a lane
+    ((1, 1, 24, 75), (1, 1, 5, 5), (2, 2), (2, 2), ((0, 0), (0, 0))),       # on five columns of workers
+    ((2, 1, 15, 36), (1, 1, 3, 5), (2, 2), (2, 2), ((0, 1), (0, 1))),       # padded at the end
+    ((1, 1, 20, 188), (1, 1, 2, 4), (2, 2), (2, 2), ((1, 1), (1, 1))),      # and at both
 ]
 
 

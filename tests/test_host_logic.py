@@ -348,3 +348,50 @@ def test_calls_check_their_arguments_before_the_library_sees_them():
         distdl.stencil3d_fwd(part, y, [[1, 2, 3], [1, 2, 3], [1, 2]], y, stream=0)
     raw, radius = distdl._taps(np.arange(9).reshape(3, 3))
     assert radius == 1 and np.array_equal(np.frombuffer(raw, np.float32), np.arange(9, dtype=np.float32))
+
+
+def _fused_pool_adjoint_disagreements(kernel, stride, dim, sizes, paddings):
+    """Layers in which a row (dim 0) or column (dim 1) of some worker's bulk gets other outputs than those whose windows hold it, and the
+    number of layers of which that was asked."""
+    wrong, asked = [], 0
+    for n in sizes:
+        for p in range(1, 9):
+            for pad in paddings:
+                m = (n + sum(pad) - kernel) // stride + 1
+                if n < p or m < p:
+                    continue
+                lo, hi = distdl.halo_widths_1d(n, p, kernel, stride, pad_lo=pad[0], pad_hi=pad[1])[:2]
+                across = distdl.halo_widths_1d(16, 1, kernel, stride, pad_lo=pad[0], pad_hi=pad[1])[:2]
+                shape, parts, los, his = [1, 1, 16, 16], [1] * 4, [0, 0, across[0], across[0]], [0, 0, across[1], across[1]]
+                shape[2 + dim], parts[2 + dim], los[2 + dim], his[2 + dim] = n, p, lo, hi
+                try:
+                    part = distdl.Partition(shape, parts, los, his)
+                except distdl.DistdlError:
+                    continue                                     # ghosts wider than a neighbour
+                for w in range(p):
+                    got = distdl.selftest_pool_adj_terms(part, kernel, stride, pad, distdl.POOL_AVG, w, dim)
+                    if got is None:
+                        break
+                    start, size = (v[2 + dim] for v in part.shard_extents(w)[:2])
+                    at = start + pad[0] + np.arange(size)[:, None] - np.arange(kernel)[None, :]       # first cell of the window, padded
+                    want = np.where((at >= 0) & (at % stride == 0) & (at // stride < m), at // stride, -1)
+                    if not np.array_equal(np.array(got), want):
+                        wrong.append((n, p, pad, w))
+                        break
+                else:
+                    asked += 1
+    return wrong, asked
+
+
+@pytest.mark.parametrize("dim", [0, 1])
+@pytest.mark.parametrize("kernel,stride", [(2, 2)])
+def test_fused_pool_adjoint_adds_every_output_that_holds_a_cell(kernel, stride, dim):
+    """Windows meet shard ends in as many ways as there are widths, partitions and paddings: all of them up to 160, and further on around
+    the widths whose shards end a strip of 64 or 128 columns or begin the next.  A shard that begins with a whole window of the worker on its
+    left (2 x 2 / 2, 20 columns on 4 workers) once got no gradient in its first two columns."""
+    paddings = [(a, b) for a in range(kernel) for b in range(kernel)]
+    wrong, asked = _fused_pool_adjoint_disagreements(kernel, stride, dim, range(kernel, 161), paddings)
+    ends = sorted({p * at + d for p in range(1, 9) for at in (64, 128) for d in range(-4, 5) if p * at + d > 160})
+    more = _fused_pool_adjoint_disagreements(kernel, stride, dim, ends + [1020, 1021, 1022, 1023, 1024], paddings)
+    assert not wrong + more[0], (len(wrong + more[0]), wrong[:3], more[0][:3])
+    assert asked > 1000 and more[1] > 1000
