@@ -340,7 +340,8 @@ struct PoolStrip {
         newest = col0 + lane + div_floor(S.hlw - S.j0, SW) + EW;
         cols = min(S.bw - col0 * SW, 32 * NU * SW);
         left = wc > 0 && col0 == 0 && newest - lane - (NJ - 1) < 0;
-        right = wc + 1 < wcols && col0 * SW + cols == S.bw;
+        // not in a shard's last strip only: where that is one column wide, the group at the end of the strip before it may lie under the output too
+        right = wc + 1 < wcols && newest - lane + 32 * NU - 1 >= S.ow;
     }
     // window column under which output v of a group holds the group's cell c (outside 0 .. KW - 1: it does not)
     static constexpr __host__ __device__ __forceinline__ int window(int c, int v) { return c + DW + (v - EW) * SW; }

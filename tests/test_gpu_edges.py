@@ -247,6 +247,9 @@ POOL_EDGES = [
     ((1, 1, 24, 75), (1, 1, 5, 5), (2, 2), (2, 2), ((0, 0), (0, 0))),       # on five columns of workers
     ((2, 1, 15, 36), (1, 1, 3, 5), (2, 2), (2, 2), ((0, 1), (0, 1))),       # padded at the end
     ((1, 1, 20, 188), (1, 1, 2, 4), (2, 2), (2, 2), ((1, 1), (1, 1))),      # and at both
+    ((1, 1, 9, 257), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 0), (1, 0))),       # 129 columns: the last strip is one, the one before meets the neighbour too
+    ((1, 2, 12, 386), (1, 1, 2, 3), (3, 3), (2, 2), ((0, 0), (0, 0))),
+    ((1, 1, 10, 514), (1, 1, 1, 4), (3, 3), (2, 2), ((0, 0), (0, 0))),
 ]
 
 

@@ -384,11 +384,12 @@ def _fused_pool_adjoint_disagreements(kernel, stride, dim, sizes, paddings):
 
 
 @pytest.mark.parametrize("dim", [0, 1])
-@pytest.mark.parametrize("kernel,stride", [(2, 2)])
+@pytest.mark.parametrize("kernel,stride", [(2, 2), (3, 2), (3, 1)])
 def test_fused_pool_adjoint_adds_every_output_that_holds_a_cell(kernel, stride, dim):
     """Windows meet shard ends in as many ways as there are widths, partitions and paddings: all of them up to 160, and further on around
     the widths whose shards end a strip of 64 or 128 columns or begin the next.  A shard that begins with a whole window of the worker on its
-    left (2 x 2 / 2, 20 columns on 4 workers) once got no gradient in its first two columns."""
+    left (2 x 2 / 2, 20 columns on 4 workers) once got no gradient in its first two columns; one of 128 m + 1 columns (3 x 3 / 2, 257 on 2 workers, padded on
+    the left) lost a term of the column before its last."""
     paddings = [(a, b) for a in range(kernel) for b in range(kernel)]
     wrong, asked = _fused_pool_adjoint_disagreements(kernel, stride, dim, range(kernel, 161), paddings)
     ends = sorted({p * at + d for p in range(1, 9) for at in (64, 128) for d in range(-4, 5) if p * at + d > 160})
