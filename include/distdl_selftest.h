@@ -41,8 +41,8 @@ distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition_t *p, int3
 
 /* The adjoint of the pooling layer with H* in its kernel (k x k windows, the same stride and padding in both dimensions): works out by
  * the kernel's own rules which outputs it adds to every row (dim 0) or column (dim 1) of a worker's bulk.  terms[k * q + b] = global index
- * of the output under which bulk row or column q is row or column b of the window, -1: none.  *fused = 0 if such a layer runs as two
- * kernels (then nothing else is written).  Host only; DISTDL_ERR_INVALID_ARG if the array is too small (the message gives the size needed),
+ * of the output under which bulk row or column q is row or column b of the window, -1: none.  *fused = 0: such a layer
+ * takes two kernels (then nothing else is written), 1: it could be one but is faster as two on 148 multiprocessors, 2: it is one.  Host only; DISTDL_ERR_INVALID_ARG if the array is too small (the message gives the size needed),
  * otherwise errors as the operator's. */
 distdl_status_t distdl_selftest_pool_adj_terms(const distdl_partition_t *p, int32_t k, int32_t stride, int32_t pad_lo, int32_t pad_hi,
                                                int32_t mode, int32_t worker, int32_t dim, int32_t *fused, int32_t *terms, int32_t num_terms);

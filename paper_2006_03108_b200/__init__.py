@@ -511,10 +511,11 @@ def selftest_conv_row_reads(part, k, gradients=False):
 
 
 def selftest_pool_adj_terms(part, kernel, stride, pad, mode, worker, dim):
-    """For every row (dim 0) or column (dim 1) of a worker's bulk the outputs that the pooling adjoint with H* in it adds to it, one per row or
-    column of the window, -1: none (include/distdl_selftest.h); None if the layer runs as two kernels."""
+    """(fused, terms) of the pooling adjoint with H* in it: whether the layer runs so (0: it cannot, and there are no terms; 1: two kernels are faster;
+    2: it does), and for every row (dim 0) or column (dim 1) of a worker's bulk the outputs that are added to it, one per row or column of the window,
+    -1: none (include/distdl_selftest.h)."""
     cells = part.shard_extents(worker)[1][2 + dim]
     terms, fused = (ctypes.c_int32 * (kernel * cells))(), ctypes.c_int32(0)
     _check(lib().distdl_selftest_pool_adj_terms(part.handle, kernel, stride, pad[0], pad[1], mode, worker, dim, ctypes.byref(fused), terms,
                                                 kernel * cells))
-    return [list(terms[kernel * q:kernel * q + kernel]) for q in range(cells)] if fused.value else None
+    return fused.value, [list(terms[kernel * q:kernel * q + kernel]) for q in range(cells)] if fused.value else None

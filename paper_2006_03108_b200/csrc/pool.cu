@@ -699,9 +699,8 @@ static distdl_status_t pool_dim(int64_t n, int32_t p, int32_t k, int32_t s, int3
 struct PoolPlan {
     PoolParams P;
     int fixed;                       // which of the compile-time variants, 0: the general kernels
-    bool fused;                      // adjoint with H* in it
-    int nu;                          // columns (fused: of groups) per lane
-    int64_t max_rows, max_cols;      // of the items that threads (general), lanes (fixed) and groups (adjoint, fixed) walk
+    bool fusable;                    // the adjoint's kernel can have H* in it
+    int64_t max_rows, max_cols;      // of the largest shard: outputs, of the adjoint padded cells
 };
 
 static distdl_status_t pool_plan(const distdl_partition *p, int32_t kh, int32_t kw, int32_t sh, int32_t sw, int32_t plh, int32_t phh,
@@ -748,11 +747,8 @@ static distdl_status_t pool_plan(const distdl_partition *p, int32_t kh, int32_t 
     // the compile-time variants
     const int fixed = plan.fixed = (kh == 2 && kw == 2 && sh == 2 && sw == 2) ? 1 : (kh == 3 && kw == 3 && sh == 2 && sw == 2) ? 2
                                  : (kh == 3 && kw == 3 && sh == 1 && sw == 1) ? 3 : 0;
-    // The adjoint with H* in it: where there is an H* (a ghost anywhere).  Max pooling on windows that do not overlap has one term a cell and
-    // half the registers without it, and is faster so once the launch no longer counts (2 x 2 / 2, pairs: 12 x 7 x 333 x 129 on 3 x 2 workers
-    // 22.2 -> 18.7 us; 8 x 16 x 514 x 514 on 4 x 4 101 -> 109; average pooling 93 -> 93 there, 16 x 16 x 1000 x 1000 on 3 x 3 615 -> 532).
-    bool fused = fixed && adjoint && !p->adj_host.tiles.empty() &&
-                 (mode == DISTDL_POOL_AVG || sh < kh || sw < kw || (int64_t)P.planes * P.hg * P.wg < ((int64_t)8 << 20));
+    // the adjoint with H* in it: where there is an H* (a ghost anywhere)
+    bool fused = fixed && adjoint && !p->adj_host.tiles.empty();
     for (int32_t w = 0; w < p->num_workers; ++w) {
         const int32_t r = w / p->pshape[3], c = w % p->pshape[3];
         PoolShard &S = P.s[w];
@@ -778,22 +774,70 @@ static distdl_status_t pool_plan(const distdl_partition *p, int32_t kh, int32_t 
         fused = fused && S.oh >= 1 && S.ow >= kw && S.hlw <= 16 && S.pw - S.hlw - S.bw <= 16 &&
                 (c == 0 || div_floor(S.hlw - S.j0 - kw + sw, sw) >= -1) && (c + 1 == p->pshape[3] || div_floor(S.hlw + S.bw - 1 - S.j0, sw) <= S.ow);
     }
+    plan.fusable = fused;
+    return DISTDL_OK;
+}
+
+// Rows and columns of what the threads walk, and the launch over them.
+struct PoolLaunch {
+    int64_t max_rows, max_cols;      // threads' cells or outputs (general), lanes' (fixed), groups (adjoint, fixed)
+    int nu;                          // columns (adjoint: of groups) per lane
+    int rows, tiles_x, tiles_y;      // rows per warp (fixed) or thread; tiles per plane
+};
+
+static PoolLaunch pool_launch(const PoolPlan &plan, int32_t workers, bool adjoint, bool fused, int sms) {
+    const PoolParams &P = plan.P;
+    const int fixed = plan.fixed;
+    PoolLaunch L;
+    int64_t &max_rows = L.max_rows, &max_cols = L.max_cols;
+    max_rows = plan.max_rows;
+    max_cols = plan.max_cols;
     if (fixed && adjoint && !fused) {
         // groups of sh x sw cells; the group lattice starts up to one group before cell 0
-        max_rows = max_rows / sh + 2;
-        max_cols = max_cols / sw + 2;
+        max_rows = max_rows / P.sh + 2;
+        max_cols = max_cols / P.sw + 2;
     } else if (fixed && adjoint) {
-        // the compile-time adjoint walks groups of sh x sw bulk cells, the first row of groups may begin above the bulk
+        // groups of sh x sw bulk cells, the first row of groups may begin above the bulk
         max_rows = max_cols = 0;
-        for (int32_t w = 0; w < p->num_workers; ++w) {
+        for (int32_t w = 0; w < workers; ++w) {
             const PoolShard &S = P.s[w];
-            max_rows = std::max<int64_t>(max_rows, div_floor(S.hlh + S.bh - 1 - S.i0, sh) - div_floor(S.hlh - S.i0, sh) + 1);
-            max_cols = std::max<int64_t>(max_cols, (S.bw + sw - 1) / sw);
+            max_rows = std::max<int64_t>(max_rows, div_floor(S.hlh + S.bh - 1 - S.i0, P.sh) - div_floor(S.hlh - S.i0, P.sh) + 1);
+            max_cols = std::max<int64_t>(max_cols, (S.bw + P.sw - 1) / P.sw);
         }
     }
-    plan.fused = fused;
-    plan.nu = fused && max_cols <= 32 ? 1 : kPoolCols;
-    return DISTDL_OK;
+    // the compile-time variants: 64 (or 32) columns and up to 16 rows (20 of the fused adjoint) per warp, fewer where eight warps would leave some without a row
+    // or an SM would have fewer than 16 warps
+    L.nu = fused && max_cols <= 32 ? 1 : kPoolCols;
+    const int cols = fixed ? 32 * L.nu : kPoolThreadsX;
+    L.tiles_x = (int)((max_cols + cols - 1) / cols);
+    L.rows = 1;
+    if (fixed) {
+        const int64_t all = (int64_t)workers * P.planes * L.tiles_x * max_rows;      // rows of 64 columns
+        L.rows = (int)std::min<int64_t>(fused ? 20 : 16, std::max<int64_t>(2, std::min((max_rows + kPoolThreadsY - 1) / kPoolThreadsY, all / (16 * sms))));
+    }
+    L.tiles_y = (int)((max_rows + kPoolThreadsY * L.rows - 1) / (kPoolThreadsY * L.rows));
+    if (fixed) L.rows = (int)((max_rows + kPoolThreadsY * L.tiles_y - 1) / (kPoolThreadsY * L.tiles_y));      // equal shares
+    return L;
+}
+
+// Whether the adjoint with H* in it is the faster one.  It saves H*'s launch (3 us) and passes over cells and ghosts, but a warp takes about 0.3 ns of
+// the device longer to begin: where it finds its neighbours' outputs, the column beside the shard, the ghosts to clear.  So small images in large
+// batches, whose warps have two or three rows each, are for the two kernels.  Fitted to 830 layers (both ways timed, calls back to back, 0.1 to 24 M cells, 8 to 8192 planes
+// of 10 to 1024 rows and columns on up to 4 x 4 workers): within 0.6 % of the better way on average, where fusing
+// nearly all of them was 8 % behind.
+//   2 x 2 / 2 avg, 1024 x 16 x 14 x 14 on 1 x 2 workers fused 59.6, two kernels 27.5 us;   4096 x 62 x 62 on 2 x 2 81 / 52;   64 x 258 x 258 on 4 x 4 10.5 / 12.1
+//   2 x 2 / 2 max, 1024 x 62 x 62 on 2 x 2 25.2 / 17.6;   192 x 362 x 358 on 2 x 3 36.1 / 39.5
+//   3 x 3 / 2 max, 4096 x 62 x 62 on 2 x 2 105 / 77;   192 x 362 x 358 on 2 x 3 38.2 / 47.6
+//   3 x 3 / 1 avg, 4096 x 30 x 30 on 2 x 2 91.7 / 86.9;   512 x 126 x 126 on 2 x 2 33.7 / 68.3
+static bool pool_fused_pays(const PoolPlan &plan, int32_t workers, const PoolLaunch &L, int sms) {
+    const PoolParams &P = plan.P;
+    const int64_t warps = (int64_t)workers * P.planes * L.tiles_x * ((L.max_rows + L.rows - 1) / L.rows);
+    const int64_t cells = (int64_t)P.planes * P.hg * P.wg, beside = (int64_t)P.planes * (P.wcols - 1) * P.hg;      // rows that meet a shard end
+    int64_t limit = (int64_t)sms * 74;
+    if (plan.fixed == 3) limit = (int64_t)sms * 100 + cells / 160 + beside / 4;
+    else if (plan.fixed == 2) limit += cells / 600 + beside / 40;
+    else if (P.mode == DISTDL_POOL_AVG) limit += cells / 1600;
+    return warps < limit;
 }
 
 // terms[k * q + b]: output column (counted from the shard's own) that the adjoint with H* in it adds to bulk column q as window column b.
@@ -849,23 +893,20 @@ static distdl_status_t pool_impl(const distdl_partition *p, const void *const *i
     st = halo_check_shards(p, adjoint ? out : const_cast<void *const *>(reinterpret_cast<const void *const *>(in)), what);
     if (st != DISTDL_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    const int fixed = plan.fixed, nu = plan.nu;
-    const bool fused = plan.fused;
-    const int64_t max_rows = plan.max_rows, max_cols = plan.max_cols;
-    // the compile-time variants: 64 (or 32) columns and up to 16 rows (20 of the fused adjoint) per warp, fewer where eight warps would leave some without a row
-    // or an SM would have fewer than 16 warps
-    const int cols = fixed ? 32 * nu : kPoolThreadsX;
-    const int tiles_x = (int)((max_cols + cols - 1) / cols);
-    int rows = 1;
+    const int fixed = plan.fixed;
+    int sms = 0;
     if (fixed) {
-        int dev = 0, sms = 0;
+        int dev = 0;
         DISTDL_CUDA_CHECK(cudaGetDevice(&dev));
         DISTDL_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const int64_t all = (int64_t)p->num_workers * P.planes * tiles_x * max_rows;      // rows of 64 columns
-        rows = (int)std::min<int64_t>(fused ? 20 : 16, std::max<int64_t>(2, std::min((max_rows + kPoolThreadsY - 1) / kPoolThreadsY, all / (16 * sms))));
     }
-    const int tiles_y = (int)((max_rows + kPoolThreadsY * rows - 1) / (kPoolThreadsY * rows));
-    if (fixed) rows = (int)((max_rows + kPoolThreadsY * tiles_y - 1) / (kPoolThreadsY * tiles_y));      // equal shares
+    bool fused = plan.fusable;
+    PoolLaunch L = pool_launch(plan, p->num_workers, adjoint, fused, sms);
+    if (fused && !pool_fused_pays(plan, p->num_workers, L, sms)) {
+        fused = false;
+        L = pool_launch(plan, p->num_workers, adjoint, fused, sms);
+    }
+    const int rows = L.rows, tiles_x = L.tiles_x, tiles_y = L.tiles_y, nu = L.nu;
     const int64_t blocks = (int64_t)tiles_x * tiles_y * P.planes;
     if (blocks >= ((int64_t)1 << 31)) return fail(DISTDL_ERR_UNSUPPORTED, "%s: too many tiles", what);
     const dim3 grid((unsigned)blocks, (unsigned)p->num_workers), block(kPoolThreadsX, kPoolThreadsY);
@@ -915,8 +956,12 @@ extern "C" distdl_status_t distdl_selftest_pool_adj_terms(const distdl_partition
     PoolPlan plan;
     const distdl_status_t st = pool_plan(p, k, k, stride, stride, pad_lo, pad_hi, pad_lo, pad_hi, mode, true, what, plan);
     if (st != DISTDL_OK) return st;
-    *fused = plan.fused ? 1 : 0;
-    if (!plan.fused) return DISTDL_OK;
+    *fused = 0;
+    if (!plan.fusable) return DISTDL_OK;
+    const int sms = 148;                                        // a B200's
+    const PoolLaunch launch = pool_launch(plan, p->num_workers, true, true, sms);
+    const int nu = launch.nu;
+    *fused = pool_fused_pays(plan, p->num_workers, launch, sms) ? 2 : 1;
     const PoolParams &P = plan.P;
     const PoolShard &S = P.s[worker];
     const int wr = worker / P.wcols, wc = worker % P.wcols, cells = dim ? S.bw : S.bh;
@@ -924,9 +969,9 @@ extern "C" distdl_status_t distdl_selftest_pool_adj_terms(const distdl_partition
     for (int i = 0; i < k * cells; ++i) terms[i] = -1;
     std::vector<int32_t> own(dim ? k * cells : 0, INT_MIN);
     if (dim) {
-        if (plan.fixed == 1) pool_column_terms<2, 2>(S, wc, P.wcols, plan.nu, own.data());
-        else if (plan.fixed == 2) pool_column_terms<3, 2>(S, wc, P.wcols, plan.nu, own.data());
-        else pool_column_terms<3, 1>(S, wc, P.wcols, plan.nu, own.data());
+        if (plan.fixed == 1) pool_column_terms<2, 2>(S, wc, P.wcols, nu, own.data());
+        else if (plan.fixed == 2) pool_column_terms<3, 2>(S, wc, P.wcols, nu, own.data());
+        else pool_column_terms<3, 1>(S, wc, P.wcols, nu, own.data());
     }
     std::vector<int32_t> first(dim ? P.wcols : P.wrows, 0);          // outputs of the workers before each
     for (size_t w = 1; w < first.size(); ++w) first[w] = first[w - 1] + (dim ? P.s[w - 1].ow : P.s[(w - 1) * P.wcols].oh);

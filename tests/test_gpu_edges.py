@@ -250,6 +250,9 @@ POOL_EDGES = [
     ((1, 1, 9, 257), (1, 1, 1, 2), (3, 3), (2, 2), ((1, 0), (1, 0))),       # 129 columns: the last strip is one, the one before meets the neighbour too
     ((1, 2, 12, 386), (1, 1, 2, 3), (3, 3), (2, 2), ((0, 0), (0, 0))),
     ((1, 1, 10, 514), (1, 1, 1, 4), (3, 3), (2, 2), ((0, 0), (0, 0))),
+    ((60, 50, 14, 14), (1, 1, 1, 2), (2, 2), (2, 2), ((0, 0), (0, 0))),     # small images in large batches: the local adjoint, then H*
+    ((50, 50, 20, 21), (1, 1, 2, 2), (3, 3), (2, 2), ((1, 1), (1, 1))),
+    ((60, 50, 14, 13), (1, 1, 1, 2), (3, 3), (1, 1), ((1, 1), (1, 1))),
 ]
 
 

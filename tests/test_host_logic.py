@@ -369,8 +369,8 @@ def _fused_pool_adjoint_disagreements(kernel, stride, dim, sizes, paddings):
                 except distdl.DistdlError:
                     continue                                     # ghosts wider than a neighbour
                 for w in range(p):
-                    got = distdl.selftest_pool_adj_terms(part, kernel, stride, pad, distdl.POOL_AVG, w, dim)
-                    if got is None:
+                    fused, got = distdl.selftest_pool_adj_terms(part, kernel, stride, pad, distdl.POOL_AVG, w, dim)
+                    if not fused:
                         break
                     start, size = (v[2 + dim] for v in part.shard_extents(w)[:2])
                     at = start + pad[0] + np.arange(size)[:, None] - np.arange(kernel)[None, :]       # first cell of the window, padded
@@ -396,3 +396,23 @@ def test_fused_pool_adjoint_adds_every_output_that_holds_a_cell(kernel, stride, 
     more = _fused_pool_adjoint_disagreements(kernel, stride, dim, ends + [1020, 1021, 1022, 1023, 1024], paddings)
     assert not wrong + more[0], (len(wrong + more[0]), wrong[:3], more[0][:3])
     assert asked > 1000 and more[1] > 1000
+
+
+@pytest.mark.parametrize("kernel,stride,mode,shape,parts,fused", [
+    # B200, adjoint, one kernel against two (us)
+    (2, 2, "avg", (512, 16, 14, 14), (1, 2), False),             # 59.6 / 27.5
+    (2, 2, "max", (64, 16, 62, 62), (2, 2), False),              # 25.2 / 17.6
+    (3, 2, "max", (256, 16, 62, 62), (2, 2), False),             # 105 / 77
+    (3, 1, "avg", (256, 16, 30, 30), (2, 2), False),             # 91.7 / 86.9
+    (2, 2, "avg", (4, 16, 258, 258), (4, 4), True),              # 10.5 / 12.1
+    (2, 2, "max", (12, 16, 362, 358), (2, 3), True),             # 36.1 / 39.5
+    (3, 2, "max", (16, 16, 1024, 1024), (4, 4), True),           # 350 / 417
+    (3, 2, "avg", (128, 16, 126, 126), (2, 2), True),            # 68.7 / 77.8
+    (3, 1, "max", (32, 16, 126, 126), (2, 2), True),             # 40.9 / 75.3
+])
+def test_pool_adjoint_takes_the_faster_of_one_kernel_and_two(kernel, stride, mode, shape, parts, fused):
+    pad = (0, 0) if kernel == 2 else (1, 1)
+    w = [distdl.halo_widths_1d(shape[2 + d], parts[d], kernel, stride, pad_lo=pad[0], pad_hi=pad[1]) for d in range(2)]
+    part = distdl.Partition(shape, (1, 1) + parts, [0, 0, w[0][0], w[1][0]], [0, 0, w[0][1], w[1][1]])
+    code = distdl.POOL_AVG if mode == "avg" else distdl.POOL_MAX
+    assert distdl.selftest_pool_adj_terms(part, kernel, stride, pad, code, 0, 0)[0] == (2 if fused else 1)
