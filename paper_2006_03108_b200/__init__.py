@@ -101,8 +101,9 @@ def lib():
 
 
 def _check(status):
+    """Raises what a call returned, a status or (csrc/binding.cpp) what is wrong with a list of shards."""
     if status != 0:
-        raise DistdlError(status, lib().distdl_last_error().decode())
+        raise DistdlError(1, status) if isinstance(status, str) else DistdlError(status, lib().distdl_last_error().decode())
 
 
 def _ptr(t):
@@ -283,19 +284,23 @@ def halo_widths_1d(n, p, kernel, stride=1, dilation=1, pad_lo=0, pad_hi=0):
 
 
 def broadcast_fwd(src, dsts, stream=None):
-    _check((_calls or _load()).broadcast_fwd(src, dsts, len(dsts), src.numel(), _dtype_code(src), stream))
+    n = len(dsts)
+    _check((_calls or _load()).broadcast_fwd(src, dsts, n, src.numel(), _dtype_code(src), stream, n))
 
 
 def sumreduce_adj(dy, dxs, stream=None):
-    _check((_calls or _load()).sumreduce_adj(dy, dxs, len(dxs), dy.numel(), _dtype_code(dy), stream))
+    n = len(dxs)
+    _check((_calls or _load()).sumreduce_adj(dy, dxs, n, dy.numel(), _dtype_code(dy), stream, n))
 
 
 def sumreduce_fwd(srcs, dst, stream=None):
-    _check((_calls or _load()).sumreduce_fwd(srcs, dst, len(srcs), dst.numel(), _dtype_code(dst), stream))
+    n = len(srcs)
+    _check((_calls or _load()).sumreduce_fwd(srcs, dst, n, dst.numel(), _dtype_code(dst), stream, n))
 
 
 def broadcast_adj(dys, dx, stream=None):
-    _check((_calls or _load()).broadcast_adj(dys, dx, len(dys), dx.numel(), _dtype_code(dx), stream))
+    n = len(dys)
+    _check((_calls or _load()).broadcast_adj(dys, dx, n, dx.numel(), _dtype_code(dx), stream, n))
 
 
 def _partition_pair(src_pshape, dst_pshape, small):
@@ -323,11 +328,11 @@ def partition_broadcast_adj(src_pshape, dst_pshape, dy, dx, stream=None):
 
 
 def halo_fwd(part, shards, stream=None):
-    _check((_calls or _load()).halo_fwd(part.handle.value, shards, stream))
+    _check((_calls or _load()).halo_fwd(part.handle.value, shards, stream, part.num_workers))
 
 
 def halo_adj(part, shards, stream=None):
-    _check((_calls or _load()).halo_adj(part.handle.value, shards, stream))
+    _check((_calls or _load()).halo_adj(part.handle.value, shards, stream, part.num_workers))
 
 
 def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dtype=F32, stream=None):
@@ -344,12 +349,14 @@ def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dt
 
 def conv_fwd(part, x, w, bias, y, stream=None):
     kh, kw = w.shape[-2:]
-    _check((_calls or _load()).conv_fwd(part.handle.value, x, w, bias, kh, kw, y, stream))
+    n = part.num_workers
+    _check((_calls or _load()).conv_fwd(part.handle.value, x, w, bias, kh, kw, y, stream, n, n))
 
 
 def conv_adj(part, dy, w, dx, stream=None):
     kh, kw = w.shape[-2:]
-    _check((_calls or _load()).conv_adj(part.handle.value, dy, w, kh, kw, dx, stream))
+    n = part.num_workers
+    _check((_calls or _load()).conv_adj(part.handle.value, dy, w, kh, kw, dx, stream, n, n))
 
 
 def _taps(w):
@@ -362,23 +369,33 @@ def _taps(w):
 
 def stencil3d_fwd(part, x, w, y, stream=None):
     taps, radius = _taps(w)
-    _check(_calls.stencil3d_fwd(part.handle.value, x, taps, radius, y, stream))
+    n = part.num_workers
+    _check(_calls.stencil3d_fwd(part.handle.value, x, taps, radius, y, stream, n, n))
 
 
 def stencil3d_adj(part, dy, w, dx, stream=None):
     taps, radius = _taps(w)
-    _check(_calls.stencil3d_adj(part.handle.value, dy, taps, radius, dx, stream))
+    n = part.num_workers
+    _check(_calls.stencil3d_adj(part.handle.value, dy, taps, radius, dx, stream, n, n))
+
+
+def _convg_counts(px, pco):
+    """Input shards, blocks of weights, output shards."""
+    pci = px.partition_shape[1] if px.rank == 4 else 1
+    return px.num_workers, pco * pci, pco * px.num_workers // pci
 
 
 def convg_fwd(px, nco, pco, x, w, bias, y, stream=None):
     """Channel-partitioned convolution layer; w: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j."""
     kh, kw = w[0].shape[-2:]
-    _check((_calls or _load()).convg_fwd(px.handle.value, nco, pco, x, w, bias, kh, kw, y, stream))
+    n, blocks, m = _convg_counts(px, pco)
+    _check((_calls or _load()).convg_fwd(px.handle.value, nco, pco, x, w, bias, kh, kw, y, stream, n, blocks, pco, m))
 
 
 def convg_adj(px, nco, pco, dy, w, dx, stream=None):
     kh, kw = w[0].shape[-2:]
-    _check((_calls or _load()).convg_adj(px.handle.value, nco, pco, dy, w, kh, kw, dx, stream))
+    n, blocks, m = _convg_counts(px, pco)
+    _check((_calls or _load()).convg_adj(px.handle.value, nco, pco, dy, w, kh, kw, dx, stream, m, blocks, n))
 
 
 def convg_adj_params_workspace(px, nco, pco, kh, kw):
@@ -389,8 +406,9 @@ def convg_adj_params_workspace(px, nco, pco, kh, kw):
 
 def convg_adj_params(px, nco, pco, x, dy, kernel, dw, db, workspace, stream=None):
     """dw: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j; db: list of [nco_i] or None."""
+    n, blocks, m = _convg_counts(px, pco)
     _check((_calls or _load()).convg_adj_params(px.handle.value, nco, pco, x, dy, kernel[0], kernel[1], dw, db, workspace,
-                                                workspace.numel() * workspace.element_size(), stream))
+                                                workspace.numel() * workspace.element_size(), stream, n, m, blocks, pco))
 
 
 class Repartition:
@@ -430,15 +448,16 @@ class Repartition:
 
 
 def repartition_fwd(rep, src, dst, stream=None):
-    _check((_calls or _load()).repartition_fwd(rep.handle.value, src, dst, stream))
+    _check((_calls or _load()).repartition_fwd(rep.handle.value, src, dst, stream, rep.num_src, rep.num_dst))
 
 
 def repartition_adj(rep, dy, dx, stream=None):
-    _check((_calls or _load()).repartition_adj(rep.handle.value, dy, dx, stream))
+    _check((_calls or _load()).repartition_adj(rep.handle.value, dy, dx, stream, rep.num_dst, rep.num_src))
 
 
 def allreduce(bufs, stream=None):
-    _check((_calls or _load()).allreduce(bufs, len(bufs), bufs[0].numel(), _dtype_code(bufs[0]), stream))
+    n = len(bufs)
+    _check((_calls or _load()).allreduce(bufs, n, bufs[0].numel(), _dtype_code(bufs[0]), stream, n))
 
 
 POOL_AVG, POOL_MAX = 0, 1
@@ -446,26 +465,28 @@ POOL_AVG, POOL_MAX = 0, 1
 
 def pool_fwd(part, x, kernel, stride, pad, mode, y, argmax=None, stream=None):
     """kernel = (kh, kw), stride = (sh, sw), pad = ((lo_h, hi_h), (lo_w, hi_w)); x is updated in place by H."""
+    n = part.num_workers
     _check((_calls or _load()).pool_fwd(part.handle.value, x, kernel[0], kernel[1], stride[0], stride[1], pad[0][0], pad[0][1],
-                                        pad[1][0], pad[1][1], mode, y, argmax, stream))
+                                        pad[1][0], pad[1][1], mode, y, argmax, stream, n, n, n if mode == POOL_MAX else 0))
 
 
 def pool_adj(part, dy, argmax, kernel, stride, pad, mode, dx, stream=None):
+    n = part.num_workers
     _check((_calls or _load()).pool_adj(part.handle.value, dy, argmax, kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
-                                        pad[0][1], pad[1][0], pad[1][1], mode, dx, stream))
+                                        pad[0][1], pad[1][0], pad[1][1], mode, dx, stream, n, n if mode == POOL_MAX else 0, n))
 
 
 def affine_fwd(nb, nfi, nfo, pfo, pfi, x, w, bias, y, stream=None):
-    _check((_calls or _load()).affine_fwd(nb, nfi, nfo, pfo, pfi, x, w, bias, y, stream))
+    _check((_calls or _load()).affine_fwd(nb, nfi, nfo, pfo, pfi, x, w, bias, y, stream, pfi, pfo * pfi, pfo, pfo))
 
 
 def affine_adj(nb, nfi, nfo, pfo, pfi, dy, w, dx, stream=None):
-    _check((_calls or _load()).affine_adj(nb, nfi, nfo, pfo, pfi, dy, w, dx, stream))
+    _check((_calls or _load()).affine_adj(nb, nfi, nfo, pfo, pfi, dy, w, dx, stream, pfo, pfo * pfi, pfi))
 
 
 def affine_adj_params(nb, nfi, nfo, pfo, pfi, dy, x, dw, db=None, stream=None):
     """dW blocks (worker order i * pfi + j) and, if given, the db blocks of the adjoint affine algorithm."""
-    _check((_calls or _load()).affine_adj_params(nb, nfi, nfo, pfo, pfi, dy, x, dw, db, stream))
+    _check((_calls or _load()).affine_adj_params(nb, nfi, nfo, pfo, pfi, dy, x, dw, db, stream, pfo, pfi, pfo * pfi, pfo))
 
 
 def conv_adj_params_workspace(part, kh, kw):
@@ -477,8 +498,9 @@ def conv_adj_params_workspace(part, kh, kw):
 
 def conv_adj_params(part, x, dy, kernel, dw, db, workspace, stream=None):
     """dw [C, kh, kw] and db [C] (or None) of the adjoint convolution algorithm; workspace: a uint8 tensor."""
+    n = part.num_workers
     _check((_calls or _load()).conv_adj_params(part.handle.value, x, dy, kernel[0], kernel[1], dw, db, workspace,
-                                               workspace.numel() * workspace.element_size(), stream))
+                                               workspace.numel() * workspace.element_size(), stream, n, n))
 
 
 def device_status(stream=None):

@@ -10,6 +10,7 @@
 #include <stdint.h>
 
 #include <tuple>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -75,21 +76,22 @@ struct Arg<const float *> {                           // what taps() returns
     const float *get() { return value; }
 };
 
-struct Pointers {                                     // shards; None: no array.  Ones that are not there are NULL
+struct Pointers {                                     // shards; None: no array
     void *few[64] = {};
     std::vector<void *> many;
     void **p = nullptr;
+    Py_ssize_t size = 0;
     bool read(PyObject *o, bool) {
         if (o == Py_None) return true;
         PyObject *s = PySequence_Fast(o, "a sequence of shards is needed");
         if (!s) return false;
         const Py_ssize_t n = PySequence_Fast_GET_SIZE(s);
-        if (n > 64) many.resize((size_t)(n > DISTDL_MAX_WORKERS ? n : DISTDL_MAX_WORKERS));
+        if (n > 64) many.resize((size_t)n);
         p = n > 64 ? many.data() : few;
         bool ok = true;
-        for (Py_ssize_t i = 0; ok && i < n && i < PySequence_Fast_GET_SIZE(s); ++i) {      // another thread may change a list meanwhile
-            PyObject *shard = Py_NewRef(PySequence_Fast_GET_ITEM(s, i));
-            ok = address(shard, p + i);
+        for (; ok && size < n && size < PySequence_Fast_GET_SIZE(s); ++size) {      // another thread may change a list meanwhile
+            PyObject *shard = Py_NewRef(PySequence_Fast_GET_ITEM(s, size));
+            ok = address(shard, p + size);
             Py_DECREF(shard);
         }
         Py_DECREF(s);
@@ -105,15 +107,37 @@ struct Arg<const void *const *> : Pointers {
     const void *const *get() { return p; }
 };
 
-// The stream is every function's last argument.
+// What the library reads of a list: as many entries as the caller says the layer has.  A list that is too short is refused here, optional ones too (a
+// missing bias or position would read as "none").  Beyond any layer's number the library refuses the layer before it reads the list.
+constexpr long long kMostEntries = 4096;
+static_assert(kMostEntries >= DISTDL_MAX_WORKERS, "");
+template <typename T>
+bool too_short(const Arg<T> &arg, PyObject *const *&need, int at, PyObject **why) {
+    if constexpr (std::is_base_of_v<Pointers, Arg<T>>) {
+        const long long entries = PyLong_AsLongLong(*need++);
+        if (entries == -1 && PyErr_Occurred()) return true;
+        if (arg.p && arg.size < entries && entries <= kMostEntries) {
+            *why = PyUnicode_FromFormat("argument %d is a list of %zd entries, %lld are needed", at + 1, arg.size, entries);
+            return true;
+        }
+    }
+    return false;
+}
+
+// The stream is every function's last argument.  Behind it: how many entries each list has to have, in the lists' order.  Returns the status, or what is
+// wrong with a list.
 template <auto Function>
 struct Call;
 template <typename... A, distdl_status_t (*Function)(A...)>
 struct Call<Function> {
+    static constexpr size_t kLists = (std::is_base_of_v<Pointers, Arg<A>> + ... + 0);
     template <size_t... I>
     static PyObject *run(PyObject *const *args, std::index_sequence<I...>) {
         std::tuple<Arg<A>...> a;
         if (!(std::get<I>(a).read(args[I], I + 1 == sizeof...(A)) && ...)) return nullptr;
+        PyObject *const *need = args + sizeof...(A);
+        PyObject *why = nullptr;
+        if ((too_short(std::get<I>(a), need, (int)I, &why) || ...)) return why;
         distdl_status_t status;
         Py_BEGIN_ALLOW_THREADS
         status = Function(std::get<I>(a).get()...);
@@ -121,7 +145,8 @@ struct Call<Function> {
         return PyLong_FromLong((long)status);
     }
     static PyObject *entry(PyObject *, PyObject *const *args, Py_ssize_t n) {
-        if (n != (Py_ssize_t)sizeof...(A)) return PyErr_Format(PyExc_TypeError, "%zd arguments, %zd needed", n, (Py_ssize_t)sizeof...(A));
+        constexpr Py_ssize_t needed = (Py_ssize_t)(sizeof...(A) + kLists);
+        if (n != needed) return PyErr_Format(PyExc_TypeError, "%zd arguments, %zd needed", n, needed);
         return run(args, std::index_sequence_for<A...>{});
     }
 };

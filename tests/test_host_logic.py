@@ -330,7 +330,7 @@ def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
 
 
 def test_calls_check_their_arguments_before_the_library_sees_them():
-    """Shards missing from a list are NULL (an error), not whatever lies behind it; wrong types are exceptions."""
+    """Lists that are too short are errors, not whatever lies behind them; wrong types are exceptions."""
     part = distdl.Partition((8, 8), (2, 2), (1, 1), (1, 1))
     y, few = [256] * 4, [256, 512]
     conv = distdl.Partition((1, 1, 8, 8), (1, 1, 2, 2), (0, 0, 1, 1), (0, 0, 1, 1))
@@ -416,3 +416,63 @@ def test_pool_adjoint_takes_the_faster_of_one_kernel_and_two(kernel, stride, mod
     part = distdl.Partition(shape, (1, 1) + parts, [0, 0, w[0][0], w[1][0]], [0, 0, w[0][1], w[1][1]])
     code = distdl.POOL_AVG if mode == "avg" else distdl.POOL_MAX
     assert distdl.selftest_pool_adj_terms(part, kernel, stride, pad, code, 0, 0)[0] == (2 if fused else 1)
+
+
+class _Block:
+    """A block of weights at some address."""
+
+    def __init__(self, *shape):
+        self.shape = shape
+
+    def data_ptr(self):
+        return 0x10000
+
+    def numel(self):
+        return 1 << 20
+
+    def element_size(self):
+        return 1
+
+
+def test_short_lists_are_refused_whatever_they_hold():
+    """Also where an entry may be missing (bias, positions, db), and where the list is as long as the calls' own array."""
+    a, w = [0x10000 * (i + 1) for i in range(256)], _Block(3, 3, 5, 5)
+
+    def refuses(needed, fn, *args):
+        with pytest.raises(distdl.DistdlError, match="%d are needed" % needed) as e:
+            fn(*args, stream=0)
+        assert e.value.status == 1
+
+    for workers in (65, 100, 256):
+        part = distdl.Partition((1024,), (workers,), (1,), (1,))
+        for n in {0, 10, 63, 64, workers - 1}:
+            refuses(workers, distdl.halo_fwd, part, a[:n])
+            refuses(workers, distdl.halo_adj, part, tuple(a[:n]))
+    rep = distdl.Repartition((8, 8), (4, 1), (1, 2))
+    refuses(4, distdl.repartition_fwd, rep, a[:3], a[:2])
+    refuses(2, distdl.repartition_fwd, rep, a[:4], a[:1])
+    refuses(2, distdl.repartition_adj, rep, a[:1], a[:4])
+    conv = distdl.Partition((1, 1, 8, 8), (1, 1, 2, 2), (0, 0, 2, 2), (0, 0, 2, 2))
+    refuses(4, distdl.conv_fwd, conv, a[:4], w, None, a[:3])
+    refuses(4, distdl.conv_adj, conv, a[:3], w, a[:4])
+    refuses(4, distdl.conv_adj_params, conv, a[:4], a[:2], (5, 5), 256, None, w)
+    px = distdl.Partition((1, 6, 16, 16), (1, 2, 2, 2), (0, 0, 2, 2), (0, 0, 2, 2))            # 8 input shards, 12 output shards, 6 blocks
+    for lists, needed in [((a[:7], [w] * 6, a[:3], a[:12]), 8), ((a[:8], [w] * 5, None, a[:12]), 6), ((a[:8], [w] * 6, [None] * 2, a[:12]), 3),
+                          ((a[:8], [w] * 6, None, a[:11]), 12)]:
+        refuses(needed, distdl.convg_fwd, px, 9, 3, *lists)
+    refuses(12, distdl.convg_adj, px, 9, 3, a[:11], [w] * 6, a[:8])
+    refuses(8, distdl.convg_adj, px, 9, 3, a[:12], [w] * 6, a[:7])
+    refuses(3, distdl.convg_adj_params, px, 9, 3, a[:8], a[:12], (5, 5), a[:6], a[:2], w)
+    refuses(6, distdl.convg_adj_params, px, 9, 3, a[:8], a[:12], (5, 5), a[:5], None, w)
+    st = distdl.Partition((8, 8, 8), (2, 1, 1), (1, 1, 1), (1, 1, 1))
+    refuses(2, distdl.stencil3d_fwd, st, a[:2], np.ones((3, 3)), a[:1])
+    refuses(2, distdl.stencil3d_adj, st, a[:1], np.ones((3, 3)), a[:2])
+    pool = distdl.Partition((1, 1, 8, 8), (1, 1, 2, 2))
+    layer = ((2, 2), (2, 2), ((0, 0), (0, 0)))
+    refuses(4, distdl.pool_fwd, pool, a[:4], *layer, distdl.POOL_MAX, a[:4], a[:3])
+    refuses(4, distdl.pool_adj, pool, a[:4], a[:3], *layer, distdl.POOL_MAX, a[:4])
+    refuses(4, distdl.pool_fwd, pool, a[:4], *layer, distdl.POOL_AVG, a[:3])
+    refuses(2, distdl.affine_fwd, 16, 256, 256, 2, 4, a[:4], a[:8], [None], a[:2])
+    refuses(4, distdl.affine_fwd, 16, 256, 256, 2, 4, a[:3], a[:8], None, a[:2])
+    refuses(8, distdl.affine_adj, 16, 256, 256, 2, 4, a[:2], a[:7], a[:4])
+    refuses(2, distdl.affine_adj_params, 16, 256, 256, 2, 4, a[:2], a[:4], a[:8], a[:1])
