@@ -10,6 +10,7 @@ PyTorch is used by callers for device memory and streams; this module only reads
 
 import ctypes
 import importlib
+import math
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -303,10 +304,19 @@ def broadcast_adj(dys, dx, stream=None):
     _check((_calls or _load()).broadcast_adj(dys, dx, n, dx.numel(), _dtype_code(dx), stream, n))
 
 
-def _partition_pair(src_pshape, dst_pshape, small):
+def _check_shards(shards, pshape):
+    """One shard per worker of a partition (of more workers than any partition has, the library refuses the partition)."""
+    n = math.prod(int(v) for v in pshape)
+    if len(shards) < n <= 4096:
+        raise DistdlError(1, "a list of %d shards, %d are needed" % (len(shards), n))
+
+
+def _partition_pair(src_pshape, dst_pshape, small, large):
     rank = len(src_pshape)
     if len(dst_pshape) != rank:
         raise ValueError("partition shapes differ in rank")
+    _check_shards(small, src_pshape)
+    _check_shards(large, dst_pshape)
     sp = (ctypes.c_int32 * rank)(*[int(v) for v in src_pshape])
     dp = (ctypes.c_int32 * rank)(*[int(v) for v in dst_pshape])
     el = (ctypes.c_int64 * len(small))(*[t.numel() for t in small])
@@ -315,14 +325,14 @@ def _partition_pair(src_pshape, dst_pshape, small):
 
 def partition_broadcast_fwd(src_pshape, dst_pshape, src, dst, stream=None):
     """dst[w] <- src[source of w]: broadcast along the partition dimensions where src_pshape is 1."""
-    rank, sp, dp, el = _partition_pair(src_pshape, dst_pshape, src)
+    rank, sp, dp, el = _partition_pair(src_pshape, dst_pshape, src, dst)
     _check(lib().distdl_partition_broadcast_fwd(rank, sp, dp, el, _ptr_array(src), _ptr_array(dst), _dtype_code(src[0]),
                                                 _stream(stream)))
 
 
 def partition_broadcast_adj(src_pshape, dst_pshape, dy, dx, stream=None):
     """dx[j] <- sum, in worker order, of the dy[w] whose source is j: the sum-reduce back to the smaller partition."""
-    rank, sp, dp, el = _partition_pair(src_pshape, dst_pshape, dx)
+    rank, sp, dp, el = _partition_pair(src_pshape, dst_pshape, dx, dy)
     _check(lib().distdl_partition_broadcast_adj(rank, sp, dp, el, _ptr_array(dy), _ptr_array(dx), _dtype_code(dx[0]),
                                                 _stream(stream)))
 
@@ -340,6 +350,7 @@ def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dt
     tables go into a fixed 1 MiB device array of the library instead of a cudaMalloc'd block
     (see distdl_halo_fwd_noalloc in include/distdl.h for the limits and the sharing rules)."""
     rank = len(global_shape)
+    _check_shards(shards, partition_shape)
     gs = (ctypes.c_int64 * rank)(*[int(v) for v in global_shape])
     ps = (ctypes.c_int32 * rank)(*[int(v) for v in partition_shape])
     lo = None if halo_lo is None else (ctypes.c_int32 * rank)(*[int(v) for v in halo_lo])

@@ -476,3 +476,9 @@ def test_short_lists_are_refused_whatever_they_hold():
     refuses(4, distdl.affine_fwd, 16, 256, 256, 2, 4, a[:3], a[:8], None, a[:2])
     refuses(8, distdl.affine_adj, 16, 256, 256, 2, 4, a[:2], a[:7], a[:4])
     refuses(2, distdl.affine_adj_params, 16, 256, 256, 2, 4, a[:2], a[:4], a[:8], a[:1])
+    t = [_FakeTensor(v) for v in a]
+    refuses(4, distdl.partition_broadcast_fwd, (2, 1), (2, 2), t[:2], t[:3])
+    refuses(2, distdl.partition_broadcast_fwd, (2, 1), (2, 2), t[:1], t[:4])
+    refuses(4, distdl.partition_broadcast_adj, (2, 1), (2, 2), t[:3], t[:2])
+    with pytest.raises(distdl.DistdlError, match="4 are needed"):
+        distdl.halo_fwd_noalloc((8, 8), (2, 2), (1, 1), (1, 1), t[:3], stream=0)
