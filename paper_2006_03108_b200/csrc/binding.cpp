@@ -156,22 +156,26 @@ PyObject *taps(PyObject *, PyObject *w) {
     PyObject *rows = PySequence_Fast(w, "taps must have shape [3][2R+1]");
     if (!rows) return nullptr;
     std::vector<float> v;
-    Py_ssize_t width = -1;
-    bool shaped = PySequence_Fast_GET_SIZE(rows) == 3, failed = false;
-    for (Py_ssize_t r = 0; !failed && r < PySequence_Fast_GET_SIZE(rows); ++r) {
-        PyObject *row = PySequence_Fast(PySequence_Fast_GET_ITEM(rows, r), "taps must have shape [3][2R+1]");
+    Py_ssize_t width = -1, count = 0;
+    bool shaped = true, failed = false;
+    // a number's own conversion may change the lists meanwhile: sizes are looked up at each step, and what is in hand is held
+    for (; !failed && count < PySequence_Fast_GET_SIZE(rows); ++count) {
+        PyObject *item = Py_NewRef(PySequence_Fast_GET_ITEM(rows, count)), *row = PySequence_Fast(item, "taps must have shape [3][2R+1]");
+        Py_DECREF(item);
         failed = !row;
-        const Py_ssize_t n = row ? PySequence_Fast_GET_SIZE(row) : 0;
-        shaped = shaped && n % 2 == 1 && (width < 0 || n == width);
-        width = n;
-        for (Py_ssize_t k = 0; !failed && k < n; ++k) {
-            PyObject *f = PyNumber_Float(PySequence_Fast_GET_ITEM(row, k));
+        Py_ssize_t n = 0;
+        for (; !failed && n < PySequence_Fast_GET_SIZE(row); ++n) {
+            PyObject *number = Py_NewRef(PySequence_Fast_GET_ITEM(row, n)), *f = PyNumber_Float(number);
+            Py_DECREF(number);
             failed = !f;
             if (f) v.push_back((float)PyFloat_AS_DOUBLE(f));
             Py_XDECREF(f);
         }
         Py_XDECREF(row);
+        shaped = shaped && n % 2 == 1 && (width < 0 || n == width);
+        width = n;
     }
+    shaped = shaped && count == 3;
     Py_DECREF(rows);
     if (failed) return nullptr;
     if (!shaped) Py_RETURN_NONE;

@@ -418,6 +418,32 @@ def test_pool_adjoint_takes_the_faster_of_one_kernel_and_two(kernel, stride, mod
     assert distdl.selftest_pool_adj_terms(part, kernel, stride, pad, code, 0, 0)[0] == (2 if fused else 1)
 
 
+class _Change:
+    """A number whose conversion changes the list that it is in."""
+
+    def __init__(self, change):
+        self.change = change
+
+    def __float__(self):
+        self.change()
+        return 2.0
+
+
+def test_taps_that_change_while_they_are_read():
+    for at in range(3):
+        rows = [[1.0] * 5 for _ in range(3)]
+        rows[at][1] = _Change(rows[at].clear)
+        with pytest.raises(ValueError):
+            distdl._taps(rows)
+        rows = [[1.0] * 5 for _ in range(3)]
+        rows[at][4] = _Change(rows.clear)
+        if at < 2:
+            with pytest.raises(ValueError):
+                distdl._taps(rows)
+        else:
+            assert np.array_equal(np.frombuffer(distdl._taps(rows)[0], np.float32), [1] * 14 + [2])
+
+
 class _Block:
     """A block of weights at some address."""
 
