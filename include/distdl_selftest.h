@@ -32,12 +32,13 @@ distdl_status_t distdl_selftest_wait_timeout(int64_t limit_cycles, void *stream)
 distdl_status_t distdl_selftest_row_plan(const distdl_partition_t *p, int32_t adjoint, int32_t *header, int32_t header_words,
                                          int32_t *records, int32_t record_words, int32_t *num_records);
 
-/* The depthwise convolution copies rows in whole 16-byte blocks.  For every row and strip of every shard that the adjoint
- * with a k x k kernel (gradients != 0: the parameter gradients) reads from arrays without ghosts, works out by the kernels' own
- * rules what is copied: *floats_past_end = the most floats beyond the end of a shard's array that a block takes in,
- * *rows_by_cell = rows copied cell by cell instead.  Host only; errors as the operators'. */
+/* The depthwise convolution copies rows in whole 16-byte blocks; where the last block of a row would reach past the end of its
+ * array, only the blocks before it, and the cells behind them one by one.  For every row and strip of every shard that the adjoint with a k x k
+ * kernel (gradients != 0: the parameter gradients) reads from arrays without ghosts, works out by the kernels' own rules what is copied:
+ * *floats_past_end = the most floats beyond the end of a shard's array that a block takes in, *rows_cut = rows that end in
+ * single cells (up to three).  Host only; errors as the operators'. */
 distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition_t *p, int32_t k, int32_t gradients, int64_t *floats_past_end,
-                                               int64_t *rows_by_cell);
+                                               int64_t *rows_cut);
 
 /* The adjoint of the pooling layer with H* in its kernel (k x k windows, the same stride and padding in both dimensions): works out by
  * the kernel's own rules which outputs it adds to every row (dim 0) or column (dim 1) of a worker's bulk.  terms[k * q + b] = global index

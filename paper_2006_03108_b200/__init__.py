@@ -536,11 +536,11 @@ def selftest_row_plan(part, adjoint=False):
 
 
 def selftest_conv_row_reads(part, k, gradients=False):
-    """(floats read past the end of a shard's array at most, rows copied cell by cell) of the depthwise convolution's copies
-    from arrays without ghosts (include/distdl_selftest.h)."""
-    past, cells = ctypes.c_int64(0), ctypes.c_int64(0)
-    _check(lib().distdl_selftest_conv_row_reads(part.handle, int(k), 1 if gradients else 0, ctypes.byref(past), ctypes.byref(cells)))
-    return past.value, cells.value
+    """(floats that a block takes in past the end of a shard's array at most, rows that end in single cells) of the depthwise convolution's
+    copies from arrays without ghosts (include/distdl_selftest.h)."""
+    past, rows = ctypes.c_int64(0), ctypes.c_int64(0)
+    _check(lib().distdl_selftest_conv_row_reads(part.handle, int(k), 1 if gradients else 0, ctypes.byref(past), ctypes.byref(rows)))
+    return past.value, rows.value
 
 
 def selftest_pool_adj_terms(part, kernel, stride, pad, mode, worker, dim):

@@ -95,6 +95,11 @@ __host__ __device__ inline bool dw_may_pass_end(int i, int bh, int bw) { return 
 __host__ __device__ inline bool dw_past_end(const float *first, int n, const float *end) {
     return first + ((n + 3 + (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3)) & ~3) - (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3) > end;
 }
+// Cells of such a row that its whole blocks hold; the up to three behind them are copied one by one.
+__host__ __device__ inline int dw_whole(const float *first, int n) {
+    const int tail = (n + (int)((reinterpret_cast<uintptr_t>(first) >> 2) & 3)) & 3;
+    return n > tail ? n - tail : 0;
+}
 
 // One warp's work: plane, shard (r, c), first row and column, rows and columns of the segment.
 struct DwItem {
@@ -243,7 +248,7 @@ struct DwRing {
                     // the last row of a shard (or the last few): its whole blocks at once, then up to three cells.  Cell by cell, one load
                     // after another, the lane kept a small layer waiting (3 x 3, 9 x 2 x 43 x 101 on 4 x 1 workers, adjoint / gradients 9.1 / 14.1
                     // -> 7.1 / 12.2 us).
-                    const int tail = (n + (int)((reinterpret_cast<uintptr_t>(f) >> 2) & 3)) & 3, whole = n > tail ? n - tail : 0;
+                    const int whole = dw_whole(f, n);
                     if (whole) {
                         o = row_copy(f, whole, col, slot, bar);
                     } else {
@@ -265,7 +270,7 @@ struct DwRing {
                     mbar_expect_tx(bar, 0);
                 } else if (dw_may_pass_end(i, P.bh[t.r], bw) &&
                            dw_past_end(f, t.cols, P.dy[t.r * P.pw + t.c] + (size_t)P.planes * (uint32_t)(P.bh[t.r] * bw))) {
-                    const int tail = (t.cols + (int)((reinterpret_cast<uintptr_t>(f) >> 2) & 3)) & 3, whole = t.cols > tail ? t.cols - tail : 0;
+                    const int whole = dw_whole(f, t.cols);
                     if (whole) o = row_copy(f, whole, 0, slot, bar);
                     else mbar_expect_tx(bar, 0);
                     for (int e = whole; e < t.cols; ++e) cp_async4_to(smem_u32(slot + o + e), f + e);
@@ -934,16 +939,16 @@ extern "C" distdl_status_t distdl_conv_adj(const distdl_partition_t *p, const vo
 
 // Every row that the adjoint (gradients: the parameter gradients) copies out of arrays without ghosts, by the rules of the kernels.
 extern "C" distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition_t *p, int32_t k, int32_t gradients, int64_t *floats_past_end,
-                                                          int64_t *rows_by_cell) {
+                                                          int64_t *rows_cut) {
     using namespace distdl;
     clear_error();
-    if (!floats_past_end || !rows_by_cell) return fail(DISTDL_ERR_INVALID_ARG, "selftest_conv_row_reads: NULL argument");
+    if (!floats_past_end || !rows_cut) return fail(DISTDL_ERR_INVALID_ARG, "selftest_conv_row_reads: NULL argument");
     DwParams P;
     memset(&P, 0, sizeof(P));
     int64_t max_bh = 0, max_bw = 0;
     const distdl_status_t st = dw_geometry(p, k, k, "selftest_conv_row_reads", &P, &max_bh, &max_bw);
     if (st != DISTDL_OK) return st;
-    *floats_past_end = *rows_by_cell = 0;
+    *floats_past_end = *rows_cut = 0;
     const int strip = dw_narrow(P, max_bh, max_bw) ? 64 : 128;
     const uintptr_t base = 256;                                 // never read: addresses only
     for (int32_t w = 0; w < p->num_workers; ++w) {
@@ -955,12 +960,11 @@ extern "C" distdl_status_t distdl_selftest_conv_row_reads(const distdl_partition
                 const int cols = std::min(strip, bw - j0);
                 const int halo = gradients ? 0 : k / 2, ja = std::max(j0 - halo, 0), n = std::min(j0 + cols + halo, bw) - ja;
                 const uintptr_t first = base + 4 * (uintptr_t)(row * bw + ja);
-                if (dw_may_pass_end((int)(row % bh), bh, bw) && dw_past_end(reinterpret_cast<const float *>(first), n, end)) {
-                    ++*rows_by_cell;
-                    continue;
-                }
-                const int lead = (int)((first >> 2) & 3);
-                *floats_past_end = std::max<int64_t>(*floats_past_end, row * bw + ja - lead + ((lead + n + 3) & ~3) - cells);
+                const float *f = reinterpret_cast<const float *>(first);
+                const bool cut = dw_may_pass_end((int)(row % bh), bh, bw) && dw_past_end(f, n, end);
+                const int lead = (int)((first >> 2) & 3), in_blocks = cut ? dw_whole(f, n) : n;
+                *rows_cut += cut;
+                if (in_blocks) *floats_past_end = std::max<int64_t>(*floats_past_end, row * bw + ja - lead + ((lead + in_blocks + 3) & ~3) - cells);
             }
     }
     return DISTDL_OK;

@@ -291,8 +291,8 @@ def test_partition_broadcast_rejects_shapes_that_do_not_broadcast():
 @pytest.mark.parametrize("gradients", [False, True])
 @pytest.mark.parametrize("k", [3, 5, 7])
 def test_depthwise_convolution_copies_end_inside_their_arrays(k, gradients):
-    """Rows of arrays without ghosts travel in 16-byte blocks: none may begin before the array's end and reach past it, and
-    the rows that would are the few of the last 12 bytes."""
+    """Rows of arrays without ghosts travel in 16-byte blocks: none may begin before the array's end and reach past it.  The rows whose
+    last block would are the few of the last 12 bytes; they travel in their whole blocks and single cells."""
     h = (0, 0, k // 2, k // 2)
     for planes in (1, 2, 3, 4):
         for rows in range(1, 12):
@@ -304,6 +304,11 @@ def test_depthwise_convolution_copies_end_inside_their_arrays(k, gradients):
         part = distdl.Partition((1, 1, 6, 3), (1, 1, 1, 3), h, h)
         past, by_cell = distdl.selftest_conv_row_reads(part, k, gradients)
         assert past <= 0 and by_cell <= 3 * 3
+    for parts in ((1, 1), (2, 3)):
+        for cols in range(3 * parts[1], 280):                    # the last row ends anywhere in a block, in strips of 64 and 128 columns
+            part = distdl.Partition((1, 701 if cols > 200 else 1, 3 * parts[0], cols), (1, 1) + parts, h, h)
+            past, cut = distdl.selftest_conv_row_reads(part, k, gradients)
+            assert past <= 0 and (cut > 0 or cols % 4 == 0 or parts != (1, 1)), (parts, cols, past, cut)
 
 
 def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
