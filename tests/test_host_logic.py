@@ -314,7 +314,7 @@ def test_depthwise_convolution_copies_end_inside_their_arrays(k, gradients):
 def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
     """Kernels are launched while their predecessors in the stream run; what those wrote is visible to a kernel only after its
     own wait.  So every kernel launched that way begins with stream_enter(), under no condition, and nothing else lets
-    successors in."""
+    successors in.  A few set themselves up ahead of it, with nothing but their launch's parameters, shared and tensor memory."""
     src = os.path.join(ROOT, "paper_2006_03108_b200", "csrc")
     bodies, triggers = {}, 0
     for name in sorted(os.listdir(src)):
@@ -332,6 +332,15 @@ def test_every_kernel_waits_for_the_stream_before_it_touches_memory():
     for kernel, body in sorted(bodies.items()):
         assert len(re.findall(r"^    stream_enter\(\);", body, re.M)) == 1, kernel
         assert body.count("stream_enter") == 1 and body.count("griddepcontrol") == 0, kernel
+        before = re.sub(r"static_assert\([^;]*;|constexpr [^;]*;|extern __shared__ [^;]*;", "", body[:body.index("stream_enter();")])
+        if kernel not in ("convg_kernel", "affine_kernel_pair", "affine_kernel_split", "affine_kernel_quad", "affine_dw_kernel"):
+            assert not before.strip(), kernel
+            continue
+        assert not re.search(r"__ldg|cp_async|bulk|tma_|atomic|\bld_|\bst_|\breturn\b", before), kernel
+        assert not re.search(r"\b[GPQ]\.(p\.)?(in|out|w|x|y|dx|dy|dw|db|bias|partial|\w*map)\b", before), kernel      # what points to device memory
+        assert all(re.match(r"tcgen05\.(alloc|relinquish_alloc_permit)\.", a) for a in re.findall(r'asm volatile\("([^"]*)"', before)), kernel
+        assert set(re.findall(r"\b(\w+)\[[^\]]*\] = ", before)) <= {"table", "tiles", "wbuf"}, kernel
+        assert set(re.findall(r"\*(\w+) = ", before)) - {"aligned", "bars", "tmem_slot", "abort_flag", "tiles", "wbuf", "table", "ptrs"} == set(), kernel
 
 
 def test_calls_check_their_arguments_before_the_library_sees_them():
