@@ -95,6 +95,14 @@ CONV_EDGES = [
     ((5, 3, 19, 45), (1, 1, 3, 2), 5),       # shards of 7, 6, 6 rows and 23, 22 columns
     ((37, 16, 8, 128), (1, 1, 1, 1), 5),     # strips of 64 columns: as many of 128 as the device has schedulers
     ((37, 16, 9, 128), (1, 1, 1, 1), 5),     # strips of 128: twice as many segments
+    # layers that fill the device, in strips of 128 columns (forward, adjoint, gradients: 16-byte reads or not); 250 and 251 columns
+    # end the arrays without ghosts off a 16-byte boundary
+    ((19, 17, 9, 250), (1, 1, 1, 1), 3),     # 16, not, not
+    ((5, 21, 22, 504), (1, 1, 2, 2), 3),     # not, 16, not
+    ((19, 17, 9, 251), (1, 1, 1, 1), 5),     # not, not, not
+    ((5, 21, 22, 504), (1, 1, 2, 2), 5),     # 16, 16, 16
+    ((19, 17, 9, 250), (1, 1, 1, 1), 7),     # 16, not, not
+    ((5, 21, 22, 504), (1, 1, 2, 2), 7),     # not, 16, not
 ]
 
 
@@ -301,6 +309,9 @@ STENCIL_EDGES = [
     ((8, 16, 193), (1, 1, 1), 1),            # one column in the last of four tiles
     ((6, 8, 128), (1, 1, 1), 4),             # one tile of 8 rows x 128 columns, two of the others
     ((6, 24, 65), (1, 1, 1), 2),             # 4-byte copies, fewer tiles of 8 x 128
+    ((6, 8, 128), (1, 1, 1), 1),             # tiles of 8 x 128 and, in the adjoint, 16-byte copies
+    ((9, 8, 256), (1, 1, 2), 2),
+    ((11, 24, 200), (2, 3, 1), 3),
 ]
 
 
