@@ -735,10 +735,17 @@ static distdl_status_t dw_geometry(const distdl_partition *p, int32_t kh, int32_
 // Nor where wide strips, in segments of eight rows, leave a scheduler of the device with one warp at most: it goes at the pace of one warp's
 // instructions, and half the columns are half of them (forward, adjoint and gradients, 7 x 7, 1 x 10 x 375 x 111: 33.7 -> 26.1 us; 5 x 5, 1 x 3
 // x 33 x 169 on 1 x 2 workers 26.0 -> 22.0, 2 x 1 x 217 x 753 on 4 x 3 24.7 -> 22.1).
-constexpr int64_t kDwFewItems = 592;       // schedulers of a B200
+static int64_t dw_schedulers() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        sms = 148;                          // no device: a B200's
+    }
+    return 4 * (int64_t)sms;
+}
 static bool dw_narrow(const DwParams &P, int64_t max_bh, int64_t max_bw) {
     if (2 * ((max_bw + 63) / 64) * 7 < 4 * ((max_bw + 127) / 128) * 6) return true;
-    return ((max_bw + 127) / 128) * ((max_bh + 7) / 8) * P.ph * P.pw * P.planes <= kDwFewItems;
+    return ((max_bw + 127) / 128) * ((max_bh + 7) / 8) * P.ph * P.pw * P.planes <= dw_schedulers();
 }
 
 // Rows per segment: the smallest estimated time, turns of the resident warps times rows an item reads (its halo, whole
