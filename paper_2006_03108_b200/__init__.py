@@ -1,8 +1,9 @@
 """Thin Python binding of the C-ABI library (include/distdl.h).
 
-Argument marshalling only: tensors are turned into device pointers and sizes (for the operators in _binding.so,
+Argument marshalling only: tensors are turned into device pointers and sizes (for the operators in the extension _binding,
 csrc/binding.cpp), every step of every operator runs in the CUDA kernels of libdistdl.so.  There is no CPU or PyTorch fallback:
-if the library is missing or a call fails, an exception is raised.
+if the library is missing or a call fails, an exception is raised: DistdlError with the library's status (a list of shards that is
+too short: status 1), TypeError or AttributeError for an argument of another type.  Whole numbers may be of any type with __index__ (NumPy's too).
 
 PyTorch is used by callers for device memory and streams; this module only reads
 `tensor.data_ptr()` and the current stream handle.

@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdistdl.so")
-BINDING = os.path.join(HERE, "_binding.so")          # the calls from Python, a CPython extension
+BINDING = os.path.join(HERE, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))    # the calls from Python, an extension of this interpreter
 
 SOURCES = ["planner.cpp", "partition.cu", "bcast_reduce.cu", "halo.cu", "convd.cu", "convg.cu", "pool.cu", "stencil3d.cu", "affine.cu"]
 

@@ -522,3 +522,33 @@ def test_short_lists_are_refused_whatever_they_hold():
     refuses(4, distdl.partition_broadcast_adj, (2, 1), (2, 2), t[:3], t[:2])
     with pytest.raises(distdl.DistdlError, match="4 are needed"):
         distdl.halo_fwd_noalloc((8, 8), (2, 2), (1, 1), (1, 1), t[:3], stream=0)
+
+
+def test_extension_is_named_after_the_interpreter_it_is_built_for():
+    import sysconfig
+    assert os.path.basename(distdl._load().__file__) == "_binding" + sysconfig.get_config_var("EXT_SUFFIX")
+
+
+def test_prototypes_agree_with_the_headers():
+    """distdl.lib() gives the library's functions to callers of their own; csrc/binding.cpp takes the types from the headers themselves."""
+    text = "".join(open(os.path.join(ROOT, "include", h)).read() for h in ("distdl.h", "distdl_selftest.h"))
+    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+    scalars = {"int32_t": ctypes.c_int32, "int64_t": ctypes.c_int64, "distdl_dtype_t": ctypes.c_int32, "size_t": ctypes.c_size_t}
+    kinds = {ctypes.POINTER(ctypes.c_int32): "int32_t*", ctypes.POINTER(ctypes.c_int64): "int64_t*", ctypes.POINTER(ctypes.c_float): "float*",
+             ctypes.POINTER(ctypes.POINTER(ctypes.c_int32)): "int32_t**"}
+    seen = set()
+    for name, args in re.findall(r"\b(distdl_[a-z0-9_]+)\s*\(([^()]*)\)\s*;", text):
+        types = getattr(distdl.lib(), name).argtypes
+        if types is None:
+            continue
+        seen.add(name)
+        declared = [] if args.strip() in ("", "void") else [re.sub(r"\bconst\b|\s", "", re.sub(r"\w+\s*$", "", a.strip())) for a in args.split(",")]
+        assert len(declared) == len(types), name
+        for want, got in zip(declared, types):
+            if want in scalars:
+                assert got is scalars[want], (name, want)
+            elif want.rstrip("*") in ("int32_t", "int64_t", "float"):
+                assert kinds[got] == want, (name, want)
+            else:                                            # handles, buffers: void *; arrays of them: void **
+                assert got is (ctypes.POINTER(ctypes.c_void_p) if want.endswith("**") else ctypes.c_void_p), (name, want)
+    assert len(seen) >= 40, sorted(seen)
