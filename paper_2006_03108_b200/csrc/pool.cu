@@ -6,8 +6,9 @@
 // forward = halo exchange H (the library's in-place kernel), then the local sliding kernel over
 // each worker's padded shard, starting at the first input the worker's block of the evenly split
 // output needs; adjoint = local adjoint into every cell of the padded shard (ghosts included),
-// then H*.  The local adjoint is evaluated in gather form -- a cell sums over the outputs whose
-// window holds it, in ascending output order -- so overlapping windows need no atomics.
+// then H*: as these two kernels, or (common windows, pool_adj_fused) as one that adds up the neighbours'
+// outputs where H* would have brought their ghosts.  The local adjoint is evaluated in gather form -- a cell
+// sums over the outputs whose window holds it, in ascending output order -- so overlapping windows need no atomics.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -562,10 +563,10 @@ pool_adj_fused(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, i
     else pool_adj_strip<KH, KW, SH, SW, MODE, SW - 1, NU>(P, blockIdx.y, plane, first_row, rows, col0, threadIdx.x);
 }
 
-// Adjoint of the local layer alone (H* follows), where a shard meets more than a column of a neighbour's outputs: a lane owns the SH x SW
-// cells {i0 + SH * gi + r, j0 + SW * gj + c} of a group and marches down gi.  The outputs whose window holds cell (r, c) of the group are (gi - t, gj - v) with window positions a = r + t * SH < KH, b = c + v * SW < KW, all
-// known at compile time; the outputs (gi - t, .) of the rows above stay in registers, and every cell picks its terms
-// (ascending output order = descending t, v).
+// Adjoint of the local layer alone (H* follows), where a shard meets more than a column of a neighbour's outputs or the images are small and many: a
+// lane owns the SH x SW cells {i0 + SH * gi + r, j0 + SW * gj + c} of a group and marches down gi.  The outputs whose window holds cell (r, c) of the
+// group are (gi - t, gj - v) with window positions a = r + t * SH < KH, b = c + v * SW < KW, all known at compile time; the outputs (gi - t, .) of the
+// rows above stay in registers, and every cell picks its terms (ascending output order = descending t, v).
 template <int KH, int KW, int SH, int SW, int MODE>
 __global__ void __launch_bounds__(kPoolThreadsX *kPoolThreadsY)
 pool_adj_fixed(const __grid_constant__ PoolParams P, int tiles_x, int tiles_y, int rows) {

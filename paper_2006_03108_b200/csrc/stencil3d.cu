@@ -219,7 +219,7 @@ stencil3d_kernel(const __grid_constant__ StencilParams P) {
                         ((uint32_t)(yo + io) * (uint32_t)ipx + (uint32_t)(xc + io));
         }
     }
-    // threads 0 .. 8 * 2R - 1: one cell of an extra column
+    // threads 0 .. kStRows * 2R - 1: one cell of an extra column
     const int hc_row = threadIdx.x / (2 * R), hc_c = threadIdx.x % (2 * R);
     const bool hc_active = (int)threadIdx.x < kStRows * 2 * R && y0 + hc_row < by;
     const int hc_x = hc_c < R ? x0 - R + hc_c : x0 + tw + (hc_c - R);
