@@ -230,6 +230,7 @@ class Partition:
             hi = None if halo_hi is None else (ctypes.c_int32 * rank)(*[int(v) for v in halo_hi])
             _check(L.distdl_partition_create(rank, gs, ps, lo, hi, dtype, ctypes.byref(self._h)))
         self.dtype = dtype
+        self._address = self._h.value
         self.num_workers = L.distdl_partition_num_workers(self._h)
 
     @property
@@ -265,7 +266,7 @@ class Partition:
     def close(self):
         if self._h:
             lib().distdl_partition_destroy(self._h)
-            self._h = ctypes.c_void_p()
+            self._h, self._address = ctypes.c_void_p(), None
 
     def __del__(self):
         try:
@@ -339,11 +340,11 @@ def partition_broadcast_adj(src_pshape, dst_pshape, dy, dx, stream=None):
 
 
 def halo_fwd(part, shards, stream=None):
-    _check((_calls or _load()).halo_fwd(part.handle.value, shards, stream, part.num_workers))
+    _check((_calls or _load()).halo_fwd(part._address, shards, stream, part.num_workers))
 
 
 def halo_adj(part, shards, stream=None):
-    _check((_calls or _load()).halo_adj(part.handle.value, shards, stream, part.num_workers))
+    _check((_calls or _load()).halo_adj(part._address, shards, stream, part.num_workers))
 
 
 def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dtype=F32, stream=None):
@@ -362,13 +363,13 @@ def halo_fwd_noalloc(global_shape, partition_shape, halo_lo, halo_hi, shards, dt
 def conv_fwd(part, x, w, bias, y, stream=None):
     kh, kw = w.shape[-2:]
     n = part.num_workers
-    _check((_calls or _load()).conv_fwd(part.handle.value, x, w, bias, kh, kw, y, stream, n, n))
+    _check((_calls or _load()).conv_fwd(part._address, x, w, bias, kh, kw, y, stream, n, n))
 
 
 def conv_adj(part, dy, w, dx, stream=None):
     kh, kw = w.shape[-2:]
     n = part.num_workers
-    _check((_calls or _load()).conv_adj(part.handle.value, dy, w, kh, kw, dx, stream, n, n))
+    _check((_calls or _load()).conv_adj(part._address, dy, w, kh, kw, dx, stream, n, n))
 
 
 def _taps(w):
@@ -382,13 +383,13 @@ def _taps(w):
 def stencil3d_fwd(part, x, w, y, stream=None):
     taps, radius = _taps(w)
     n = part.num_workers
-    _check(_calls.stencil3d_fwd(part.handle.value, x, taps, radius, y, stream, n, n))
+    _check(_calls.stencil3d_fwd(part._address, x, taps, radius, y, stream, n, n))
 
 
 def stencil3d_adj(part, dy, w, dx, stream=None):
     taps, radius = _taps(w)
     n = part.num_workers
-    _check(_calls.stencil3d_adj(part.handle.value, dy, taps, radius, dx, stream, n, n))
+    _check(_calls.stencil3d_adj(part._address, dy, taps, radius, dx, stream, n, n))
 
 
 def _convg_counts(px, pco):
@@ -401,13 +402,13 @@ def convg_fwd(px, nco, pco, x, w, bias, y, stream=None):
     """Channel-partitioned convolution layer; w: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j."""
     kh, kw = w[0].shape[-2:]
     n, blocks, m = _convg_counts(px, pco)
-    _check((_calls or _load()).convg_fwd(px.handle.value, nco, pco, x, w, bias, kh, kw, y, stream, n, blocks, pco, m))
+    _check((_calls or _load()).convg_fwd(px._address, nco, pco, x, w, bias, kh, kw, y, stream, n, blocks, pco, m))
 
 
 def convg_adj(px, nco, pco, dy, w, dx, stream=None):
     kh, kw = w[0].shape[-2:]
     n, blocks, m = _convg_counts(px, pco)
-    _check((_calls or _load()).convg_adj(px.handle.value, nco, pco, dy, w, kh, kw, dx, stream, m, blocks, n))
+    _check((_calls or _load()).convg_adj(px._address, nco, pco, dy, w, kh, kw, dx, stream, m, blocks, n))
 
 
 def convg_adj_params_workspace(px, nco, pco, kh, kw):
@@ -419,7 +420,7 @@ def convg_adj_params_workspace(px, nco, pco, kh, kw):
 def convg_adj_params(px, nco, pco, x, dy, kernel, dw, db, workspace, stream=None):
     """dw: list of blocks [nco_i, nci_j, kh, kw] in order i * P_ci + j; db: list of [nco_i] or None."""
     n, blocks, m = _convg_counts(px, pco)
-    _check((_calls or _load()).convg_adj_params(px.handle.value, nco, pco, x, dy, kernel[0], kernel[1], dw, db, workspace,
+    _check((_calls or _load()).convg_adj_params(px._address, nco, pco, x, dy, kernel[0], kernel[1], dw, db, workspace,
                                                 workspace.numel() * workspace.element_size(), stream, n, m, blocks, pco))
 
 
@@ -436,6 +437,7 @@ class Repartition:
         sp = (ctypes.c_int32 * rank)(*[int(v) for v in src_partition_shape])
         dp = (ctypes.c_int32 * rank)(*[int(v) for v in dst_partition_shape])
         _check(lib().distdl_repartition_create(rank, gs, sp, dp, dtype, ctypes.byref(self._h)))
+        self._address = self._h.value
         self.num_src = self.num_dst = 1
         for a, b in zip(src_partition_shape, dst_partition_shape):
             self.num_src *= int(a)
@@ -454,17 +456,17 @@ class Repartition:
         try:
             if self._h:
                 lib().distdl_repartition_destroy(self._h)
-                self._h = ctypes.c_void_p()
+                self._h, self._address = ctypes.c_void_p(), None
         except Exception:
             pass
 
 
 def repartition_fwd(rep, src, dst, stream=None):
-    _check((_calls or _load()).repartition_fwd(rep.handle.value, src, dst, stream, rep.num_src, rep.num_dst))
+    _check((_calls or _load()).repartition_fwd(rep._address, src, dst, stream, rep.num_src, rep.num_dst))
 
 
 def repartition_adj(rep, dy, dx, stream=None):
-    _check((_calls or _load()).repartition_adj(rep.handle.value, dy, dx, stream, rep.num_dst, rep.num_src))
+    _check((_calls or _load()).repartition_adj(rep._address, dy, dx, stream, rep.num_dst, rep.num_src))
 
 
 def allreduce(bufs, stream=None):
@@ -478,13 +480,13 @@ POOL_AVG, POOL_MAX = 0, 1
 def pool_fwd(part, x, kernel, stride, pad, mode, y, argmax=None, stream=None):
     """kernel = (kh, kw), stride = (sh, sw), pad = ((lo_h, hi_h), (lo_w, hi_w)); x is updated in place by H."""
     n = part.num_workers
-    _check((_calls or _load()).pool_fwd(part.handle.value, x, kernel[0], kernel[1], stride[0], stride[1], pad[0][0], pad[0][1],
+    _check((_calls or _load()).pool_fwd(part._address, x, kernel[0], kernel[1], stride[0], stride[1], pad[0][0], pad[0][1],
                                         pad[1][0], pad[1][1], mode, y, argmax, stream, n, n, n if mode == POOL_MAX else 0))
 
 
 def pool_adj(part, dy, argmax, kernel, stride, pad, mode, dx, stream=None):
     n = part.num_workers
-    _check((_calls or _load()).pool_adj(part.handle.value, dy, argmax, kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
+    _check((_calls or _load()).pool_adj(part._address, dy, argmax, kernel[0], kernel[1], stride[0], stride[1], pad[0][0],
                                         pad[0][1], pad[1][0], pad[1][1], mode, dx, stream, n, n if mode == POOL_MAX else 0, n))
 
 
@@ -511,7 +513,7 @@ def conv_adj_params_workspace(part, kh, kw):
 def conv_adj_params(part, x, dy, kernel, dw, db, workspace, stream=None):
     """dw [C, kh, kw] and db [C] (or None) of the adjoint convolution algorithm; workspace: a uint8 tensor."""
     n = part.num_workers
-    _check((_calls or _load()).conv_adj_params(part.handle.value, x, dy, kernel[0], kernel[1], dw, db, workspace,
+    _check((_calls or _load()).conv_adj_params(part._address, x, dy, kernel[0], kernel[1], dw, db, workspace,
                                                workspace.numel() * workspace.element_size(), stream, n, n))
 
 

@@ -360,6 +360,12 @@ def test_calls_check_their_arguments_before_the_library_sees_them():
         distdl.pool_fwd(conv, y, (3.5, 3), (1, 1), ((1, 1), (1, 1)), distdl.POOL_MAX, y, stream=0)
     with pytest.raises(ValueError):
         distdl.stencil3d_fwd(part, y, [[1, 2, 3], [1, 2, 3], [1, 2]], y, stream=0)
+    conv.close()
+    conv.close()
+    for call in (lambda: distdl.conv_fwd(conv, y, w_ptr, None, y, stream=0), lambda: distdl.halo_adj(conv, y, stream=0)):
+        with pytest.raises(distdl.DistdlError) as e:
+            call()
+        assert e.value.status == 1
     raw, radius = distdl._taps(np.arange(9).reshape(3, 3))
     assert radius == 1 and np.array_equal(np.frombuffer(raw, np.float32), np.arange(9, dtype=np.float32))
 
